@@ -1,5 +1,5 @@
 // eri_classes.cu -- instantiates the kernels of the canonical classes whose index is
-// congruent to ERI_TU modulo kNumTU, in the three arithmetic variants.  Compiled once per
+// congruent to ERI_TU modulo kNumTU, in the two arithmetic types.  Compiled once per
 // unit with -DERI_TU=<0..15> so the 55 canonical classes build in parallel.
 #include "eri_internal.h"
 #include "eri_kernels.cuh"
@@ -14,6 +14,22 @@
 
 namespace eri {
 
+template <class C>
+constexpr KernelInfo kernel_info() {
+    static_assert(C::SETUP_FIELDS * sizeof(typename C::R) <= kSetupFieldsMax * sizeof(double), "setup");
+    KernelInfo k{};
+    k.tpq = C::TPQ;
+    k.setup = C::USES_SETUP;
+    k.nrys = C::NRYS;
+    k.ltot = C::NAB + C::NCD;
+    k.sn = C::SN;
+    k.cb = C::DIRECT && C::Lb > 0 ? C::S_CB : 0;
+    k.cd = C::DIRECT && C::Ld > 0 ? C::S_CD : 0;
+    k.swab = C::SWAB_OK;
+    k.swcd = C::SWCD_OK;
+    return k;
+}
+
 template <int IDX>
 struct Register {
     static void apply(LaunchFn *table, KernelInfo *info) {
@@ -22,18 +38,12 @@ struct Register {
                 constexpr int cls = canonical_class(IDX);
                 constexpr int La = (cls >> 6) & 3, Lb = (cls >> 4) & 3, Lc = (cls >> 2) & 3,
                               Ld = cls & 3;
-                table[cls * kNumVariants + 0] = &launch_class<La, Lb, Lc, Ld, double, false>;
-                table[cls * kNumVariants + 1] = &launch_class<La, Lb, Lc, Ld, float, false>;
-                table[cls * kNumVariants + 2] = &launch_class<La, Lb, Lc, Ld, float, true>;
-                info[cls * kNumVariants + 0] = {Cfg<La, Lb, Lc, Ld, double>::TPQ,
-                                                 Cfg<La, Lb, Lc, Ld, double>::USES_SETUP};
-                info[cls * kNumVariants + 1] = {Cfg<La, Lb, Lc, Ld, float>::TPQ,
-                                                 Cfg<La, Lb, Lc, Ld, float>::USES_SETUP};
-                info[cls * kNumVariants + 2] = {false, false};  // contracted: fused kernels
-                // setup records fit the setup buffer (kSetupFieldsMax doubles per quartet)
-                static_assert(Cfg<La, Lb, Lc, Ld, double>::SETUP_FIELDS <= kSetupFieldsMax, "setup");
-                static_assert(Cfg<La, Lb, Lc, Ld, float>::SETUP_FIELDS * sizeof(float) <=
-                                  kSetupFieldsMax * sizeof(double), "setup");
+                table[cls * kNumVariants + 0] = &launch_class<La, Lb, Lc, Ld, double>;
+                table[cls * kNumVariants + 1] = &launch_class<La, Lb, Lc, Ld, float>;
+                table[cls * kNumVariants + 2] = &launch_class<La, Lb, Lc, Ld, float>;
+                info[cls * kNumVariants + 0] = kernel_info<Cfg<La, Lb, Lc, Ld, double>>();
+                info[cls * kNumVariants + 1] = kernel_info<Cfg<La, Lb, Lc, Ld, float>>();
+                info[cls * kNumVariants + 2] = kernel_info<Cfg<La, Lb, Lc, Ld, float>>();
             }
             Register<IDX + 1>::apply(table, info);
         }

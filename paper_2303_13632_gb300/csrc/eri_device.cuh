@@ -207,6 +207,7 @@ struct ClassArgs {
     const int4 *quartets;  // class-sorted shell ids, first quartet of the class
     long long nq;          // quartets of the class
     double *out_fp64;      // FP64 output of the class (null in compressed mode)
+    void *raw;             // values of primitive quartets in the recurrence type (then no other output)
     uint32_t *packed;      // first word of the class segment (null in FP64 mode)
     long long seg_words;   // words of the class segment (incl. zero padding)
     float *scales;         // eps of the class's first quartet
@@ -226,9 +227,7 @@ enum PairField { PR_P = 0, PR_IP, PR_PAX, PR_PAY, PR_PAZ, PR_KCN, kPairFields };
 // Launch options of a class kernel (see launch_class).
 struct LaunchOpts {
     int force_phase = 0;
-    unsigned long long *counter = nullptr;
-    int grid = 0;
-    int device = 0;
+    bool preset = false;      // the records are in ClassArgs::setup already
     void *scratch = nullptr;  // setup buffer for the split setup/recurrence path (K = 1)
 };
 

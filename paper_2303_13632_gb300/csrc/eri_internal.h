@@ -96,12 +96,40 @@ void eri_register_backward_3(BackwardFn *table, BackwardFn *table_mixed);
 
 // Each class translation unit fills table[cls * kNumVariants + variant] for its classes.
 constexpr int kNumTU = 16;
-// info[cls * kNumVariants + v] describes that launcher.
+// info[cls * kNumVariants + v] describes that launcher and the setup records its kernels read.
 struct KernelInfo {
     bool tpq;    // has a thread-per-quartet kernel (LaunchOpts::force_phase selects the other)
     bool setup;  // primitive (K = 1) plans run it through the setup kernel: the caller passes
                  // LaunchOpts::scratch and at most kSetupChunk quartets per launch
+    int nrys, ltot;   // roots, La + Lb + Lc + Ld
+    int sn;           // values per (quartet, root)
+    int cb, cd;       // slots of C00 on B and C00' on D (0: none)
+    bool swab, swcd;  // the VRR may be built on B (D)
 };
+constexpr int kSetupGeo = 8;  // AB, CD and the HRR directions, ahead of the per-root values
+
+// Contracted quartets (eri_contract.cu).  Every primitive quartet of the class is a unit: a setup
+// kernel writes the units' records, the class's recurrence kernel their values, and a last stage
+// sums the units of each quartet.
+struct UnitSpan {
+    const long long *ps;  // exclusive prefix sum of the primitive quartets of the plan's quartets,
+                          // at the class's first quartet (nq + 1 entries)
+    long long nq;         // quartets of the class
+    long long u0;         // first unit of the span (units are counted from the class's first)
+    int nu;               // units
+};
+// Primitive quartets of each of n quartets; out[n] = 0.
+cudaError_t unit_counts(const int4 *q, long long n, const int *nprim, long long *out, cudaStream_t s);
+// Records (layout of KernelInfo, field-major with `stride`) of the units of a span.
+cudaError_t unit_setup(const ShellsDev &sh, const Tables &tb, const ClassArgs &a, const KernelInfo &k,
+                       bool mixed, const UnitSpan &span, void *records, int stride, cudaStream_t s);
+// Sums of the units' values (values[unit - u0][n_ERIQ]) over each quartet, in unit order: FP32 with
+// Kahan compensation (mixed) or FP64; finished quartets go to a.out_fp64, or are left in the slot
+// of the quartet's first unit and compressed (Eqs. 9-10).  A quartet that the span cuts hands its
+// state to the next span through `carry` (4 n_ERIQ values, halves used in turn by `parity`).
+cudaError_t unit_contract(const ClassArgs &a, bool mixed, int neri, const UnitSpan &span, void *values,
+                          void *carry, int parity, cudaStream_t s);
+
 // One class of a plan's compressed output, as the Coulomb/exchange digestion reads it.
 struct DigestClass {
     int cls;               // generic class id

@@ -133,21 +133,19 @@ struct Cfg {
     static constexpr int NCH = cdiv(NB, BCH);
     static constexpr int ITEMS_D = NA * NC * NCH;
     // shared memory per quartet (bytes)
-    static constexpr int GEO_BYTES = G_N * 8;
     static constexpr int BC_BYTES = NRYS * SN * (int)sizeof(R);
     static constexpr int H_BYTES = (FUSE_BC || DIRECT) ? 0 : 3 * NRYS * HBLK * (int)sizeof(R);
     static constexpr int I_BYTES = 3 * NRYS * IBLKP * (int)sizeof(R);
     static constexpr int STAGE_BYTES = NERI * 3;  // worst case 24-bit codes
     static constexpr int UNION_BYTES = imax(H_BYTES + I_BYTES, STAGE_BYTES);
-    static constexpr int PERQ = GEO_BYTES + RG_N * (int)sizeof(R) + BC_BYTES + UNION_BYTES + 8;
+    static constexpr int PERQ = RG_N * (int)sizeof(R) + BC_BYTES + UNION_BYTES + 8;
     static constexpr int SMEM_BUDGET = 96 * 1024;
     static constexpr int QMAX_T = imax(1, 256 / ITEMS_D);
     static constexpr int QMAX_S = imax(1, SMEM_BUDGET / PERQ);
     static constexpr int Q = imin(128, imin(QMAX_T, QMAX_S));
     static constexpr int THREADS = imax(64, cdiv(Q * ITEMS_D, 32) * 32);
     // shared memory layout (byte offsets)
-    static constexpr int OFF_GEO = 0;
-    static constexpr int OFF_RG = OFF_GEO + Q * GEO_BYTES;
+    static constexpr int OFF_RG = 0;
     static constexpr int OFF_BC = ((OFF_RG + Q * RG_N * (int)sizeof(R) + 15) / 16) * 16;
     static constexpr int OFF_BMAX = ((OFF_BC + Q * BC_BYTES + 15) / 16) * 16;
     static constexpr int OFF_U = ((OFF_BMAX + Q * 8 + 15) / 16) * 16;
@@ -697,9 +695,23 @@ __device__ __forceinline__ void phase_direct(const typename C::R *bc, int mu, in
     }
 }
 
+// a b, with ROUND as a product the compiler must round before it enters a sum.  With one axis per
+// instantiation it knows that I(0, 0, 0, 0) is 1, turns fma(b10, 1, c * I) into b10 + c * I and fuses
+// that the other way round; the phase kernels, whose axis is a run-time value, round c * I.  The
+// units of contracted quartets keep that rounding, so that their codes do not depend on which
+// kernel form computes a class.
+template <bool ROUND, typename R>
+__device__ __forceinline__ R prod_r(R a, R b) {
+    if constexpr (ROUND && sizeof(R) == 4)
+        return __fmul_rn(a, b);
+    else
+        return a * b;
+}
+
 // VRR + bra HRR + ket HRR of one (root, axis) entirely in registers: I[(i, k, j, l)] in the
-// layout of i_index for fixed (xi, mu).  Used by the thread-per-quartet kernel.
-template <class C>
+// layout of i_index for fixed (xi, mu).  Used by the thread-per-quartet kernel.  ROUND: see
+// prod_r.
+template <class C, bool ROUND>
 __device__ __forceinline__ void axis_2d(const typename C::R *b, const typename C::R *rg, int xi,
                                         typename C::R (&I)[C::IBLK]) {
     using R = typename C::R;
@@ -711,7 +723,7 @@ __device__ __forceinline__ void axis_2d(const typename C::R *b, const typename C
     cur[0] = (xi == 2) ? b[S_WZ] : (R)1;
 #pragma unroll
     for (int i = 0; i < C::NAB; ++i)
-        cur[i + 1] = c00 * cur[i] + (i > 0 ? (R)i * b10 * cur[i - 1] : (R)0);
+        cur[i + 1] = c00 * cur[i] + (i > 0 ? prod_r<ROUND>((R)i * b10, cur[i - 1]) : (R)0);
 #pragma unroll
     for (int i = 0; i <= C::NAB; ++i) prev[i] = (R)0;
     R hk[C::La + 1][C::Lb + 1][C::NCD + 1];
@@ -727,7 +739,7 @@ __device__ __forceinline__ void axis_2d(const typename C::R *b, const typename C
             R nxt[C::NAB + 1];
 #pragma unroll
             for (int i = 0; i <= C::NAB; ++i) {
-                R v = c01 * cur[i];
+                R v = prod_r<ROUND>(c01, cur[i]);
                 if (k > 0) v = fma((R)k * b01, prev[i], v);
                 if (i > 0) v = fma((R)i * b00, cur[i - 1], v);
                 nxt[i] = v;
@@ -773,30 +785,21 @@ __device__ __forceinline__ void phase_ket(const typename C::R *rg, int mu, int x
         for (int l = 0; l <= C::Ld; ++l) Iq[i_index<C>(xi, mu, i, k, j, l)] = o[k][l];
 }
 
-// Phase D for b-chunk CH: acc[bb][d] (+)= sum_mu X[bx][dx] Y[by][dy] Z[bz][dz], where X, Y, Z
+// Phase D for b-chunk CH: acc[bb][d] = sum_mu X[bx][dx] Y[by][dy] Z[bz][dz], where X, Y, Z
 // are the (j, l) blocks of I at (i, k) = (a_xi, c_xi) for xi = x, y, z.
-template <class C, int CH, bool KAHAN>
+template <class C, int CH>
 __device__ __forceinline__ void quad_chunk(const typename C::R *Iq, int a, int c,
-                                           typename C::R (&acc)[C::BCH][C::ND],
-                                           typename C::R (&comp)[C::BCH][C::ND], bool first) {
+                                           typename C::R (&acc)[C::BCH][C::ND]) {
     using R = typename C::R;
     constexpr int B0 = CH * C::BCH;
     constexpr int NBC = imin(C::BCH, C::NB - B0);
     constexpr int LD1 = C::Ld + 1;
     const int ax = c_cart[C::La][a][0], ay = c_cart[C::La][a][1], az = c_cart[C::La][a][2];
     const int cx = c_cart[C::Lc][c][0], cy = c_cart[C::Lc][c][1], cz = c_cart[C::Lc][c][2];
-    R part[KAHAN ? C::BCH : 1][KAHAN ? C::ND : 1];
-    if constexpr (KAHAN) {
 #pragma unroll
-        for (int bb = 0; bb < C::BCH; ++bb)
+    for (int bb = 0; bb < C::BCH; ++bb)
 #pragma unroll
-            for (int d = 0; d < C::ND; ++d) part[bb][d] = (R)0;
-    } else if (first) {
-#pragma unroll
-        for (int bb = 0; bb < C::BCH; ++bb)
-#pragma unroll
-            for (int d = 0; d < C::ND; ++d) acc[bb][d] = (R)0;
-    }
+        for (int d = 0; d < C::ND; ++d) acc[bb][d] = (R)0;
     const R *px = Iq + i_index<C>(0, 0, ax, cx, 0, 0);
     const R *py = Iq + i_index<C>(1, 0, ay, cy, 0, 0);
     const R *pz = Iq + i_index<C>(2, 0, az, cz, 0, 0);
@@ -805,8 +808,6 @@ __device__ __forceinline__ void quad_chunk(const typename C::R *Iq, int a, int c
     for (int mu = 0; mu < C::NRYS; ++mu) {
 #pragma unroll
         for (int bb = 0; bb < NBC; ++bb) {
-            constexpr int dummy = 0;
-            (void)dummy;
             const int b = B0 + bb;
             const int bx = cart_x(C::Lb, b), by = cart_y(C::Lb, b), bz = cart_z(C::Lb, b);
             R X[LD1], Y[LD1], Z[LD1];
@@ -820,79 +821,56 @@ __device__ __forceinline__ void quad_chunk(const typename C::R *Iq, int a, int c
             for (int d = 0; d < C::ND; ++d) {
                 const int dx = cart_x(C::Ld, d), dy = cart_y(C::Ld, d), dz = cart_z(C::Ld, d);
                 R xy = X[dx] * Y[dy];
-                if constexpr (KAHAN)
-                    part[bb][d] = fma(xy, Z[dz], part[bb][d]);
-                else
-                    acc[bb][d] = fma(xy, Z[dz], acc[bb][d]);
+                acc[bb][d] = fma(xy, Z[dz], acc[bb][d]);
             }
         }
         px += MU_STRIDE;
         py += MU_STRIDE;
         pz += MU_STRIDE;
     }
-    if constexpr (KAHAN) {
-#pragma unroll
-        for (int bb = 0; bb < C::BCH; ++bb)
-#pragma unroll
-            for (int d = 0; d < C::ND; ++d) {
-                if (first) {
-                    acc[bb][d] = part[bb][d];
-                    comp[bb][d] = (R)0;
-                } else {
-                    // Kahan-compensated sum over primitive quartets
-                    R y = part[bb][d] - comp[bb][d];
-                    R t = acc[bb][d] + y;
-                    comp[bb][d] = (t - acc[bb][d]) - y;
-                    acc[bb][d] = t;
-                }
-            }
-    }
 }
 
-template <class C, bool KAHAN>
+template <class C>
 __device__ __forceinline__ void quad_dispatch(int ch, const typename C::R *Iq, int a, int c,
-                                              typename C::R (&acc)[C::BCH][C::ND],
-                                              typename C::R (&comp)[C::BCH][C::ND], bool first) {
+                                              typename C::R (&acc)[C::BCH][C::ND]) {
     if constexpr (C::NCH == 1) {
-        quad_chunk<C, 0, KAHAN>(Iq, a, c, acc, comp, first);
+        quad_chunk<C, 0>(Iq, a, c, acc);
     } else {
         switch (ch) {
-            case 0: quad_chunk<C, 0, KAHAN>(Iq, a, c, acc, comp, first); break;
-            case 1: if constexpr (C::NCH > 1) quad_chunk<C, 1, KAHAN>(Iq, a, c, acc, comp, first); break;
-            case 2: if constexpr (C::NCH > 2) quad_chunk<C, 2, KAHAN>(Iq, a, c, acc, comp, first); break;
-            case 3: if constexpr (C::NCH > 3) quad_chunk<C, 3, KAHAN>(Iq, a, c, acc, comp, first); break;
-            case 4: if constexpr (C::NCH > 4) quad_chunk<C, 4, KAHAN>(Iq, a, c, acc, comp, first); break;
-            case 5: if constexpr (C::NCH > 5) quad_chunk<C, 5, KAHAN>(Iq, a, c, acc, comp, first); break;
-            case 6: if constexpr (C::NCH > 6) quad_chunk<C, 6, KAHAN>(Iq, a, c, acc, comp, first); break;
-            case 7: if constexpr (C::NCH > 7) quad_chunk<C, 7, KAHAN>(Iq, a, c, acc, comp, first); break;
-            case 8: if constexpr (C::NCH > 8) quad_chunk<C, 8, KAHAN>(Iq, a, c, acc, comp, first); break;
-            case 9: if constexpr (C::NCH > 9) quad_chunk<C, 9, KAHAN>(Iq, a, c, acc, comp, first); break;
+            case 0: quad_chunk<C, 0>(Iq, a, c, acc); break;
+            case 1: if constexpr (C::NCH > 1) quad_chunk<C, 1>(Iq, a, c, acc); break;
+            case 2: if constexpr (C::NCH > 2) quad_chunk<C, 2>(Iq, a, c, acc); break;
+            case 3: if constexpr (C::NCH > 3) quad_chunk<C, 3>(Iq, a, c, acc); break;
+            case 4: if constexpr (C::NCH > 4) quad_chunk<C, 4>(Iq, a, c, acc); break;
+            case 5: if constexpr (C::NCH > 5) quad_chunk<C, 5>(Iq, a, c, acc); break;
+            case 6: if constexpr (C::NCH > 6) quad_chunk<C, 6>(Iq, a, c, acc); break;
+            case 7: if constexpr (C::NCH > 7) quad_chunk<C, 7>(Iq, a, c, acc); break;
+            case 8: if constexpr (C::NCH > 8) quad_chunk<C, 8>(Iq, a, c, acc); break;
+            case 9: if constexpr (C::NCH > 9) quad_chunk<C, 9>(Iq, a, c, acc); break;
             default: break;
         }
     }
 }
 
 // ---------------------------------------------------------------------------------------
-// One tile of Q quartets (tile index `tile`) of the phase kernel.  PRESET: phases A0/A1 were
-// done by eri_setup_kernel and their results are read from args.setup.
-template <class C, bool KAHAN, bool PRESET = false>
-__device__ __forceinline__ void class_tile(const ShellsDev &sh, const Tables &tb,
-                                           const ClassArgs &args, long long tile,
-                                           unsigned char *smem) {
+// One tile of Q quartets (tile index `tile`) of the phase kernel; the setup stage (phases A0 and
+// A1) was done by a setup kernel and its records are read from args.setup.  With args.raw the
+// "quartets" are primitive quartets whose values are stored as they are, to be summed over the
+// primitives afterwards (eri_contract.cu).
+template <class C>
+__device__ __forceinline__ void class_tile(const ClassArgs &args, long long tile, unsigned char *smem) {
     using R = typename C::R;
-    double *geo_s = reinterpret_cast<double *>(smem + C::OFF_GEO);
     R *rg_s = reinterpret_cast<R *>(smem + C::OFF_RG);
     R *bc_s = reinterpret_cast<R *>(smem + C::OFF_BC);
     unsigned long long *bmax_s = reinterpret_cast<unsigned long long *>(smem + C::OFF_BMAX);
     R *H_s = reinterpret_cast<R *>(smem + C::OFF_H);
     R *I_s = reinterpret_cast<R *>(smem + C::OFF_I);
-    __shared__ int maxprim_s;
 
     const int tid = threadIdx.x;
     const long long q0 = tile * C::Q;
     const int qn = (int)((args.nq - q0) < C::Q ? (args.nq - q0) : C::Q);
 
-    // phase D item of this thread (fixed across primitive iterations)
+    // phase D item of this thread
     const bool has_item = tid < C::Q * C::ITEMS_D;
     int dq = 0, da = 0, dc = 0, dch = 0;
     if (has_item) {
@@ -903,109 +881,68 @@ __device__ __forceinline__ void class_tile(const ShellsDev &sh, const Tables &tb
         dch = r % C::NCH;
     }
     R acc[C::BCH][C::ND];
-    R comp[C::BCH][C::ND];  // Kahan compensation; eliminated when KAHAN is false
-
-    if (tid == 0) maxprim_s = 1;
+    {
+        // setup values of the tile, field-major in the setup buffer (coalesced loads)
+        const R *su = reinterpret_cast<const R *>(args.setup) + q0;
+        const int ss = (int)args.setup_stride;  // <= 2^20: 32-bit offsets
+        for (int it = tid; it < C::Q * C::SETUP_GEO; it += C::THREADS) {
+            int f = it / C::Q, q = it % C::Q;
+            rg_s[q * RG_N + f] = q < qn ? su[f * ss + q] : (R)0;
+        }
+        for (int it = tid; it < C::Q * C::NRYS * C::SN; it += C::THREADS) {
+            int f = it / C::Q, q = it % C::Q;
+            bc_s[q * C::NRYS * C::SN + f] = q < qn ? su[(C::SETUP_GEO + f) * ss + q] : (R)0;
+        }
+    }
     __syncthreads();
-    for (int prim = 0; prim < maxprim_s; ++prim) {
-        if constexpr (PRESET) {
-            // setup values of the tile, field-major in the setup buffer (coalesced loads)
-            const R *su = reinterpret_cast<const R *>(args.setup) + q0;
-            const int ss = (int)args.setup_stride;  // <= 2^20: 32-bit offsets
-            for (int it = tid; it < C::Q * C::SETUP_GEO; it += C::THREADS) {
-                int f = it / C::Q, q = it % C::Q;
-                rg_s[q * RG_N + f] = q < qn ? su[f * ss + q] : (R)0;
-            }
-            for (int it = tid; it < C::Q * C::NRYS * C::SN; it += C::THREADS) {
-                int f = it / C::Q, q = it % C::Q;
-                bc_s[q * C::NRYS * C::SN + f] = q < qn ? su[(C::SETUP_GEO + f) * ss + q] : (R)0;
-            }
-            __syncthreads();
-        } else {
-            // A0: geometry per quartet (canonical shell order)
-            for (int q = tid; q < C::Q; q += C::THREADS) {
-                int np = 0;
-                double *geo = geo_s + q * G_N;
-                if (q < qn) {
-                    int4 g = args.quartets[q0 + q];
-                    int4 qt = make_int4(pick(g, args.perm[0]), pick(g, args.perm[1]),
-                                        pick(g, args.perm[2]), pick(g, args.perm[3]));
-                    geometry_of<C>(sh, args, qt, prim, geo, np);
-                } else {
-                    geo[G_PREF] = 0.0;
-                    geo[G_T] = 0.0;
-                    for (int s = G_P; s < G_N; ++s)
-                        geo[s] = (s == G_P || s == G_Q || s == G_IP || s == G_IQ) ? 1.0
-                                                                                  : (s == G_IPQ ? 0.5 : 0.0);
-                }
-                if (prim == 0 && np > 1) atomicMax(&maxprim_s, np);
-                R *rg = rg_s + q * RG_N;
-                rg[RG_ABX] = to_r<R>(geo[G_ABX]);
-                rg[RG_ABY] = to_r<R>(geo[G_ABY]);
-                rg[RG_ABZ] = to_r<R>(geo[G_ABZ]);
-                rg[RG_CDX] = to_r<R>(geo[G_CDX]);
-                rg[RG_CDY] = to_r<R>(geo[G_CDY]);
-                rg[RG_CDZ] = to_r<R>(geo[G_CDZ]);
-                rg[RG_SWAB] = to_r<R>(geo[G_SWAB]);
-                rg[RG_SWCD] = to_r<R>(geo[G_SWCD]);
-            }
-            __syncthreads();
-            // A1: roots, weights, B and C per (quartet, root).  For primitive plans (no Kahan
-            // sums) the mixed path forms B and C in two-float FP32 exactly as the split path's
-            // setup kernel does (the persistent form of those plans then matches the per-class
-            // launches bit for bit); contracted plans keep the FP64 formation, cheaper per item
-            for (int it = tid; it < C::Q * C::NRYS; it += C::THREADS) {
-                int q = it / C::NRYS, mu = it % C::NRYS;
-                if constexpr (sizeof(R) == 4 && !KAHAN) {
-                    const double *geo = geo_s + q * G_N;
-                    SetupTF<C> pre;
-                    pre.init(geo);
-                    double x, w;
-                    root_mixed<C>(tb, geo[G_T], mu, x, w);
-                    pre.root(x, w, bc_s + (q * C::NRYS + mu) * C::SN);
-                } else {
-                    phase_setup<C>(tb, geo_s + q * G_N, mu, bc_s + (q * C::NRYS + mu) * C::SN);
-                }
-            }
-            __syncthreads();
+    // B: VRR (+ bra HRR, + ket HRR when fused), or the four-index recursion, per
+    // (quartet, root, axis)
+    for (int it = tid; it < C::Q * C::NRYS * 3; it += C::THREADS) {
+        int q = it / (C::NRYS * 3), r = it % (C::NRYS * 3);
+        int mu = r / 3, xi = r % 3;
+        if constexpr (C::DIRECT)
+            phase_direct<C>(bc_s + q * C::NRYS * C::SN, mu, xi,
+                            I_s + (size_t)q * (C::I_BYTES / sizeof(R)));
+        else
+            phase_vrr<C>(bc_s + q * C::NRYS * C::SN, rg_s + q * RG_N, mu, xi,
+                         H_s + (size_t)q * (C::H_BYTES / sizeof(R)),
+                         I_s + (size_t)q * (C::I_BYTES / sizeof(R)));
+    }
+    __syncthreads();
+    if constexpr (!C::FUSE_BC && !C::DIRECT) {
+        constexpr int NIJ = (C::La + 1) * (C::Lb + 1);
+        for (int it = tid; it < C::Q * C::NRYS * 3 * NIJ; it += C::THREADS) {
+            int q = it / (C::NRYS * 3 * NIJ), r = it % (C::NRYS * 3 * NIJ);
+            int mu = r / (3 * NIJ);
+            r %= 3 * NIJ;
+            int xi = r / NIJ, ij = r % NIJ;
+            phase_ket<C>(rg_s + q * RG_N, mu, xi, ij / (C::Lb + 1), ij % (C::Lb + 1),
+                         H_s + (size_t)q * (C::H_BYTES / sizeof(R)),
+                         I_s + (size_t)q * (C::I_BYTES / sizeof(R)));
         }
-        // B: VRR (+ bra HRR, + ket HRR when fused), or the four-index recursion, per
-        // (quartet, root, axis)
-        for (int it = tid; it < C::Q * C::NRYS * 3; it += C::THREADS) {
-            int q = it / (C::NRYS * 3), r = it % (C::NRYS * 3);
-            int mu = r / 3, xi = r % 3;
-            if constexpr (C::DIRECT)
-                phase_direct<C>(bc_s + q * C::NRYS * C::SN, mu, xi,
-                                I_s + (size_t)q * (C::I_BYTES / sizeof(R)));
-            else
-                phase_vrr<C>(bc_s + q * C::NRYS * C::SN, rg_s + q * RG_N, mu, xi,
-                             H_s + (size_t)q * (C::H_BYTES / sizeof(R)),
-                             I_s + (size_t)q * (C::I_BYTES / sizeof(R)));
-        }
-        __syncthreads();
-        if constexpr (!C::FUSE_BC && !C::DIRECT) {
-            constexpr int NIJ = (C::La + 1) * (C::Lb + 1);
-            for (int it = tid; it < C::Q * C::NRYS * 3 * NIJ; it += C::THREADS) {
-                int q = it / (C::NRYS * 3 * NIJ), r = it % (C::NRYS * 3 * NIJ);
-                int mu = r / (3 * NIJ);
-                r %= 3 * NIJ;
-                int xi = r / NIJ, ij = r % NIJ;
-                phase_ket<C>(rg_s + q * RG_N, mu, xi, ij / (C::Lb + 1), ij % (C::Lb + 1),
-                             H_s + (size_t)q * (C::H_BYTES / sizeof(R)),
-                             I_s + (size_t)q * (C::I_BYTES / sizeof(R)));
-            }
-            __syncthreads();
-        }
-        // D: quadrature into register accumulators
-        if (has_item)
-            quad_dispatch<C, KAHAN>(dch, I_s + (size_t)dq * (C::I_BYTES / sizeof(R)), da, dc, acc,
-                                    comp, prim == 0);
         __syncthreads();
     }
-
+    // D: quadrature into register accumulators
+    if (has_item)
+        quad_dispatch<C>(dch, I_s + (size_t)dq * (C::I_BYTES / sizeof(R)), da, dc, acc);
+    __syncthreads();
     const bool live = has_item && dq < qn;
     const int st0 = args.ostride[0], st1 = args.ostride[1], st2 = args.ostride[2],
               st3 = args.ostride[3];
+    if (args.raw != nullptr) {
+        if (live) {
+            R *o = reinterpret_cast<R *>(args.raw) + (q0 + dq) * (long long)C::NERI + da * st0 + dc * st2;
+#pragma unroll
+            for (int bb = 0; bb < C::BCH; ++bb) {
+                int b = dch * C::BCH + bb;
+                if (b < C::NB) {
+#pragma unroll
+                    for (int d = 0; d < C::ND; ++d) o[b * st1 + d * st3] = acc[bb][d];
+                }
+            }
+        }
+        return;
+    }
     if (args.out_fp64 != nullptr) {
         // FP64 output in the generic class's row-major order
         if (live) {
@@ -1146,11 +1083,11 @@ __device__ __forceinline__ void class_tile(const ShellsDev &sh, const Tables &tb
     }
 }
 
-template <class C, bool KAHAN, bool PRESET = false>
+template <class C>
 __global__ void __launch_bounds__(C::THREADS)
-eri_class_kernel(ShellsDev sh, Tables tb, ClassArgs args) {
+eri_class_kernel(ClassArgs args) {
     extern __shared__ __align__(16) unsigned char smem[];
-    class_tile<C, KAHAN, PRESET>(sh, tb, args, blockIdx.x, smem);
+    class_tile<C>(args, blockIdx.x, smem);
 }
 
 // Setup stage of the split path (primitive quartets, K = 1): one thread per quartet computes
@@ -1202,28 +1139,9 @@ eri_setup_kernel(ShellsDev sh, Tables tb, ClassArgs args, typename C::R *out, lo
     }
 }
 
-// Persistent form: a grid sized to the resident CTAs pulls tiles from a work counter
-// (atomicAdd, no waiting) until the class is exhausted; quartets of uneven contraction
-// degree therefore balance dynamically.  The counter must be zero at launch.
-template <class C, bool KAHAN>
-__global__ void __launch_bounds__(C::THREADS)
-eri_class_persistent(ShellsDev sh, Tables tb, ClassArgs args, unsigned long long *counter) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ long long tile_s;
-    const long long n_tiles = (args.nq + C::Q - 1) / C::Q;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) tile_s = (long long)atomicAdd(counter, 1ull);
-        __syncthreads();
-        const long long t = tile_s;
-        if (t >= n_tiles) break;
-        class_tile<C, KAHAN>(sh, tb, args, t, smem);
-    }
-}
-
 // The four-index recursion of phase_direct for one (root, axis) in registers, in the layout of
 // axis_2d (I[((i * (Lc+1) + k) * (Lb+1) + j) * (Ld+1) + l]); thread-per-quartet kernels.
-template <class C>
+template <class C, bool ROUND>
 __device__ __forceinline__ void axis_direct(const typename C::R *b, int xi,
                                             typename C::R (&I)[C::IBLK]) {
     using R = typename C::R;
@@ -1237,7 +1155,7 @@ __device__ __forceinline__ void axis_direct(const typename C::R *b, int xi,
     I[0] = (xi == 2) ? b[S_WZ] : (R)1;
 #pragma unroll
     for (int i = 1; i <= C::La; ++i) {
-        R v = cA * I[ERI_IX(i - 1, 0, 0, 0)];
+        R v = prod_r<ROUND>(cA, I[ERI_IX(i - 1, 0, 0, 0)]);
         if (i > 1) v = fma((R)(i - 1) * b10, I[ERI_IX(i - 2, 0, 0, 0)], v);
         I[ERI_IX(i, 0, 0, 0)] = v;
     }
@@ -1245,7 +1163,7 @@ __device__ __forceinline__ void axis_direct(const typename C::R *b, int xi,
     for (int j = 1; j <= C::Lb; ++j)
 #pragma unroll
         for (int i = 0; i <= C::La; ++i) {
-            R v = cB * I[ERI_IX(i, 0, j - 1, 0)];
+            R v = prod_r<ROUND>(cB, I[ERI_IX(i, 0, j - 1, 0)]);
             if (j > 1) v = fma((R)(j - 1) * b10, I[ERI_IX(i, 0, j - 2, 0)], v);
             if (i > 0) v = fma((R)i * b10, I[ERI_IX(i - 1, 0, j - 1, 0)], v);
             I[ERI_IX(i, 0, j, 0)] = v;
@@ -1256,7 +1174,7 @@ __device__ __forceinline__ void axis_direct(const typename C::R *b, int xi,
         for (int i = 0; i <= C::La; ++i)
 #pragma unroll
             for (int j = 0; j <= C::Lb; ++j) {
-                R v = cC * I[ERI_IX(i, k - 1, j, 0)];
+                R v = prod_r<ROUND>(cC, I[ERI_IX(i, k - 1, j, 0)]);
                 if (k > 1) v = fma((R)(k - 1) * b01, I[ERI_IX(i, k - 2, j, 0)], v);
                 if (i > 0) v = fma((R)i * b00, I[ERI_IX(i - 1, k - 1, j, 0)], v);
                 if (j > 0) v = fma((R)j * b00, I[ERI_IX(i, k - 1, j - 1, 0)], v);
@@ -1270,7 +1188,7 @@ __device__ __forceinline__ void axis_direct(const typename C::R *b, int xi,
             for (int i = 0; i <= C::La; ++i)
 #pragma unroll
                 for (int j = 0; j <= C::Lb; ++j) {
-                    R v = cD * I[ERI_IX(i, k, j, l - 1)];
+                    R v = prod_r<ROUND>(cD, I[ERI_IX(i, k, j, l - 1)]);
                     if (l > 1) v = fma((R)(l - 1) * b01, I[ERI_IX(i, k, j, l - 2)], v);
                     if (k > 0) v = fma((R)k * b01, I[ERI_IX(i, k - 1, j, l - 1)], v);
                     if (i > 0) v = fma((R)i * b00, I[ERI_IX(i - 1, k, j, l - 1)], v);
@@ -1287,19 +1205,19 @@ __device__ __forceinline__ void axis_direct(const typename C::R *b, int xi,
 // PRESET: the geometry and per-root setup come from the setup kernel's records (FP32 only).
 
 // 2-D integrals of one root and the quadrature (Eq. 8) into the thread's accumulators.
-template <class C>
+template <class C, bool ROUND>
 __device__ __forceinline__ void tpq_root(const typename C::R *bc, const typename C::R *rg,
                                          typename C::R (&acc)[C::NERI]) {
     using R = typename C::R;
     R X[C::IBLK], Y[C::IBLK], Z[C::IBLK];
     if constexpr (C::DIRECT) {
-        axis_direct<C>(bc, 0, X);
-        axis_direct<C>(bc, 1, Y);
-        axis_direct<C>(bc, 2, Z);
+        axis_direct<C, ROUND>(bc, 0, X);
+        axis_direct<C, ROUND>(bc, 1, Y);
+        axis_direct<C, ROUND>(bc, 2, Z);
     } else {
-        axis_2d<C>(bc, rg, 0, X);
-        axis_2d<C>(bc, rg, 1, Y);
-        axis_2d<C>(bc, rg, 2, Z);
+        axis_2d<C, ROUND>(bc, rg, 0, X);
+        axis_2d<C, ROUND>(bc, rg, 1, Y);
+        axis_2d<C, ROUND>(bc, rg, 2, Z);
     }
 #pragma unroll
     for (int a = 0; a < C::NA; ++a)
@@ -1318,7 +1236,11 @@ __device__ __forceinline__ void tpq_root(const typename C::R *bc, const typename
                 }
 }
 
-template <class C, bool PRESET = false>
+// Form of the thread-per-quartet kernel: setup inline, from the setup kernel's records, or over the
+// units of contracted quartets (records in, values out in R).
+enum TpqForm { TPQ_INLINE = 0, TPQ_PRESET, TPQ_UNITS };
+
+template <class C, int FORM>
 __device__ __forceinline__ void tpq_tile(const ShellsDev &sh, const Tables &tb,
                                          const ClassArgs &args, long long tile,
                                          unsigned char *smem) {
@@ -1331,7 +1253,7 @@ __device__ __forceinline__ void tpq_tile(const ShellsDev &sh, const Tables &tb,
 #pragma unroll
     for (int o = 0; o < C::NERI; ++o) acc[o] = (R)0;
     if (live) {
-        if constexpr (PRESET) {
+        if constexpr (FORM != TPQ_INLINE) {
             // field-major setup records: consecutive threads read consecutive words
             const R *su = reinterpret_cast<const R *>(args.setup) + (q0 + tid);
             const int ss = (int)args.setup_stride;  // <= 2^20: 32-bit offsets
@@ -1343,7 +1265,7 @@ __device__ __forceinline__ void tpq_tile(const ShellsDev &sh, const Tables &tb,
                 R bc[C::SN];
 #pragma unroll
                 for (int f = 0; f < C::SN; ++f) bc[f] = su[(C::SETUP_GEO + mu * C::SN + f) * ss];
-                tpq_root<C>(bc, rg, acc);
+                tpq_root<C, FORM == TPQ_UNITS>(bc, rg, acc);
             }
         } else {
             int4 g = args.quartets[q0 + tid];
@@ -1370,14 +1292,14 @@ __device__ __forceinline__ void tpq_tile(const ShellsDev &sh, const Tables &tb,
                         root_mixed<C>(tb, geo[G_T], mu, x, w);
                         R bc[C::SN];
                         pre.root(x, w, bc);
-                        tpq_root<C>(bc, rg, acc);
+                        tpq_root<C, false>(bc, rg, acc);
                     }
                 } else {
 #pragma unroll 1
                     for (int mu = 0; mu < C::NRYS; ++mu) {
                         R bc[C::SN];
                         phase_setup<C>(tb, geo, mu, bc);
-                        tpq_root<C>(bc, rg, acc);
+                        tpq_root<C, false>(bc, rg, acc);
                     }
                 }
             }
@@ -1385,6 +1307,22 @@ __device__ __forceinline__ void tpq_tile(const ShellsDev &sh, const Tables &tb,
     }
     const int st0 = args.ostride[0], st1 = args.ostride[1], st2 = args.ostride[2],
               st3 = args.ostride[3];
+    if constexpr (FORM == TPQ_UNITS) {
+        if (live) {
+            R *out = reinterpret_cast<R *>(args.raw) + (q0 + tid) * (long long)C::NERI;
+#pragma unroll
+            for (int a = 0; a < C::NA; ++a)
+#pragma unroll
+                for (int b = 0; b < C::NB; ++b)
+#pragma unroll
+                    for (int c = 0; c < C::NC; ++c)
+#pragma unroll
+                        for (int d = 0; d < C::ND; ++d)
+                            out[a * st0 + b * st1 + c * st2 + d * st3] =
+                                acc[((a * C::NB + b) * C::NC + c) * C::ND + d];
+        }
+        return;
+    }
     if (args.out_fp64 != nullptr) {
         if (live) {
             double *out = args.out_fp64 + (q0 + tid) * (long long)C::NERI;
@@ -1490,120 +1428,62 @@ __device__ __forceinline__ void tpq_tile(const ShellsDev &sh, const Tables &tb,
     }
 }
 
-template <class C, bool PRESET = false>
+template <class C, int FORM>
 __global__ void __launch_bounds__(C::TPQ_THREADS, C::TPQ_MINB)
 eri_tpq_kernel(ShellsDev sh, Tables tb, ClassArgs args) {
     extern __shared__ __align__(16) unsigned char smem[];
-    tpq_tile<C, PRESET>(sh, tb, args, blockIdx.x, smem);
+    tpq_tile<C, FORM>(sh, tb, args, blockIdx.x, smem);
 }
 
-template <class C>
-__global__ void __launch_bounds__(C::TPQ_THREADS, C::TPQ_MINB)
-eri_tpq_persistent(ShellsDev sh, Tables tb, ClassArgs args, unsigned long long *counter) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ long long tile_s;
-    const long long n_tiles = (args.nq + C::TPQ_THREADS - 1) / C::TPQ_THREADS;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) tile_s = (long long)atomicAdd(counter, 1ull);
-        __syncthreads();
-        const long long t = tile_s;
-        if (t >= n_tiles) break;
-        tpq_tile<C>(sh, tb, args, t, smem);
-    }
-}
-
-// Host-side launch helper for one canonical class.
+// Host-side launch helper for one canonical class in one arithmetic type.  Without o.preset:
+// primitive (K = 1) quartets, through the setup kernel and o.scratch where the class uses it.
+// With o.preset: only the recurrence/quadrature kernel, over args.nq records of args.setup.
 //   o.force_phase  use the shared-memory phase kernel even where the thread-per-quartet
 //                  kernel exists (autotuning)
-//   o.counter      non-null: persistent launch pulling tiles from this zeroed counter with
-//                  o.grid CTAs (o.grid <= 0: every resident CTA, from the occupancy API)
-template <int La, int Lb, int Lc, int Ld, typename R, bool KAHAN>
+template <int La, int Lb, int Lc, int Ld, typename R>
 cudaError_t launch_class(const ShellsDev &sh, const Tables &tb, const ClassArgs &args,
                          cudaStream_t stream, const LaunchOpts &o) {
     using C = Cfg<La, Lb, Lc, Ld, R>;
     if (args.nq <= 0) return cudaSuccess;
-    int sms = 0;
-    if (o.counter) {
-        cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, o.device);
+    if (args.nq > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const bool tpq = C::TPQ && !o.force_phase;
+    ClassArgs a = args;
+    if constexpr (C::TPQ_SMALL) {
+        if (tpq && !o.preset) {
+            size_t smem = args.out_fp64 ? 0 : ((size_t)C::TPQ_THREADS * C::NERI * args.bits + 31) / 32 * 4 + 16;
+            const unsigned tiles = (unsigned)((args.nq + C::TPQ_THREADS - 1) / C::TPQ_THREADS);
+            eri_tpq_kernel<C, TPQ_INLINE><<<tiles, C::TPQ_THREADS, smem, stream>>>(sh, tb, args);
+            return cudaGetLastError();
+        }
+    }
+    if (!o.preset) {
+        // FP64 setup kernel, then the recurrence/quadrature kernel
+        if (!o.scratch) return cudaErrorInvalidValue;
+        a.setup = o.scratch;
+        a.setup_stride = (args.nq + 31) / 32 * 32;
+        eri_setup_kernel<C><<<(unsigned)((args.nq + 127) / 128), 128, 0, stream>>>(
+            sh, tb, args, reinterpret_cast<R *>(o.scratch), a.setup_stride);
+        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    if constexpr (C::TPQ && !KAHAN) {
-        if (!o.force_phase) {
-            size_t smem = 0;
-            if (args.out_fp64 == nullptr)
-                smem = ((size_t)C::TPQ_THREADS * C::NERI * args.bits + 31) / 32 * 4 + 16;
-            long long tiles = (args.nq + C::TPQ_THREADS - 1) / C::TPQ_THREADS;
-            if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-            if (!o.counter) {
-                if constexpr (C::TPQ_SPLIT) {
-                    if (o.scratch) {
-                        // FP64 setup kernel, then the FP32 thread-per-quartet kernel
-                        const long long stride = (args.nq + 31) / 32 * 32;
-                        eri_setup_kernel<C><<<(unsigned)((args.nq + 127) / 128), 128, 0, stream>>>(
-                            sh, tb, args, reinterpret_cast<R *>(o.scratch), stride);
-                        cudaError_t e = cudaGetLastError();
-                        if (e != cudaSuccess) return e;
-                        ClassArgs a2 = args;
-                        a2.setup = o.scratch;
-                        a2.setup_stride = stride;
-                        eri_tpq_kernel<C, true><<<(unsigned)tiles, C::TPQ_THREADS, smem, stream>>>(sh, tb, a2);
-                        return cudaGetLastError();
-                    }
-                }
-                eri_tpq_kernel<C><<<(unsigned)tiles, C::TPQ_THREADS, smem, stream>>>(sh, tb, args);
+    if constexpr (C::TPQ) {
+        if (tpq) {
+            const unsigned tiles = (unsigned)((args.nq + C::TPQ_THREADS - 1) / C::TPQ_THREADS);
+            if (args.raw) {
+                eri_tpq_kernel<C, TPQ_UNITS><<<tiles, C::TPQ_THREADS, 0, stream>>>(sh, tb, a);
                 return cudaGetLastError();
             }
-            int per_sm = 0;
-            cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &per_sm, eri_tpq_persistent<C>, C::TPQ_THREADS, smem);
-            if (e != cudaSuccess) return e;
-            long long grid = o.grid > 0 ? o.grid : (long long)per_sm * sms;
-            grid = grid < tiles ? grid : tiles;
-            eri_tpq_persistent<C><<<(unsigned)grid, C::TPQ_THREADS, smem, stream>>>(sh, tb, args,
-                                                                                     o.counter);
-            return cudaGetLastError();
+            if constexpr (C::TPQ_SPLIT) {
+                size_t smem = args.out_fp64 ? 0 : ((size_t)C::TPQ_THREADS * C::NERI * args.bits + 31) / 32 * 4 + 16;
+                eri_tpq_kernel<C, TPQ_PRESET><<<tiles, C::TPQ_THREADS, smem, stream>>>(sh, tb, a);
+                return cudaGetLastError();
+            }
         }
     }
-    if constexpr (!KAHAN) {
-        if (o.scratch && !o.counter) {
-            // split path: FP64 setup kernel, then the recurrence/quadrature kernel
-            long long blocks = (args.nq + 127) / 128;
-            if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-            const long long stride = (args.nq + 31) / 32 * 32;
-            eri_setup_kernel<C><<<(unsigned)blocks, 128, 0, stream>>>(
-                sh, tb, args, reinterpret_cast<R *>(o.scratch), stride);
-            cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            ClassArgs a2 = args;
-            a2.setup = o.scratch;
-            a2.setup_stride = stride;
-            auto k2 = eri_class_kernel<C, false, true>;
-            e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-            if (e != cudaSuccess) return e;
-            long long tiles = (args.nq + C::Q - 1) / C::Q;
-            k2<<<(unsigned)tiles, C::THREADS, C::SMEM, stream>>>(sh, tb, a2);
-            return cudaGetLastError();
-        }
-    }
-    auto kern = eri_class_kernel<C, KAHAN>;
-    auto pkern = eri_class_persistent<C, KAHAN>;
-    cudaError_t e = cudaFuncSetAttribute(o.counter ? (const void *)pkern : (const void *)kern,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    auto k2 = eri_class_kernel<C>;
+    cudaError_t e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
-    long long tiles = (args.nq + C::Q - 1) / C::Q;
-    if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    if (!o.counter) {
-        kern<<<(unsigned)tiles, C::THREADS, C::SMEM, stream>>>(sh, tb, args);
-        return cudaGetLastError();
-    }
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pkern, C::THREADS, C::SMEM);
-    if (e != cudaSuccess) return e;
-    long long grid = o.grid > 0 ? o.grid : (long long)per_sm * sms;
-    grid = grid < tiles ? grid : tiles;
-    if (grid < 1) grid = 1;
-    pkern<<<(unsigned)grid, C::THREADS, C::SMEM, stream>>>(sh, tb, args, o.counter);
+    k2<<<(unsigned)((args.nq + C::Q - 1) / C::Q), C::THREADS, C::SMEM, stream>>>(a);
     return cudaGetLastError();
 }
 

@@ -168,8 +168,6 @@ extern "C" eri_status_t eri_compute_class_noalloc(int32_t cls, int32_t precision
     std::call_once(g_table_once, fill_table);
     DeviceState *st = nullptr;
     if (device_state(&st) != cudaSuccess) return ERI_E_CUDA;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return ERI_E_CUDA;
     ClassArgs a{};
     int ccls = 0;
     canonical(cls, a.perm, a.ostride, &ccls);
@@ -186,7 +184,6 @@ extern "C" eri_status_t eri_compute_class_noalloc(int32_t cls, int32_t precision
     if (cudaGetLastError() != cudaSuccess) return ERI_E_CUDA;
     ShellsDev sh{d_cx, d_cy, d_cz, d_pofs, d_nprim, d_exps, d_cn};
     LaunchOpts o;
-    o.device = dev;
     o.scratch = st->scratch;
     return fn(sh, st->tables, a, s, o) == cudaSuccess ? ERI_OK : ERI_E_CUDA;
 }

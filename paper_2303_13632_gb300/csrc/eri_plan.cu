@@ -2,6 +2,7 @@
 // normalisation (Sec. II-A), device-side stable sort of quartets by class, the output
 // layouts, and the per-class kernel launches.
 #include <cub/device/device_radix_sort.cuh>
+#include <cub/device/device_scan.cuh>
 
 #include <algorithm>
 #include <cmath>
@@ -221,9 +222,13 @@ struct eri_plan_s {
     double *d_pairs = nullptr;    // primitive-pair table (n_prims^2 records), or null
     int *d_prim_shell = nullptr;  // shell of every primitive (with the pair table)
     std::vector<int> h_L, h_nprim;  // per shell, for eri_plan_update_shells
-    // batched form: tile counters of the persistent kernels (scratch), streams, graph cache
-    unsigned long long *d_counters = nullptr;
-    static constexpr int kSide = 4;
+    // contracted plans: prefix sum of the sorted quartets' primitive quartets (nq + 1 entries), the
+    // primitive quartets of each class, and the partial sums of quartets cut between two spans
+    long long *d_pstart = nullptr;
+    long long units[kNumClassIds] = {0};
+    void *d_carry = nullptr;
+    // side streams over which the classes of a call are spread, and the graph of the batched form
+    static constexpr int kSide = 8;
     cudaStream_t side[kSide] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[kSide] = {};
     // streamed copies to the host: copy stream and one event per class
@@ -237,9 +242,8 @@ struct eri_plan_s {
     // per-class precision (-1: the plan's) and the calibrated mixed-path error per class
     int class_prec[kNumClassIds];
     float class_err[kNumClassIds];
-    // autotuned launch choice per canonical class and variant (grid 0 = all resident CTAs)
+    // autotuned launch choice per canonical class and variant
     int tune_phase[256 * kNumVariants] = {0};
-    int tune_grid[256 * kNumVariants] = {0};
     // host layout
     long long count[kNumClassIds] = {0};
     long long first[kNumClassIds] = {0};
@@ -268,7 +272,8 @@ void free_plan(eri_plan_s *p) {
     cudaFree(p->d_setup);
     cudaFree(p->d_pairs);
     cudaFree(p->d_prim_shell);
-    cudaFree(p->d_counters);
+    cudaFree(p->d_pstart);
+    cudaFree(p->d_carry);
     if (p->graph) cudaGraphExecDestroy(p->graph);
     for (int i = 0; i < eri_plan_s::kSide; ++i) {
         if (p->side[i]) cudaStreamDestroy(p->side[i]);
@@ -438,16 +443,83 @@ ClassArgs class_args(eri_plan_s *p, int cls, double *d_out, int bits, void *d_pa
     return a;
 }
 
+// values of one quartet's partial sums carried between two spans: two halves, FP64 or FP32 with
+// the Kahan compensation, of at most 10000 outputs
+constexpr size_t kCarryBytes = 2 * 10000 * sizeof(double);
+
+// Share of the plan's scratch that a launch may use: slice `index` of `count` equal ones (classes
+// on different streams use different slices).
+struct Slice {
+    int index = 0, count = 1;
+};
+
+bool is_contracted(const eri_plan_s *p) { return p->max_nprim > 1; }
+
+// units of a span of class cls with `bytes` of scratch: a record and n_ERIQ values each
+int span_units(const KernelInfo &k, int neri, bool mixed, size_t bytes) {
+    const size_t per = (size_t)(kSetupGeo + k.nrys * k.sn + neri) * (mixed ? sizeof(float) : sizeof(double));
+    return (int)(std::min<size_t>(kSetupChunk, bytes / per) / 32 * 32);
+}
+
+// A contracted class: spans of primitive quartets through the setup, class and contraction kernels
+// (eri_contract.cu).  q_first: the class position of a.quartets.
+eri_status_t launch_contracted(eri_plan_s *p, int cls, const ClassArgs &a, int variant, long long q_first,
+                               Slice sl, int force_phase, cudaStream_t stream) {
+    const int cc = canonicalise(cls).cls, k = cc * kNumVariants + variant, neri = class_neri(cls);
+    const KernelInfo &info = g_info[k];
+    const bool mixed = variant != 0;
+    UnitSpan span{};
+    span.ps = p->d_pstart + p->first[cls] + q_first;
+    span.nq = a.nq;
+    long long total = p->units[cls];
+    if (q_first != 0 || a.nq != p->count[cls]) {  // part of a class (plan-time calls only)
+        long long ends[2];
+        cudaError_t e = cudaMemcpyAsync(&ends[0], span.ps, sizeof(long long), cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&ends[1], span.ps + a.nq, sizeof(long long), cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) return cuda_status(e);
+        total = ends[1] - ends[0];
+    }
+    const size_t bytes = kScratchBytes / sl.count / 256 * 256;
+    char *records = static_cast<char *>(p->d_setup) + sl.index * bytes;
+    char *carry = static_cast<char *>(p->d_carry) + sl.index * kCarryBytes;
+    const int cap = span_units(info, neri, mixed, bytes);
+    ShellsDev sh{p->d_cx, p->d_cy, p->d_cz, p->d_pofs, p->d_nprim, p->d_exps, p->d_cn};
+    const size_t rec_bytes = (size_t)(kSetupGeo + info.nrys * info.sn) * (mixed ? sizeof(float) : sizeof(double));
+    int parity = 0;
+    for (span.u0 = 0; span.u0 < total; span.u0 += cap, parity ^= 1) {
+        span.nu = (int)std::min<long long>(cap, total - span.u0);
+        cudaError_t e = unit_setup(sh, p->tables, a, info, mixed, span, records, cap, stream);
+        if (e != cudaSuccess) return cuda_status(e);
+        ClassArgs au = a;
+        au.nq = span.nu;
+        au.setup = records;
+        au.setup_stride = cap;
+        au.raw = records + (size_t)cap * rec_bytes;
+        LaunchOpts o;
+        o.preset = true;
+        o.force_phase = force_phase;
+        e = g_launch[k](sh, p->tables, au, stream, o);
+        if (e == cudaSuccess) e = unit_contract(a, mixed, neri, span, au.raw, carry, parity, stream);
+        if (e != cudaSuccess) return cuda_status(e);
+    }
+    return ERI_OK;
+}
+
 // Launches the kernels of generic class cls with prepared arguments `a` (its quartets, count
 // and output) in precision variant `variant`; primitive plans run the split setup/recurrence
 // path in chunks of kSetupChunk quartets where the class has no thread-per-quartet form.
+// q_first: the class position of a.quartets; `sl`: the scratch the launches may use.
 eri_status_t launch_class_args(eri_plan_s *p, int cls, const ClassArgs &a, int variant,
-                               cudaStream_t stream) {
+                               cudaStream_t stream, long long q_first = 0, Slice sl = Slice(),
+                               int force_phase = 0) {
     if (a.nq == 0) return ERI_OK;
     Canon c = canonicalise(cls);
     ShellsDev sh{p->d_cx, p->d_cy, p->d_cz, p->d_pofs, p->d_nprim, p->d_exps, p->d_cn};
     const int neri = class_neri(cls);
     const int bits = a.bits;
+    const size_t slice_bytes = kScratchBytes / sl.count / 256 * 256;
     if (class_has_g(c.cls)) {
         int L[4];
         class_ls(c.cls, L);
@@ -455,25 +527,27 @@ eri_status_t launch_class_args(eri_plan_s *p, int cls, const ClassArgs &a, int v
             cudaError_t e = ensure_scratch(p);
             if (e != cudaSuccess) return cuda_status(e);
         }
-        return cuda_status(launch_generic(sh, p->tables, a, L, variant != 0, static_cast<double *>(p->d_setup),
-                                          kScratchBytes, stream));
+        return cuda_status(launch_generic(sh, p->tables, a, L, variant != 0,
+                                          reinterpret_cast<double *>(static_cast<char *>(p->d_setup) + sl.index * slice_bytes),
+                                          slice_bytes, stream));
     }
     LaunchFn fn = g_launch[c.cls * kNumVariants + variant];
     if (!fn) return ERI_E_UNSUPPORTED;
+    if (is_contracted(p)) return launch_contracted(p, cls, a, variant, q_first, sl, force_phase, stream);
     LaunchOpts o;
-    o.device = p->device;
-    const bool split = p->max_nprim == 1 && g_info[c.cls * kNumVariants + variant].setup;
-    if (!split) return cuda_status(fn(sh, p->tables, a, stream, o));
+    o.force_phase = force_phase;
+    if (!g_info[c.cls * kNumVariants + variant].setup && !force_phase) return cuda_status(fn(sh, p->tables, a, stream, o));
     {
         cudaError_t e = ensure_scratch(p);
         if (e != cudaSuccess) return cuda_status(e);
     }
-    o.scratch = p->d_setup;
-    // chunks of kSetupChunk quartets (multiples of 32: every chunk starts on a packed word)
-    for (long long c0 = 0; c0 < a.nq; c0 += kSetupChunk) {
+    o.scratch = static_cast<char *>(p->d_setup) + sl.index * slice_bytes;
+    // chunks that fit the scratch (multiples of 32: every chunk starts on a packed word)
+    const long long chunk = kSetupChunk / sl.count / 32 * 32;
+    for (long long c0 = 0; c0 < a.nq; c0 += chunk) {
         ClassArgs ac = a;
         ac.quartets = a.quartets + c0;
-        ac.nq = std::min<long long>(kSetupChunk, a.nq - c0);
+        ac.nq = std::min<long long>(chunk, a.nq - c0);
         if (a.out_fp64) {
             ac.out_fp64 = a.out_fp64 + c0 * neri;
         } else {
@@ -526,7 +600,7 @@ eri_status_t schwarz_factors(const eri_shell_t *shells, int n_shells, int device
             a.quartets += c0;
             a.nq = std::min(chunk, sp->count[c] - c0);
             a.out_fp64 = buf;
-            st = launch_class_args(sp, c, a, 0, nullptr);
+            st = launch_class_args(sp, c, a, 0, nullptr, c0);
             if (st == ERI_OK) e = screen_absmax_sqrt(buf, a.nq, neri, Qs + sp->first[c] + c0, nullptr);
             if (e != cudaSuccess) st = cuda_status(e);
         }
@@ -552,12 +626,45 @@ eri_status_t launch_one(eri_plan_s *p, int cls, double *d_out, int bits, void *d
     return launch_class_args(p, cls, a, class_variant(p, cls), stream);
 }
 
-eri_status_t ensure_batched_resources(eri_plan_s *p) {
+eri_status_t ensure_side_streams(eri_plan_s *p);
+
+// What the compute calls of a contracted plan need: the prefix sum of the primitive quartets, the
+// scratch, the carried sums and the side streams.  Called once the class layout is known.
+eri_status_t prepare_contracted(eri_plan_s *p) {
+    const long long n = p->nq;
+    long long *d_counts = nullptr;
+    void *d_tmp = nullptr;
+    size_t tmp = 0;
+    cudaError_t e = plan_malloc(&d_counts, (n + 1) * sizeof(long long));
+    if (e == cudaSuccess) e = plan_malloc(&p->d_pstart, (n + 1) * sizeof(long long));
+    if (e == cudaSuccess) e = plan_malloc(&p->d_setup, kScratchBytes);
+    if (e == cudaSuccess) e = plan_malloc(&p->d_carry, eri_plan_s::kSide * kCarryBytes);
+    if (e == cudaSuccess) e = unit_counts(p->d_quartets, n, p->d_nprim, d_counts, nullptr);
+    if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(nullptr, tmp, d_counts, p->d_pstart, n + 1);
+    if (e == cudaSuccess) e = plan_malloc(&d_tmp, std::max<size_t>(tmp, 1));
+    if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(d_tmp, tmp, d_counts, p->d_pstart, n + 1);
+    for (int c = 0; e == cudaSuccess && c < kNumClassIds; ++c)
+        if (p->count[c] > 0)
+            e = cudaMemcpyAsync(&p->units[c], p->d_pstart + p->first[c] + p->count[c], sizeof(long long),
+                                cudaMemcpyDeviceToHost, nullptr);
+    const cudaError_t se = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = se;
+    cudaFree(d_counts);
+    cudaFree(d_tmp);
+    if (e != cudaSuccess) return cuda_status(e);
+    long long before = 0;  // the copies hold the prefix at each class's end
+    for (int c = 0; c < kNumClassIds; ++c)
+        if (p->count[c] > 0) {
+            const long long end = p->units[c];
+            p->units[c] = end - before;
+            before = end;
+        }
+    return ensure_side_streams(p);
+}
+
+// side streams and events
+eri_status_t ensure_side_streams(eri_plan_s *p) {
     cudaError_t e = cudaSuccess;
-    if (!p->d_counters) e = cudaMalloc(&p->d_counters, 256 * sizeof(unsigned long long));
-    bool has_g = false;
-    for (int c = 256; c < kNumClassIds; ++c) has_g |= p->count[c] > 0;
-    if (e == cudaSuccess && has_g) e = ensure_scratch(p);  // before any stream capture
     for (int i = 0; e == cudaSuccess && i < eri_plan_s::kSide; ++i) {
         if (!p->side[i]) e = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking);
         if (e == cudaSuccess && !p->join_ev[i])
@@ -567,12 +674,12 @@ eri_status_t ensure_batched_resources(eri_plan_s *p) {
     return cuda_status(e);
 }
 
-// Persistent launches of every non-empty class on the plan's side streams (forked from and
-// joined back into `stream`); the classes go to the side streams by decreasing quartet count.
-eri_status_t enqueue_batched(eri_plan_s *p, int bits, void *d_packed, float *d_scales,
-                             cudaStream_t stream) {
-    cudaError_t e = cudaMemsetAsync(p->d_counters, 0, 256 * sizeof(unsigned long long), stream);
-    if (e == cudaSuccess) e = cudaEventRecord(p->fork_ev, stream);
+// Every non-empty class on the plan's side streams (forked from and joined back into `stream`),
+// each with its slice of the scratch; the classes go to the side streams by decreasing work.
+// d_out: FP64 output, else compressed.  tuned: with the kernel choices of eri_autotune.
+eri_status_t enqueue_forked(eri_plan_s *p, double *d_out, int bits, void *d_packed, float *d_scales,
+                            bool tuned, cudaStream_t stream) {
+    cudaError_t e = cudaEventRecord(p->fork_ev, stream);
     for (int i = 0; e == cudaSuccess && i < eri_plan_s::kSide; ++i)
         e = cudaStreamWaitEvent(p->side[i], p->fork_ev, 0);
     if (e != cudaSuccess) return cuda_status(e);
@@ -581,41 +688,27 @@ eri_status_t enqueue_batched(eri_plan_s *p, int bits, void *d_packed, float *d_s
     size_t o = 0;
     for (int c = 0; c < kNumClassIds; ++c) {
         off[c] = o;
-        o += packed_segment_bytes(p->count[c], class_neri(c), bits);
+        if (!d_out) o += packed_segment_bytes(p->count[c], class_neri(c), bits);
         if (p->count[c] > 0) cls.push_back(c);
     }
-    std::sort(cls.begin(), cls.end(), [&](int x, int y) {
-        return p->count[x] * class_neri(x) > p->count[y] * class_neri(y);
-    });
-    ShellsDev sh{p->d_cx, p->d_cy, p->d_cz, p->d_pofs, p->d_nprim, p->d_exps, p->d_cn};
-    for (size_t i = 0; i < cls.size(); ++i) {
-        int c = cls[i];
-        int cc = canonicalise(c).cls;
-        const int variant = class_variant(p, c);
-        if (class_has_g(cc)) {
-            // plain launches of the run-time-L kernels; all on the first side stream, since
-            // they share the plan's scratch
-            ClassArgs a = class_args(p, c, nullptr, bits, d_packed, d_scales, off[c]);
-            eri_status_t st = launch_class_args(p, c, a, variant, p->side[0]);
-            if (st != ERI_OK) return st;
-            continue;
-        }
-        LaunchFn fn = g_launch[cc * kNumVariants + variant];
-        if (!fn) return ERI_E_UNSUPPORTED;
-        ClassArgs a = class_args(p, c, nullptr, bits, d_packed, d_scales, off[c]);
-        LaunchOpts lo;
-        lo.device = p->device;
-        lo.counter = p->d_counters + c;
-        lo.force_phase = p->tune_phase[cc * kNumVariants + variant];
-        lo.grid = p->tune_grid[cc * kNumVariants + variant];
-        e = fn(sh, p->tables, a, p->side[i % eri_plan_s::kSide], lo);
-        if (e != cudaSuccess) return cuda_status(e);
+    auto work = [&](int c) {
+        return (is_contracted(p) && !class_has_g(c) ? p->units[c] : p->count[c]) * class_neri(c);
+    };
+    std::sort(cls.begin(), cls.end(), [&](int x, int y) { return work(x) > work(y); });
+    eri_status_t st = ERI_OK;
+    for (size_t i = 0; i < cls.size() && st == ERI_OK; ++i) {
+        const int c = cls[i], s = (int)(i % eri_plan_s::kSide), variant = class_variant(p, c);
+        ClassArgs a = class_args(p, c, d_out, bits, d_packed, d_scales, off[c]);
+        const int phase = tuned && !class_has_g(c) ? p->tune_phase[canonicalise(c).cls * kNumVariants + variant] : 0;
+        st = launch_class_args(p, c, a, variant, p->side[s], 0, Slice{s, eri_plan_s::kSide}, phase);
     }
-    for (int i = 0; e == cudaSuccess && i < eri_plan_s::kSide; ++i) {
-        e = cudaEventRecord(p->join_ev[i], p->side[i]);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, p->join_ev[i], 0);
+    // joined also after an error: the side streams' work stays ordered before the caller's
+    for (int i = 0; i < eri_plan_s::kSide; ++i) {
+        cudaError_t je = cudaEventRecord(p->join_ev[i], p->side[i]);
+        if (je == cudaSuccess) je = cudaStreamWaitEvent(stream, p->join_ev[i], 0);
+        if (e == cudaSuccess) e = je;
     }
-    return cuda_status(e);
+    return st != ERI_OK ? st : cuda_status(e);
 }
 
 }  // namespace
@@ -880,6 +973,14 @@ eri_status_t eri_plan_create(const eri_shell_t *shells, int32_t n_shells, const 
         f += p->count[c];
         off += p->count[c] * neri;
     }
+    if (is_contracted(p) && p->nq > 0) {
+        // the compute calls of a contracted plan allocate nothing (they may be captured)
+        eri_status_t st = prepare_contracted(p);
+        if (st != ERI_OK) {
+            free_plan(p);
+            return st;
+        }
+    }
     *out = p;
     return ERI_OK;
 }
@@ -1055,6 +1156,8 @@ eri_status_t eri_compute(eri_plan_t plan, double *d_out, void *stream) {
     if (!plan || (!d_out && plan->nq > 0)) return ERI_E_INVALID;
     if (reinterpret_cast<uintptr_t>(d_out) % 8) return ERI_E_INVALID;
     cudaSetDevice(plan->device);
+    if (is_contracted(plan) && plan->nq > 0)
+        return enqueue_forked(plan, d_out, 0, nullptr, nullptr, false, (cudaStream_t)stream);
     for (int c = 0; c < kNumClassIds; ++c) {
         eri_status_t s = launch_one(plan, c, d_out, 0, nullptr, nullptr, 0, (cudaStream_t)stream);
         if (s != ERI_OK) return s;
@@ -1081,6 +1184,8 @@ eri_status_t eri_compute_compressed(eri_plan_t plan, int32_t bits, void *d_packe
     if (reinterpret_cast<uintptr_t>(d_packed) % 4 || reinterpret_cast<uintptr_t>(d_scales) % 4)
         return ERI_E_INVALID;
     cudaSetDevice(plan->device);
+    if (is_contracted(plan) && plan->nq > 0)
+        return enqueue_forked(plan, nullptr, bits, d_packed, d_scales, false, (cudaStream_t)stream);
     size_t off = 0;
     for (int c = 0; c < kNumClassIds; ++c) {
         const int neri = class_neri(c);
@@ -1185,7 +1290,8 @@ eri_status_t eri_compute_compressed_batched(eri_plan_t plan, int32_t bits, void 
         return ERI_E_INVALID;
     if (plan->nq == 0) return ERI_OK;
     cudaSetDevice(plan->device);
-    eri_status_t st = ensure_batched_resources(plan);
+    eri_status_t st = ensure_side_streams(plan);
+    if (st == ERI_OK) st = cuda_status(ensure_scratch(plan));  // before the capture
     if (st != ERI_OK) return st;
     if (!plan->graph || plan->g_bits != bits || plan->g_prec != plan->precision ||
         plan->g_packed != d_packed || plan->g_scales != d_scales) {
@@ -1202,7 +1308,7 @@ eri_status_t eri_compute_compressed_batched(eri_plan_t plan, int32_t bits, void 
             cudaStreamDestroy(origin);
             return cuda_status(e);
         }
-        st = enqueue_batched(plan, bits, d_packed, d_scales, origin);
+        st = enqueue_forked(plan, nullptr, bits, d_packed, d_scales, true, origin);
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(origin, &g);
         cudaStreamDestroy(origin);
@@ -1263,7 +1369,7 @@ eri_status_t eri_autotune(eri_plan_t plan, int32_t bits, void *d_packed, float *
     if (!plan || bits < 2 || bits > 24) return ERI_E_INVALID;
     if (plan->nq > 0 && (!d_packed || !d_scales)) return ERI_E_INVALID;
     cudaSetDevice(plan->device);
-    eri_status_t st = ensure_batched_resources(plan);
+    eri_status_t st = cuda_status(ensure_scratch(plan));
     if (st != ERI_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
     cudaDeviceProp prop;
@@ -1280,7 +1386,6 @@ eri_status_t eri_autotune(eri_plan_t plan, int32_t bits, void *d_packed, float *
             while (std::fscanf(f, "%255s %d %d %d %d %d", name, &v, &b, &c, &fp, &gr) == 6)
                 if (gpu == name && v >= 0 && v < kNumVariants && b == bits && c >= 0 && c < 256) {
                     plan->tune_phase[c * kNumVariants + v] = fp;
-                    plan->tune_grid[c * kNumVariants + v] = gr;
                     known[c * kNumVariants + v] = 1;
                 }
             std::fclose(f);
@@ -1289,7 +1394,6 @@ eri_status_t eri_autotune(eri_plan_t plan, int32_t bits, void *d_packed, float *
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    ShellsDev sh{plan->d_cx, plan->d_cy, plan->d_cz, plan->d_pofs, plan->d_nprim, plan->d_exps, plan->d_cn};
     std::vector<std::string> lines;
     size_t o = 0;
     std::vector<size_t> off(kNumClassIds);
@@ -1304,43 +1408,32 @@ eri_status_t eri_autotune(eri_plan_t plan, int32_t bits, void *d_packed, float *
         const int variant = class_variant(plan, c);
         if (known[cc * kNumVariants + variant] || done[cc * kNumVariants + variant]) continue;
         done[cc * kNumVariants + variant] = 1;
-        LaunchFn fn = g_launch[cc * kNumVariants + variant];
         ClassArgs a = class_args(plan, c, nullptr, bits, d_packed, d_scales, off[c]);
-        int cand_phase[2] = {0, 1};
-        int n_phase = g_info[cc * kNumVariants + variant].tpq ? 2 : 1;
-        int grids[3] = {0, prop.multiProcessorCount, 2 * prop.multiProcessorCount};
+        const int n_phase = g_info[cc * kNumVariants + variant].tpq ? 2 : 1;
         float best = 1e30f;
-        int bp = 0, bg = 0;
-        for (int ip = 0; ip < n_phase; ++ip)
-            for (int ig = 0; ig < 3; ++ig) {
-                LaunchOpts lo;
-                lo.device = plan->device;
-                lo.counter = plan->d_counters + c;
-                lo.force_phase = n_phase == 2 ? cand_phase[ip] : 0;
-                lo.grid = grids[ig];
-                float ms = 0.0f;
-                for (int rep = 0; rep < 2; ++rep) {  // first run warms up
-                    cudaMemsetAsync(plan->d_counters + c, 0, sizeof(unsigned long long), s);
-                    cudaEventRecord(e0, s);
-                    if (fn(sh, plan->tables, a, s, lo) != cudaSuccess) {
-                        cudaEventDestroy(e0);
-                        cudaEventDestroy(e1);
-                        return ERI_E_CUDA;
-                    }
-                    cudaEventRecord(e1, s);
-                    cudaEventSynchronize(e1);
-                    cudaEventElapsedTime(&ms, e0, e1);
+        int bp = 0;
+        for (int ip = 0; ip < n_phase; ++ip) {
+            float ms = 0.0f;
+            for (int rep = 0; rep < 2; ++rep) {  // first run warms up
+                cudaEventRecord(e0, s);
+                st = launch_class_args(plan, c, a, variant, s, 0, Slice(), ip);
+                if (st != ERI_OK) {
+                    cudaEventDestroy(e0);
+                    cudaEventDestroy(e1);
+                    return st;
                 }
-                if (ms < best) {
-                    best = ms;
-                    bp = lo.force_phase;
-                    bg = lo.grid;
-                }
+                cudaEventRecord(e1, s);
+                cudaEventSynchronize(e1);
+                cudaEventElapsedTime(&ms, e0, e1);
             }
+            if (ms < best) {
+                best = ms;
+                bp = ip;
+            }
+        }
         plan->tune_phase[cc * kNumVariants + variant] = bp;
-        plan->tune_grid[cc * kNumVariants + variant] = bg;
         char buf[512];
-        std::snprintf(buf, sizeof(buf), "%s %d %d %d %d %d\n", gpu.c_str(), variant, bits, cc, bp, bg);
+        std::snprintf(buf, sizeof(buf), "%s %d %d %d %d %d\n", gpu.c_str(), variant, bits, cc, bp, 0);
         lines.push_back(buf);
     }
     cudaEventDestroy(e0);
@@ -1371,21 +1464,20 @@ eri_status_t eri_plan_class_kernels(eri_plan_t plan, int32_t cls, char *buf, siz
     }
     const int k = c.cls * kNumVariants + v;
     if (!g_launch[k]) return ERI_E_UNSUPPORTED;
-    const bool split = plan->max_nprim == 1 && g_info[k].setup;
-    const bool tpq = g_info[k].tpq && v != 2;
     char cfg[64];
     std::snprintf(cfg, sizeof(cfg), "Cfg<%d, %d, %d, %d, %s>", (c.cls >> 6) & 3, (c.cls >> 4) & 3,
                   (c.cls >> 2) & 3, c.cls & 3, v == 0 ? "double" : "float");
     // the launch choice of launch_class (eri_kernels.cuh) for a per-class call
+    const bool units = is_contracted(plan);
     std::string name;
-    if (tpq && split)
-        name = std::string("eri_setup_kernel<") + cfg + "> + eri_tpq_kernel<" + cfg + ", 1>";
-    else if (tpq)
-        name = std::string("eri_tpq_kernel<") + cfg + ", 0>";
-    else if (split)
-        name = std::string("eri_setup_kernel<") + cfg + "> + eri_class_kernel<" + cfg + ", 0, 1>";
+    if (g_info[k].tpq)
+        name = std::string("eri_tpq_kernel<") + cfg + (units ? ", 2>" : (g_info[k].setup ? ", 1>" : ", 0>"));
     else
-        name = std::string("eri_class_kernel<") + cfg + (v == 2 ? ", 1, 0>" : ", 0, 0>");
+        name = std::string("eri_class_kernel<") + cfg + ">";
+    if (units)
+        name = "unit_setup_kernel + " + name + " + contract_kernel + pack_kernel";
+    else if (g_info[k].setup)
+        name = std::string("eri_setup_kernel<") + cfg + "> + " + name;
     if (name.size() + 1 > len) return ERI_E_INVALID;
     std::memcpy(buf, name.c_str(), name.size() + 1);
     return ERI_OK;
@@ -1402,8 +1494,12 @@ eri_status_t eri_plan_class_launches(eri_plan_t plan, int32_t cls, int32_t *n_la
     }
     const int k = canonicalise(cls).cls * kNumVariants + v;
     if (!g_launch[k]) return ERI_E_UNSUPPORTED;
-    const bool split = plan->max_nprim == 1 && g_info[k].setup;
-    *n_launches = split ? 2 * (int32_t)((plan->count[cls] + kSetupChunk - 1) / kSetupChunk) : 1;
+    if (is_contracted(plan)) {
+        const long long cap = span_units(g_info[k], class_neri(cls), v != 0, kScratchBytes);
+        *n_launches = 4 * (int32_t)((plan->units[cls] + cap - 1) / cap);
+    } else {
+        *n_launches = g_info[k].setup ? 2 * (int32_t)((plan->count[cls] + kSetupChunk - 1) / kSetupChunk) : 1;
+    }
     return ERI_OK;
 }
 
