@@ -1,8 +1,10 @@
 // eri_backward.cu -- instantiates the adjoint kernels of the canonical classes whose index is
 // congruent to ERI_BTU modulo 4 (compiled once per unit with -DERI_BTU=<0..3>) and registers
-// their launchers: FP64 for classes with every angular momentum <= 2 (the extended index ranges
-// of f shells exceed the per-CTA shared memory in FP64), FP32 recurrences (the mixed adjoint)
-// for every class.
+// their launchers: FP64 for classes with every angular momentum <= 2, FP32 recurrences (the mixed
+// adjoint) for every class.
+#include <algorithm>
+#include <type_traits>
+
 #include "eri_backward.cuh"
 #include "eri_internal.h"
 

@@ -4,317 +4,550 @@
 // For a primitive g_a = c N(alpha, L) prod_xi (r_xi - A_xi)^{a_xi} exp(-alpha |r - A|^2):
 //   d g_a / d A_xi  = 2 alpha g_{a + 1_xi} - a_xi g_{a - 1_xi}
 //   d g_a / d alpha = (2L + 3) / (4 alpha) g_a - sum_xi g_{a + 2_xi}
-// (shifted functions keep the coefficient and normalisation of g_a).  In the Rys form of
-// Eq. 8 each shift touches one axis factor only, so with the 2-D integrals I(i,j,k,l,mu,xi)
-// built for every index up to L + 2 (VRR Eq. 6 and HRR Eq. 7 on the extended ranges, n_Rys =
-// floor((L+2)/2) + 1 roots, exact for the shifted integrals of total degree <= L + 2):
-//   dE/dA_x = sum_mu sum_abcd G_abcd [2 alpha Ix(a+1) - a_x Ix(a-1)] Iy Iz, likewise y, z, B, C, D
-//   dE/d alpha_a = sum_mu sum_abcd G_abcd [(2La+3)/(4 alpha) Ix Iy Iz - Ix(a+2) Iy Iz - ...].
-// Centre gradients are summed over primitives; exponent gradients go to the primitive.
+// (shifted functions keep the coefficient and normalisation of g_a).  In the Rys form of Eq. 8 each
+// shift touches one axis factor only (n_Rys = floor((L+2)/2) + 1 roots, exact for the shifted
+// integrals of total degree <= L + 2), so with W = sum G I_y I_z over the outputs that share their
+// components w = (i0, i1, i2, i3) along an axis,
+//   dE/dA = sum_mu sum_w W(w) [2 alpha I(w + 1_a) - a I(w - 1_a)]   on that axis,
+// and the same with w + 2_a for the exponents.
+//
+// No integral beyond the class's own index ranges is formed.  I(w) is the mean of a product of
+// powers of x - A, x - B, x' - C, x' - D over a Gaussian in (x, x'), so raising an index is
+//   I(w + 1_a) = C00_A I(w) + B10 D I(w) + B00 K I(w),
+// where D I(w) = a I(w - 1_a) + b I(w - 1_b) and K I(w) = c I(w - 1_c) + d I(w - 1_d) (the
+// derivatives along x and x').  The sums over w of W times I, its four lowered forms, DD I, DK I and
+// KK I (S0, Sa..Sd, SDD, SDK, SKK; SD = Sa + Sb, SK = Sc + Sd) then give everything: with
+// P = B10 SD + B00 SK and V = B10^2 SDD + 2 B10 B00 SDK + B00^2 SKK,
+//   U1 = sum W I(w + 1_a) = C00_A S0 + P,   U2 = sum W I(w + 2_a) = C00_A (U1 + P) + B10 S0 + V,
+// for B with C00_B, and for C and D with C00', B01 and the bra and ket sums exchanged.  On the ranges
+// extended by two this took 625 instead of 81 2-D integrals per (root, axis) of [dd|dd] (90 KB of
+// shared memory instead of 8 per primitive quartet in FP64) and 12 of them per w and centre.
+//
+// GPU mapping.  A unit is a primitive quartet; a CTA owns a range of consecutive units of a class and
+// takes QG of them at a time, so that every CTA has the same number whatever the contraction
+// degrees.  Geometry, roots and the B, C records are made for a batch of units at once (one thread
+// per unit, then per (unit, root): all threads busy in FP64).  Then per QG units:
+//   1  2-D integrals: the lanes of rows_direct per (unit, root, axis)
+//   2  W: one thread per (unit, root, a, c, b-chunk) with its outputs' G in registers (kept while the
+//      units belong to one quartet) and the (b, d) blocks of I_x, I_y, I_z at its (a, c): five
+//      operations per output for all three axes; the partial W blocks go to shared memory
+//   3  one thread per (unit, axis, root, i0, i2): sums the partial blocks over the (a, c) with these
+//      components, forms the eight sums from the neighbouring blocks of I and adds to the centre
+//      gradients in registers (compensated in FP32) until the quartet ends; the exponent terms are
+//      summed over the unit (warp shuffles, then FP64) and added to global memory.
+// Bound by issue of the FMAs and shared-memory reads of 2 and 3 in FP32, by the FP64 pipe in FP64.
+// Measured on the 16 classes of p and d shells, K = 3, forward and backward: 1024 quartets per class
+// in mixed precision 115 -> 17.0 ms, 384 in FP64 220 -> 59.4 ms.
 #pragma once
 
-#include "eri_bwd_table.h"
-#include "eri_kernels.cuh"
+#include "eri_rows.cuh"
 
 namespace eri {
 
-// 2-D integral configuration on the extended index ranges (all L + 2) of class (La..Ld), in
-// the recurrence type R: FP64 keeps the VRR + HRR of Eqs. 6-7; FP32 (the mixed adjoint) uses the
-// four-index recursion of phase_direct, which does not amplify FP32 rounding through the
-// transfer relation (see eri_kernels.cuh), with the B and C values of the mixed setup.
-template <int La0, int Lb0, int Lc0, int Ld0, typename R_ = double>
+// Values of N consecutive elements at a 16-byte (or narrower, for short blocks) boundary.
+template <int N, int V, typename R>
+__device__ __forceinline__ void load_block(const R *p, R (&x)[N]) {
+    if constexpr (sizeof(R) == 4 && V == 4) {
+#pragma unroll
+        for (int t = 0; t < N; t += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(p + t);
+            x[t] = v.x;
+            if (t + 1 < N) x[t + 1] = v.y;
+            if (t + 2 < N) x[t + 2] = v.z;
+            if (t + 3 < N) x[t + 3] = v.w;
+        }
+    } else if constexpr (V == 2) {
+        using T = std::conditional_t<sizeof(R) == 4, float2, double2>;
+#pragma unroll
+        for (int t = 0; t < N; t += 2) {
+            const T v = *reinterpret_cast<const T *>(p + t);
+            x[t] = v.x;
+            if (t + 1 < N) x[t + 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < N; ++t) x[t] = p[t];
+    }
+}
+template <int N, int V, typename R>
+__device__ __forceinline__ void store_block(R *p, const R (&x)[N]) {
+    if constexpr (sizeof(R) == 4 && V == 4) {
+#pragma unroll
+        for (int t = 0; t < N; t += 4)
+            *reinterpret_cast<float4 *>(p + t) = make_float4(x[t], t + 1 < N ? x[t + 1] : 0.0f,
+                                                             t + 2 < N ? x[t + 2] : 0.0f, t + 3 < N ? x[t + 3] : 0.0f);
+    } else if constexpr (V == 2) {
+#pragma unroll
+        for (int t = 0; t < N; t += 2) {
+            if constexpr (sizeof(R) == 4)
+                *reinterpret_cast<float2 *>(p + t) = make_float2(x[t], t + 1 < N ? x[t + 1] : 0.0f);
+            else
+                *reinterpret_cast<double2 *>(p + t) = make_double2(x[t], t + 1 < N ? x[t + 1] : 0.0);
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < N; ++t) p[t] = x[t];
+    }
+}
+
+template <int La_, int Lb_, int Lc_, int Ld_, typename R_>
 struct GCfg {
     using R = R_;
-    static constexpr int oLa = La0, oLb = Lb0, oLc = Lc0, oLd = Ld0;
-    static constexpr int oNA = ncart(La0), oNB = ncart(Lb0), oNC = ncart(Lc0), oND = ncart(Ld0);
-    static constexpr int oNERI = oNA * oNB * oNC * oND;
-    static constexpr int La = La0 + 2, Lb = Lb0 + 2, Lc = Lc0 + 2, Ld = Ld0 + 2;
-    static constexpr int NAB = La + Lb, NCD = Lc + Ld;
-    static constexpr int NRYS = (La0 + Lb0 + Lc0 + Ld0 + 2) / 2 + 1;
-    static constexpr int RB = (int)sizeof(R);
-    static constexpr bool FUSE_BC = false;
-    static constexpr bool DIRECT = sizeof(R) == 4;
-    static constexpr bool SWAB_OK = !DIRECT, SWCD_OK = !DIRECT;
-    static constexpr int S_CB = S_N;
-    static constexpr int S_CD = S_N + (DIRECT ? 3 : 0);
-    static constexpr int SN = S_CD + (DIRECT ? 3 : 0);
-    static constexpr int JL = (Lb + 1) * (Ld + 1);
-    static constexpr int IBLK = (La + 1) * (Lc + 1) * JL;
-    static constexpr int JLP = (JL % 2) ? JL : JL + 1;
-    static constexpr int IBLKP = (La + 1) * (Lc + 1) * JLP;
-    static constexpr int HBLK = (La + 1) * (Lb + 1) * (NCD + 1);
-    static constexpr int GEO_BYTES = G_N * 8;
-    static constexpr int BC_BYTES = NRYS * SN * RB;
-    static constexpr int H_BYTES = DIRECT ? 0 : 3 * NRYS * HBLK * RB;
-    static constexpr int I_BYTES = 3 * NRYS * IBLKP * RB;
-    static constexpr int NACC = 17;  // dR[4][3], dalpha-part[4], E
-    static constexpr int PERQ = GEO_BYTES + RG_N * RB + BC_BYTES + H_BYTES + I_BYTES + NACC * 8 +
-                                oNERI * RB + 160;
-    static constexpr int Q = imax(1, imin(8, (100 * 1024) / PERQ));
+    static constexpr int La = La_, Lb = Lb_, Lc = Lc_, Ld = Ld_;
+    static constexpr int NA = ncart(La), NB = ncart(Lb), NC = ncart(Lc), ND = ncart(Ld);
+    static constexpr int NERI = NA * NB * NC * ND;
+    static constexpr int NRYS = (La + Lb + Lc + Ld + 2) / 2 + 1;
+    static constexpr bool SWAB_OK = false, SWCD_OK = false;
+    static constexpr int S_CB = S_N, S_CD = S_N + 3, SN = S_N + 6;
+    static constexpr int NI = La + 1, NJ = Lb + 1, NK = Lc + 1, NL = Ld + 1, JL = NJ * NL;
+    // (j, l) blocks: 16-byte vectors, an odd number of them (the blocks of a quarter warp start in
+    // distinct banks)
+    static constexpr int VJ = JL == 1 ? 1 : (sizeof(R) == 8 || JL == 2 ? 2 : 4);
+    static constexpr int JP0 = (JL + VJ - 1) / VJ * VJ;
+    static constexpr int JP = (VJ > 1 && JL > 2 && (JP0 / VJ) % 2 == 0) ? JP0 + VJ : JP0;
+    static constexpr int AC = NI * NK;
+    static constexpr int IB = AC * JP;  // 2-D integrals per (root, axis)
     static constexpr int THREADS = 256;
-    static constexpr int OFF_GEO = 0;
-    static constexpr int OFF_RG = Q * GEO_BYTES;
-    static constexpr int OFF_BC = ((OFF_RG + Q * RG_N * RB + 15) / 16) * 16;
-    static constexpr int OFF_ACC = ((OFF_BC + Q * BC_BYTES + 15) / 16) * 16;
-    static constexpr int OFF_DR = OFF_ACC + Q * NACC * 8;        // centre gradients, all primitives
-    static constexpr int OFF_PRIM = OFF_DR + Q * 12 * 8;          // primitive ids + exponents
-    static constexpr int OFF_H = ((OFF_PRIM + Q * 8 * 8 + 15) / 16) * 16;
-    static constexpr int OFF_I = OFF_H + Q * H_BYTES;
-    static constexpr int OFF_G = OFF_I + Q * I_BYTES;  // the tile's upstream G, generic order
-    static constexpr int SMEM = OFF_G + Q * oNERI * RB + 16;
+    // outputs (G values) per thread of step 2
+    static constexpr int BCH = imax(1, imin(NB, (sizeof(R) == 8 ? 18 : 50) / ND));
+    static constexpr int NCH = cdiv(NB, BCH);
+    static constexpr int ACN = NA * NC * NCH;
+    // roots taken together, in passes of equal length
+    static constexpr int NPASS = cdiv(NRYS, imin(NRYS, imax(1, THREADS / ACN)));
+    static constexpr int RG = cdiv(NRYS, NPASS);
+    static constexpr int WT = RG * ACN;
+    // threads of step 3 per (unit, axis), padded to whole segments of a warp
+    static constexpr int SA = RG * AC;
+    static constexpr int SEG = SA <= 32 ? pow2ceil(SA) : cdiv(SA, 32) * 32;
+    static constexpr int SW = SEG < 32 ? SEG : 32;   // lanes summed by shuffles
+    static constexpr int NSW = SEG / SW;
+    static constexpr int ST = 3 * SEG;
+    static constexpr int I_VALS = 3 * NRYS * IB;     // per unit
+    static constexpr int W_VALS = 3 * RG * ACN * JP;
+    static constexpr int UNIT_BYTES = (I_VALS + W_VALS) * (int)sizeof(R);
+    static constexpr int QG = imax(1, imin(imin(THREADS / WT, THREADS / ST), (48 * 1024) / UNIT_BYTES));
+    // units per batch of the setup stages
+    static constexpr int NBU = imax(1, imin(32, THREADS / (QG * NRYS))) * QG;
+    static constexpr int align16(int n) { return (n + 15) / 16 * 16; }
+    static constexpr int OFF_BC = 0;
+    static constexpr int OFF_META = align16(NBU * NRYS * SN * (int)sizeof(R));
+    static constexpr int OFF_EA = align16(OFF_META + NBU * 8 * 4);
+    static constexpr int OFF_RED = align16(OFF_EA + NBU * 4 * (int)sizeof(R));
+    static constexpr int OFF_I = align16(OFF_RED + QG * 3 * NSW * 5 * (int)sizeof(R));
+    static constexpr int OFF_W = align16(OFF_I + QG * I_VALS * (int)sizeof(R));
+    // the batch's geometry is dead before steps 1 to 3 start
+    static constexpr int SMEM = imax(OFF_W + QG * W_VALS * (int)sizeof(R), OFF_I + NBU * G_N * 8) + 16;
 };
 
-template <class C>
-__device__ __forceinline__ typename C::R gI(const typename C::R *Iq, int xi, int mu, int i, int j, int k,
-                                            int l) {
-    return Iq[i_index<C>(xi, mu, i, k, j, l)];
+// Units of a class: its quartets' primitive quartets, quartet after quartet.
+struct GradUnits {
+    const long long *ps;  // prefix sum of the primitive quartets at the class's first quartet, or
+                          // null for a primitive plan (one unit per quartet)
+    long long units;
+    int steps;            // groups of QG units per CTA
+};
+
+template <class C, int CH>
+__device__ __forceinline__ void load_g(const double *__restrict__ G, const ClassArgs &args, int a, int c,
+                                       typename C::R (&g)[C::BCH][C::ND]) {
+#pragma unroll
+    for (int bb = 0; bb < C::BCH; ++bb)
+#pragma unroll
+        for (int d = 0; d < C::ND; ++d)
+            if (CH * C::BCH + bb < C::NB)
+                g[bb][d] = to_r<typename C::R>(__ldg(G + a * args.ostride[0] + (CH * C::BCH + bb) * args.ostride[1] +
+                                                     c * args.ostride[2] + d * args.ostride[3]));
 }
 
-// The index table of the grouped contraction (eri_bwd_table.h), as device data, one per canonical
-// class.
-template <int A, int B, int Cc, int D>
-__device__ const BwdTab<A, B, Cc, D> kBwdTab = make_bwd_tab<A, B, Cc, D>();
+// Step 2 for b-chunk CH: the thread's partial W blocks along the three axes.
+template <class C, int CH>
+__device__ __forceinline__ void w_chunk(const typename C::R (&g)[C::BCH][C::ND], const typename C::R (&X)[C::JL],
+                                        const typename C::R (&Y)[C::JL], const typename C::R (&Z)[C::JL],
+                                        typename C::R (&WX)[C::JL], typename C::R (&WY)[C::JL],
+                                        typename C::R (&WZ)[C::JL]) {
+    using R = typename C::R;
+#pragma unroll
+    for (int bb = 0; bb < C::BCH; ++bb) {
+        if constexpr (CH * C::BCH < C::NB) {
+            const int b = CH * C::BCH + bb;
+            if (b < C::NB) {
+#pragma unroll
+                for (int d = 0; d < C::ND; ++d) {
+                    const int jx = cart_x(C::Lb, b) * C::NL + cart_x(C::Ld, d);
+                    const int jy = cart_y(C::Lb, b) * C::NL + cart_y(C::Ld, d);
+                    const int jz = cart_z(C::Lb, b) * C::NL + cart_z(C::Ld, d);
+                    const R gy = g[bb][d] * Y[jy], gx = g[bb][d] * X[jx];
+                    WX[jx] = fma(gy, Z[jz], WX[jx]);
+                    WZ[jz] = fma(gy, X[jx], WZ[jz]);
+                    WY[jy] = fma(gx, Z[jz], WY[jy]);
+                }
+            }
+        }
+    }
+}
+
+// f(std::integral_constant<int, CH>) for the run-time chunk ch
+template <class C, int CH = 0, class F>
+__device__ __forceinline__ void with_chunk(int ch, F f) {
+    if constexpr (CH + 1 >= C::NCH) {
+        f(std::integral_constant<int, CH>{});
+    } else {
+        if (ch == CH)
+            f(std::integral_constant<int, CH>{});
+        else
+            with_chunk<C, CH + 1>(ch, f);
+    }
+}
 
 template <class C>
-__device__ __forceinline__ void backward_tile(const ShellsDev &sh, const Tables &tb,
-                                              const ClassArgs &args, const double *__restrict__ G,
-                                              double *__restrict__ dR, double *__restrict__ dalpha) {
+__device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables &tb, const ClassArgs &args,
+                                               const GradUnits &un, const double *__restrict__ G,
+                                               double *__restrict__ dR, double *__restrict__ dalpha) {
     using R = typename C::R;
+    constexpr int T = C::THREADS, JL = C::JL, JP = C::JP;
     extern __shared__ __align__(16) unsigned char smem[];
-    double *geo_s = reinterpret_cast<double *>(smem + C::OFF_GEO);
-    R *rg_s = reinterpret_cast<R *>(smem + C::OFF_RG);
     R *bc_s = reinterpret_cast<R *>(smem + C::OFF_BC);
-    double *acc_s = reinterpret_cast<double *>(smem + C::OFF_ACC);
-    double *dr_s = reinterpret_cast<double *>(smem + C::OFF_DR);
-    double *prim_s = reinterpret_cast<double *>(smem + C::OFF_PRIM);  // [q][0..3] exps, [4..7] prim ids
-    R *H_s = reinterpret_cast<R *>(smem + C::OFF_H);
+    int *meta_s = reinterpret_cast<int *>(smem + C::OFF_META);  // quartet, its four shells' primitives
+    R *ea_s = reinterpret_cast<R *>(smem + C::OFF_EA);          // 2 alpha of the four primitives
+    R *red_s = reinterpret_cast<R *>(smem + C::OFF_RED);
     R *I_s = reinterpret_cast<R *>(smem + C::OFF_I);
-    __shared__ int maxprim_s;
-    __shared__ int4 qt_s[C::Q];
-    __shared__ R ea_s[C::Q * 4];  // 2 alpha of the quartet's four primitives, in R
+    R *W_s = reinterpret_cast<R *>(smem + C::OFF_W);
+    double *geo_s = reinterpret_cast<double *>(smem + C::OFF_I);
+    __shared__ int range_s[2];
 
     const int tid = threadIdx.x;
-    const long long q0 = (long long)blockIdx.x * C::Q;
-    const int qn = (int)((args.nq - q0) < C::Q ? (args.nq - q0) : C::Q);
-    if (tid == 0) maxprim_s = 1;
-    for (int i = tid; i < C::Q * 12; i += C::THREADS) dr_s[i] = 0.0;
-    for (int q = tid; q < C::Q; q += C::THREADS) {
-        int4 g = q < qn ? args.quartets[q0 + q] : make_int4(0, 0, 0, 0);
-        qt_s[q] = make_int4(pick(g, args.perm[0]), pick(g, args.perm[1]), pick(g, args.perm[2]),
-                            pick(g, args.perm[3]));
-    }
-    // the tile's G (contiguous per quartet in the class's generic layout), read once for all
-    // primitives into the canonical component order (rounded to FP32 once for the mixed adjoint)
-    R *G_s = reinterpret_cast<R *>(smem + C::OFF_G);
-    {
-        const int st0 = args.ostride[0], st1 = args.ostride[1], st2 = args.ostride[2],
-                  st3 = args.ostride[3];
-        for (int t = tid; t < qn * C::oNERI; t += C::THREADS) {
-            const int q = t / C::oNERI, e = t - q * C::oNERI;
-            const int id = e % C::oND, ic = (e / C::oND) % C::oNC, ib = (e / (C::oND * C::oNC)) % C::oNB,
-                      ia = e / (C::oND * C::oNC * C::oNB);
-            G_s[t] = to_r<R>(G[(q0 + q) * C::oNERI + ia * st0 + ib * st1 + ic * st2 + id * st3]);
+    const long long U0 = (long long)blockIdx.x * un.steps * C::QG;
+    const long long U1 = min(un.units, U0 + (long long)un.steps * C::QG);
+    const long long base = un.ps ? un.ps[0] : 0;
+    if (un.ps && tid < 2) {  // quartets of the CTA's first and last unit
+        const long long u = tid ? U1 - 1 : U0;
+        int lo = 0, hi = (int)args.nq - 1;
+        while (lo < hi) {
+            const int mid = lo + (hi - lo + 1) / 2;
+            if (__ldg(un.ps + mid) - base <= u) lo = mid; else hi = mid - 1;
         }
+        range_s[tid] = lo;
     }
-    __syncthreads();
+    // step 2: (group, root of the pass, a, c, chunk); step 3: (group, axis, root of the pass, i0, i2)
+    const int wg = tid / C::WT, wr = tid - wg * C::WT;
+    const int wmu = wr / C::ACN, witem = wr - wmu * C::ACN;
+    const int wch = witem % C::NCH, wc = (witem / C::NCH) % C::NC, wa = witem / (C::NCH * C::NC);
+    int wo[3];
+#pragma unroll
+    for (int x = 0; x < 3; ++x) wo[x] = (c_cart[C::La][wa % C::NA][x] * C::NK + c_cart[C::Lc][wc][x]) * JP;
+    R g[C::BCH][C::ND];
+    int gq = -1;  // the quartet whose G the thread holds
+    const int sg = tid / C::ST, sx = (tid - sg * C::ST) / C::SEG, se = (tid - sg * C::ST) % C::SEG;
+    const bool s_on = sg < C::QG && se < C::SA;
+    const int smu = se / C::AC, si = (se % C::AC) / C::NK, sk = se % C::NK;
+    R dacc[4], dcomp[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dacc[k] = dcomp[k] = (R)0;
 
-    for (int prim = 0; prim < maxprim_s; ++prim) {
-        for (int i = tid; i < C::Q * C::NACC; i += C::THREADS) acc_s[i] = 0.0;
-        for (int q = tid; q < C::Q; q += C::THREADS) {
-            double *geo = geo_s + q * G_N;
-            int np = 0;
-            if (q < qn) {
-                int4 qt = qt_s[q];
-                phase_geometry<C>(sh, qt, prim, geo, np);
-                if (prim < np) {
-                    int nb = sh.nprim[qt.y], nc = sh.nprim[qt.z], nd = sh.nprim[qt.w];
-                    int id = prim % nd, t = prim / nd;
-                    int ic = t % nc;
-                    t /= nc;
-                    int ib = t % nb, ia = t / nb;
-                    int pk[4] = {sh.pofs[qt.x] + ia, sh.pofs[qt.y] + ib, sh.pofs[qt.z] + ic,
-                                 sh.pofs[qt.w] + id};
-                    for (int k = 0; k < 4; ++k) {
-                        prim_s[q * 8 + k] = sh.exps[pk[k]];
-                        prim_s[q * 8 + 4 + k] = (double)pk[k];
-                        ea_s[q * 4 + k] = to_r<R>(2.0 * sh.exps[pk[k]]);
-                    }
+    for (long long ub = U0; ub < U1; ub += C::NBU) {
+        const int nu = (int)min((long long)C::NBU, U1 - ub);
+        __syncthreads();
+        for (int i = tid; i < nu; i += T) {
+            const long long u = ub + i;
+            int q, prim = 0;
+            if (un.ps) {
+                int lo = range_s[0], hi = range_s[1];
+                while (lo < hi) {
+                    const int mid = lo + (hi - lo + 1) / 2;
+                    if (__ldg(un.ps + mid) - base <= u) lo = mid; else hi = mid - 1;
                 }
+                q = lo;
+                prim = (int)(u - (__ldg(un.ps + q) - base));
             } else {
-                geo[G_PREF] = 0.0;
-                geo[G_T] = 0.0;
-                for (int s = G_P; s < G_N; ++s)
-                    geo[s] = (s == G_P || s == G_Q || s == G_IP || s == G_IQ) ? 1.0
-                                                                              : (s == G_IPQ ? 0.5 : 0.0);
+                q = (int)u;
             }
-            if (prim == 0 && np > 1) atomicMax(&maxprim_s, np);
-            R *rg = rg_s + q * RG_N;
-            rg[RG_ABX] = to_r<R>(geo[G_ABX]);
-            rg[RG_ABY] = to_r<R>(geo[G_ABY]);
-            rg[RG_ABZ] = to_r<R>(geo[G_ABZ]);
-            rg[RG_CDX] = to_r<R>(geo[G_CDX]);
-            rg[RG_CDY] = to_r<R>(geo[G_CDY]);
-            rg[RG_CDZ] = to_r<R>(geo[G_CDZ]);
-            rg[RG_SWAB] = to_r<R>(geo[G_SWAB]);
-            rg[RG_SWCD] = to_r<R>(geo[G_SWCD]);
-            if (q >= qn || prim >= np) {
-                for (int k = 0; k < 4; ++k) {
-                    prim_s[q * 8 + k] = 1.0;
-                    prim_s[q * 8 + 4 + k] = -1.0;
-                    ea_s[q * 4 + k] = (R)2;
-                }
+            const int4 gqt = args.quartets[q];
+            const int4 qt = make_int4(pick(gqt, args.perm[0]), pick(gqt, args.perm[1]), pick(gqt, args.perm[2]),
+                                      pick(gqt, args.perm[3]));
+            int np = 0;
+            geometry_of<C>(sh, args, qt, prim, geo_s + i * G_N, np);
+            const int nb = sh.nprim[qt.y], nc = sh.nprim[qt.z], nd = sh.nprim[qt.w];
+            int t = prim;
+            const int id = t % nd;
+            t /= nd;
+            const int ic = t % nc;
+            t /= nc;
+            const int pk[4] = {sh.pofs[qt.x] + t / nb, sh.pofs[qt.y] + t % nb, sh.pofs[qt.z] + ic,
+                               sh.pofs[qt.w] + id};
+            meta_s[i * 8] = q;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                meta_s[i * 8 + 1 + k] = pk[k];
+                ea_s[i * 4 + k] = to_r<R>(2.0 * sh.exps[pk[k]]);
             }
         }
         __syncthreads();
-        for (int it = tid; it < C::Q * C::NRYS; it += C::THREADS) {
-            int q = it / C::NRYS, mu = it % C::NRYS;
-            phase_setup<C>(tb, geo_s + q * G_N, mu, bc_s + (q * C::NRYS + mu) * C::SN);
+        for (int it = tid; it < nu * C::NRYS; it += T) {
+            const int i = it / C::NRYS, mu = it - i * C::NRYS;
+            const double *geo = geo_s + i * G_N;
+            double x, w;
+            rys_root<sizeof(R) == 4>(tb, C::NRYS, mu, geo[G_T], x, w);
+            R *b = bc_s + it * C::SN;
+            const double ipq = geo[G_IPQ], fq = geo[G_Q] * x * ipq, fp = geo[G_P] * x * ipq;
+            b[S_WZ] = to_r<R>(geo[G_PREF] * w);
+            b[S_B00] = to_r<R>(0.5 * x * ipq);
+            b[S_B10] = to_r<R>((1.0 - fq) * (0.5 * geo[G_IP]));
+            b[S_B01] = to_r<R>((1.0 - fp) * (0.5 * geo[G_IQ]));
+#pragma unroll
+            for (int s = 0; s < 3; ++s) {
+                const double pq = geo[G_PQX + s];
+                b[S_C0X + s] = to_r<R>(geo[G_PAX + s] - fq * pq);
+                b[C::S_CB + s] = to_r<R>((geo[G_PAX + s] + geo[G_ABX + s]) - fq * pq);
+                b[S_C1X + s] = to_r<R>(geo[G_QCX + s] + fp * pq);
+                b[C::S_CD + s] = to_r<R>((geo[G_QCX + s] + geo[G_CDX + s]) + fp * pq);
+            }
         }
-        __syncthreads();
-        for (int it = tid; it < C::Q * C::NRYS * 3; it += C::THREADS) {
-            int q = it / (C::NRYS * 3), r = it % (C::NRYS * 3);
-            if constexpr (C::DIRECT)
-                phase_direct<C>(bc_s + q * C::NRYS * C::SN, r / 3, r % 3, I_s + (size_t)q * (C::I_BYTES / C::RB));
-            else
-                phase_vrr<C>(bc_s + q * C::NRYS * C::SN, rg_s + q * RG_N, r / 3, r % 3,
-                             H_s + (size_t)q * (C::H_BYTES / C::RB), I_s + (size_t)q * (C::I_BYTES / C::RB));
-        }
-        __syncthreads();
-        if constexpr (!C::DIRECT) {
-            constexpr int NIJ = (C::La + 1) * (C::Lb + 1);
-            for (int it = tid; it < C::Q * C::NRYS * 3 * NIJ; it += C::THREADS) {
-                int q = it / (C::NRYS * 3 * NIJ), r = it % (C::NRYS * 3 * NIJ);
-                int mu = r / (3 * NIJ);
-                r %= 3 * NIJ;
-                int xi = r / NIJ, ij = r % NIJ;
-                phase_ket<C>(rg_s + q * RG_N, mu, xi, ij / (C::Lb + 1), ij % (C::Lb + 1),
-                             H_s + (size_t)q * (C::H_BYTES / C::RB), I_s + (size_t)q * (C::I_BYTES / C::RB));
+        for (int u0 = 0; u0 < nu; u0 += C::QG) {
+            __syncthreads();  // records are written; I and W of the units before are read
+            // 1: 2-D integrals
+            constexpr int NIP = pow2ceil(C::NI), RITEMS = C::QG * C::NRYS * 3 * NIP;
+            for (int it = tid; it < cdiv(RITEMS, 32) * 32; it += T) {
+                const int blk = it / NIP, i = it % NIP;
+                const int gu = blk / (3 * C::NRYS);
+                const bool live = it < RITEMS && i < C::NI && u0 + gu < nu;
+                // lanes without a unit repeat the first one (in range, not stored)
+                const int r = live ? blk - gu * 3 * C::NRYS : 0, unit = live ? u0 + gu : u0;
+                rows_direct<C, JP>(bc_s + (unit * C::NRYS + r / 3) * C::SN, r % 3, i, live,
+                                   I_s + (live ? gu : 0) * C::I_VALS + ((r % 3) * C::NRYS + r / 3) * C::IB);
             }
             __syncthreads();
-        }
-        // contraction with G, grouped by axis: for axis x and the x-components (i0, i1, i2, i3)
-        // of the four centres, W = sum of G I_y I_z over the outputs with those x-components
-        // (y, z the other two axes); each derivative factor of axis x then multiplies W once
-        // instead of once per output.
-        {
-            constexpr int W1 = C::oLa + 1, W2 = C::oLb + 1, W3 = C::oLc + 1, W4 = C::oLd + 1;
-            constexpr int WN = W1 * W2 * W3 * W4;
-            constexpr int ITEMS = C::NRYS * 3 * WN;
-            const auto &tab = kBwdTab<C::oLa, C::oLb, C::oLc, C::oLd>;
-            using Tab = BwdTab<C::oLa, C::oLb, C::oLc, C::oLd>;
-            static_assert(Tab::WN == WN && Tab::N == C::oNERI && Tab::LC1 == C::Lc + 1 && Tab::LD1 == C::Ld + 1 &&
-                              Tab::JLP == C::JLP,
-                          "index table and 2-D integral layout disagree");
-            const int lane = tid & 31;
-            for (int q = 0; q < qn; ++q) {
-                const R *Iq = I_s + (size_t)q * (C::I_BYTES / C::RB);
-                const R *Gq = G_s + q * C::oNERI;
-                R ea[4];
+            const bool w_unit = wg < C::QG && u0 + wg < nu;
+            if (w_unit) {
+                const int q = meta_s[(u0 + wg) * 8];
+                if (q != gq) {
+                    gq = q;
+                    with_chunk<C>(wch, [&](auto ch) {
+                        load_g<C, decltype(ch)::value>(G + (long long)q * C::NERI, args, wa, wc, g);
+                    });
+                }
+            }
+            const bool s_unit = s_on && u0 + sg < nu;
+            R up2[4], e0 = (R)0;  // exponent terms of the unit
 #pragma unroll
-                for (int k = 0; k < 4; ++k) ea[k] = ea_s[q * 4 + k];
-                // the thread's sums (in R)
-                R r[C::NACC];
+            for (int k = 0; k < 4; ++k) up2[k] = (R)0;
+#pragma unroll 1
+            for (int pass = 0; pass < C::NPASS; ++pass) {
+                const int m0 = pass * C::RG;
+                if (pass > 0) __syncthreads();
+                // 2: partial W blocks
+                if (w_unit && m0 + wmu < C::NRYS) {
+                    const R *Iu = I_s + wg * C::I_VALS + (m0 + wmu) * C::IB;
+                    R X[JL], Y[JL], Z[JL], WX[JL], WY[JL], WZ[JL];
+                    load_block<JL, C::VJ>(Iu + wo[0], X);
+                    load_block<JL, C::VJ>(Iu + C::NRYS * C::IB + wo[1], Y);
+                    load_block<JL, C::VJ>(Iu + 2 * C::NRYS * C::IB + wo[2], Z);
 #pragma unroll
-                for (int k = 0; k < C::NACC; ++k) r[k] = (R)0;
-                for (int it = tid; it < ITEMS; it += C::THREADS) {
-                    const int mu = it / (3 * WN), rem = it % (3 * WN);
-                    const int x = rem / WN, w = rem % WN;
-                    const int i3 = w % W4, i2 = (w / W4) % W3, i1 = (w / (W4 * W3)) % W2,
-                              i0 = w / (W4 * W3 * W2);
-                    const int y = x == 2 ? 0 : x + 1, z = x == 0 ? 2 : x - 1;
-                    const R *Iy = Iq + i_index<C>(y, mu, 0, 0, 0, 0), *Iz = Iq + i_index<C>(z, mu, 0, 0, 0, 0);
-                    const unsigned long long *ent = tab.e + x * C::oNERI;
-                    R W = (R)0;
-                    for (int k = tab.start[w], k1 = tab.start[w + 1]; k < k1; ++k) {
-                        const unsigned long long v = ent[k];
-                        W = fma(Gq[(int)(v & 0xffffu)] * Iy[(int)((v >> 16) & 0xffffu)], Iz[(int)(v >> 32)], W);
+                    for (int t = 0; t < JL; ++t) WX[t] = WY[t] = WZ[t] = (R)0;
+                    with_chunk<C>(wch, [&](auto ch) { w_chunk<C, decltype(ch)::value>(g, X, Y, Z, WX, WY, WZ); });
+                    R *Wu = W_s + wg * C::W_VALS + (wmu * C::ACN + witem) * JP;
+                    store_block<JL, C::VJ>(Wu, WX);
+                    store_block<JL, C::VJ>(Wu + C::RG * C::ACN * JP, WY);
+                    store_block<JL, C::VJ>(Wu + 2 * C::RG * C::ACN * JP, WZ);
+                }
+                __syncthreads();
+                // 3: the sums over w of the thread's (i0, i2)
+                if (s_unit && m0 + smu < C::NRYS) {
+                    const R *Wu = W_s + sg * C::W_VALS + (sx * C::RG + smu) * C::ACN * JP;
+                    R Wb[JL];
+#pragma unroll
+                    for (int t = 0; t < JL; ++t) Wb[t] = (R)0;
+                    // components with value v along the axis: x: r = La - v fixed, y and z: r = v..La
+                    // (r = La - a_x; index r (r+1) / 2 + a_z)
+                    for (int na = 0; na <= C::La - si; ++na) {
+                        const int ra = sx == 0 ? C::La - si : si + na, za = sx == 0 ? na : (sx == 1 ? ra - si : si);
+                        for (int nc = 0; nc <= C::Lc - sk; ++nc) {
+                            const int rc = sx == 0 ? C::Lc - sk : sk + nc, zc = sx == 0 ? nc : (sx == 1 ? rc - sk : sk);
+                            const R *p = Wu + ((ra * (ra + 1) / 2 + za) * C::NC + rc * (rc + 1) / 2 + zc) * C::NCH * JP;
+#pragma unroll
+                            for (int ch = 0; ch < C::NCH; ++ch, p += JP) {
+                                R v[JL];
+                                load_block<JL, C::VJ>(p, v);
+#pragma unroll
+                                for (int t = 0; t < JL; ++t) Wb[t] += v[t];
+                            }
+                        }
                     }
+                    const R *Ib = I_s + sg * C::I_VALS + (sx * C::NRYS + m0 + smu) * C::IB + (si * C::NK + sk) * JP;
+                    const R fi = (R)si, fk = (R)sk;
+                    R S0 = (R)0, Sa = (R)0, Sb = (R)0, Sc = (R)0, Sd = (R)0, DD = (R)0, DK = (R)0, KK = (R)0;
+                    R v[JL];
+                    load_block<JL, C::VJ>(Ib, v);
+#pragma unroll
+                    for (int j = 0; j < C::NJ; ++j)
+#pragma unroll
+                        for (int l = 0; l < C::NL; ++l) {
+                            const R w = Wb[j * C::NL + l];
+                            S0 = fma(w, v[j * C::NL + l], S0);
+                            if (j > 0) Sb = fma((R)j * w, v[(j - 1) * C::NL + l], Sb);
+                            if (l > 0) Sd = fma((R)l * w, v[j * C::NL + l - 1], Sd);
+                            if (j > 1) DD = fma((R)(j * (j - 1)) * w, v[(j - 2) * C::NL + l], DD);
+                            if (l > 1) KK = fma((R)(l * (l - 1)) * w, v[j * C::NL + l - 2], KK);
+                            if (j > 0 && l > 0) DK = fma((R)(j * l) * w, v[(j - 1) * C::NL + l - 1], DK);
+                        }
+                    if constexpr (C::La > 0) {
+                        if (si > 0) {
+                            R s = (R)0, sb = (R)0, sd = (R)0;
+                            load_block<JL, C::VJ>(Ib - C::NK * JP, v);
+#pragma unroll
+                            for (int j = 0; j < C::NJ; ++j)
+#pragma unroll
+                                for (int l = 0; l < C::NL; ++l) {
+                                    const R w = Wb[j * C::NL + l];
+                                    s = fma(w, v[j * C::NL + l], s);
+                                    if (j > 0) sb = fma((R)j * w, v[(j - 1) * C::NL + l], sb);
+                                    if (l > 0) sd = fma((R)l * w, v[j * C::NL + l - 1], sd);
+                                }
+                            Sa = fi * s;
+                            DD = fma((R)2 * fi, sb, DD);
+                            DK = fma(fi, sd, DK);
+                        }
+                    }
+                    if constexpr (C::Lc > 0) {
+                        if (sk > 0) {
+                            R s = (R)0, sb = (R)0, sd = (R)0;
+                            load_block<JL, C::VJ>(Ib - JP, v);
+#pragma unroll
+                            for (int j = 0; j < C::NJ; ++j)
+#pragma unroll
+                                for (int l = 0; l < C::NL; ++l) {
+                                    const R w = Wb[j * C::NL + l];
+                                    s = fma(w, v[j * C::NL + l], s);
+                                    if (j > 0) sb = fma((R)j * w, v[(j - 1) * C::NL + l], sb);
+                                    if (l > 0) sd = fma((R)l * w, v[j * C::NL + l - 1], sd);
+                                }
+                            Sc = fk * s;
+                            KK = fma((R)2 * fk, sd, KK);
+                            DK = fma(fk, sb, DK);
+                        }
+                    }
+                    auto dot = [&](const R *p) -> R {
+                        R s = (R)0;
+                        load_block<JL, C::VJ>(p, v);
+#pragma unroll
+                        for (int t = 0; t < JL; ++t) s = fma(Wb[t], v[t], s);
+                        return s;
+                    };
+                    if constexpr (C::La > 1)
+                        if (si > 1) DD = fma(fi * (fi - (R)1), dot(Ib - 2 * C::NK * JP), DD);
+                    if constexpr (C::Lc > 1)
+                        if (sk > 1) KK = fma(fk * (fk - (R)1), dot(Ib - 2 * JP), KK);
+                    if constexpr (C::La > 0 && C::Lc > 0)
+                        if (si > 0 && sk > 0) DK = fma(fi * fk, dot(Ib - (C::NK + 1) * JP), DK);
+                    const R *b = bc_s + ((u0 + sg) * C::NRYS + m0 + smu) * C::SN;
+                    const R b00 = b[S_B00], b10 = b[S_B10], b01 = b[S_B01];
+                    const R SD = Sa + Sb, SK = Sc + Sd;
+                    const R P = fma(b10, SD, b00 * SK), Q = fma(b01, SK, b00 * SD);
+                    const R x2 = (R)2 * b00 * DK;
+                    const R VP = fma(b10, fma(b10, DD, x2), b00 * b00 * KK) + b10 * S0;
+                    const R VQ = fma(b01, fma(b01, KK, x2), b00 * b00 * DD) + b01 * S0;
+                    const R *ea = ea_s + (u0 + sg) * 4;
+                    const R cf[4] = {b[S_C0X + sx], b[C::S_CB + sx], b[S_C1X + sx], b[C::S_CD + sx]};
+                    const R low[4] = {Sa, Sb, Sc, Sd};
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const int nk = k == 0 ? i0 : (k == 1 ? i1 : (k == 2 ? i2 : i3));
-                        const int e0 = (k == 0), e1 = (k == 1), e2 = (k == 2), e3 = (k == 3);
-                        const R up = gI<C>(Iq, x, mu, i0 + e0, i1 + e1, i2 + e2, i3 + e3);
-                        const R up2 = gI<C>(Iq, x, mu, i0 + 2 * e0, i1 + 2 * e1, i2 + 2 * e2, i3 + 2 * e3);
-                        const R dn = nk > 0 ? gI<C>(Iq, x, mu, i0 - e0, i1 - e1, i2 - e2, i3 - e3) : (R)0;
-                        const R t = W * (ea[k] * up - (R)nk * dn);
-                        // r[k * 3 + x] with x known only at run time: select, no dynamic indexing
-                        r[k * 3 + 0] += x == 0 ? t : (R)0;
-                        r[k * 3 + 1] += x == 1 ? t : (R)0;
-                        r[k * 3 + 2] += x == 2 ? t : (R)0;
-                        r[12 + k] -= W * up2;
+                        const R p = k < 2 ? P : Q;
+                        const R u1 = fma(cf[k], S0, p);
+                        up2[k] += fma(cf[k], u1 + p, k < 2 ? VP : VQ);
+                        const R t = fma(ea[k], u1, -low[k]);
+                        if constexpr (sizeof(R) == 4) {  // compensated over the quartet's units
+                            const R y = __fsub_rn(t, dcomp[k]), n = __fadd_rn(dacc[k], y);
+                            dcomp[k] = __fsub_rn(__fsub_rn(n, dacc[k]), y);
+                            dacc[k] = n;
+                        } else {
+                            dacc[k] += t;
+                        }
                     }
-                    if (x == 0) r[16] += W * gI<C>(Iq, 0, mu, i0, i1, i2, i3);
-                }
-                // warp sums in R (FP32 in the mixed adjoint: the FP64 pipe is the scarce one there),
-                // then FP64 across warps, primitives and quartets
-#pragma unroll
-                for (int k = 0; k < C::NACC; ++k) {
-                    R v = r[k];
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-                    if (lane == 0 && v != (R)0) atomicAdd(acc_s + q * C::NACC + k, RTraits<R>::to_f64(v));
+                    if (sx == 0) e0 += S0;
                 }
             }
-        }
-        __syncthreads();
-        // per quartet: exponent gradients of this primitive quartet, centre gradients summed
-        for (int q = tid; q < qn; q += C::THREADS) {
-            const double *acc = acc_s + q * C::NACC;
-            const double *ex = prim_s + q * 8;
-            const int Lk[4] = {C::oLa, C::oLb, C::oLc, C::oLd};
-            if (ex[4] >= 0.0) {
+            // exponent terms of the unit: over the segment, then over segments and axes in FP64
+#pragma unroll
+            for (int off = C::SW / 2; off > 0; off >>= 1) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) up2[k] += __shfl_down_sync(0xffffffffu, up2[k], off, C::SW);
+                e0 += __shfl_down_sync(0xffffffffu, e0, off, C::SW);
+            }
+            if (sg < C::QG && se % C::SW == 0) {
+                R *r = red_s + ((sg * 3 + sx) * C::NSW + se / C::SW) * 5;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) r[k] = up2[k];
+                r[4] = e0;
+            }
+            // centre gradients when the group's next unit is not of this quartet (or not of this batch)
+            const int mine = (sg < C::QG && u0 + sg < nu) ? meta_s[(u0 + sg) * 8] : -1;
+            const bool flush = mine >= 0 && (u0 + sg + C::QG >= nu || meta_s[(u0 + sg + C::QG) * 8] != mine);
+            if (__any_sync(0xffffffffu, flush)) {
+                R v[4];
+#pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    double v = (2.0 * Lk[k] + 3.0) / (4.0 * ex[k]) * acc[16] + acc[12 + k];
-                    atomicAdd(dalpha + (long long)ex[4 + k], v);
+                    v[k] = flush ? dacc[k] - dcomp[k] : (R)0;
+#pragma unroll
+                    for (int off = C::SW / 2; off > 0; off >>= 1)
+                        v[k] += __shfl_down_sync(0xffffffffu, v[k], off, C::SW);
                 }
-                for (int i = 0; i < 12; ++i) dr_s[q * 12 + i] += acc[i];
+                if (flush) {
+                    if (se % C::SW == 0) {
+                        const int4 gqt = args.quartets[mine];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            atomicAdd(dR + 3LL * pick(gqt, args.perm[k]) + sx, RTraits<R>::to_f64(v[k]));
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) dacc[k] = dcomp[k] = (R)0;
+                }
+            }
+            __syncthreads();
+            if (tid < C::QG * 4 && u0 + tid / 4 < nu) {
+                const int gu = tid / 4, k = tid % 4;
+                constexpr int Lk[4] = {C::La, C::Lb, C::Lc, C::Ld};
+                const R *r = red_s + gu * 3 * C::NSW * 5;
+                double s2 = 0.0, e = 0.0;
+#pragma unroll
+                for (int t = 0; t < 3 * C::NSW; ++t) {
+                    s2 += RTraits<R>::to_f64(r[t * 5 + k]);
+                    if (t < C::NSW) e += RTraits<R>::to_f64(r[t * 5 + 4]);
+                }
+                const int pk = meta_s[(u0 + gu) * 8 + 1 + k];
+                const int L = k == 0 ? Lk[0] : (k == 1 ? Lk[1] : (k == 2 ? Lk[2] : Lk[3]));
+                atomicAdd(dalpha + pk, (2.0 * L + 3.0) / (4.0 * sh.exps[pk]) * e - s2);
             }
         }
-        __syncthreads();
-    }
-    for (int it = tid; it < qn * 12; it += C::THREADS) {
-        int q = it / 12, i = it % 12, k = i / 3, x = i % 3;
-        int4 qt = qt_s[q];
-        int s = pick(qt, k);
-        atomicAdd(dR + 3LL * s + x, dr_s[q * 12 + i]);
     }
 }
 
-template <class C>
-__global__ void __launch_bounds__(C::THREADS)
-eri_backward_kernel(ShellsDev sh, Tables tb, ClassArgs args, const double *__restrict__ G,
+template <class C, int MINB>
+__global__ void __launch_bounds__(C::THREADS, MINB)
+eri_backward_kernel(ShellsDev sh, Tables tb, ClassArgs args, GradUnits un, const double *__restrict__ G,
                     double *__restrict__ dR, double *__restrict__ dalpha) {
-    backward_tile<C>(sh, tb, args, G, dR, dalpha);
+    backward_units<C>(sh, tb, args, un, G, dR, dalpha);
 }
 
-// The same for the mixed adjoint of classes with an f shell, compiled for one resident CTA per
-// SM: under the default bound ptxas caps some of them at 128 registers with large spills, and
-// [ff|pp] then returned wrong exponent gradients for its first centre (the emulated kernel
-// arithmetic and the oracle agree); with the whole register file available none spills.
-template <class C>
-__global__ void __launch_bounds__(C::THREADS, 1)
-eri_backward_kernel_wide(ShellsDev sh, Tables tb, ClassArgs args, const double *__restrict__ G,
-                         double *__restrict__ dR, double *__restrict__ dalpha) {
-    backward_tile<C>(sh, tb, args, G, dR, dalpha);
-}
-
-template <int La, int Lb, int Lc, int Ld, typename R = double>
+template <int La, int Lb, int Lc, int Ld, typename R>
 cudaError_t launch_backward(const ShellsDev &sh, const Tables &tb, const ClassArgs &args,
-                            const double *G, double *dR, double *dalpha, cudaStream_t stream) {
+                            const long long *ps, long long units, const double *G, double *dR,
+                            double *dalpha, cudaStream_t stream) {
     using C = GCfg<La, Lb, Lc, Ld, R>;
     static_assert(C::SMEM <= 227 * 1024, "adjoint tile exceeds shared memory");
-    if (args.nq <= 0) return cudaSuccess;
-    constexpr bool wide = sizeof(R) == 4 && (La == 3 || Lb == 3 || Lc == 3 || Ld == 3);
-    void (*kern)(ShellsDev, Tables, ClassArgs, const double *, double *, double *);
-    if constexpr (wide)
-        kern = eri_backward_kernel_wide<C>;
-    else
-        kern = eri_backward_kernel<C>;
+    static_assert(C::WT <= C::THREADS && C::ST <= C::THREADS, "adjoint thread layout");
+    if (args.nq <= 0 || units <= 0) return cudaSuccess;
+    // registers: two CTAs per SM; the wide blocks of f shells and FP64 take the register file of one
+    constexpr int MINB = (sizeof(R) == 8 || C::JL > 9) ? 1 : 2;
+    auto kern = eri_backward_kernel<C, MINB>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
-    long long grid = (args.nq + C::Q - 1) / C::Q;
+    // whole batches per CTA, at most 64 steps, about eight CTAs per SM when there are enough units
+    constexpr int batch = C::NBU / C::QG;
+    const long long want = units / ((long long)C::QG * 152 * 8);
+    GradUnits un{ps, units, (int)std::max<long long>(1, std::min<long long>(64, want))};
+    if (un.steps > batch) un.steps = un.steps / batch * batch;
+    const long long per = (long long)un.steps * C::QG, grid = (units + per - 1) / per;
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-    kern<<<(unsigned)grid, C::THREADS, C::SMEM, stream>>>(sh, tb, args, G, dR, dalpha);
+    kern<<<(unsigned)grid, C::THREADS, C::SMEM, stream>>>(sh, tb, args, un, G, dR, dalpha);
     return cudaGetLastError();
 }
 

@@ -1,5 +1,6 @@
-// eri_bwd_table.h -- index table of the adjoint's grouped contraction (plain C++17, evaluated at
-// compile time; eri_backward.cuh places one per canonical class in device memory).
+// eri_bwd_table.h -- index table of the adjoint's contraction grouped by axis (plain C++17, evaluated
+// at compile time), written out entry by entry.  The adjoint kernel (eri_backward.cuh) forms the same
+// groups from its thread layout and reads no table; this header states them for the CPU test.
 //
 // The adjoint contracts G with the 2-D integrals axis by axis: for axis x and the x-components
 // w = (i0, i1, i2, i3) of the four centres, W = sum of G I_y I_z over the outputs sharing them
@@ -9,7 +10,7 @@
 // canonical index ((ia * NB + ib) * NC + ic) * ND + id (bits 0-15), the offset of its
 // y-components (bits 16-31) and of its z-components (bits 32-47) inside one (axis, root) block of
 // the 2-D integrals on the index ranges extended by two, layout [a][c][b][d] with the (b, d)
-// blocks padded to an odd length JLP.
+// blocks padded to an odd length JLP (the layout of an adjoint that forms the extended integrals).
 #pragma once
 
 namespace eri {

@@ -85,9 +85,11 @@ using LaunchFn = cudaError_t (*)(const ShellsDev &sh, const Tables &tb, const Cl
 // Variants: 0 = FP64, 1 = mixed, 2 = mixed with Kahan-compensated primitive sums.
 constexpr int kNumVariants = 3;
 
-// Launcher of one canonical class's adjoint kernel (FP64).
+// Launcher of one canonical class's adjoint kernel: `units` primitive quartets, ps their prefix sum
+// at the class's first quartet (null: one per quartet).
 using BackwardFn = cudaError_t (*)(const ShellsDev &sh, const Tables &tb, const ClassArgs &args,
-                                   const double *G, double *dR, double *dalpha, cudaStream_t stream);
+                                   const long long *ps, long long units, const double *G, double *dR,
+                                   double *dalpha, cudaStream_t stream);
 // Each adjoint unit fills the FP64 and the mixed-precision table for its classes.
 void eri_register_backward_0(BackwardFn *table, BackwardFn *table_mixed);
 void eri_register_backward_1(BackwardFn *table, BackwardFn *table_mixed);

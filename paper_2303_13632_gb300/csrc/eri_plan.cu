@@ -1276,7 +1276,11 @@ eri_status_t eri_backward(eri_plan_t plan, const double *d_G, double *d_dR, doub
         a.quartets = plan->d_quartets + plan->first[c];
         a.nq = plan->count[c];
         a.err = plan->d_err;
-        e = backward_of(c)(sh, plan->tables, a, d_G + plan->fp64_off[c], d_dR, d_dalpha, st);
+        a.pairs = plan->d_pairs;
+        a.np = plan->n_prims;
+        const bool units = is_contracted(plan);
+        e = backward_of(c)(sh, plan->tables, a, units ? plan->d_pstart + plan->first[c] : nullptr,
+                           units ? plan->units[c] : plan->count[c], d_G + plan->fp64_off[c], d_dR, d_dalpha, st);
         if (e != cudaSuccess) return cuda_status(e);
     }
     return ERI_OK;
