@@ -203,12 +203,17 @@ pack_kernel(ClassArgs args, int neri, int qt, UnitSpan span, const R *__restrict
     __shared__ R inv_s[kMaxQ];
     __shared__ unsigned long long part_raw_s[kThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long base = span.ps[0], u1 = span.u0 + span.nu;
+    const long long base = span.ps ? span.ps[0] : 0, u1 = span.u0 + span.nu;
     if (tid == 0) {
-        q_s[0] = quartet_of(span.ps, base, span.u0, 0, (int)span.nq - 1);
-        int b = quartet_of(span.ps, base, u1 - 1, 0, (int)span.nq - 1);
-        if (span.ps[b + 1] - base > u1) --b;  // continues in the next span
-        q_s[1] = b;
+        if (span.ps) {
+            q_s[0] = quartet_of(span.ps, base, span.u0, 0, (int)span.nq - 1);
+            int b = quartet_of(span.ps, base, u1 - 1, 0, (int)span.nq - 1);
+            if (span.ps[b + 1] - base > u1) --b;  // continues in the next span
+            q_s[1] = b;
+        } else {  // values of whole quartets
+            q_s[0] = 0;
+            q_s[1] = span.nu - 1;
+        }
     }
     __syncthreads();
     const long long q0 = q_s[0] + (long long)blockIdx.x * qt;
@@ -217,7 +222,7 @@ pack_kernel(ClassArgs args, int neri, int qt, UnitSpan span, const R *__restrict
     const int bits = args.bits;
     const R M = (R)((1u << (bits - 1)) - 1u);
     for (int q = tid; q < qn; q += kThreads)
-        slot_s[q] = (int)(max(span.ps[q0 + q] - base, span.u0) - span.u0);
+        slot_s[q] = span.ps ? (int)(max(span.ps[q0 + q] - base, span.u0) - span.u0) : (int)(q0 + q);
     __syncthreads();
     // non-negative IEEE values order like their bit patterns (and a NaN stays the largest)
     using U = std::conditional_t<sizeof(R) == 8, unsigned long long, unsigned int>;
@@ -317,6 +322,14 @@ cudaError_t setup_r(const ShellsDev &sh, const Tables &tb, const ClassArgs &a, c
     return cudaGetLastError();
 }
 
+// nq: quartets the span can hold at most
+template <typename R>
+cudaError_t pack_r(const ClassArgs &a, int neri, long long nq, const UnitSpan &span, const R *values, cudaStream_t s) {
+    const int qt = std::max(1, std::min(128, 4096 / neri));
+    pack_kernel<R><<<(unsigned)((nq + qt - 1) / qt), kThreads, 0, s>>>(a, neri, qt, span, values);
+    return cudaGetLastError();
+}
+
 template <typename R>
 cudaError_t contract_r(const ClassArgs &a, int neri, const UnitSpan &span, R *values, R *carry, int parity,
                        cudaStream_t s) {
@@ -330,9 +343,7 @@ cudaError_t contract_r(const ClassArgs &a, int neri, const UnitSpan &span, R *va
     contract_kernel<R, false><<<blocks, kThreads, 0, s>>>(a, neri, span, values, carry, parity);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int qt = std::max(1, std::min(128, 4096 / neri));
-    pack_kernel<R><<<(unsigned)((nq + qt - 1) / qt), kThreads, 0, s>>>(a, neri, qt, span, values);
-    return cudaGetLastError();
+    return pack_r(a, neri, nq, span, values, s);
 }
 
 }  // namespace
@@ -346,6 +357,13 @@ cudaError_t unit_setup(const ShellsDev &sh, const Tables &tb, const ClassArgs &a
                        bool mixed, const UnitSpan &span, void *records, int stride, cudaStream_t s) {
     return mixed ? setup_r(sh, tb, a, k, span, static_cast<float *>(records), stride, s)
                  : setup_r(sh, tb, a, k, span, static_cast<double *>(records), stride, s);
+}
+
+cudaError_t pack_values(const ClassArgs &a, int neri, const double *values, cudaStream_t s) {
+    UnitSpan whole{};
+    whole.nq = a.nq;
+    whole.nu = (int)a.nq;
+    return pack_r(a, neri, a.nq, whole, values, s);
 }
 
 cudaError_t unit_contract(const ClassArgs &a, bool mixed, int neri, const UnitSpan &span, void *values,

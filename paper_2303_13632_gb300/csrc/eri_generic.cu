@@ -7,16 +7,16 @@
 // better part of an hour ([gg|gg] alone compiles for more than seven minutes in three variants),
 // so these classes share one kernel per precision with the same stages of Sec. II-C in run-time
 // loops over shared memory:
-//   A0 geometry and prefactor        one thread per quartet (FP64, as the specialised kernels)
-//   A1 Rys root/weight, B and C      one thread per (quartet, root) (FP64, rounded to R)
-//   B  2-D integrals I(i, j, k, l)   one thread per (quartet, root, axis): the four-index Rys
-//                                    recursion in which every index is raised with the C value of
-//                                    its own centre (the recurrences behind Eqs. 6-7 before the
-//                                    transfer relation; exact arithmetic gives the VRR + HRR values)
-//   D  quadrature (Eq. 8)            one thread per (quartet, output), summed over the roots in R
-//                                    and over primitives in FP64 (in the output or the scratch)
-// Compressed output (Sec. II-D) then takes two more launches over the FP64 values: b_max and eps
-// per quartet (Eq. 9), and the codes (Eq. 10) packed one output word per thread.
+//   geometry and prefactor        FP64, as the specialised kernels
+//   Rys root/weight, B and C      FP64, rounded to R
+//   2-D integrals I(i, j, k, l)   the four-index Rys recursion in which every index is raised with
+//                                 the C value of its own centre (the recurrences behind Eqs. 6-7
+//                                 before the transfer relation; exact arithmetic gives the VRR +
+//                                 HRR values)
+//   quadrature (Eq. 8)            summed over the roots in R and over primitives in FP64 (in the
+//                                 output or the scratch)
+// Compressed output (Sec. II-D) then takes one more launch over the FP64 values (pack_kernel of
+// eri_contract.cu).
 #include <algorithm>
 #include <vector>
 
@@ -28,11 +28,13 @@ namespace eri {
 namespace {
 
 constexpr int kGenThreads = 256;
-constexpr int kGenAcc = 8;  // outputs per thread summed over primitives in registers
-// B, C values per (quartet, root): the slots of phase_setup plus C00 relative to B and C00'
+constexpr int kGenQmax = 64;      // quartets per tile
+constexpr int kGenUnits = 128;    // units (primitive quartets) per batch
+constexpr int kGenSmem = 96 * 1024;
+// B, C values per (unit, root): the slots of phase_setup plus C00 relative to B and C00'
 // relative to D
 constexpr int kGenCB = S_N, kGenCD = S_N + 3, kGenSN = S_N + 6;
-constexpr int kGenSNP = kGenSN + 1;  // odd stride of the (quartet, root) records: distinct banks
+constexpr int kGenSNP = kGenSN + 1;  // odd stride of the (unit, root) records: distinct banks
 
 // geometry without the choice of transfer direction (the four-index recursion needs none)
 struct GenGeo {
@@ -43,15 +45,21 @@ struct GenShape {
     int L[4];        // canonical angular momenta
     int n[4];        // Cartesian components per shell
     int nrys, neri;  // roots, ERIs per quartet
-    int iblk;        // 2-D integrals per (root, axis): (La+1)(Lb+1)(Lc+1)(Ld+1)
-    int iblkp;       // their stride in shared memory, odd so that the blocks the threads of a
-                     // warp build start in distinct banks
-    int q;           // quartets per CTA
-    int bc_off, i_off, smem;  // dynamic shared memory layout (bytes)
+    int iblkp;       // stride of the (La+1)(Lb+1)(Lc+1)(Ld+1) integrals of a (unit, root, axis), odd
+                     // so that the blocks the lanes of a warp build start in distinct banks
+    int lanes;       // lanes per (unit, root, axis): (La+1)(Lb+1) rounded up to a power of two
+    int q;           // quartets per tile
+    int units;       // units per batch
+    unsigned m_neri, m_ncd;  // ceil(2^32 / d) for n_ERIQ, n_c n_d (0: d = 1)
+    int geo_off, bc_off, i_off, smem;  // dynamic shared memory layout (bytes)
 };
 
+unsigned div_magic(int d) { return d == 1 ? 0u : (unsigned)(((1ull << 32) + d - 1) / d); }
+// n / d for n d < 2^32 with the magic of d
+__device__ __forceinline__ int div_by(int n, unsigned m) { return m ? (int)__umulhi((unsigned)n, m) : n; }
+
 template <typename R>
-GenShape gen_shape(const int L[4], int qmax = 64) {
+GenShape gen_shape(const int L[4], bool contracted) {
     GenShape g{};
     for (int k = 0; k < 4; ++k) {
         g.L[k] = L[k];
@@ -59,64 +67,165 @@ GenShape gen_shape(const int L[4], int qmax = 64) {
     }
     g.nrys = (L[0] + L[1] + L[2] + L[3]) / 2 + 1;
     g.neri = g.n[0] * g.n[1] * g.n[2] * g.n[3];
-    g.iblk = (L[0] + 1) * (L[1] + 1) * (L[2] + 1) * (L[3] + 1);
-    g.iblkp = g.iblk | 1;
-    const int geo = G_N * 8, bc = g.nrys * kGenSNP * (int)sizeof(R), ib = 3 * g.nrys * g.iblkp * (int)sizeof(R);
-    const int perq = geo + bc + ib + 16;
-    // quartets per CTA: within the shared-memory budget, and (for classes of at most
-    // kGenThreads * kGenAcc outputs) few enough that the primitive sums stay in registers
-    g.q = std::max(1, std::min(qmax, (96 * 1024) / perq));
-    if (g.neri <= kGenThreads * kGenAcc) g.q = std::max(1, std::min(g.q, kGenThreads * kGenAcc / g.neri));
-    g.bc_off = g.q * geo;
-    g.i_off = ((g.bc_off + g.q * bc + 15) / 16) * 16;
-    g.smem = g.i_off + g.q * ib;
+    g.iblkp = ((L[0] + 1) * (L[1] + 1) * (L[2] + 1) * (L[3] + 1)) | 1;
+    g.lanes = 1;
+    while (g.lanes < (L[0] + 1) * (L[1] + 1)) g.lanes *= 2;
+    g.m_neri = div_magic(g.neri);
+    g.m_ncd = div_magic(g.n[2] * g.n[3]);
+    const int tab = 2 * 4 * (g.n[0] * g.n[1] + g.n[2] * g.n[3]) + 4 * (kGenUnits + 2 * kGenQmax + 2);
+    g.geo_off = (tab + 15) / 16 * 16;
+    const int perunit = G_N * 8 + g.nrys * kGenSNP * (int)sizeof(R) + 3 * g.nrys * g.iblkp * (int)sizeof(R);
+    g.units = std::max(1, std::min(kGenUnits, (kGenSmem - g.geo_off) / perunit));
+    // a tile of primitive quartets is one batch; contracted quartets have batches of their own, and
+    // short tiles keep the longest of them from holding up the end of a launch
+    g.q = contracted ? (g.neri >= 64 ? 1 : 4) : std::min(kGenQmax, g.units);
+    g.bc_off = g.geo_off + g.units * G_N * 8;
+    g.i_off = (g.bc_off + g.units * g.nrys * kGenSNP * (int)sizeof(R) + 15) / 16 * 16;
+    g.smem = g.i_off + g.units * 3 * g.nrys * g.iblkp * (int)sizeof(R);
     return g;
+}
+
+// 2-D integrals of one (unit, root, axis) by g.lanes lanes of a warp, lane (i, j) holding its value of
+// the plane (k, l).  Raising k or l takes the values of lanes (i - 1, j) and (i, j - 1) by shuffles
+// and the lane's own lower planes from registers; every index is raised with its own centre.  Every
+// lane of the warp calls it; live lanes store I(i, j, k, l) at i si + j sj + k sk + l.
+template <typename R>
+__device__ __forceinline__ void plane_recursion(const GenShape &g, const R *b, int xi, int e, bool live, R *I) {
+    const int La = g.L[0], Lb = g.L[1], Lc = g.L[2], Ld = g.L[3], nj = Lb + 1, w = g.lanes;
+    const int i = e / nj, j = e - i * nj;
+    const int sk = Ld + 1, sj = (Lc + 1) * sk, si = nj * sj;
+    const R cA = b[S_C0X + xi], cB = b[kGenCB + xi], cC = b[S_C1X + xi], cD = b[kGenCD + xi];
+    const R b00 = b[S_B00], b10 = b[S_B10], b01 = b[S_B01];
+    const R ib00 = (R)i * b00, jb00 = (R)j * b00, ib10 = (R)i * b10;
+    // the plane (0, 0): I(i, 0), then up to I(i, j) on every lane of row i
+    R lo = (R)0, v = xi == 2 ? b[S_WZ] : (R)1, mine;
+    for (int t = 1; t <= La; ++t) {
+        R n = cA * v;
+        if (t > 1) n = fma((R)(t - 1) * b10, lo, n);
+        if (t <= i) {
+            lo = v;
+            v = n;
+        }
+    }
+    mine = v;
+    lo = (R)0;
+    for (int t = 1; t <= Lb; ++t) {
+        const R u = __shfl_up_sync(0xffffffffu, v, nj, w);
+        R n = cB * v;
+        if (t > 1) n = fma((R)(t - 1) * b10, lo, n);
+        if (i > 0) n = fma(ib10, u, n);
+        lo = v;
+        v = n;
+        if (t == j) mine = n;
+    }
+    R *out = I + i * si + j * sj;
+    R p1 = (R)0, p2 = (R)0, low[kLmax + 1];  // (k-1, 0), (k-2, 0), (k-1, l)
+#pragma unroll
+    for (int l = 0; l <= kLmax; ++l) low[l] = (R)0;
+    for (int k = 0; k <= Lc; ++k, out += sk) {
+        if (k > 0) {
+            const R u = __shfl_up_sync(0xffffffffu, p1, nj, w), s = __shfl_up_sync(0xffffffffu, p1, 1, w);
+            R n = cC * p1;
+            if (k > 1) n = fma((R)(k - 1) * b01, p2, n);
+            if (i > 0) n = fma(ib00, u, n);
+            if (j > 0) n = fma(jb00, s, n);
+            mine = n;
+        }
+        p2 = p1;
+        p1 = mine;
+        if (live) out[0] = mine;
+        R q1 = mine, q2 = (R)0, below = low[0];
+        low[0] = mine;
+        const R kb01 = (R)k * b01;
+#pragma unroll
+        for (int l = 1; l <= kLmax; ++l) {
+            if (l <= Ld) {
+                const R u = __shfl_up_sync(0xffffffffu, q1, nj, w), s = __shfl_up_sync(0xffffffffu, q1, 1, w);
+                R n = cD * q1;
+                if (l > 1) n = fma((R)(l - 1) * b01, q2, n);
+                if (k > 0) n = fma(kb01, below, n);
+                if (i > 0) n = fma(ib00, u, n);
+                if (j > 0) n = fma(jb00, s, n);
+                if (live) out[l] = n;
+                q2 = q1;
+                q1 = n;
+                below = low[l];
+                low[l] = n;
+            }
+        }
+    }
 }
 
 // One tile: quartets [q0, q0 + qn) of the class of `args`, ERIs summed over primitive quartets
 // in FP64 into out[q * n_ERIQ + generic index], q = 0..qn-1 (out = the tile's first quartet).
+// The tile's primitive quartets are taken in batches of g.units, whatever quartet they belong to:
+//   geometry        one thread per unit
+//   roots, B and C  one thread per (unit, root)
+//   2-D integrals   plane_recursion, (La+1)(Lb+1) lanes per (unit, root, axis)
+//   quadrature      one thread per (quartet, output), or several that share the quartet's units
+// One primitive quartet per quartet at a time left most of the CTA idle in all but the last of these:
+// 35,000 quartets of a 40-atom molecule (K up to 6, FP32) from the work queue 133 -> 12.8 ms; the 369
+// classes with a g shell, 2^20 ERIs each, 16-bit codes 45 -> 38 ms (11.0 ms with the classes spread
+// over side streams).  Bound by shared-memory reads: three per root and output for two operations.
 // Every thread of the CTA calls it; it begins and ends with a barrier.
 template <typename R>
 __device__ __forceinline__ void generic_tile(const ShellsDev &sh, const Tables &tb, const ClassArgs &args,
                                              const GenShape &g, long long q0, int qn, double *__restrict__ out,
-                                             unsigned char *smem, int &maxprim_s) {
-    double *geo_s = reinterpret_cast<double *>(smem);
+                                             unsigned char *smem) {
+    const int nab = g.n[0] * g.n[1], ncd = g.n[2] * g.n[3];
+    // per (a, b) and (c, d): offsets of the components in a block along the three axes (10 bits
+    // each; they add without carry) and the position in the caller's order
+    unsigned *off_s = reinterpret_cast<unsigned *>(smem);
+    int *pos_s = reinterpret_cast<int *>(off_s + nab + ncd);
+    int *uq_s = pos_s + nab + ncd;        // quartet of each unit of the batch
+    int *first_s = uq_s + kGenUnits;      // first unit of each quartet of the tile; [qn] = units
+    double *geo_s = reinterpret_cast<double *>(smem + g.geo_off);
     R *bc_s = reinterpret_cast<R *>(smem + g.bc_off);
     R *I_s = reinterpret_cast<R *>(smem + g.i_off);
     const int tid = threadIdx.x;
     const int La = g.L[0], Lb = g.L[1], Lc = g.L[2], Ld = g.L[3];
-    // strides of I(i, j, k, l) within one (root, axis) block
     const int sk = Ld + 1, sj = (Lc + 1) * sk, si = (Lb + 1) * sj;
-    const bool in_regs = qn * g.neri <= kGenThreads * kGenAcc;
-    double acc[kGenAcc];
-#pragma unroll
-    for (int k = 0; k < kGenAcc; ++k) acc[k] = 0.0;
+    auto shells_of = [&](int q) {
+        const int4 gq = args.quartets[q0 + q];
+        return make_int4(pick(gq, args.perm[0]), pick(gq, args.perm[1]), pick(gq, args.perm[2]), pick(gq, args.perm[3]));
+    };
     __syncthreads();
-    if (tid == 0) maxprim_s = 1;
+    for (int t = tid; t < nab + ncd; t += kGenThreads) {
+        const bool bra = t < nab;
+        const int e = bra ? t : t - nab, n2 = bra ? g.n[1] : g.n[3];
+        const int e1 = e / n2, e2 = e - e1 * n2;
+        const int l1 = bra ? La : Lc, l2 = bra ? Lb : Ld, s1 = bra ? si : sk, s2 = bra ? sj : 1;
+        unsigned o = 0;
+        for (int x = 0; x < 3; ++x) o |= (unsigned)(c_cart[l1][e1][x] * s1 + c_cart[l2][e2][x] * s2) << (10 * x);
+        off_s[t] = o;
+        pos_s[t] = e1 * args.ostride[bra ? 0 : 2] + e2 * args.ostride[bra ? 1 : 3];
+    }
+    if (tid == 0) first_s[0] = 0;
+    for (int q = tid; q < qn; q += kGenThreads) {
+        const int4 qt = shells_of(q);
+        first_s[q + 1] = sh.nprim[qt.x] * sh.nprim[qt.y] * sh.nprim[qt.z] * sh.nprim[qt.w];
+    }
     __syncthreads();
-    for (int prim = 0; prim < maxprim_s; ++prim) {
-        // A0: geometry of primitive quartet `prim` of each quartet
-        for (int q = tid; q < g.q; q += kGenThreads) {
-            double *geo = geo_s + q * G_N;
-            int np = 0;
-            if (q < qn) {
-                const int4 gq = args.quartets[q0 + q];
-                const int4 qt = make_int4(pick(gq, args.perm[0]), pick(gq, args.perm[1]),
-                                          pick(gq, args.perm[2]), pick(gq, args.perm[3]));
-                geometry_of<GenGeo>(sh, args, qt, prim, geo, np);
-            } else {
-                geo[G_PREF] = 0.0;
-                geo[G_T] = 0.0;
-                for (int s = G_P; s < G_N; ++s)
-                    geo[s] = (s == G_P || s == G_Q || s == G_IP || s == G_IQ) ? 1.0 : (s == G_IPQ ? 0.5 : 0.0);
+    if (tid == 0)
+        for (int q = 0; q < qn; ++q) first_s[q + 1] += first_s[q];
+    __syncthreads();
+    const int total = first_s[qn];
+    for (int ub = 0; ub < total; ub += g.units) {
+        const int nu = min(g.units, total - ub);
+        for (int i = tid; i < nu; i += kGenThreads) {
+            int lo = 0, hi = qn - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) / 2;
+                if (first_s[mid] <= ub + i) lo = mid; else hi = mid - 1;
             }
-            if (prim == 0 && np > 1) atomicMax(&maxprim_s, np);
+            int np = 0;
+            geometry_of<GenGeo>(sh, args, shells_of(lo), ub + i - first_s[lo], geo_s + i * G_N, np);
+            uq_s[i] = lo;
         }
         __syncthreads();
-        // A1: root and weight, B and C of each (quartet, root)
-        for (int it = tid; it < g.q * g.nrys; it += kGenThreads) {
-            const int q = it / g.nrys, mu = it - q * g.nrys;
-            const double *geo = geo_s + q * G_N;
+        for (int it = tid; it < nu * g.nrys; it += kGenThreads) {
+            const int u = it / g.nrys, mu = it - u * g.nrys;
+            const double *geo = geo_s + u * G_N;
             double x, w;
             rys_root<sizeof(R) == 4>(tb, g.nrys, mu, geo[G_T], x, w);
             R *b = bc_s + (size_t)it * kGenSNP;
@@ -135,97 +244,42 @@ __device__ __forceinline__ void generic_tile(const ShellsDev &sh, const Tables &
             b[S_WZ] = to_r<R>(geo[G_PREF] * w);
         }
         __syncthreads();
-        // B: I(i, j, k, l) of each (quartet, root, axis), every index raised with its own centre
-        for (int it = tid; it < g.q * g.nrys * 3; it += kGenThreads) {
-            const int q = it / (g.nrys * 3), r = it - q * g.nrys * 3;
-            const int mu = r / 3, xi = r - mu * 3;
-            const R *b = bc_s + (size_t)(q * g.nrys + mu) * kGenSNP;
-            R *I = I_s + (size_t)it * g.iblkp;  // block (q, mu, xi): consecutive threads, odd stride
-            const R cA = b[S_C0X + xi], cB = b[kGenCB + xi], cC = b[S_C1X + xi], cD = b[kGenCD + xi];
-            const R b00 = b[S_B00], b10 = b[S_B10], b01 = b[S_B01];
-            I[0] = xi == 2 ? b[S_WZ] : (R)1;
-            for (int i = 1; i <= La; ++i) {
-                R v = cA * I[(i - 1) * si];
-                if (i > 1) v = fma((R)(i - 1) * b10, I[(i - 2) * si], v);
-                I[i * si] = v;
-            }
-            for (int j = 1; j <= Lb; ++j)
-                for (int i = 0; i <= La; ++i) {
-                    const int e = i * si + j * sj;
-                    R v = cB * I[e - sj];
-                    if (j > 1) v = fma((R)(j - 1) * b10, I[e - 2 * sj], v);
-                    if (i > 0) v = fma((R)i * b10, I[e - si - sj], v);
-                    I[e] = v;
-                }
-            for (int k = 1; k <= Lc; ++k)
-                for (int i = 0; i <= La; ++i)
-                    for (int j = 0; j <= Lb; ++j) {
-                        const int e = i * si + j * sj + k * sk;
-                        R v = cC * I[e - sk];
-                        if (k > 1) v = fma((R)(k - 1) * b01, I[e - 2 * sk], v);
-                        if (i > 0) v = fma((R)i * b00, I[e - si - sk], v);
-                        if (j > 0) v = fma((R)j * b00, I[e - sj - sk], v);
-                        I[e] = v;
-                    }
-            for (int l = 1; l <= Ld; ++l)
-                for (int k = 0; k <= Lc; ++k)
-                    for (int i = 0; i <= La; ++i)
-                        for (int j = 0; j <= Lb; ++j) {
-                            const int e = i * si + j * sj + k * sk + l;
-                            R v = cD * I[e - 1];
-                            if (l > 1) v = fma((R)(l - 1) * b01, I[e - 2], v);
-                            if (k > 0) v = fma((R)k * b01, I[e - sk - 1], v);
-                            if (i > 0) v = fma((R)i * b00, I[e - si - 1], v);
-                            if (j > 0) v = fma((R)j * b00, I[e - sj - 1], v);
-                            I[e] = v;
-                        }
+        const int groups = nu * g.nrys * 3, nij = (La + 1) * (Lb + 1);
+        for (int it = tid; it - (tid & 31) < groups * g.lanes; it += kGenThreads) {
+            const int r = it / g.lanes, e = it % g.lanes;
+            const bool live = r < groups && e < nij;
+            const int m = r < groups ? r : 0;  // lanes past the last group repeat the first (not stored)
+            plane_recursion<R>(g, bc_s + (size_t)(m / 3) * kGenSNP, m % 3, e < nij ? e : 0, live,
+                               I_s + (size_t)m * g.iblkp);
         }
         __syncthreads();
-        // D: quadrature of each (quartet, output); primitive quartets summed in FP64, in the
-        // thread's registers when the tile has at most kGenAcc outputs per thread (the same
-        // outputs every primitive), else in `out`
-        const bool last = prim + 1 == maxprim_s;
-        auto quad = [&](int it, double *&dst) -> R {
-            const int q = it / g.neri, o = it - q * g.neri;
-            int t = o;
-            const int id = t % g.n[3];
-            t /= g.n[3];
-            const int ic = t % g.n[2];
-            t /= g.n[2];
-            const int ib = t % g.n[1], ia = t / g.n[1];
-            int off[3];
-            for (int x = 0; x < 3; ++x)
-                off[x] = c_cart[La][ia][x] * si + c_cart[Lb][ib][x] * sj + c_cart[Lc][ic][x] * sk +
-                         c_cart[Ld][id][x];
-            const R *I0 = I_s + (size_t)q * g.nrys * 3 * g.iblkp;
-            const R *Ix = I0 + off[0], *Iy = I0 + g.iblkp + off[1], *Iz = I0 + 2 * g.iblkp + off[2];
-            const int ms = 3 * g.iblkp;  // next root
-            R s = (R)0;
-            for (int mu = 0; mu < g.nrys; ++mu) s = fma(Ix[mu * ms] * Iy[mu * ms], Iz[mu * ms], s);
-            dst = out + q * (long long)g.neri + ia * args.ostride[0] + ib * args.ostride[1] + ic * args.ostride[2] +
-                  id * args.ostride[3];
-            return s;
-        };
-        if (in_regs) {
-#pragma unroll
-            for (int k = 0; k < kGenAcc; ++k) {
-                const int it = tid + k * kGenThreads;
-                if (it < qn * g.neri) {
-                    double *dst;
-                    acc[k] += RTraits<R>::to_f64(quad(it, dst));
-                    if (last) {
-                        *dst = acc[k];
-                        if (!(fabs(acc[k]) <= 1.7976931348623157e308)) atomicOr(args.err, 1);
-                    }
-                }
+        // quadrature: `parts` neighbouring lanes share the units of one (quartet, output)
+        const int qa = uq_s[0], nseg = uq_s[nu - 1] - qa + 1, ms = 3 * g.iblkp;
+        int parts = 1;
+        while (parts < 32 && 2 * parts * nseg * g.neri <= kGenThreads && 2 * parts * nseg <= nu) parts *= 2;
+        const int items = nseg * g.neri * parts;
+        for (int it = tid; it - (tid & 31) < items; it += kGenThreads) {
+            const bool on = it < items;
+            const int t = on ? it / parts : 0, part = it & (parts - 1);
+            const int seg = div_by(t, g.m_neri), o = t - seg * g.neri, q = qa + seg;
+            const int ab = div_by(o, g.m_ncd), cd = o - ab * ncd;
+            const unsigned off = off_s[ab] + off_s[nab + cd];
+            const int u0 = max(first_s[q] - ub, 0), u1 = on ? min(first_s[q + 1] - ub, nu) : 0;
+            double sum = 0.0;
+            for (int u = u0 + part; u < u1; u += parts) {
+                const R *I0 = I_s + (size_t)u * g.nrys * ms;
+                const R *Ix = I0 + (off & 1023u), *Iy = I0 + g.iblkp + ((off >> 10) & 1023u),
+                        *Iz = I0 + 2 * g.iblkp + (off >> 20);
+                R s = (R)0;
+                for (int mu = 0; mu < g.nrys; ++mu, Ix += ms, Iy += ms, Iz += ms) s = fma(*Ix * *Iy, *Iz, s);
+                sum += RTraits<R>::to_f64(s);
             }
-        } else {
-            for (int it = tid; it < qn * g.neri; it += kGenThreads) {
-                double *dst;
-                const R s = quad(it, dst);
-                const double v = (prim == 0 ? 0.0 : *dst) + RTraits<R>::to_f64(s);
-                *dst = v;
-                if (last && !(fabs(v) <= 1.7976931348623157e308)) atomicOr(args.err, 1);
+            for (int d = parts / 2; d > 0; d >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, d, parts);
+            if (on && part == 0) {
+                double *dst = out + (long long)q * g.neri + pos_s[ab] + pos_s[nab + cd];
+                if (first_s[q] < ub) sum += *dst;
+                *dst = sum;
+                if (first_s[q + 1] <= ub + nu && !(fabs(sum) <= 1.7976931348623157e308)) atomicOr(args.err, 1);
             }
         }
         __syncthreads();
@@ -236,50 +290,9 @@ template <typename R>
 __global__ void __launch_bounds__(kGenThreads)
 eri_generic_kernel(ShellsDev sh, Tables tb, ClassArgs args, GenShape g, double *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int maxprim_s;
     const long long q0 = (long long)blockIdx.x * g.q;
     const int qn = (int)((args.nq - q0) < g.q ? (args.nq - q0) : g.q);
-    generic_tile<R>(sh, tb, args, g, q0, qn, out + q0 * (long long)g.neri, smem, maxprim_s);
-}
-
-// eps = b_max / (2^(bits-1) - 1) of each quartet (Eq. 9), b_max from the FP64 values; one warp
-// per quartet
-__global__ void generic_scales_kernel(const double *__restrict__ v, long long nq, int neri, int bits,
-                                      float *__restrict__ scales) {
-    const long long q = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / 32;
-    const int lane = threadIdx.x & 31;
-    if (q >= nq) return;
-    const double *x = v + q * neri;
-    double m = 0.0;
-    for (int i = lane; i < neri; i += 32) m = fmax(m, fabs(x[i]));
-    for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
-    if (lane == 0) scales[q] = (float)(m / (double)((1u << (bits - 1)) - 1u));
-}
-
-// n-bit codes q = ANINT(x / eps) (Eq. 10), clamped to +-(2^(bits-1) - 1), packed LSB first: one
-// thread per output word gathers the (parts of the) codes that fall in it; words past the last
-// code are zero
-__global__ void generic_pack_kernel(const double *__restrict__ v, long long nvals, int neri, int bits,
-                                    const float *__restrict__ scales, uint32_t *__restrict__ packed,
-                                    long long nwords) {
-    const double M = (double)((1u << (bits - 1)) - 1u);
-    const uint32_t mask = (1u << bits) - 1u;
-    for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < nwords;
-         w += (long long)gridDim.x * blockDim.x) {
-        const long long b0 = w * 32;
-        const long long first = b0 / bits, lastc = (b0 + 31) / bits;
-        uint32_t word = 0u;
-        for (long long c = first; c <= lastc && c < nvals; ++c) {
-            const float eps = scales[c / neri];
-            const double inv = eps > 0.0f ? 1.0 / (double)eps : 0.0;
-            double r = round(v[c] * inv);
-            r = r > M ? M : (r < -M ? -M : r);
-            const uint32_t code = (uint32_t)(int)r & mask;
-            const long long s = c * bits - b0;
-            word |= s >= 0 ? code << s : code >> (-s);
-        }
-        packed[w] = word;
-    }
+    generic_tile<R>(sh, tb, args, g, q0, qn, out + q0 * (long long)g.neri, smem);
 }
 
 template <typename R>
@@ -315,20 +328,17 @@ struct QueueClass {
     long long first_tile;  // first tile of the class in the queue
 };
 
-constexpr int kQueueQmax = 128;
-
 template <typename R>
 __global__ void __launch_bounds__(kGenThreads)
 eri_queue_kernel(ShellsDev sh, Tables tb, const QueueClass *__restrict__ classes, int n_classes,
                  long long n_tiles, unsigned long long *counter, double *__restrict__ scratch,
                  long long slot_doubles, int bits, int *err) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int maxprim_s;
     __shared__ long long item_s;
     __shared__ int cls_s;
-    __shared__ unsigned long long bmax_s[kQueueQmax];
-    __shared__ float eps_s[kQueueQmax];
-    const int tid = threadIdx.x;
+    __shared__ unsigned long long bmax_s[kGenQmax];
+    __shared__ double inv_s[kGenQmax];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double *vals = scratch + (long long)blockIdx.x * slot_doubles;
     const double M = (double)((1u << (bits - 1)) - 1u);
     const uint32_t mask = (1u << bits) - 1u;
@@ -350,44 +360,44 @@ eri_queue_kernel(ShellsDev sh, Tables tb, const QueueClass *__restrict__ classes
         const GenShape g = qc.g;
         const long long q0 = (item - qc.first_tile) * g.q;
         const int qn = (int)((a.nq - q0) < g.q ? (a.nq - q0) : g.q);
-        generic_tile<R>(sh, tb, a, g, q0, qn, vals, smem, maxprim_s);
-        // b_max per quartet (non-negative IEEE values order like their bit patterns)
+        generic_tile<R>(sh, tb, a, g, q0, qn, vals, smem);
+        // b_max per quartet (non-negative IEEE values order like their bit patterns): all warps on
+        // a large quartet, a warp per small one
         for (int q = tid; q < qn; q += kGenThreads) bmax_s[q] = 0ull;
         __syncthreads();
-        for (int it = tid; it < qn * g.neri; it += kGenThreads) {
-            const double v = fabs(vals[it]);
-            if (!(v <= 1.7976931348623157e308)) atomicOr(err, 1);
-            atomicMax(bmax_s + it / g.neri, (unsigned long long)__double_as_longlong(v));
+        const int wstep = g.neri >= 512 ? kGenThreads : 32, wfirst = g.neri >= 512 ? tid : lane;
+        for (int q = g.neri >= 512 ? 0 : warp; q < qn; q += g.neri >= 512 ? 1 : kGenThreads / 32) {
+            unsigned long long m = 0ull;
+            for (int o = wfirst; o < g.neri; o += wstep)
+                m = max(m, (unsigned long long)__double_as_longlong(fabs(vals[(long long)q * g.neri + o])));
+            for (int d = 16; d > 0; d >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, d));
+            if (lane == 0) atomicMax(bmax_s + q, m);
         }
         __syncthreads();
         for (int q = tid; q < qn; q += kGenThreads) {
             const float e = (float)(__longlong_as_double((long long)bmax_s[q]) / M);
-            eps_s[q] = e;
+            inv_s[q] = e > 0.0f ? 1.0 / (double)e : 0.0;
             a.scales[q0 + q] = e;
         }
         __syncthreads();
-        // codes of the tile's values [c0, c1) at stream bits [c0 * bits, c1 * bits)
-        const long long c0 = q0 * g.neri, c1 = (q0 + qn) * (long long)g.neri;
-        const long long b0 = c0 * bits, b1 = c1 * bits;
-        for (long long w = (b0 >> 5) + tid; w < ((b1 + 31) >> 5); w += kGenThreads) {
-            const long long wb = w * 32;
-            long long first = wb / bits, last = (wb + 31) / bits;
-            first = first < c0 ? c0 : first;
-            last = last >= c1 ? c1 - 1 : last;
+        // the tile's words of the stream, positions relative to the tile's first bit
+        const long long bit0 = q0 * g.neri * bits, bit1 = (q0 + qn) * (long long)g.neri * bits;
+        const long long w0 = bit0 >> 5;
+        const int head = (int)(bit0 & 31), nw = (int)(((bit1 + 31) >> 5) - w0), nv = qn * g.neri;
+        for (int w = tid; w < nw; w += kGenThreads) {
+            const int b0 = w * 32 - head;
+            int c = b0 <= 0 ? 0 : (int)((unsigned)b0 / (unsigned)bits);
             uint32_t word = 0u;
-            for (long long c = first; c <= last; ++c) {
-                const float e = eps_s[(c - c0) / g.neri];
-                const double inv = e > 0.0f ? 1.0 / (double)e : 0.0;
-                double r = round(vals[c - c0] * inv);
+            for (int s = c * bits - b0; s < 32 && c < nv; ++c, s += bits) {
+                double r = round(vals[c] * inv_s[div_by(c, g.m_neri)]);
                 r = r > M ? M : (r < -M ? -M : r);
                 const uint32_t code = (uint32_t)(int)r & mask;
-                const long long sh_ = c * bits - wb;
-                word |= sh_ >= 0 ? code << sh_ : code >> (-sh_);
+                word |= s >= 0 ? code << s : code >> (-s);
             }
-            if (wb >= b0 && wb + 32 <= b1)
-                a.packed[w] = word;
+            if (b0 >= 0 && b0 + 32 <= nv * bits)
+                a.packed[w0 + w] = word;
             else
-                atomicOr(a.packed + w, word);
+                atomicOr(a.packed + w0 + w, word);
         }
         __syncthreads();
     }
@@ -396,7 +406,7 @@ eri_queue_kernel(ShellsDev sh, Tables tb, const QueueClass *__restrict__ classes
 }  // namespace
 
 cudaError_t launch_queue(const ShellsDev &sh, const Tables &tb, const QueueSpec *classes, int n_classes,
-                         bool mixed, int bits, int *err, void *d_table, unsigned long long *d_counter,
+                         bool mixed, bool contracted, int bits, int *err, void *d_table, unsigned long long *d_counter,
                          double *scratch, size_t scratch_bytes, int device, cudaStream_t stream) {
     if (n_classes <= 0) return cudaSuccess;
     std::vector<QueueClass> qc(n_classes);
@@ -405,7 +415,7 @@ cudaError_t launch_queue(const ShellsDev &sh, const Tables &tb, const QueueSpec 
     long long slot = 1;
     for (int i = 0; i < n_classes; ++i) {
         qc[i].a = classes[i].a;
-        qc[i].g = mixed ? gen_shape<float>(classes[i].L, kQueueQmax) : gen_shape<double>(classes[i].L, kQueueQmax);
+        qc[i].g = mixed ? gen_shape<float>(classes[i].L, contracted) : gen_shape<double>(classes[i].L, contracted);
         qc[i].first_tile = tiles;
         tiles += (classes[i].a.nq + qc[i].g.q - 1) / qc[i].g.q;
         smem = std::max(smem, qc[i].g.smem);
@@ -434,9 +444,10 @@ cudaError_t launch_queue(const ShellsDev &sh, const Tables &tb, const QueueSpec 
 size_t queue_table_bytes() { return (size_t)kNumClassIds * sizeof(QueueClass); }
 
 cudaError_t launch_generic(const ShellsDev &sh, const Tables &tb, const ClassArgs &a, const int L[4],
-                           bool mixed, double *scratch, size_t scratch_bytes, cudaStream_t stream) {
+                           bool mixed, bool contracted, double *scratch, size_t scratch_bytes,
+                           cudaStream_t stream) {
     if (a.nq <= 0) return cudaSuccess;
-    const GenShape g = mixed ? gen_shape<float>(L) : gen_shape<double>(L);
+    const GenShape g = mixed ? gen_shape<float>(L, contracted) : gen_shape<double>(L, contracted);
     if (g.smem > 227 * 1024) return cudaErrorInvalidValue;
     if (a.out_fp64)
         return mixed ? run_values<float>(sh, tb, a, g, a.out_fp64, stream)
@@ -450,15 +461,11 @@ cudaError_t launch_generic(const ShellsDev &sh, const Tables &tb, const ClassArg
         cudaError_t e = mixed ? run_values<float>(sh, tb, ac, g, scratch, stream)
                               : run_values<double>(sh, tb, ac, g, scratch, stream);
         if (e != cudaSuccess) return e;
-        generic_scales_kernel<<<(unsigned)((ac.nq * 32 + 255) / 256), 256, 0, stream>>>(
-            scratch, ac.nq, g.neri, a.bits, a.scales + c0);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const long long w0 = c0 * g.neri * a.bits / 32;
-        const long long nw = (c0 + ac.nq == a.nq) ? a.seg_words - w0 : ac.nq * g.neri * a.bits / 32;
-        const long long blocks = std::min<long long>((nw + 255) / 256, 152LL * 16);
-        generic_pack_kernel<<<(unsigned)std::max<long long>(1, blocks), 256, 0, stream>>>(
-            scratch, ac.nq * g.neri, g.neri, a.bits, a.scales + c0, a.packed + w0, nw);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        ac.packed = a.packed + w0;
+        ac.scales = a.scales + c0;
+        ac.seg_words = (c0 + ac.nq == a.nq) ? a.seg_words - w0 : ac.nq * g.neri * a.bits / 32;
+        if ((e = pack_values(ac, g.neri, scratch, stream)) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
@@ -467,13 +474,12 @@ int generic_launches(long long nq, int neri, bool compressed, size_t scratch_byt
     if (nq <= 0) return 0;
     if (!compressed) return 1;
     const long long chunk = chunk_quartets(neri, scratch_bytes);
-    return chunk > 0 ? 3 * (int)((nq + chunk - 1) / chunk) : 0;
+    return chunk > 0 ? 2 * (int)((nq + chunk - 1) / chunk) : 0;
 }
 
 const char *generic_kernel_names(bool mixed, bool compressed) {
     if (compressed)
-        return mixed ? "eri_generic_kernel<float> + generic_scales_kernel + generic_pack_kernel"
-                     : "eri_generic_kernel<double> + generic_scales_kernel + generic_pack_kernel";
+        return mixed ? "eri_generic_kernel<float> + pack_kernel<double>" : "eri_generic_kernel<double> + pack_kernel<double>";
     return mixed ? "eri_generic_kernel<float>" : "eri_generic_kernel<double>";
 }
 

@@ -52,7 +52,8 @@ inline bool class_has_g(int cls) { return cls >= 256; }
 // scratch_bytes / (8 n_ERIQ) quartets at a time).  mixed: FP32 recurrences and quadrature from
 // FP64 setup values, FP64 sums over primitives.
 cudaError_t launch_generic(const ShellsDev &sh, const Tables &tb, const ClassArgs &a, const int L[4],
-                           bool mixed, double *scratch, size_t scratch_bytes, cudaStream_t stream);
+                           bool mixed, bool contracted, double *scratch, size_t scratch_bytes,
+                           cudaStream_t stream);
 // launches launch_generic makes for nq quartets of n_ERIQ = neri, and the kernel names
 int generic_launches(long long nq, int neri, bool compressed, size_t scratch_bytes);
 const char *generic_kernel_names(bool mixed, bool compressed);
@@ -68,7 +69,7 @@ struct QueueSpec {
 };
 size_t queue_table_bytes();
 cudaError_t launch_queue(const ShellsDev &sh, const Tables &tb, const QueueSpec *classes, int n_classes,
-                         bool mixed, int bits, int *err, void *d_table, unsigned long long *d_counter,
+                         bool mixed, bool contracted, int bits, int *err, void *d_table, unsigned long long *d_counter,
                          double *scratch, size_t scratch_bytes, int device, cudaStream_t stream);
 
 // Quartets per launch of the split setup/recurrence path (a multiple of 32 so that every chunk
@@ -131,6 +132,10 @@ cudaError_t unit_setup(const ShellsDev &sh, const Tables &tb, const ClassArgs &a
 // state to the next span through `carry` (4 n_ERIQ values, halves used in turn by `parity`).
 cudaError_t unit_contract(const ClassArgs &a, bool mixed, int neri, const UnitSpan &span, void *values,
                           void *carry, int parity, cudaStream_t s);
+
+// Compressed output of a.nq whole quartets from their FP64 values (values[q * n_ERIQ]); a.seg_words
+// covers the words from a.packed on.
+cudaError_t pack_values(const ClassArgs &a, int neri, const double *values, cudaStream_t s);
 
 // One class of a plan's compressed output, as the Coulomb/exchange digestion reads it.
 struct DigestClass {

@@ -527,7 +527,7 @@ eri_status_t launch_class_args(eri_plan_s *p, int cls, const ClassArgs &a, int v
             cudaError_t e = ensure_scratch(p);
             if (e != cudaSuccess) return cuda_status(e);
         }
-        return cuda_status(launch_generic(sh, p->tables, a, L, variant != 0,
+        return cuda_status(launch_generic(sh, p->tables, a, L, variant != 0, is_contracted(p),
                                           reinterpret_cast<double *>(static_cast<char *>(p->d_setup) + sl.index * slice_bytes),
                                           slice_bytes, stream));
     }
@@ -1361,7 +1361,8 @@ eri_status_t eri_compute_compressed_queue(eri_plan_t plan, int32_t bits, void *d
         off += packed_segment_bytes(plan->count[c], class_neri(c), bits);
     }
     ShellsDev sh{plan->d_cx, plan->d_cy, plan->d_cz, plan->d_pofs, plan->d_nprim, plan->d_exps, plan->d_cn};
-    e = launch_queue(sh, plan->tables, spec.data(), (int)spec.size(), plan->precision == ERI_MIXED, bits,
+    e = launch_queue(sh, plan->tables, spec.data(), (int)spec.size(), plan->precision == ERI_MIXED,
+                     is_contracted(plan), bits,
                      plan->d_err, plan->d_queue,
                      reinterpret_cast<unsigned long long *>(static_cast<char *>(plan->d_queue) + table),
                      static_cast<double *>(plan->d_setup), kScratchBytes, plan->device, s);
