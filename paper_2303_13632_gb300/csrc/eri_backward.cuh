@@ -40,55 +40,9 @@
 // in mixed precision 115 -> 17.0 ms, 384 in FP64 220 -> 59.4 ms.
 #pragma once
 
-#include "eri_rows.cuh"
+#include "eri_kernels.cuh"
 
 namespace eri {
-
-// Values of N consecutive elements at a 16-byte (or narrower, for short blocks) boundary.
-template <int N, int V, typename R>
-__device__ __forceinline__ void load_block(const R *p, R (&x)[N]) {
-    if constexpr (sizeof(R) == 4 && V == 4) {
-#pragma unroll
-        for (int t = 0; t < N; t += 4) {
-            const float4 v = *reinterpret_cast<const float4 *>(p + t);
-            x[t] = v.x;
-            if (t + 1 < N) x[t + 1] = v.y;
-            if (t + 2 < N) x[t + 2] = v.z;
-            if (t + 3 < N) x[t + 3] = v.w;
-        }
-    } else if constexpr (V == 2) {
-        using T = std::conditional_t<sizeof(R) == 4, float2, double2>;
-#pragma unroll
-        for (int t = 0; t < N; t += 2) {
-            const T v = *reinterpret_cast<const T *>(p + t);
-            x[t] = v.x;
-            if (t + 1 < N) x[t + 1] = v.y;
-        }
-    } else {
-#pragma unroll
-        for (int t = 0; t < N; ++t) x[t] = p[t];
-    }
-}
-template <int N, int V, typename R>
-__device__ __forceinline__ void store_block(R *p, const R (&x)[N]) {
-    if constexpr (sizeof(R) == 4 && V == 4) {
-#pragma unroll
-        for (int t = 0; t < N; t += 4)
-            *reinterpret_cast<float4 *>(p + t) = make_float4(x[t], t + 1 < N ? x[t + 1] : 0.0f,
-                                                             t + 2 < N ? x[t + 2] : 0.0f, t + 3 < N ? x[t + 3] : 0.0f);
-    } else if constexpr (V == 2) {
-#pragma unroll
-        for (int t = 0; t < N; t += 2) {
-            if constexpr (sizeof(R) == 4)
-                *reinterpret_cast<float2 *>(p + t) = make_float2(x[t], t + 1 < N ? x[t + 1] : 0.0f);
-            else
-                *reinterpret_cast<double2 *>(p + t) = make_double2(x[t], t + 1 < N ? x[t + 1] : 0.0);
-        }
-    } else {
-#pragma unroll
-        for (int t = 0; t < N; ++t) p[t] = x[t];
-    }
-}
 
 template <int La_, int Lb_, int Lc_, int Ld_, typename R_>
 struct GCfg {
@@ -100,13 +54,10 @@ struct GCfg {
     static constexpr bool SWAB_OK = false, SWCD_OK = false;
     static constexpr int S_CB = S_N, S_CD = S_N + 3, SN = S_N + 6;
     static constexpr int NI = La + 1, NJ = Lb + 1, NK = Lc + 1, NL = Ld + 1, JL = NJ * NL;
-    // (j, l) blocks: 16-byte vectors, an odd number of them (the blocks of a quarter warp start in
-    // distinct banks)
-    static constexpr int VJ = JL == 1 ? 1 : (sizeof(R) == 8 || JL == 2 ? 2 : 4);
-    static constexpr int JP0 = (JL + VJ - 1) / VJ * VJ;
-    static constexpr int JP = (VJ > 1 && JL > 2 && (JP0 / VJ) % 2 == 0) ? JP0 + VJ : JP0;
+    using IB_ = JBlock<JL, NK, (int)sizeof(R)>;
+    static constexpr int VJ = IB_::V, JP = IB_::P;
     static constexpr int AC = NI * NK;
-    static constexpr int IB = AC * JP;  // 2-D integrals per (root, axis)
+    static constexpr int IR = IB_::ROW, IB = NI * IR;  // 2-D integrals per row and per (root, axis)
     static constexpr int THREADS = 256;
     // outputs (G values) per thread of step 2
     static constexpr int BCH = imax(1, imin(NB, (sizeof(R) == 8 ? 18 : 50) / ND));
@@ -186,19 +137,6 @@ __device__ __forceinline__ void w_chunk(const typename C::R (&g)[C::BCH][C::ND],
     }
 }
 
-// f(std::integral_constant<int, CH>) for the run-time chunk ch
-template <class C, int CH = 0, class F>
-__device__ __forceinline__ void with_chunk(int ch, F f) {
-    if constexpr (CH + 1 >= C::NCH) {
-        f(std::integral_constant<int, CH>{});
-    } else {
-        if (ch == CH)
-            f(std::integral_constant<int, CH>{});
-        else
-            with_chunk<C, CH + 1>(ch, f);
-    }
-}
-
 template <class C>
 __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables &tb, const ClassArgs &args,
                                                const GradUnits &un, const double *__restrict__ G,
@@ -231,10 +169,11 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
     // step 2: (group, root of the pass, a, c, chunk); step 3: (group, axis, root of the pass, i0, i2)
     const int wg = tid / C::WT, wr = tid - wg * C::WT;
     const int wmu = wr / C::ACN, witem = wr - wmu * C::ACN;
-    const int wch = witem % C::NCH, wc = (witem / C::NCH) % C::NC, wa = witem / (C::NCH * C::NC);
+    // the chunk is the slowest part of an item, so that most warps run the code of one chunk
+    const int wch = witem / (C::NA * C::NC), wc = witem % C::NC, wa = (witem / C::NC) % C::NA;
     int wo[3];
 #pragma unroll
-    for (int x = 0; x < 3; ++x) wo[x] = (c_cart[C::La][wa % C::NA][x] * C::NK + c_cart[C::Lc][wc][x]) * JP;
+    for (int x = 0; x < 3; ++x) wo[x] = c_cart[C::La][wa][x] * C::IR + c_cart[C::Lc][wc][x] * JP;
     R g[C::BCH][C::ND];
     int gq = -1;  // the quartet whose G the thread holds
     const int sg = tid / C::ST, sx = (tid - sg * C::ST) / C::SEG, se = (tid - sg * C::ST) % C::SEG;
@@ -309,10 +248,10 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
             for (int it = tid; it < cdiv(RITEMS, 32) * 32; it += T) {
                 const int blk = it / NIP, i = it % NIP;
                 const int gu = blk / (3 * C::NRYS);
-                const bool live = it < RITEMS && i < C::NI && u0 + gu < nu;
+                const bool live = it < RITEMS && u0 + gu < nu;
                 // lanes without a unit repeat the first one (in range, not stored)
                 const int r = live ? blk - gu * 3 * C::NRYS : 0, unit = live ? u0 + gu : u0;
-                rows_direct<C, JP>(bc_s + (unit * C::NRYS + r / 3) * C::SN, r % 3, i, live,
+                rows_direct<C, typename C::IB_, NIP>(bc_s + (unit * C::NRYS + r / 3) * C::SN, r % 3, i, live,
                                    I_s + (live ? gu : 0) * C::I_VALS + ((r % 3) * C::NRYS + r / 3) * C::IB);
             }
             __syncthreads();
@@ -321,7 +260,7 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                 const int q = meta_s[(u0 + wg) * 8];
                 if (q != gq) {
                     gq = q;
-                    with_chunk<C>(wch, [&](auto ch) {
+                    with_chunk<C::NCH>(wch, [&](auto ch) {
                         load_g<C, decltype(ch)::value>(G + (long long)q * C::NERI, args, wa, wc, g);
                     });
                 }
@@ -343,7 +282,7 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                     load_block<JL, C::VJ>(Iu + 2 * C::NRYS * C::IB + wo[2], Z);
 #pragma unroll
                     for (int t = 0; t < JL; ++t) WX[t] = WY[t] = WZ[t] = (R)0;
-                    with_chunk<C>(wch, [&](auto ch) { w_chunk<C, decltype(ch)::value>(g, X, Y, Z, WX, WY, WZ); });
+                    with_chunk<C::NCH>(wch, [&](auto ch) { w_chunk<C, decltype(ch)::value>(g, X, Y, Z, WX, WY, WZ); });
                     R *Wu = W_s + wg * C::W_VALS + (wmu * C::ACN + witem) * JP;
                     store_block<JL, C::VJ>(Wu, WX);
                     store_block<JL, C::VJ>(Wu + C::RG * C::ACN * JP, WY);
@@ -362,9 +301,9 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                         const int ra = sx == 0 ? C::La - si : si + na, za = sx == 0 ? na : (sx == 1 ? ra - si : si);
                         for (int nc = 0; nc <= C::Lc - sk; ++nc) {
                             const int rc = sx == 0 ? C::Lc - sk : sk + nc, zc = sx == 0 ? nc : (sx == 1 ? rc - sk : sk);
-                            const R *p = Wu + ((ra * (ra + 1) / 2 + za) * C::NC + rc * (rc + 1) / 2 + zc) * C::NCH * JP;
+                            const R *p = Wu + ((ra * (ra + 1) / 2 + za) * C::NC + rc * (rc + 1) / 2 + zc) * JP;
 #pragma unroll
-                            for (int ch = 0; ch < C::NCH; ++ch, p += JP) {
+                            for (int ch = 0; ch < C::NCH; ++ch, p += C::NA * C::NC * JP) {
                                 R v[JL];
                                 load_block<JL, C::VJ>(p, v);
 #pragma unroll
@@ -372,7 +311,7 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                             }
                         }
                     }
-                    const R *Ib = I_s + sg * C::I_VALS + (sx * C::NRYS + m0 + smu) * C::IB + (si * C::NK + sk) * JP;
+                    const R *Ib = I_s + sg * C::I_VALS + (sx * C::NRYS + m0 + smu) * C::IB + si * C::IR + sk * JP;
                     const R fi = (R)si, fk = (R)sk;
                     R S0 = (R)0, Sa = (R)0, Sb = (R)0, Sc = (R)0, Sd = (R)0, DD = (R)0, DK = (R)0, KK = (R)0;
                     R v[JL];
@@ -392,7 +331,7 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                     if constexpr (C::La > 0) {
                         if (si > 0) {
                             R s = (R)0, sb = (R)0, sd = (R)0;
-                            load_block<JL, C::VJ>(Ib - C::NK * JP, v);
+                            load_block<JL, C::VJ>(Ib - C::IR, v);
 #pragma unroll
                             for (int j = 0; j < C::NJ; ++j)
 #pragma unroll
@@ -433,11 +372,11 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                         return s;
                     };
                     if constexpr (C::La > 1)
-                        if (si > 1) DD = fma(fi * (fi - (R)1), dot(Ib - 2 * C::NK * JP), DD);
+                        if (si > 1) DD = fma(fi * (fi - (R)1), dot(Ib - 2 * C::IR), DD);
                     if constexpr (C::Lc > 1)
                         if (sk > 1) KK = fma(fk * (fk - (R)1), dot(Ib - 2 * JP), KK);
                     if constexpr (C::La > 0 && C::Lc > 0)
-                        if (si > 0 && sk > 0) DK = fma(fi * fk, dot(Ib - (C::NK + 1) * JP), DK);
+                        if (si > 0 && sk > 0) DK = fma(fi * fk, dot(Ib - C::IR - JP), DK);
                     const R *b = bc_s + ((u0 + sg) * C::NRYS + m0 + smu) * C::SN;
                     const R b00 = b[S_B00], b10 = b[S_B10], b01 = b[S_B01];
                     const R SD = Sa + Sb, SK = Sc + Sd;

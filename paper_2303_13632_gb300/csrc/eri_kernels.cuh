@@ -30,6 +30,8 @@
 // recurrences and quadrature, Kahan-compensated sums over primitives).
 #pragma once
 
+#include <type_traits>
+
 #include "eri_device.cuh"
 
 namespace eri {
@@ -67,6 +69,119 @@ __host__ __device__ constexpr int imax(int a, int b) { return a > b ? a : b; }
 __host__ __device__ constexpr int bch_fit(int nanc, int nb, int b) {
     while (b < nb && nanc * cdiv(nb, b) > 1024) ++b;
     return b;
+}
+
+constexpr int kStagePad = 32;  // staged codes ahead of and behind a tile's (read by edge words, masked)
+
+__host__ __device__ constexpr int pow2ceil(int n) { return n <= 1 ? 1 : 2 * pow2ceil((n + 1) / 2); }
+
+// (j, l) blocks of 2-D integrals in shared memory, moved as vectors: V values per access (16 bytes
+// where the block is long enough), P values from one block (i, k) to the next k, ROW from one i to
+// the next.  Both are an odd number of vectors, so that the vectors of a quarter warp (the rows that
+// rows_direct stores, the blocks that the quadrature loads) fall into distinct banks: with scalar
+// stores and rows of a multiple of 32 values, [fd|fd] spent 48 of 110 million shared-memory
+// wavefronts on store conflicts.
+template <int JL, int NK, int BYTES>
+struct JBlock {
+    static constexpr int V = JL == 1 ? 1 : (BYTES == 8 || JL == 2 ? 2 : 4);
+    static constexpr int odd(int n) { return V > 1 && JL > 2 && (n / V) % 2 == 0 ? n + V : n; }
+    static constexpr int P = odd((JL + V - 1) / V * V);
+    static constexpr int ROW = odd(NK * P);
+};
+
+// N consecutive values at a boundary of V values.
+template <int N, int V, typename R>
+__device__ __forceinline__ void load_block(const R *p, R *x) {
+    if constexpr (sizeof(R) == 4 && V == 4) {
+#pragma unroll
+        for (int t = 0; t < N; t += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(p + t);
+            x[t] = v.x;
+            if (t + 1 < N) x[t + 1] = v.y;
+            if (t + 2 < N) x[t + 2] = v.z;
+            if (t + 3 < N) x[t + 3] = v.w;
+        }
+    } else if constexpr (V == 2) {
+        using T = std::conditional_t<sizeof(R) == 4, float2, double2>;
+#pragma unroll
+        for (int t = 0; t < N; t += 2) {
+            const T v = *reinterpret_cast<const T *>(p + t);
+            x[t] = v.x;
+            if (t + 1 < N) x[t + 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < N; ++t) x[t] = p[t];
+    }
+}
+
+// N values to consecutive elements at a boundary of V values (up to V - 1 more are written).
+template <int N, int V, typename R>
+__device__ __forceinline__ void store_block(R *p, const R *x) {
+    if constexpr (sizeof(R) == 4 && V == 4) {
+#pragma unroll
+        for (int t = 0; t < N; t += 4)
+            *reinterpret_cast<float4 *>(p + t) = make_float4(x[t], t + 1 < N ? x[t + 1] : 0.0f,
+                                                             t + 2 < N ? x[t + 2] : 0.0f, t + 3 < N ? x[t + 3] : 0.0f);
+    } else if constexpr (V == 2) {
+#pragma unroll
+        for (int t = 0; t < N; t += 2) {
+            if constexpr (sizeof(R) == 4)
+                *reinterpret_cast<float2 *>(p + t) = make_float2(x[t], t + 1 < N ? x[t + 1] : 0.0f);
+            else
+                *reinterpret_cast<double2 *>(p + t) = make_double2(x[t], t + 1 < N ? x[t + 1] : 0.0);
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < N; ++t) p[t] = x[t];
+    }
+}
+
+// The low 16 bits (up to 22 where fewer than 23 are kept) are those of round_half_away(x) in two's
+// complement, x = v * inv below 2^22 in magnitude, without conversion instructions: |x| + 1/2 and the
+// addition of 2^23 both round toward zero, so the low bits of the sum are floor(|x| + 1/2).
+__device__ __forceinline__ uint32_t code_of(float v, float inv) {
+    const float x = __fmul_rn(v, inv);
+    const uint32_t n = __float_as_uint(__fadd_rz(__fadd_rz(fabsf(x), 0.5f), 8388608.0f));
+    const uint32_t s = (uint32_t)(__float_as_int(x) >> 31);
+    return (n ^ s) - s;
+}
+
+// v << n, 0 from n = 32 on
+__device__ __forceinline__ uint32_t shl(uint32_t v, int n) {
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
+    return r;
+}
+
+// max(m, |a|, |b|), NaN if one is
+__device__ __forceinline__ float max3_abs(float m, float a, float b) {
+    float r;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(a), "f"(b));
+    return r;
+}
+
+// n elements of `size` bytes (1, 2 or 4) from shared to global memory, both at the same offset from
+// a 16-byte boundary: whole vectors, and single elements at the ends.
+template <int T>
+__device__ __forceinline__ void copy_out(unsigned char *dst, const unsigned char *src, int n, int size) {
+    const int bytes = n * size;
+    int lead = (int)(-reinterpret_cast<uintptr_t>(dst) & 15);
+    lead = lead < bytes ? lead : bytes;
+    const int vecs = (bytes - lead) / 16, tail = lead + 16 * vecs;
+    for (int i = threadIdx.x; i < vecs; i += T)
+        reinterpret_cast<uint4 *>(dst + lead)[i] = reinterpret_cast<const uint4 *>(src + lead)[i];
+    // at most 15 bytes at either end
+    const int e = threadIdx.x * size;
+    const int o = e < lead ? e : tail + (e - lead);
+    if (o < bytes && (e < lead || o >= tail)) {
+        if (size == 4)
+            *reinterpret_cast<uint32_t *>(dst + o) = *reinterpret_cast<const uint32_t *>(src + o);
+        else if (size == 2)
+            *reinterpret_cast<uint16_t *>(dst + o) = *reinterpret_cast<const uint16_t *>(src + o);
+        else
+            dst[o] = src[o];
+    }
 }
 
 // ids[k] of an int4 without dynamic register indexing.
@@ -152,6 +267,33 @@ struct Cfg {
     static constexpr int OFF_H = OFF_U;
     static constexpr int OFF_I = OFF_U + Q * H_BYTES;
     static constexpr int SMEM = OFF_U + ((Q * UNION_BYTES + 16 + 15) / 16) * 16 + 16;
+    // the tile of rows_kernel (DIRECT classes): a thread takes all outputs of one a where they fit
+    // its registers (ROW_C), else of one (a, c) and a chunk of b
+    using RB = JBlock<JL, Lc + 1, (int)sizeof(R)>;
+    static constexpr int RIB = (La + 1) * RB::ROW;  // 2-D integrals per (root, axis)
+    static constexpr int ROW_OUT = 40;
+    static constexpr bool ROW_C = NB * NC * ND <= ROW_OUT;
+    static constexpr int ROW_NCH = ROW_C ? 1 : cdiv(NB, imax(1, imin(NB, ROW_OUT / ND)));
+    static constexpr int ROW_BCH = cdiv(NB, ROW_NCH);
+    static constexpr int ROW_ITEMS = ROW_C ? NA : NA * NC * ROW_NCH;
+    static constexpr int ROW_BC = NRYS * SN * 4, ROW_I = 3 * NRYS * RIB * 4;
+    static constexpr int ROW_Q = imin(64, imax(1, imin(256 / ROW_ITEMS, (56 * 1024) / (2 * ROW_BC + ROW_I + NERI * 2))));
+    static constexpr int ROW_THREADS = imax(128, cdiv(ROW_Q * ROW_ITEMS, 32) * 32);
+    // lanes per (quartet, root, axis) of rows_direct: the smallest number that occupies three tenths
+    // of the CTA and leaves a lane at most nine values of a plane (sixteen without l planes)
+    static constexpr bool nip_ok(int n) {
+        return ROW_Q * NRYS * 3 * n * 10 >= 3 * ROW_THREADS && cdiv(La + 1, n) * (Lb + 1) <= (Ld > 0 ? 9 : 16);
+    }
+    static constexpr int NIP = nip_ok(1) ? 1 : (nip_ok(2) && La > 0 ? 2 : pow2ceil(La + 1));
+    static constexpr int ROW_OFF_I = (2 * ROW_Q * ROW_BC + 15) / 16 * 16;
+    static constexpr int ROW_OFF_BMAX = ROW_OFF_I + (ROW_Q * ROW_I + 15) / 16 * 16;
+    static constexpr int ROW_OFF_STAGE = ROW_OFF_BMAX + (ROW_Q * 4 + 15) / 16 * 16;
+    // staged codes (bytes, halfwords or words, kStagePad of them ahead) or FP32 values (bits = 0)
+    static constexpr int row_smem(int bits) {
+        return ROW_OFF_STAGE + (ROW_Q * NERI + 2 * kStagePad) * (bits == 0 || bits > 16 ? 4 : (bits == 8 ? 1 : 2)) + 16;
+    }
+    // registers for three resident CTAs of 256 threads
+    static constexpr int ROW_MINB = imax(1, 65536 / (ROW_THREADS * 84));
     // values per quartet written by the separate setup kernel (K = 1 plans)
     static constexpr int SETUP_GEO = 8;  // AB, CD, swab, swcd
     static constexpr int SETUP_FIELDS = SETUP_GEO + NRYS * SN;
@@ -610,87 +752,119 @@ __device__ __forceinline__ void phase_vrr(const typename C::R *bc, const typenam
 //   I(i, j, k, l+1) = C00'_D I(l) + l B01 I(l-1) + k B01 I(k-1, l) + (i I(i-1) + j I(j-1)) B00
 // where C00_X = (P - X) - q x / (p+q) (P - Q), C00'_Y = (Q - Y) + p x / (p+q) (P - Q).
 // Exact arithmetic gives the VRR + HRR values; in FP32 no step subtracts transferred
-// values of a larger magnitude, so the rounding is not amplified.  The (i, j) plane of the
-// current (k, l) is kept in registers, lower planes are read back from the I block already
-// written (a small register footprint next to the accumulators of phase D).
-template <class C>
-__device__ __forceinline__ void phase_direct(const typename C::R *bc, int mu, int xi,
-                                             typename C::R *Iq) {
+// values of a larger magnitude, so the rounding is not amplified.
+//
+// The block is built by NIP neighbouring lanes, lane g holding RPL = (La + 1) / NIP (rounded up) rows
+// i = g RPL.. of all j.  Raising k or l needs row i - 1 (the lane's own, or one shuffle per value for
+// its first row) and the rows of lower planes, which stay in registers: a plane costs no
+// shared-memory read and its values are independent.  Through shared memory one thread per (quartet,
+// root, axis) walked (La+1)(Lb+1)(Lc+1)(Ld+1) dependent steps: for [ff|ff] 21 busy threads of 224
+// and 256 steps per quartet.  One lane per block needs the fewest instructions, more lanes the
+// shortest time: NIP is the smallest that occupies three tenths of the CTA (Cfg::NIP).
+//
+// C: La..Ld, R, S_CB, S_CD (the slots of C00 on B and C00' on D).  b: the B, C record of the root;
+// xi: axis; g: the lane of the group; blk: the block of (quartet, root, axis) in the layout B (a
+// JBlock); live: the lane stores its rows.  Every lane of the warp calls it.
+// Each value is formed by the operations of axis_direct in their order.
+template <class C, class B, int NIP>
+__device__ __forceinline__ void rows_direct(const typename C::R *b, int xi, int g, bool live,
+                                            typename C::R *blk) {
     using R = typename C::R;
-    constexpr int NI = C::La + 1, NJ = C::Lb + 1;
-    const R *b = bc + mu * C::SN;
+    constexpr int NI = C::La + 1, NJ = C::Lb + 1, NK = C::Lc + 1, NL = C::Ld + 1, RPL = cdiv(NI, NIP);
     const R cA = b[S_C0X + xi], cC = b[S_C1X + xi];
     R cB = (R)0, cD = (R)0;
     if constexpr (C::Lb > 0) cB = b[C::S_CB + xi];
     if constexpr (C::Ld > 0) cD = b[C::S_CD + xi];
     const R b00 = b[S_B00], b10 = b[S_B10], b01 = b[S_B01];
-    R *blk = Iq + i_index<C>(xi, mu, 0, 0, 0, 0);
-    // plane (k, l) = (0, 0)
-    R pl[NI][NJ];
-    pl[0][0] = (xi == 2) ? b[S_WZ] : (R)1;
+    const int i0 = g * RPL;  // first row
+    // row i - 1 at j of the plane p: the lane's own row, or the last one of the lane before
+    auto below = [&](const R (&p)[RPL][NJ], int r, int j) -> R {
+        if (r > 0) return p[r - 1][j];
+        if constexpr (NIP == 1)
+            return (R)0;
+        else
+            return __shfl_up_sync(0xffffffffu, p[RPL - 1][j], 1, NIP);
+    };
+    // i (integer) times f for row r, and whether i > 0
+    R ib00[RPL], ib10[RPL];
 #pragma unroll
-    for (int i = 1; i < NI; ++i)
-        pl[i][0] = i > 1 ? fma((R)(i - 1) * b10, pl[i - 2][0], cA * pl[i - 1][0]) : cA * pl[i - 1][0];
+    for (int r = 0; r < RPL; ++r) {
+        ib00[r] = (R)(i0 + r) * b00;
+        ib10[r] = (R)(i0 + r) * b10;
+    }
+    auto raised = [&](int r) { return NIP == 1 ? r > 0 : (r > 0 || i0 > 0); };
+    // plane (0, 0): I(i, 0), every lane running the chain up to its own rows, then over j
+    R pl[RPL][NJ];
+    {
+        R c[NIP * RPL];
+        c[0] = (xi == 2) ? b[S_WZ] : (R)1;
+#pragma unroll
+        for (int t = 1; t < NIP * RPL; ++t) {
+            c[t] = cA * c[t - 1];
+            if (t > 1) c[t] = fma((R)(t - 1) * b10, c[t - 2], c[t]);
+        }
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) {
+            pl[r][0] = c[r];
+#pragma unroll
+            for (int t = 1; t < NIP; ++t)
+                if (t == g) pl[r][0] = c[t * RPL + r];
+        }
+    }
 #pragma unroll
     for (int j = 1; j < NJ; ++j)
 #pragma unroll
-        for (int i = 0; i < NI; ++i) {
-            R v = cB * pl[i][j - 1];
-            if (j > 1) v = fma((R)(j - 1) * b10, pl[i][j - 2], v);
-            if (i > 0) v = fma((R)i * b10, pl[i - 1][j - 1], v);
-            pl[i][j] = v;
+        for (int r = 0; r < RPL; ++r) {
+            const R u = below(pl, r, j - 1);
+            R v = cB * pl[r][j - 1];
+            if (j > 1) v = fma((R)(j - 1) * b10, pl[r][j - 2], v);
+            if (raised(r)) v = fma(ib10[r], u, v);
+            pl[r][j] = v;
         }
+    R p1[RPL][NJ], p2[RPL][NJ], lo[NL][RPL][NJ];  // planes (k-1, 0), (k-2, 0) and (k-1, l)
 #pragma unroll
-    for (int k = 0; k <= C::Lc; ++k) {
-        if (k > 0) {
-            // raise k at l = 0 from the planes (k-1, 0) and (k-2, 0) read back from the I block
+    for (int k = 0; k < NK; ++k) {
+        R cur[NL][RPL][NJ];
 #pragma unroll
-            for (int i = 0; i < NI; ++i)
+        for (int r = 0; r < RPL; ++r)
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                if (k == 0) {
+                    cur[0][r][j] = pl[r][j];
+                    continue;
+                }
+                const R u = below(p1, r, j);
+                R v = cC * p1[r][j];
+                if (k > 1) v = fma((R)(k - 1) * b01, p2[r][j], v);
+                if (raised(r)) v = fma(ib00[r], u, v);
+                if (j > 0) v = fma((R)j * b00, p1[r][j - 1], v);
+                cur[0][r][j] = v;
+            }
+#pragma unroll
+        for (int l = 1; l < NL; ++l)
+#pragma unroll
+            for (int r = 0; r < RPL; ++r)
 #pragma unroll
                 for (int j = 0; j < NJ; ++j) {
-                    const int e = (i * (C::Lc + 1) + k) * C::JLP + j * (C::Ld + 1);
-                    R v = cC * blk[e - C::JLP];
-                    if (k > 1) v = fma((R)(k - 1) * b01, blk[e - 2 * C::JLP], v);
-                    if (i > 0) v = fma((R)i * b00, blk[e - (C::Lc + 2) * C::JLP], v);
-                    if (j > 0) v = fma((R)j * b00, blk[e - C::JLP - (C::Ld + 1)], v);
-                    pl[i][j] = v;
+                    const R u = below(cur[l - 1], r, j);
+                    R v = cD * cur[l - 1][r][j];
+                    if (l > 1) v = fma((R)(l - 1) * b01, cur[l > 1 ? l - 2 : 0][r][j], v);
+                    if (k > 0) v = fma((R)k * b01, lo[l - 1][r][j], v);
+                    if (raised(r)) v = fma(ib00[r], u, v);
+                    if (j > 0) v = fma((R)j * b00, cur[l - 1][r][j - 1], v);
+                    cur[l][r][j] = v;
                 }
-        }
 #pragma unroll
-        for (int i = 0; i < NI; ++i)
+        for (int r = 0; r < RPL; ++r) {
+            R out[NJ * NL];
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) blk[(i * (C::Lc + 1) + k) * C::JLP + j * (C::Ld + 1)] = pl[i][j];
-        if constexpr (C::Ld > 0) {
-            // raise l: the plane (k, l-1) stays in registers, (k, l-2) and (k-1, l-1) are read
-            // back from the I block (keeps the register footprint at two planes)
-            R q1[NI][NJ];
+            for (int j = 0; j < NJ; ++j) {
+                if (k > 0) p2[r][j] = p1[r][j];
+                p1[r][j] = cur[0][r][j];
 #pragma unroll
-            for (int i = 0; i < NI; ++i)
-#pragma unroll
-                for (int j = 0; j < NJ; ++j) q1[i][j] = pl[i][j];
-#pragma unroll
-            for (int l = 1; l <= C::Ld; ++l) {
-                R nw[NI][NJ];
-#pragma unroll
-                for (int i = 0; i < NI; ++i)
-#pragma unroll
-                    for (int j = 0; j < NJ; ++j) {
-                        const int e = (i * (C::Lc + 1) + k) * C::JLP + j * (C::Ld + 1) + l;
-                        R v = cD * q1[i][j];
-                        if (l > 1) v = fma((R)(l - 1) * b01, blk[e - 2], v);
-                        if (k > 0) v = fma((R)k * b01, blk[e - C::JLP - 1], v);
-                        if (i > 0) v = fma((R)i * b00, q1[i - 1][j], v);
-                        if (j > 0) v = fma((R)j * b00, q1[i][j - 1], v);
-                        nw[i][j] = v;
-                    }
-#pragma unroll
-                for (int i = 0; i < NI; ++i)
-#pragma unroll
-                    for (int j = 0; j < NJ; ++j) {
-                        blk[(i * (C::Lc + 1) + k) * C::JLP + j * (C::Ld + 1) + l] = nw[i][j];
-                        q1[i][j] = nw[i][j];
-                    }
+                for (int l = 0; l < NL; ++l) out[j * NL + l] = lo[l][r][j] = cur[l][r][j];
             }
+            if (live && i0 + r < NI) store_block<NJ * NL, B::V>(blk + (i0 + r) * B::ROW + k * B::P, out);
         }
     }
 }
@@ -876,9 +1050,10 @@ __device__ __forceinline__ void class_tile(const ClassArgs &args, long long tile
     if (has_item) {
         dq = tid / C::ITEMS_D;
         int r = tid % C::ITEMS_D;
-        da = r / (C::NC * C::NCH);
-        dc = (r / C::NCH) % C::NC;
-        dch = r % C::NCH;
+        // the chunk is the slowest part, so that most warps run the code of one chunk
+        dch = r / (C::NA * C::NC);
+        da = (r / C::NC) % C::NA;
+        dc = r % C::NC;
     }
     R acc[C::BCH][C::ND];
     {
@@ -895,21 +1070,16 @@ __device__ __forceinline__ void class_tile(const ClassArgs &args, long long tile
         }
     }
     __syncthreads();
-    // B: VRR (+ bra HRR, + ket HRR when fused), or the four-index recursion, per
-    // (quartet, root, axis)
+    // B: VRR (+ bra HRR, + ket HRR when fused) per (quartet, root, axis)
     for (int it = tid; it < C::Q * C::NRYS * 3; it += C::THREADS) {
         int q = it / (C::NRYS * 3), r = it % (C::NRYS * 3);
         int mu = r / 3, xi = r % 3;
-        if constexpr (C::DIRECT)
-            phase_direct<C>(bc_s + q * C::NRYS * C::SN, mu, xi,
-                            I_s + (size_t)q * (C::I_BYTES / sizeof(R)));
-        else
-            phase_vrr<C>(bc_s + q * C::NRYS * C::SN, rg_s + q * RG_N, mu, xi,
-                         H_s + (size_t)q * (C::H_BYTES / sizeof(R)),
-                         I_s + (size_t)q * (C::I_BYTES / sizeof(R)));
+        phase_vrr<C>(bc_s + q * C::NRYS * C::SN, rg_s + q * RG_N, mu, xi,
+                     H_s + (size_t)q * (C::H_BYTES / sizeof(R)),
+                     I_s + (size_t)q * (C::I_BYTES / sizeof(R)));
     }
     __syncthreads();
-    if constexpr (!C::FUSE_BC && !C::DIRECT) {
+    if constexpr (!C::FUSE_BC) {
         constexpr int NIJ = (C::La + 1) * (C::Lb + 1);
         for (int it = tid; it < C::Q * C::NRYS * 3 * NIJ; it += C::THREADS) {
             int q = it / (C::NRYS * 3 * NIJ), r = it % (C::NRYS * 3 * NIJ);
@@ -1090,6 +1260,276 @@ eri_class_kernel(ClassArgs args) {
     class_tile<C>(args, blockIdx.x, smem);
 }
 
+// ---------------------------------------------------------------------------------------
+// The FP32 classes of the four-index path (Cfg::DIRECT) from the setup kernel's records: each CTA
+// walks tiles of ROW_Q quartets, a grid apart, in three phases per tile:
+//   the records of the next tile are copied to shared memory (cp.async) behind all of them
+//   2-D integrals: rows_direct, (La + 1) lanes per (quartet, root, axis)
+//   quadrature: per root the thread's (b, d) blocks of I along the three axes as vector loads, then
+//     two operations per output from registers
+//   b_max (one warp maximum per quartet and warp), codes into the tile's words, whole-word stores
+// What bounds it: issue slots and shared-memory reads (3 blocks of (Lb+1)(Ld+1) values per root for
+// NB ND outputs of two operations each): the kernel issues in 57 to 70% of the cycles.  Against one
+// thread per (quartet, root, axis) for the integrals, scalar shared-memory accesses, atomics or
+// conversions per code and a new CTA per tile (16 bits): [dp|ds] 200,000 quartets 131 -> 50 us,
+// [dd|dd] 60,000 147 -> 129, [fd|fd] 40,001 327 -> 271, [ff|ff] 8,000 281 -> 165; the instructions of
+// [dp|ds] fell from 110 to 38 million, of [ff|ff] from 204 to 120.
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+template <class C>
+__device__ __forceinline__ void rows_prefetch(const ClassArgs &args, long long q0, float *bc) {
+    const int last = (int)((args.nq - q0) < C::ROW_Q ? (args.nq - q0) : C::ROW_Q) - 1;
+    const float *su = reinterpret_cast<const float *>(args.setup) + q0;
+    const int ss = (int)args.setup_stride;  // <= 2^20: 32-bit offsets
+    for (int it = threadIdx.x; it < C::ROW_Q * C::NRYS * C::SN; it += C::ROW_THREADS) {
+        const int f = it / C::ROW_Q, q = it % C::ROW_Q;
+        // quartets past the last one repeat it (computed, not stored)
+        cp_async4(bc + q * C::NRYS * C::SN + f, su + (C::SETUP_GEO + f) * ss + (q < last ? q : last));
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Quadrature of the thread's outputs.  ROW_C: those of a (acc[c][b][d]); else of (a, c) and b-chunk CH.
+template <class C, int CH>
+__device__ __forceinline__ void rows_quad(const float *Iq, int ox, int oy, int oz, float *acc) {
+    constexpr int JL = C::JL, P = C::RB::P, V = C::RB::V, LD1 = C::Ld + 1;
+    constexpr int NKB = C::ROW_C ? C::Lc + 1 : 1, NCC = C::ROW_C ? C::NC : 1;
+    constexpr int B0 = CH * C::ROW_BCH, NBC = imin(C::ROW_BCH, C::NB - B0);
+#pragma unroll
+    for (int o = 0; o < NCC * C::ROW_BCH * C::ND; ++o) acc[o] = 0.0f;
+#pragma unroll 1
+    for (int mu = 0; mu < C::NRYS; ++mu, Iq += C::RIB) {
+        float X[NKB * JL], Y[NKB * JL], Z[NKB * JL];
+#pragma unroll
+        for (int k = 0; k < NKB; ++k) {
+            load_block<JL, V>(Iq + ox + k * P, X + k * JL);
+            load_block<JL, V>(Iq + oy + k * P, Y + k * JL);
+            load_block<JL, V>(Iq + oz + k * P, Z + k * JL);
+        }
+#pragma unroll
+        for (int c = 0; c < NCC; ++c)
+#pragma unroll
+            for (int bb = 0; bb < NBC; ++bb)
+#pragma unroll
+                for (int d = 0; d < C::ND; ++d) {
+                    const int b = B0 + bb;
+                    const int kx = C::ROW_C ? cart_x(C::Lc, c) : 0, ky = C::ROW_C ? cart_y(C::Lc, c) : 0,
+                              kz = C::ROW_C ? cart_z(C::Lc, c) : 0;
+                    const float x = X[kx * JL + cart_x(C::Lb, b) * LD1 + cart_x(C::Ld, d)];
+                    const float y = Y[ky * JL + cart_y(C::Lb, b) * LD1 + cart_y(C::Ld, d)];
+                    const float z = Z[kz * JL + cart_z(C::Lb, b) * LD1 + cart_z(C::Ld, d)];
+                    const int o = (c * C::ROW_BCH + bb) * C::ND + d;
+                    acc[o] = fmaf(x * y, z, acc[o]);
+                }
+    }
+}
+
+// f(std::integral_constant<int, CH>) for the run-time chunk ch of N
+template <int N, int CH = 0, class F>
+__device__ __forceinline__ void with_chunk(int ch, F f) {
+    if constexpr (CH + 1 >= N) {
+        f(std::integral_constant<int, CH>{});
+    } else {
+        if (ch == CH)
+            f(std::integral_constant<int, CH>{});
+        else
+            with_chunk<N, CH + 1>(ch, f);
+    }
+}
+
+template <class C>
+__global__ void __launch_bounds__(C::ROW_THREADS, C::ROW_MINB)
+rows_kernel(ClassArgs args) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int T = C::ROW_THREADS, Q = C::ROW_Q, P = C::RB::P;
+    constexpr int NCC = C::ROW_C ? C::NC : 1, NOUT = NCC * C::ROW_BCH * C::ND;
+    float *bc_s = reinterpret_cast<float *>(smem);
+    float *I_s = reinterpret_cast<float *>(smem + C::ROW_OFF_I);
+    unsigned int *bmax_s = reinterpret_cast<unsigned int *>(smem + C::ROW_OFF_BMAX);
+    unsigned char *stage = smem + C::ROW_OFF_STAGE;
+    const int tid = threadIdx.x;
+    const bool has_item = tid < Q * C::ROW_ITEMS;
+    const int dq = has_item ? tid / C::ROW_ITEMS : 0, item = has_item ? tid % C::ROW_ITEMS : 0;
+    // the chunk is the slowest part of an item, so that most warps run the code of one chunk
+    const int ch = C::ROW_C ? 0 : item / (C::NA * C::NC), dc = C::ROW_C ? 0 : item % C::NC,
+              da = C::ROW_C ? item : (item / C::NC) % C::NA;
+    // block offsets of the thread's (a, c) within a (root, axis) block, and its outputs' positions
+    const int ox = c_cart[C::La][da][0] * C::RB::ROW + (C::ROW_C ? 0 : c_cart[C::Lc][dc][0]) * P;
+    const int oy = c_cart[C::La][da][1] * C::RB::ROW + (C::ROW_C ? 0 : c_cart[C::Lc][dc][1]) * P + C::NRYS * C::RIB;
+    const int oz = c_cart[C::La][da][2] * C::RB::ROW + (C::ROW_C ? 0 : c_cart[C::Lc][dc][2]) * P + 2 * C::NRYS * C::RIB;
+    // positions of the thread's outputs in the staged tile, in bytes
+    const int bits = args.bits;
+    const bool coded = args.raw == nullptr && args.out_fp64 == nullptr;
+    const int size = !coded || bits > 16 ? 4 : (bits == 8 ? 1 : 2);
+    const int st1 = args.ostride[1] * size, st2 = args.ostride[2] * size, st3 = args.ostride[3] * size;
+    const int ebase = (dq * C::NERI + da * args.ostride[0] + dc * args.ostride[2]) * size;
+    const unsigned int bits_magic = coded ? (unsigned int)(0xffffffffu / (unsigned int)bits + 1u) : 0u;
+    const unsigned int same_q = __match_any_sync(0xffffffffu, has_item ? dq : -1);
+    const bool leader = (tid & 31) == __ffs(same_q) - 1;
+    const long long tiles = (args.nq + Q - 1) / Q;
+    rows_prefetch<C>(args, blockIdx.x * (long long)Q, bc_s);
+    int buf = 0;
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf ^= 1) {
+        const long long q0 = tile * Q;
+        const int qn = (int)((args.nq - q0) < Q ? (args.nq - q0) : Q);
+        const float *bc = bc_s + buf * Q * C::NRYS * C::SN;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // the tile's records are in; the tile before is stored
+        if (tile + gridDim.x < tiles)
+            rows_prefetch<C>(args, q0 + (long long)gridDim.x * Q, bc_s + (buf ^ 1) * Q * C::NRYS * C::SN);
+        {
+            constexpr int NIP = C::NIP, ITEMS = Q * C::NRYS * 3 * NIP;
+            for (int it = tid; it < cdiv(ITEMS, 32) * 32; it += T) {
+                const int g = it % NIP, r = it / NIP;
+                const bool live = it < ITEMS;
+                const int q = live ? r / (3 * C::NRYS) : 0, m = live ? r % (3 * C::NRYS) : 0;
+                rows_direct<C, typename C::RB, NIP>(bc + (q * C::NRYS + m / 3) * C::SN, m % 3, g, live,
+                                                    I_s + ((q * 3 + m % 3) * C::NRYS + m / 3) * C::RIB);
+            }
+        }
+        if (coded)
+            for (int q = tid; q < Q; q += T) bmax_s[q] = 0u;
+        __syncthreads();
+        const bool live = has_item && dq < qn;
+        float acc[NOUT];
+        const float *Iq = I_s + dq * 3 * C::NRYS * C::RIB;
+        with_chunk<C::ROW_NCH>(ch, [&](auto k) { rows_quad<C, decltype(k)::value>(Iq, ox, oy, oz, acc); });
+        // values and whole-byte codes are staged at the offset from a 16-byte boundary that their
+        // place in memory has; other codes behind kStagePad of them
+        unsigned char *dst = nullptr;
+        if (args.raw != nullptr)
+            dst = reinterpret_cast<unsigned char *>(reinterpret_cast<float *>(args.raw) + q0 * C::NERI);
+        else if (bits == 16 || bits == 8)
+            dst = reinterpret_cast<unsigned char *>(args.packed) + q0 * C::NERI * (bits / 8);
+        unsigned char *st = stage + (dst != nullptr ? (int)(reinterpret_cast<uintptr_t>(dst) & 15) : kStagePad * size);
+        // f(output, its staged place) over the thread's outputs
+        auto outputs = [&](auto f) {
+#pragma unroll
+            for (int c = 0; c < NCC; ++c)
+#pragma unroll
+                for (int bb = 0; bb < C::ROW_BCH; ++bb) {
+                    const int b = ch * C::ROW_BCH + bb;
+                    if (b < C::NB) {
+#pragma unroll
+                        for (int d = 0; d < C::ND; ++d)
+                            f(acc[(c * C::ROW_BCH + bb) * C::ND + d], st + (ebase + c * st2 + b * st1 + d * st3));
+                    }
+                }
+        };
+        if (!coded) {
+            // values through shared memory: the outputs of a thread are strided, the tile is contiguous
+            if (live) outputs([&](float v, unsigned char *e) { *reinterpret_cast<float *>(e) = v; });
+            __syncthreads();
+            if (args.raw != nullptr) {
+                copy_out<T>(dst, st, qn * C::NERI, 4);
+            } else {
+                const float *vals = reinterpret_cast<const float *>(st);
+                double *o = args.out_fp64 + q0 * C::NERI;
+                bool bad = false;
+                for (int e = tid; e < qn * C::NERI; e += T) {
+                    bad |= !RTraits<float>::finite(vals[e]);
+                    o[e] = RTraits<float>::to_f64(vals[e]);
+                }
+                if (bad) atomicOr(args.err, 1);
+            }
+            continue;
+        }
+        // b_max: non-negative IEEE values order like their bit patterns
+        float mf = 0.0f;
+        if (live) {
+            constexpr int NV = NCC * C::ROW_BCH * C::ND;
+            // a chunk shorter than ROW_BCH leaves zeros behind its outputs
+#pragma unroll
+            for (int o = 0; o < NV; o += 2) mf = max3_abs(mf, acc[o], acc[o + 1 < NV ? o + 1 : o]);
+        }
+        unsigned int mb = __float_as_uint(mf);
+        if (mb >= 0x7f800000u) atomicOr(args.err, 1);  // inf or nan
+        mb = __reduce_max_sync(same_q, mb);
+        if (leader && live) atomicMax(bmax_s + dq, mb);
+        __syncthreads();
+        const uint32_t mask = (1u << bits) - 1u;
+        if (live) {
+            // eps = b_max / M rounded to FP32 (Eq. 9): b_max is an FP32 value and M exact
+            const float M = (float)((1u << (bits - 1)) - 1u);
+            const float eps = __uint_as_float(bmax_s[dq]) / M;
+            const float inv = eps > 0.0f ? 1.0f / eps : 0.0f;
+            if (item == 0) args.scales[q0 + dq] = eps;
+            // |x| <= M (1 + 3 2^-24), so up to 22 bits no code exceeds M; non-finite values, and an eps
+            // whose reciprocal overflows, take the checked form as well
+            if (bits > 22 || !(eps <= 3.4028234663852886e38f && inv <= 3.4028234663852886e38f)) {
+                outputs([&](float v, unsigned char *e) {
+                    float r = roundf(v * inv);
+                    r = r > M ? M : (r < -M ? -M : r);
+                    const uint32_t code = to_code<float>(r, bits) & mask;
+                    if (size == 2) *reinterpret_cast<uint16_t *>(e) = (uint16_t)code;
+                    else if (size == 1) *e = (unsigned char)code;
+                    else *reinterpret_cast<uint32_t *>(e) = code;
+                });
+            } else if (bits == 16) {
+                outputs([&](float v, unsigned char *e) { *reinterpret_cast<uint16_t *>(e) = (uint16_t)code_of(v, inv); });
+            } else if (bits == 8) {
+                outputs([&](float v, unsigned char *e) { *e = (unsigned char)code_of(v, inv); });
+            } else if (size == 2) {
+                outputs([&](float v, unsigned char *e) { *reinterpret_cast<uint16_t *>(e) = (uint16_t)(code_of(v, inv) & mask); });
+            } else {
+                outputs([&](float v, unsigned char *e) { *reinterpret_cast<uint32_t *>(e) = code_of(v, inv) & mask; });
+            }
+        }
+        const int nv = qn * C::NERI;
+        const bool last_tile = (q0 + qn) >= args.nq;
+        if (dst == nullptr && tid < 2 * kStagePad) {  // codes that an edge word reads ahead of and past the tile's
+            const int e = tid < kStagePad ? -1 - tid : nv + tid - kStagePad;
+            if (size == 2) reinterpret_cast<uint16_t *>(st)[e] = 0;
+            else reinterpret_cast<uint32_t *>(st)[e] = 0u;
+        }
+        __syncthreads();
+        const long long bit1 = (q0 + qn) * (long long)C::NERI * bits, w1 = (bit1 + 31) >> 5;
+        if (dst != nullptr) {  // whole bytes: no other tile writes them
+            copy_out<T>(dst, st, nv, size);
+            if (last_tile) {  // zeros up to the segment's end
+                const long long end = args.seg_words * 4;
+                for (long long o = (bit1 >> 3) + tid; o < w1 * 4 && o < end; o += T)
+                    reinterpret_cast<unsigned char *>(args.packed)[o] = 0;
+            }
+        } else {
+            // the tile's words, each gathered from its codes; partial edge words are merged with the
+            // neighbour tile's bits
+            const long long bit0 = q0 * (long long)C::NERI * bits, w0 = bit0 >> 5;
+            const int nw = (int)(w1 - w0), head = (int)(bit0 & 31), tail = (int)(bit1 & 31);
+            for (int w = tid; w < nw; w += T) {
+                const int b0 = w * 32 - head;  // the word's first bit, at or above -31
+                const int c = (int)__umulhi((unsigned int)(b0 + kStagePad * bits), bits_magic) - kStagePad;
+                int s = c * bits - b0;  // <= 0: the first code's place
+                uint32_t v;
+                if (size == 4) {  // 17 to 24 bits: at most three codes
+                    const uint32_t *p = reinterpret_cast<const uint32_t *>(st) + c;
+                    v = p[0] >> -s | shl(p[1], s + bits) | shl(p[2], s + 2 * bits);
+                } else {
+                    const uint16_t *p = reinterpret_cast<const uint16_t *>(st) + c;
+                    v = (uint32_t)p[0] >> -s;
+                    if (bits >= 11)  // at most four codes
+                        v |= shl(p[1], s + bits) | shl(p[2], s + 2 * bits) | shl(p[3], s + 3 * bits);
+                    else
+                        for (s += bits; s < 32; s += bits) v |= (uint32_t)*++p << s;
+                }
+                uint32_t keep = 0xffffffffu;  // bits of this word owned by this tile
+                if (w == 0 && head) keep &= ~((1u << head) - 1u);
+                if (w == nw - 1 && tail && !last_tile) keep &= (1u << tail) - 1u;
+                if (keep == 0xffffffffu) {
+                    args.packed[w0 + w] = v;
+                } else {
+                    atomicAnd(args.packed + w0 + w, ~keep);
+                    atomicOr(args.packed + w0 + w, v & keep);
+                }
+            }
+        }
+        if (last_tile)
+            for (long long w = w1 + tid; w < args.seg_words; w += T) args.packed[w] = 0u;
+    }
+}
+
 // Setup stage of the split path (primitive quartets, K = 1): one thread per quartet computes
 // the Gaussian-product geometry, the Rys roots and weights and the B, C arrays in FP64 and
 // stores them (type R) field-major, so that every thread of this kernel does FP64 work and
@@ -1108,14 +1548,16 @@ eri_setup_kernel(ShellsDev sh, Tables tb, ClassArgs args, typename C::R *out, lo
     int np = 0;
     geometry_of<C>(sh, args, qt, 0, geo, np);
     R *o = out + q;
-    o[0 * st] = to_r<R>(geo[G_ABX]);
-    o[1 * st] = to_r<R>(geo[G_ABY]);
-    o[2 * st] = to_r<R>(geo[G_ABZ]);
-    o[3 * st] = to_r<R>(geo[G_CDX]);
-    o[4 * st] = to_r<R>(geo[G_CDY]);
-    o[5 * st] = to_r<R>(geo[G_CDZ]);
-    o[6 * st] = to_r<R>(geo[G_SWAB]);
-    o[7 * st] = to_r<R>(geo[G_SWCD]);
+    if constexpr (!C::DIRECT) {  // the four-index path reads no transfer vectors
+        o[0 * st] = to_r<R>(geo[G_ABX]);
+        o[1 * st] = to_r<R>(geo[G_ABY]);
+        o[2 * st] = to_r<R>(geo[G_ABZ]);
+        o[3 * st] = to_r<R>(geo[G_CDX]);
+        o[4 * st] = to_r<R>(geo[G_CDY]);
+        o[5 * st] = to_r<R>(geo[G_CDZ]);
+        o[6 * st] = to_r<R>(geo[G_SWAB]);
+        o[7 * st] = to_r<R>(geo[G_SWCD]);
+    }
     if constexpr (sizeof(R) == 4) {
         SetupTF<C> pre;
         pre.init(geo);
@@ -1258,8 +1700,10 @@ __device__ __forceinline__ void tpq_tile(const ShellsDev &sh, const Tables &tb,
             const R *su = reinterpret_cast<const R *>(args.setup) + (q0 + tid);
             const int ss = (int)args.setup_stride;  // <= 2^20: 32-bit offsets
             R rg[RG_N];
+            if constexpr (!C::DIRECT) {
 #pragma unroll
-            for (int f = 0; f < RG_N; ++f) rg[f] = su[f * ss];
+                for (int f = 0; f < RG_N; ++f) rg[f] = su[f * ss];
+            }
 #pragma unroll 1
             for (int mu = 0; mu < C::NRYS; ++mu) {
                 R bc[C::SN];
@@ -1308,8 +1752,10 @@ __device__ __forceinline__ void tpq_tile(const ShellsDev &sh, const Tables &tb,
     const int st0 = args.ostride[0], st1 = args.ostride[1], st2 = args.ostride[2],
               st3 = args.ostride[3];
     if constexpr (FORM == TPQ_UNITS) {
+        // values through shared memory: a thread's outputs are contiguous, a warp's are not
+        R *vals = reinterpret_cast<R *>(smem);
         if (live) {
-            R *out = reinterpret_cast<R *>(args.raw) + (q0 + tid) * (long long)C::NERI;
+            R *out = vals + tid * C::NERI;
 #pragma unroll
             for (int a = 0; a < C::NA; ++a)
 #pragma unroll
@@ -1321,6 +1767,9 @@ __device__ __forceinline__ void tpq_tile(const ShellsDev &sh, const Tables &tb,
                             out[a * st0 + b * st1 + c * st2 + d * st3] =
                                 acc[((a * C::NB + b) * C::NC + c) * C::ND + d];
         }
+        __syncthreads();
+        R *o = reinterpret_cast<R *>(args.raw) + q0 * (long long)C::NERI;
+        for (int e = tid; e < qn * C::NERI; e += C::TPQ_THREADS) o[e] = vals[e];
         return;
     }
     if (args.out_fp64 != nullptr) {
@@ -1470,7 +1919,11 @@ cudaError_t launch_class(const ShellsDev &sh, const Tables &tb, const ClassArgs 
         if (tpq) {
             const unsigned tiles = (unsigned)((args.nq + C::TPQ_THREADS - 1) / C::TPQ_THREADS);
             if (args.raw) {
-                eri_tpq_kernel<C, TPQ_UNITS><<<tiles, C::TPQ_THREADS, 0, stream>>>(sh, tb, a);
+                constexpr int smem = C::TPQ_THREADS * C::NERI * (int)sizeof(R);
+                auto ku = eri_tpq_kernel<C, TPQ_UNITS>;
+                cudaError_t e = cudaFuncSetAttribute(ku, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                if (e != cudaSuccess) return e;
+                ku<<<tiles, C::TPQ_THREADS, smem, stream>>>(sh, tb, a);
                 return cudaGetLastError();
             }
             if constexpr (C::TPQ_SPLIT) {
@@ -1480,11 +1933,22 @@ cudaError_t launch_class(const ShellsDev &sh, const Tables &tb, const ClassArgs 
             }
         }
     }
-    auto k2 = eri_class_kernel<C>;
-    cudaError_t e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-    k2<<<(unsigned)((args.nq + C::Q - 1) / C::Q), C::THREADS, C::SMEM, stream>>>(a);
-    return cudaGetLastError();
+    if constexpr (C::DIRECT) {
+        auto k3 = rows_kernel<C>;
+        const int smem = C::row_smem(args.out_fp64 || args.raw ? 0 : args.bits);
+        cudaError_t e = cudaFuncSetAttribute(k3, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        // at most eight CTAs per SM: with fewer resident, the last wave stays short
+        const long long tiles = (args.nq + C::ROW_Q - 1) / C::ROW_Q;
+        k3<<<(unsigned)(tiles < 8 * 152 ? tiles : 8 * 152), C::ROW_THREADS, smem, stream>>>(a);
+        return cudaGetLastError();
+    } else {
+        auto k2 = eri_class_kernel<C>;
+        cudaError_t e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        if (e != cudaSuccess) return e;
+        k2<<<(unsigned)((args.nq + C::Q - 1) / C::Q), C::THREADS, C::SMEM, stream>>>(a);
+        return cudaGetLastError();
+    }
 }
 
 // The 55 canonical classes (Sec. II-B, Eq. 3): La >= Lb, Lc >= Ld, n_ga n_gb >= n_gc n_gd.

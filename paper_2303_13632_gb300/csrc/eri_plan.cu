@@ -1478,7 +1478,7 @@ eri_status_t eri_plan_class_kernels(eri_plan_t plan, int32_t cls, char *buf, siz
     if (g_info[k].tpq)
         name = std::string("eri_tpq_kernel<") + cfg + (units ? ", 2>" : (g_info[k].setup ? ", 1>" : ", 0>"));
     else
-        name = std::string("eri_class_kernel<") + cfg + ">";
+        name = std::string(v != 0 ? "rows_kernel<" : "eri_class_kernel<") + cfg + ">";
     if (units)
         name = "unit_setup_kernel + " + name + " + contract_kernel + pack_kernel";
     else if (g_info[k].setup)
