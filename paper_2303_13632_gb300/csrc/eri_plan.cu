@@ -674,41 +674,73 @@ eri_status_t ensure_side_streams(eri_plan_s *p) {
     return cuda_status(e);
 }
 
-// Every non-empty class on the plan's side streams (forked from and joined back into `stream`),
-// each with its slice of the scratch; the classes go to the side streams by decreasing work.
-// d_out: FP64 output, else compressed.  tuned: with the kernel choices of eri_autotune.
-eri_status_t enqueue_forked(eri_plan_s *p, double *d_out, int bits, void *d_packed, float *d_scales,
-                            bool tuned, cudaStream_t stream) {
+// Side streams that a call over all classes spreads its classes over, so that small classes share the
+// GPU and the FP64 setup of one overlaps the recurrences of another; 0: none, the classes run on the
+// caller's stream one after the other.  A primitive plan makes its side streams (and, with
+// `scratch`, its scratch) on first use, which a capture does not allow: such a call keeps to the
+// caller's stream.
+//   The 256-class sweep, 16-bit codes, on 0 / 2 / 8 streams: 2^14 ERIs per class 5.4 / 2.8 / 1.0 ms,
+// 2^21 8.9 / 6.6 / 5.6 ms, 2^23 18.3 / 19.7 / 21.6 ms, 2^24 30.5 / 34.4 / 43.8 ms; FP64 at 2^19
+// 11.3 / 7.2 / 5.3 ms.  From about 2^25 quartets on (2^23 ERIs per class are 2^25.7) every class
+// fills the GPU by itself, and several at a time only spread the random reads of the pair table.
+// Sixteen streams gain another tenth on a small contracted molecule and lose it on the sweep.
+eri_status_t fork_streams(eri_plan_s *p, cudaStream_t stream, bool scratch, int *n) {
+    *n = 0;
+    int classes = 0;
+    for (int c = 0; c < kNumClassIds; ++c) classes += p->count[c] > 0;
+    if (classes < 2 || (!is_contracted(p) && p->nq >= (1LL << 25))) return ERI_OK;
+    if (!p->join_ev[eri_plan_s::kSide - 1] || !p->fork_ev || (scratch && !p->d_setup)) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return ERI_OK;
+        eri_status_t e = ensure_side_streams(p);
+        if (e == ERI_OK && scratch) e = cuda_status(ensure_scratch(p));
+        if (e != ERI_OK) return e;
+    }
+    *n = std::min(classes, (int)eri_plan_s::kSide);
+    return ERI_OK;
+}
+
+// The plan's non-empty classes on n side streams, forked from and joined back into `stream`: run(class,
+// stream, index of the stream) in decreasing order of work, dealt out in turn.
+template <class Run>
+eri_status_t on_side_streams(eri_plan_s *p, cudaStream_t stream, int n, Run run) {
     cudaError_t e = cudaEventRecord(p->fork_ev, stream);
-    for (int i = 0; e == cudaSuccess && i < eri_plan_s::kSide; ++i)
-        e = cudaStreamWaitEvent(p->side[i], p->fork_ev, 0);
+    for (int i = 0; e == cudaSuccess && i < n; ++i) e = cudaStreamWaitEvent(p->side[i], p->fork_ev, 0);
     if (e != cudaSuccess) return cuda_status(e);
     std::vector<int> cls;
-    std::vector<size_t> off(kNumClassIds, 0);
-    size_t o = 0;
-    for (int c = 0; c < kNumClassIds; ++c) {
-        off[c] = o;
-        if (!d_out) o += packed_segment_bytes(p->count[c], class_neri(c), bits);
+    for (int c = 0; c < kNumClassIds; ++c)
         if (p->count[c] > 0) cls.push_back(c);
-    }
     auto work = [&](int c) {
         return (is_contracted(p) && !class_has_g(c) ? p->units[c] : p->count[c]) * class_neri(c);
     };
-    std::sort(cls.begin(), cls.end(), [&](int x, int y) { return work(x) > work(y); });
+    std::stable_sort(cls.begin(), cls.end(), [&](int x, int y) { return work(x) > work(y); });
     eri_status_t st = ERI_OK;
-    for (size_t i = 0; i < cls.size() && st == ERI_OK; ++i) {
-        const int c = cls[i], s = (int)(i % eri_plan_s::kSide), variant = class_variant(p, c);
-        ClassArgs a = class_args(p, c, d_out, bits, d_packed, d_scales, off[c]);
-        const int phase = tuned && !class_has_g(c) ? p->tune_phase[canonicalise(c).cls * kNumVariants + variant] : 0;
-        st = launch_class_args(p, c, a, variant, p->side[s], 0, Slice{s, eri_plan_s::kSide}, phase);
-    }
+    for (size_t i = 0; i < cls.size() && st == ERI_OK; ++i) st = run(cls[i], p->side[i % n], (int)(i % n));
     // joined also after an error: the side streams' work stays ordered before the caller's
-    for (int i = 0; i < eri_plan_s::kSide; ++i) {
+    for (int i = 0; i < n; ++i) {
         cudaError_t je = cudaEventRecord(p->join_ev[i], p->side[i]);
         if (je == cudaSuccess) je = cudaStreamWaitEvent(stream, p->join_ev[i], 0);
         if (e == cudaSuccess) e = je;
     }
     return st != ERI_OK ? st : cuda_status(e);
+}
+
+// Every class, each stream with its slice of the scratch.  d_out: FP64 output, else compressed.
+// tuned: with the kernel choices of eri_autotune.
+eri_status_t enqueue_forked(eri_plan_s *p, double *d_out, int bits, void *d_packed, float *d_scales,
+                            bool tuned, int n, cudaStream_t stream) {
+    std::vector<size_t> off(kNumClassIds, 0);
+    size_t o = 0;
+    for (int c = 0; c < kNumClassIds; ++c) {
+        off[c] = o;
+        if (!d_out) o += packed_segment_bytes(p->count[c], class_neri(c), bits);
+    }
+    return on_side_streams(p, stream, n, [&](int c, cudaStream_t s, int i) {
+        const int variant = class_variant(p, c);
+        ClassArgs a = class_args(p, c, d_out, bits, d_packed, d_scales, off[c]);
+        const int phase = tuned && !class_has_g(c) ? p->tune_phase[canonicalise(c).cls * kNumVariants + variant] : 0;
+        return launch_class_args(p, c, a, variant, s, 0, Slice{i, n}, phase);
+    });
 }
 
 }  // namespace
@@ -1156,8 +1188,10 @@ eri_status_t eri_compute(eri_plan_t plan, double *d_out, void *stream) {
     if (!plan || (!d_out && plan->nq > 0)) return ERI_E_INVALID;
     if (reinterpret_cast<uintptr_t>(d_out) % 8) return ERI_E_INVALID;
     cudaSetDevice(plan->device);
-    if (is_contracted(plan) && plan->nq > 0)
-        return enqueue_forked(plan, d_out, 0, nullptr, nullptr, false, (cudaStream_t)stream);
+    int n = 0;
+    eri_status_t fs = fork_streams(plan, (cudaStream_t)stream, true, &n);
+    if (fs != ERI_OK) return fs;
+    if (n > 0) return enqueue_forked(plan, d_out, 0, nullptr, nullptr, false, n, (cudaStream_t)stream);
     for (int c = 0; c < kNumClassIds; ++c) {
         eri_status_t s = launch_one(plan, c, d_out, 0, nullptr, nullptr, 0, (cudaStream_t)stream);
         if (s != ERI_OK) return s;
@@ -1184,8 +1218,10 @@ eri_status_t eri_compute_compressed(eri_plan_t plan, int32_t bits, void *d_packe
     if (reinterpret_cast<uintptr_t>(d_packed) % 4 || reinterpret_cast<uintptr_t>(d_scales) % 4)
         return ERI_E_INVALID;
     cudaSetDevice(plan->device);
-    if (is_contracted(plan) && plan->nq > 0)
-        return enqueue_forked(plan, nullptr, bits, d_packed, d_scales, false, (cudaStream_t)stream);
+    int n = 0;
+    eri_status_t fs = fork_streams(plan, (cudaStream_t)stream, true, &n);
+    if (fs != ERI_OK) return fs;
+    if (n > 0) return enqueue_forked(plan, nullptr, bits, d_packed, d_scales, false, n, (cudaStream_t)stream);
     size_t off = 0;
     for (int c = 0; c < kNumClassIds; ++c) {
         const int neri = class_neri(c);
@@ -1265,8 +1301,8 @@ eri_status_t eri_backward(eri_plan_t plan, const double *d_G, double *d_dR, doub
     if (e == cudaSuccess) e = cudaMemsetAsync(d_dalpha, 0, sizeof(double) * (size_t)plan->n_prims, st);
     if (e != cudaSuccess) return cuda_status(e);
     ShellsDev sh{plan->d_cx, plan->d_cy, plan->d_cz, plan->d_pofs, plan->d_nprim, plan->d_exps, plan->d_cn};
-    for (int c = 0; c < kNumClassIds; ++c) {
-        if (plan->count[c] == 0) continue;
+    const bool units = is_contracted(plan);
+    auto run = [&](int c, cudaStream_t s, int) -> eri_status_t {
         Canon cn = canonicalise(c);
         ClassArgs a{};
         for (int k = 0; k < 4; ++k) {
@@ -1278,11 +1314,16 @@ eri_status_t eri_backward(eri_plan_t plan, const double *d_G, double *d_dR, doub
         a.err = plan->d_err;
         a.pairs = plan->d_pairs;
         a.np = plan->n_prims;
-        const bool units = is_contracted(plan);
-        e = backward_of(c)(sh, plan->tables, a, units ? plan->d_pstart + plan->first[c] : nullptr,
-                           units ? plan->units[c] : plan->count[c], d_G + plan->fp64_off[c], d_dR, d_dalpha, st);
-        if (e != cudaSuccess) return cuda_status(e);
-    }
+        return cuda_status(backward_of(c)(sh, plan->tables, a, units ? plan->d_pstart + plan->first[c] : nullptr,
+                                          units ? plan->units[c] : plan->count[c], d_G + plan->fp64_off[c], d_dR,
+                                          d_dalpha, s));
+    };
+    int n = 0;
+    eri_status_t fs = fork_streams(plan, st, false, &n);
+    if (fs != ERI_OK) return fs;
+    if (n > 0) return on_side_streams(plan, st, n, run);
+    for (int c = 0; c < kNumClassIds; ++c)
+        if (plan->count[c] > 0 && (fs = run(c, st, 0)) != ERI_OK) return fs;
     return ERI_OK;
 }
 
@@ -1312,7 +1353,10 @@ eri_status_t eri_compute_compressed_batched(eri_plan_t plan, int32_t bits, void 
             cudaStreamDestroy(origin);
             return cuda_status(e);
         }
-        st = enqueue_forked(plan, nullptr, bits, d_packed, d_scales, true, origin);
+        // (the resources exist: one stream at least, for the plan's autotuned choices)
+        int n = 0;
+        st = fork_streams(plan, origin, true, &n);
+        if (st == ERI_OK) st = enqueue_forked(plan, nullptr, bits, d_packed, d_scales, true, std::max(1, n), origin);
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(origin, &g);
         cudaStreamDestroy(origin);
