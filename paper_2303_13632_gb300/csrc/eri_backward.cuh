@@ -32,12 +32,16 @@
 //      units belong to one quartet) and the (b, d) blocks of I_x, I_y, I_z at its (a, c): five
 //      operations per output for all three axes; the partial W blocks go to shared memory
 //   3  one thread per (unit, axis, root, i0, i2): sums the partial blocks over the (a, c) with these
-//      components, forms the eight sums from the neighbouring blocks of I and adds to the centre
-//      gradients in registers (compensated in FP32) until the quartet ends; the exponent terms are
-//      summed over the unit (warp shuffles, then FP64) and added to global memory.
-// Bound by issue of the FMAs and shared-memory reads of 2 and 3 in FP32, by the FP64 pipe in FP64.
-// Measured on the 16 classes of p and d shells, K = 3, forward and backward: 1024 quartets per class
-// in mixed precision 115 -> 17.0 ms, 384 in FP64 220 -> 59.4 ms.
+//      components, forms the eight sums from the neighbouring blocks of I and adds to the centre and
+//      exponent gradients in registers (compensated in FP32) until the quartet or the primitive
+//      changes; then they are summed over the segment's lanes and added to global memory in FP64.
+// Step 3 of a unit and step 1 of the next one share a barrier interval (the first from the low
+// threads up, the second from the high ones down, I in two buffers): two barriers per QG units.
+// Bound by barriers between short steps and issue in FP32 (two CTAs per SM, 35% of the issue slots),
+// by the FP64 pipe in FP64.  Measured on the 16 classes of p and d shells, K = 3, forward and backward:
+// 1024 quartets per class in mixed precision 115 -> 12.7 ms, 384 in FP64 220 -> 50.4 ms.  Sharing the
+// barrier interval of steps 3 and 1 and summing exponent terms over a primitive's units instead of
+// once per unit took these from 14.6 and 54.4 ms.
 #pragma once
 
 #include "eri_kernels.cuh"
@@ -75,7 +79,7 @@ struct GCfg {
     static constexpr int ST = 3 * SEG;
     static constexpr int I_VALS = 3 * NRYS * IB;     // per unit
     static constexpr int W_VALS = 3 * RG * ACN * JP;
-    static constexpr int UNIT_BYTES = (I_VALS + W_VALS) * (int)sizeof(R);
+    static constexpr int UNIT_BYTES = (2 * I_VALS + W_VALS) * (int)sizeof(R);
     static constexpr int QG = imax(1, imin(imin(THREADS / WT, THREADS / ST), (48 * 1024) / UNIT_BYTES));
     // units per batch of the setup stages
     static constexpr int NBU = imax(1, imin(32, THREADS / (QG * NRYS))) * QG;
@@ -83,9 +87,8 @@ struct GCfg {
     static constexpr int OFF_BC = 0;
     static constexpr int OFF_META = align16(NBU * NRYS * SN * (int)sizeof(R));
     static constexpr int OFF_EA = align16(OFF_META + NBU * 8 * 4);
-    static constexpr int OFF_RED = align16(OFF_EA + NBU * 4 * (int)sizeof(R));
-    static constexpr int OFF_I = align16(OFF_RED + QG * 3 * NSW * 5 * (int)sizeof(R));
-    static constexpr int OFF_W = align16(OFF_I + QG * I_VALS * (int)sizeof(R));
+    static constexpr int OFF_I = align16(OFF_EA + NBU * 8 * (int)sizeof(R));
+    static constexpr int OFF_W = align16(OFF_I + 2 * QG * I_VALS * (int)sizeof(R));  // I in two buffers
     // the batch's geometry is dead before steps 1 to 3 start
     static constexpr int SMEM = imax(OFF_W + QG * W_VALS * (int)sizeof(R), OFF_I + NBU * G_N * 8) + 16;
 };
@@ -146,8 +149,7 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
     extern __shared__ __align__(16) unsigned char smem[];
     R *bc_s = reinterpret_cast<R *>(smem + C::OFF_BC);
     int *meta_s = reinterpret_cast<int *>(smem + C::OFF_META);  // quartet, its four shells' primitives
-    R *ea_s = reinterpret_cast<R *>(smem + C::OFF_EA);          // 2 alpha of the four primitives
-    R *red_s = reinterpret_cast<R *>(smem + C::OFF_RED);
+    R *ea_s = reinterpret_cast<R *>(smem + C::OFF_EA);          // 2 alpha, (2L+3) / (4 alpha) of the four
     R *I_s = reinterpret_cast<R *>(smem + C::OFF_I);
     R *W_s = reinterpret_cast<R *>(smem + C::OFF_W);
     double *geo_s = reinterpret_cast<double *>(smem + C::OFF_I);
@@ -179,9 +181,34 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
     const int sg = tid / C::ST, sx = (tid - sg * C::ST) / C::SEG, se = (tid - sg * C::ST) % C::SEG;
     const bool s_on = sg < C::QG && se < C::SA;
     const int smu = se / C::AC, si = (se % C::AC) / C::NK, sk = se % C::NK;
-    R dacc[4], dcomp[4];
+    // centre gradients of the quartet (0..3) and exponent gradients (4..7), with their compensation
+    R dacc[8], dcomp[8];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) dacc[k] = dcomp[k] = (R)0;
+    for (int k = 0; k < 8; ++k) dacc[k] = dcomp[k] = (R)0;
+    auto add = [&](int k, R t) {
+        if constexpr (sizeof(R) == 4) {
+            const R y = __fsub_rn(t, dcomp[k]), n = __fadd_rn(dacc[k], y);
+            dcomp[k] = __fsub_rn(__fsub_rn(n, dacc[k]), y);
+            dacc[k] = n;
+        } else {
+            dacc[k] += t;
+        }
+    };
+    // 1: 2-D integrals of the units u0.. of the batch (nu of them) into buffer buf, by the CTA's warps
+    // from the last one down
+    auto integrals = [&](int u0, int nu, int buf) {
+        constexpr int NIP = pow2ceil(C::NI), RITEMS = C::QG * C::NRYS * 3 * NIP;
+        R *Id = I_s + buf * C::QG * C::I_VALS;
+        for (int it = (T / 32 - 1 - tid / 32) * 32 + tid % 32; it < cdiv(RITEMS, 32) * 32; it += T) {
+            const int blk = it / NIP, i = it % NIP;
+            const int gu = blk / (3 * C::NRYS);
+            const bool live = it < RITEMS && u0 + gu < nu;
+            // lanes without a unit repeat the first one (in range, not stored)
+            const int r = live ? blk - gu * 3 * C::NRYS : 0, unit = live ? u0 + gu : u0;
+            rows_direct<C, typename C::IB_, NIP>(bc_s + (unit * C::NRYS + r / 3) * C::SN, r % 3, i, live,
+                                                 Id + (live ? gu : 0) * C::I_VALS + ((r % 3) * C::NRYS + r / 3) * C::IB);
+        }
+    };
 
     for (long long ub = U0; ub < U1; ub += C::NBU) {
         const int nu = (int)min((long long)C::NBU, U1 - ub);
@@ -216,8 +243,11 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
             meta_s[i * 8] = q;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
+                constexpr int Lk[4] = {C::La, C::Lb, C::Lc, C::Ld};
+                const double al = sh.exps[pk[k]];
                 meta_s[i * 8 + 1 + k] = pk[k];
-                ea_s[i * 4 + k] = to_r<R>(2.0 * sh.exps[pk[k]]);
+                ea_s[i * 8 + k] = to_r<R>(2.0 * al);
+                ea_s[i * 8 + 4 + k] = to_r<R>((0.25 * (2 * Lk[k] + 3)) / al);
             }
         }
         __syncthreads();
@@ -241,20 +271,11 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                 b[C::S_CD + s] = to_r<R>((geo[G_QCX + s] + geo[G_CDX + s]) + fp * pq);
             }
         }
-        for (int u0 = 0; u0 < nu; u0 += C::QG) {
-            __syncthreads();  // records are written; I and W of the units before are read
-            // 1: 2-D integrals
-            constexpr int NIP = pow2ceil(C::NI), RITEMS = C::QG * C::NRYS * 3 * NIP;
-            for (int it = tid; it < cdiv(RITEMS, 32) * 32; it += T) {
-                const int blk = it / NIP, i = it % NIP;
-                const int gu = blk / (3 * C::NRYS);
-                const bool live = it < RITEMS && u0 + gu < nu;
-                // lanes without a unit repeat the first one (in range, not stored)
-                const int r = live ? blk - gu * 3 * C::NRYS : 0, unit = live ? u0 + gu : u0;
-                rows_direct<C, typename C::IB_, NIP>(bc_s + (unit * C::NRYS + r / 3) * C::SN, r % 3, i, live,
-                                   I_s + (live ? gu : 0) * C::I_VALS + ((r % 3) * C::NRYS + r / 3) * C::IB);
-            }
-            __syncthreads();
+        __syncthreads();  // records are written
+        integrals(0, nu, 0);
+        for (int u0 = 0, buf = 0; u0 < nu; u0 += C::QG, buf ^= 1) {
+            __syncthreads();  // I of these units is written, W of the units before is read
+            const R *Ic = I_s + buf * C::QG * C::I_VALS;
             const bool w_unit = wg < C::QG && u0 + wg < nu;
             if (w_unit) {
                 const int q = meta_s[(u0 + wg) * 8];
@@ -266,16 +287,13 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                 }
             }
             const bool s_unit = s_on && u0 + sg < nu;
-            R up2[4], e0 = (R)0;  // exponent terms of the unit
-#pragma unroll
-            for (int k = 0; k < 4; ++k) up2[k] = (R)0;
 #pragma unroll 1
             for (int pass = 0; pass < C::NPASS; ++pass) {
                 const int m0 = pass * C::RG;
                 if (pass > 0) __syncthreads();
                 // 2: partial W blocks
                 if (w_unit && m0 + wmu < C::NRYS) {
-                    const R *Iu = I_s + wg * C::I_VALS + (m0 + wmu) * C::IB;
+                    const R *Iu = Ic + wg * C::I_VALS + (m0 + wmu) * C::IB;
                     R X[JL], Y[JL], Z[JL], WX[JL], WY[JL], WZ[JL];
                     load_block<JL, C::VJ>(Iu + wo[0], X);
                     load_block<JL, C::VJ>(Iu + C::NRYS * C::IB + wo[1], Y);
@@ -311,57 +329,64 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                             }
                         }
                     }
-                    const R *Ib = I_s + sg * C::I_VALS + (sx * C::NRYS + m0 + smu) * C::IB + si * C::IR + sk * JP;
+                    const R *Ib = Ic + sg * C::I_VALS + (sx * C::NRYS + m0 + smu) * C::IB + si * C::IR + sk * JP;
                     const R fi = (R)si, fk = (R)sk;
                     R S0 = (R)0, Sa = (R)0, Sb = (R)0, Sc = (R)0, Sd = (R)0, DD = (R)0, DK = (R)0, KK = (R)0;
                     R v[JL];
-                    load_block<JL, C::VJ>(Ib, v);
+                    // sum of W(j, l) v(j - dj, l - dl) f(j, l) with f = 1, j, l, j (j-1), l (l-1) or j l, the
+                    // factor applied once per row or column
+                    auto over_j = [&](int dj) -> R {
+                        R s = (R)0;
 #pragma unroll
-                    for (int j = 0; j < C::NJ; ++j)
+                        for (int j = dj; j < C::NJ; ++j) {
+                            R r = (R)0;
 #pragma unroll
-                        for (int l = 0; l < C::NL; ++l) {
-                            const R w = Wb[j * C::NL + l];
-                            S0 = fma(w, v[j * C::NL + l], S0);
-                            if (j > 0) Sb = fma((R)j * w, v[(j - 1) * C::NL + l], Sb);
-                            if (l > 0) Sd = fma((R)l * w, v[j * C::NL + l - 1], Sd);
-                            if (j > 1) DD = fma((R)(j * (j - 1)) * w, v[(j - 2) * C::NL + l], DD);
-                            if (l > 1) KK = fma((R)(l * (l - 1)) * w, v[j * C::NL + l - 2], KK);
-                            if (j > 0 && l > 0) DK = fma((R)(j * l) * w, v[(j - 1) * C::NL + l - 1], DK);
+                            for (int l = 0; l < C::NL; ++l) r = fma(Wb[j * C::NL + l], v[(j - dj) * C::NL + l], r);
+                            s = dj == 0 ? s + r : fma((R)(dj == 1 ? j : j * (j - 1)), r, s);
                         }
+                        return s;
+                    };
+                    auto over_l = [&](int dl) -> R {
+                        R s = (R)0;
+#pragma unroll
+                        for (int l = dl; l < C::NL; ++l) {
+                            R r = (R)0;
+#pragma unroll
+                            for (int j = 0; j < C::NJ; ++j) r = fma(Wb[j * C::NL + l], v[j * C::NL + l - dl], r);
+                            s = fma((R)(dl == 1 ? l : l * (l - 1)), r, s);
+                        }
+                        return s;
+                    };
+                    load_block<JL, C::VJ>(Ib, v);
+                    S0 = over_j(0);
+                    if constexpr (C::NJ > 1) Sb = over_j(1);
+                    if constexpr (C::NL > 1) Sd = over_l(1);
+                    if constexpr (C::NJ > 2) DD = over_j(2);
+                    if constexpr (C::NL > 2) KK = over_l(2);
+                    if constexpr (C::NJ > 1 && C::NL > 1) {
+#pragma unroll
+                        for (int j = 1; j < C::NJ; ++j) {
+                            R r = (R)0;
+#pragma unroll
+                            for (int l = 1; l < C::NL; ++l)
+                                r = fma((R)l * Wb[j * C::NL + l], v[(j - 1) * C::NL + l - 1], r);
+                            DK = fma((R)j, r, DK);
+                        }
+                    }
                     if constexpr (C::La > 0) {
                         if (si > 0) {
-                            R s = (R)0, sb = (R)0, sd = (R)0;
                             load_block<JL, C::VJ>(Ib - C::IR, v);
-#pragma unroll
-                            for (int j = 0; j < C::NJ; ++j)
-#pragma unroll
-                                for (int l = 0; l < C::NL; ++l) {
-                                    const R w = Wb[j * C::NL + l];
-                                    s = fma(w, v[j * C::NL + l], s);
-                                    if (j > 0) sb = fma((R)j * w, v[(j - 1) * C::NL + l], sb);
-                                    if (l > 0) sd = fma((R)l * w, v[j * C::NL + l - 1], sd);
-                                }
-                            Sa = fi * s;
-                            DD = fma((R)2 * fi, sb, DD);
-                            DK = fma(fi, sd, DK);
+                            Sa = fi * over_j(0);
+                            if constexpr (C::NJ > 1) DD = fma((R)2 * fi, over_j(1), DD);
+                            if constexpr (C::NL > 1) DK = fma(fi, over_l(1), DK);
                         }
                     }
                     if constexpr (C::Lc > 0) {
                         if (sk > 0) {
-                            R s = (R)0, sb = (R)0, sd = (R)0;
                             load_block<JL, C::VJ>(Ib - JP, v);
-#pragma unroll
-                            for (int j = 0; j < C::NJ; ++j)
-#pragma unroll
-                                for (int l = 0; l < C::NL; ++l) {
-                                    const R w = Wb[j * C::NL + l];
-                                    s = fma(w, v[j * C::NL + l], s);
-                                    if (j > 0) sb = fma((R)j * w, v[(j - 1) * C::NL + l], sb);
-                                    if (l > 0) sd = fma((R)l * w, v[j * C::NL + l - 1], sd);
-                                }
-                            Sc = fk * s;
-                            KK = fma((R)2 * fk, sd, KK);
-                            DK = fma(fk, sb, DK);
+                            Sc = fk * over_j(0);
+                            if constexpr (C::NL > 1) KK = fma((R)2 * fk, over_l(1), KK);
+                            if constexpr (C::NJ > 1) DK = fma(fk, over_j(1), DK);
                         }
                     }
                     auto dot = [&](const R *p) -> R {
@@ -384,77 +409,60 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                     const R x2 = (R)2 * b00 * DK;
                     const R VP = fma(b10, fma(b10, DD, x2), b00 * b00 * KK) + b10 * S0;
                     const R VQ = fma(b01, fma(b01, KK, x2), b00 * b00 * DD) + b01 * S0;
-                    const R *ea = ea_s + (u0 + sg) * 4;
+                    const R *ea = ea_s + (u0 + sg) * 8;
                     const R cf[4] = {b[S_C0X + sx], b[C::S_CB + sx], b[S_C1X + sx], b[C::S_CD + sx]};
                     const R low[4] = {Sa, Sb, Sc, Sd};
+                    const R e0 = sx == 0 ? S0 : (R)0;  // sum over mu of e0: the quartet's energy
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const R p = k < 2 ? P : Q;
                         const R u1 = fma(cf[k], S0, p);
-                        up2[k] += fma(cf[k], u1 + p, k < 2 ? VP : VQ);
-                        const R t = fma(ea[k], u1, -low[k]);
-                        if constexpr (sizeof(R) == 4) {  // compensated over the quartet's units
-                            const R y = __fsub_rn(t, dcomp[k]), n = __fadd_rn(dacc[k], y);
-                            dcomp[k] = __fsub_rn(__fsub_rn(n, dacc[k]), y);
-                            dacc[k] = n;
-                        } else {
-                            dacc[k] += t;
-                        }
+                        add(k, fma(ea[k], u1, -low[k]));
+                        add(4 + k, fma(ea[4 + k], e0, -fma(cf[k], u1 + p, k < 2 ? VP : VQ)));
                     }
-                    if (sx == 0) e0 += S0;
                 }
             }
-            // exponent terms of the unit: over the segment, then over segments and axes in FP64
+            if (u0 + C::QG < nu) integrals(u0 + C::QG, nu, buf ^ 1);
+            // sums that end here: the exponent gradients whose primitive, and the centre gradients whose
+            // quartet is not that of the group's next unit (in this batch)
+            unsigned int ends = 0u;
+            const int *mine = meta_s + (u0 + sg) * 8;
+            if (sg < C::QG && u0 + sg < nu) {
+                const bool last = u0 + sg + C::QG >= nu;
+                const int *next = mine + C::QG * 8;
+                ends = (last || next[0] != mine[0]) ? 1u : 0u;
 #pragma unroll
-            for (int off = C::SW / 2; off > 0; off >>= 1) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) up2[k] += __shfl_down_sync(0xffffffffu, up2[k], off, C::SW);
-                e0 += __shfl_down_sync(0xffffffffu, e0, off, C::SW);
+                for (int k = 0; k < 4; ++k) ends |= (last || next[1 + k] != mine[1 + k]) ? 2u << k : 0u;
             }
-            if (sg < C::QG && se % C::SW == 0) {
-                R *r = red_s + ((sg * 3 + sx) * C::NSW + se / C::SW) * 5;
+            const unsigned int any = __reduce_or_sync(0xffffffffu, ends);
+            auto total = [&](int k, bool end) -> R {  // of the segment, on its first lane; the sum starts anew
+                R v = (R)0;
+                if (end) {
+                    v = dacc[k] - dcomp[k];
+                    dacc[k] = dcomp[k] = (R)0;
+                }
 #pragma unroll
-                for (int k = 0; k < 4; ++k) r[k] = up2[k];
-                r[4] = e0;
-            }
-            // centre gradients when the group's next unit is not of this quartet (or not of this batch)
-            const int mine = (sg < C::QG && u0 + sg < nu) ? meta_s[(u0 + sg) * 8] : -1;
-            const bool flush = mine >= 0 && (u0 + sg + C::QG >= nu || meta_s[(u0 + sg + C::QG) * 8] != mine);
-            if (__any_sync(0xffffffffu, flush)) {
-                R v[4];
+                for (int off = C::SW / 2; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off, C::SW);
+                return v;
+            };
+            const bool leader = se % C::SW == 0;
+            if (any & 1u) {
+                const bool end = ends & 1u;
+                int4 gqt = make_int4(0, 0, 0, 0);
+                if (end && leader) gqt = args.quartets[mine[0]];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    v[k] = flush ? dacc[k] - dcomp[k] : (R)0;
-#pragma unroll
-                    for (int off = C::SW / 2; off > 0; off >>= 1)
-                        v[k] += __shfl_down_sync(0xffffffffu, v[k], off, C::SW);
-                }
-                if (flush) {
-                    if (se % C::SW == 0) {
-                        const int4 gqt = args.quartets[mine];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            atomicAdd(dR + 3LL * pick(gqt, args.perm[k]) + sx, RTraits<R>::to_f64(v[k]));
-                    }
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) dacc[k] = dcomp[k] = (R)0;
+                    const R v = total(k, end);
+                    if (end && leader) atomicAdd(dR + 3LL * pick(gqt, args.perm[k]) + sx, RTraits<R>::to_f64(v));
                 }
             }
-            __syncthreads();
-            if (tid < C::QG * 4 && u0 + tid / 4 < nu) {
-                const int gu = tid / 4, k = tid % 4;
-                constexpr int Lk[4] = {C::La, C::Lb, C::Lc, C::Ld};
-                const R *r = red_s + gu * 3 * C::NSW * 5;
-                double s2 = 0.0, e = 0.0;
 #pragma unroll
-                for (int t = 0; t < 3 * C::NSW; ++t) {
-                    s2 += RTraits<R>::to_f64(r[t * 5 + k]);
-                    if (t < C::NSW) e += RTraits<R>::to_f64(r[t * 5 + 4]);
+            for (int k = 0; k < 4; ++k)
+                if (any & (2u << k)) {
+                    const bool end = ends & (2u << k);
+                    const R v = total(4 + k, end);
+                    if (end && leader) atomicAdd(dalpha + mine[1 + k], RTraits<R>::to_f64(v));
                 }
-                const int pk = meta_s[(u0 + gu) * 8 + 1 + k];
-                const int L = k == 0 ? Lk[0] : (k == 1 ? Lk[1] : (k == 2 ? Lk[2] : Lk[3]));
-                atomicAdd(dalpha + pk, (2.0 * L + 3.0) / (4.0 * sh.exps[pk]) * e - s2);
-            }
         }
     }
 }
