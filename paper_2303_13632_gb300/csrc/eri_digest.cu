@@ -23,13 +23,16 @@
 // GPU mapping: one CTA per tile of consecutive quartets of one class.  The tile's codes are decoded
 // into shared memory as FP32 integers (exact for widths <= 24) and the D blocks between the
 // quartet's four shells that the passes read are staged in FP32 (six for a symmetric D, else
-// twelve).  A thread owns one (pass, x, y) and a run of the tile's quartets: what depends on the pass
-// alone is formed once, and the values of quartets that share the destination (neighbours in a list
-// of unique quartets share their bra, many also the shell c) are summed in FP64 before they are added
-// to J and K (device atomics, so the summation order of the FP64 accumulation varies between runs).
-// One thread per (quartet, pass, x, y) spent its time on that bookkeeping and on one FP64 atomic per
-// item: 3.45 million unique quartets of s to f shells (12 atoms, 16 bits, symmetric D) 10.5 -> 8.1 ms.
+// twelve).  A warp owns a few (pass, x, y), neighbours in the list of items, and its lanes the tile's
+// quartets: the sums of a warp have the same length, what depends on the pass alone is formed once,
+// and the strides between quartets are odd, so that lanes read distinct banks.  Values with the same
+// destination (neighbours in a list of unique quartets share their bra, many also the shell c) are
+// summed in FP64 over a lane's quartets and, where all its lanes end on one destination, over the
+// lanes before they are added to J and K (device atomics, so the summation order of the FP64
+// accumulation varies between runs).  3.45 million unique quartets of s to f shells (12 atoms, 16
+// bits): 10.5 -> 6.0 ms with a symmetric D.  Bound by shared-memory reads (two per product) and issue.
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "eri_internal.h"
@@ -64,7 +67,9 @@ struct DigestArgs {
     int st[4];     // strides of the four positions in the quartet's block
     int neri;
     int T;         // quartets per tile
-    int nD;        // staged D values per quartet
+    int lanes;     // lanes of a warp over the tile's quartets (power of two); 32 / lanes items per warp
+    int se, sd;    // values per quartet in shared memory: codes, D (odd)
+    unsigned m_neri;  // ceil(2^32 / n_ERIQ): quartet of a code of the tile (0: one value per quartet)
     int nblk;      // staged D blocks
     int bx[12], by[12];  // block b holds D[x][y] of positions (bx, by)
     int boff[16];  // offset of D block (x, y) (index x*4 + y) in a quartet's D area
@@ -135,8 +140,8 @@ digest_kernel(const DigestArgs *__restrict__ args, const long long *__restrict__
     }
     __syncthreads();
     int *meta = reinterpret_cast<int *>(smem);               // T x 8: bf offsets, mask, eps
-    float *e_s = reinterpret_cast<float *>(meta + A.T * 8);  // T x neri codes
-    float *d_s = e_s + (size_t)A.T * A.neri;                 // T x nD D values
+    float *e_s = reinterpret_cast<float *>(meta + A.T * 8);  // T x se codes
+    float *d_s = e_s + (size_t)A.T * A.se;                   // T x sd D values
     const long long q0 = (tile_s & ((1LL << 40) - 1)) * A.T;
     const int tn = (int)((A.nq - q0) < A.T ? (A.nq - q0) : A.T);
     const int tid = threadIdx.x;
@@ -157,41 +162,43 @@ digest_kernel(const DigestArgs *__restrict__ args, const long long *__restrict__
     const unsigned long long bit0 = (unsigned long long)q0 * (unsigned)A.neri * (unsigned)A.bits;
     const uint32_t *words = A.packed + (bit0 >> 5);
     const int head = (int)(bit0 & 31), up = 32 - A.bits;
+    // place of the tile's value v: quartets se apart
+    const int pad = A.se - A.neri;
+    auto place = [&](int v) { return v + pad * (A.m_neri ? (int)__umulhi((unsigned)v, A.m_neri) : v); };
     if (A.bits == 16) {
         const int16_t *codes = reinterpret_cast<const int16_t *>(words) + (head >> 4);
-        for (int v = tid; v < nv; v += kDigestThreads) e_s[v] = (float)__ldg(codes + v);
+        for (int v = tid; v < nv; v += kDigestThreads) e_s[place(v)] = (float)__ldg(codes + v);
     } else {
         for (int v = tid; v < nv; v += kDigestThreads) {
             const int bit = head + v * A.bits, w = bit >> 5, off = bit & 31;
             uint32_t raw = __ldg(words + w) >> off;
             if (off + A.bits > 32) raw |= __ldg(words + w + 1) << (32 - off);
-            e_s[v] = (float)((int)(raw << up) >> up);  // sign extension
+            e_s[place(v)] = (float)((int)(raw << up) >> up);  // sign extension
         }
     }
     __syncthreads();
-    // the D blocks between the quartet's shells, D[o_x + i][o_y + j] for x != y: one thread per
-    // (quartet, block row), whose at most 10 loads are independent
+    // lane = (item of the warp, quartet)
+    const int lane = tid & 31, tl = lane & (A.lanes - 1), il = lane / A.lanes, items = 32 / A.lanes;
+    // the D blocks between the quartet's shells, D[o_x + i][o_y + j]: a block row per item, whose at
+    // most 10 loads are independent
     const int rows = A.rstart[A.nblk];
-    for (int idx = tid; idx < tn * rows; idx += kDigestThreads) {
-        const int t = idx / rows;
-        const int r = idx - t * rows;
+    for (int r = (tid >> 5) * items + il; r < rows; r += kDigestThreads / 32 * items) {
         int b = 0;
         for (int k = 1; k < A.nblk; ++k) b += r >= A.rstart[k];
         const int x = A.bx[b], y = A.by[b];
         const int i = r - A.rstart[b], ny = A.n[y];
-        const int *m = meta + t * 8;
-        const float *src = A.D + (long long)(m[x] + i) * A.nbf + m[y];
-        float *dst = d_s + t * A.nD + A.boff[x * 4 + y] + i * ny;
+        float *dst = d_s + A.boff[x * 4 + y] + i * ny;
+        for (int t = tl; t < tn; t += A.lanes) {
+            const int *m = meta + t * 8;
+            const float *src = A.D + (long long)(m[x] + i) * A.nbf + m[y];
 #pragma unroll 10
-        for (int j = 0; j < ny; ++j) dst[j] = __ldg(src + j);
+            for (int j = 0; j < ny; ++j) dst[t * A.sd + j] = __ldg(src + j);
+        }
     }
     __syncthreads();
-    // groups of threads that each cover all items, over equal runs of the tile's quartets
-    const int groups = A.NI < kDigestThreads ? min(kDigestThreads / A.NI, tn) : 1;
-    const int per = (tn + groups - 1) / groups;
-    const int grp = tid / A.NI;  // 0 where an item set needs the whole CTA
-    for (int r = A.NI < kDigestThreads ? tid - grp * A.NI : tid; r < A.NI && grp < groups;
-         r += A.NI < kDigestThreads ? A.NI : kDigestThreads) {
+    for (int r0 = (tid >> 5) * items; r0 < A.NI; r0 += kDigestThreads / 32 * items) {
+        const int r = r0 + il;
+        const bool on = r < A.NI;
         int p = 0;
 #pragma unroll
         for (int k = 1; k < 6; ++k) p += r >= A.ioff[k];
@@ -212,12 +219,11 @@ digest_kernel(const DigestArgs *__restrict__ args, const long long *__restrict__
             acc1 = acc2 = 0.0;
             pend = 0u;
         };
-        const int t1 = min(tn, (grp + 1) * per);
-        for (int t = grp * per; t < t1; ++t) {
+        for (int t = tl; on && t < tn; t += A.lanes) {
             const int *m = meta + t * 8;
             const unsigned int c = ((unsigned int)m[4] >> (4 * p)) & 15u;
             if (c == 0u) continue;
-            const float *ep = e0 + t * A.neri, *dp = d1 + t * A.nD;
+            const float *ep = e0 + t * A.se, *dp = d1 + t * A.sd, *dq = d2 + t * A.sd;
             const float eps = __int_as_float(m[5]);
             const int rw = m[x] + ix, cl = m[y] + iy;
             if (rw != row || cl != col) {
@@ -225,33 +231,48 @@ digest_kernel(const DigestArgs *__restrict__ args, const long long *__restrict__
                 row = rw;
                 col = cl;
             }
-            float S = 0.0f;
-            if constexpr (SYM) {
-                for (int iu = 0; iu < nu; ++iu, ep += su) {
-                    const float *q = ep;
-#pragma unroll 2
-                    for (int iw = 0; iw < nw; ++iw, q += sw) S = fmaf(*q, *dp++, S);
+            float S = 0.0f, S2 = 0.0f;
+            auto rows_of = [&](auto n) {  // rows of a compile-time length, in order
+                constexpr int N = decltype(n)::value;
+                for (int iu = 0; iu < nu; ++iu, ep += su, dp += N, ++dq) {
+#pragma unroll
+                    for (int iw = 0; iw < N; ++iw) {
+                        const float e = ep[iw * sw];
+                        S = fmaf(e, dp[iw], S);
+                        if constexpr (!SYM) S2 = fmaf(e, dq[iw * nu], S2);
+                    }
                 }
+            };
+            switch (nw) {
+                case 1: rows_of(std::integral_constant<int, 1>{}); break;
+                case 3: rows_of(std::integral_constant<int, 3>{}); break;
+                case 6: rows_of(std::integral_constant<int, 6>{}); break;
+                default: rows_of(std::integral_constant<int, 10>{}); break;
+            }
+            if constexpr (SYM) {
                 const float k = (float)__popc(c);
                 acc1 += f32_to_f64(S * (k * eps));
                 pend = 1u;
             } else {
-                float S2 = 0.0f;
-                const float *dq = d2 + t * A.nD;
-                for (int iu = 0; iu < nu; ++iu, ep += su, ++dq) {
-                    const float *q = ep, *dc = dq;
-#pragma unroll 2
-                    for (int iw = 0; iw < nw; ++iw, q += sw, dc += nu) {
-                        const float e = *q;
-                        S = fmaf(e, *dp++, S);
-                        S2 = fmaf(e, *dc, S2);
-                    }
-                }
                 const float v1 = ((c & 1u) ? S : 0.0f) + ((c & 2u) ? S2 : 0.0f);
                 const float v2 = ((c & 4u) ? S : 0.0f) + ((c & 8u) ? S2 : 0.0f);
                 if (c & 3u) acc1 += f32_to_f64(v1 * eps);
                 if (c & 12u) acc2 += f32_to_f64(v2 * eps);
                 pend |= ((c & 3u) ? 1u : 0u) | ((c & 12u) ? 2u : 0u);
+            }
+        }
+        // one destination over the item's lanes: one sum (lanes with nothing pending add zeros)
+        if (A.lanes > 1) {
+            const int src = lane & ~(A.lanes - 1);
+            const int row0 = __shfl_sync(0xffffffffu, row, src), col0 = __shfl_sync(0xffffffffu, col, src);
+            const bool same = pend == 0u || (row == row0 && col == col0);
+            if (__all_sync(0xffffffffu, same)) {
+                for (int off = A.lanes / 2; off > 0; off >>= 1) {
+                    acc1 += __shfl_down_sync(0xffffffffu, acc1, off, A.lanes);
+                    if constexpr (!SYM) acc2 += __shfl_down_sync(0xffffffffu, acc2, off, A.lanes);
+                    pend |= __shfl_down_sync(0xffffffffu, pend, off, A.lanes);
+                }
+                if (tl != 0) pend = 0u;
             }
         }
         flush();
@@ -346,15 +367,20 @@ cudaError_t digest_all(const DigestClass *classes, int n_classes, int bits, bool
                 A.rstart[A.nblk + 1] = A.rstart[A.nblk] + A.n[x];
                 ++A.nblk;
             }
-        A.nD = o;
+        A.se = A.neri | 1;
+        A.sd = o | 1;
         const int px[6] = {0, 2, 0, 1, 0, 1}, py[6] = {1, 3, 2, 2, 3, 3};
         A.ioff[0] = 0;
         for (int p = 0; p < 6; ++p) A.ioff[p + 1] = A.ioff[p] + A.n[px[p]] * A.n[py[p]];
         A.NI = A.ioff[6];
-        const int perq = 4 * (8 + A.neri + A.nD);
+        const int perq = 4 * (8 + A.se + A.sd);
         int T = kDigestSmem / perq;
         T = T < 1 ? 1 : (T > 128 ? 128 : T);
+        A.lanes = 1;
+        while (A.lanes < 32 && 2 * A.lanes <= T) A.lanes *= 2;
+        T = T / A.lanes * A.lanes;  // all lanes busy on every quartet of a full tile
         A.T = T;
+        A.m_neri = A.neri == 1 ? 0u : (unsigned)(((1ull << 32) + A.neri - 1) / A.neri);
         if ((size_t)T * perq > (size_t)kDigestSmem) return cudaErrorInvalidValue;
         smem_max = std::max(smem_max, (size_t)T * perq);
         start[k] = tiles;
