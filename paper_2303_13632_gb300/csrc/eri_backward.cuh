@@ -39,9 +39,10 @@
 // threads up, the second from the high ones down, I in two buffers): two barriers per QG units.
 // Bound by barriers between short steps and issue in FP32 (two CTAs per SM, 35% of the issue slots),
 // by the FP64 pipe in FP64.  Measured on the 16 classes of p and d shells, K = 3, forward and backward:
-// 1024 quartets per class in mixed precision 115 -> 12.7 ms, 384 in FP64 220 -> 50.4 ms.  Sharing the
+// 1024 quartets per class in mixed precision 115 -> 12.7 ms, 384 in FP64 220 -> 46.7 ms.  Sharing the
 // barrier interval of steps 3 and 1 and summing exponent terms over a primitive's units instead of
-// once per unit took these from 14.6 and 54.4 ms.
+// once per unit took these from 14.6 and 54.4 ms; 36 instead of 18 G values per thread in FP64 (one
+// pass over the roots of [dd|dd], no b-chunks) from 50.4.
 #pragma once
 
 #include "eri_kernels.cuh"
@@ -64,7 +65,7 @@ struct GCfg {
     static constexpr int IR = IB_::ROW, IB = NI * IR;  // 2-D integrals per row and per (root, axis)
     static constexpr int THREADS = 256;
     // outputs (G values) per thread of step 2
-    static constexpr int BCH = imax(1, imin(NB, (sizeof(R) == 8 ? 18 : 50) / ND));
+    static constexpr int BCH = imax(1, imin(NB, (sizeof(R) == 8 ? 36 : 50) / ND));
     static constexpr int NCH = cdiv(NB, BCH);
     static constexpr int ACN = NA * NC * NCH;
     // roots taken together, in passes of equal length
