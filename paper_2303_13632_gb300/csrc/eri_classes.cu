@@ -14,22 +14,6 @@
 
 namespace eri {
 
-template <class C>
-constexpr KernelInfo kernel_info() {
-    static_assert(C::SETUP_FIELDS * sizeof(typename C::R) <= kSetupFieldsMax * sizeof(double), "setup");
-    KernelInfo k{};
-    k.tpq = C::TPQ;
-    k.setup = C::USES_SETUP;
-    k.nrys = C::NRYS;
-    k.ltot = C::NAB + C::NCD;
-    k.sn = C::SN;
-    k.cb = C::DIRECT && C::Lb > 0 ? C::S_CB : 0;
-    k.cd = C::DIRECT && C::Ld > 0 ? C::S_CD : 0;
-    k.swab = C::SWAB_OK;
-    k.swcd = C::SWCD_OK;
-    return k;
-}
-
 template <int IDX>
 struct Register {
     static void apply(LaunchFn *table, KernelInfo *info) {

@@ -29,7 +29,7 @@ namespace eri {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kBatch = 32;  // units a thread of contract_kernel loads ahead of their sum
+constexpr int kBatch = 24;  // units a thread of contract_kernel loads at a time
 
 template <bool AB, bool CD>
 struct UnitGeo {
@@ -46,6 +46,33 @@ __device__ __forceinline__ int quartet_of(const long long *__restrict__ ps, long
     return lo;
 }
 
+// The same by the lanes of a warp: 32 probes at a time, so that a search of a class's quartets waits
+// for memory two or three times instead of a dozen (8 of the 19 us of a small pack_kernel).
+__device__ __forceinline__ int quartet_of_warp(const long long *__restrict__ ps, long long base, long long u,
+                                               int lo, int hi) {
+    const int lane = threadIdx.x & 31;
+    while (lo < hi) {
+        const int step = (hi - lo + 31) / 32;  // probes lo + step, lo + 2 step, .. (those above hi fail)
+        const long long at = lo + (long long)(lane + 1) * step;
+        const bool le = at <= hi && __ldg(ps + at) - base <= u;
+        const int n = __popc(__ballot_sync(0xffffffffu, le));  // the prefix sum ascends
+        const long long next = lo + (long long)(n + 1) * step - 1;
+        lo += n * step;
+        hi = next < hi ? (int)next : hi;
+    }
+    return lo;
+}
+
+// Quartets of the span's first and last unit, to q_s[0] and q_s[1] (warps 0 and 1; a barrier follows).
+__device__ __forceinline__ void span_quartets(const UnitSpan &span, long long base, long long first,
+                                              long long last, int *q_s) {
+    const int warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        const int q = quartet_of_warp(span.ps, base, warp ? last : first, 0, (int)span.nq - 1);
+        if ((threadIdx.x & 31) == 0) q_s[warp] = q;
+    }
+}
+
 __global__ void unit_counts_kernel(const int4 *__restrict__ q, long long n, const int *__restrict__ nprim,
                                    long long *__restrict__ out) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -58,53 +85,71 @@ __global__ void unit_counts_kernel(const int4 *__restrict__ q, long long n, cons
     out[i] = (long long)nprim[t.x] * nprim[t.y] * nprim[t.z] * nprim[t.w];
 }
 
-// The records of eri_setup_kernel for the units of a span, the B and C values formed in FP64 and
-// rounded (as phase_setup).
+// Setup records of the units of a span, B and C formed in FP64 and rounded (as phase_setup): geometry
+// by one thread per unit, then roots, weights, B and C by one per (unit, root).  kSetupUnits units per
+// CTA: a warp for the geometry, all four for the roots, stores coalesced over the units.  Bound by the
+// FP64 pipe on many units, by the latency of its chains on few: with one thread walking the roots of a
+// unit a class of some hundred quartets took about 30 us.
+constexpr int kSetupUnits = 32;
+
 template <typename R, bool SWAB, bool SWCD>
 __global__ void __launch_bounds__(128)
 unit_setup_kernel(ShellsDev sh, Tables tb, ClassArgs args, KernelInfo k, UnitSpan span, R *out, int st) {
     __shared__ int range_s[2];
-    const int first = blockIdx.x * 128, last = min(first + 127, span.nu - 1);
-    const long long base = span.ps[0];
-    if (threadIdx.x < 2)
-        range_s[threadIdx.x] = quartet_of(span.ps, base, span.u0 + (threadIdx.x ? last : first), 0, (int)span.nq - 1);
-    __syncthreads();
-    const int u = first + threadIdx.x;
-    if (u > last) return;
-    const int q = quartet_of(span.ps, base, span.u0 + u, range_s[0], range_s[1]);
-    const int prim = (int)(span.u0 + u - (__ldg(span.ps + q) - base));
-    const int4 g = args.quartets[q];
-    const int4 qt = make_int4(pick(g, args.perm[0]), pick(g, args.perm[1]), pick(g, args.perm[2]),
-                              pick(g, args.perm[3]));
-    double geo[G_N];
-    int np = 0;
-    geometry_of<UnitGeo<SWAB, SWCD>>(sh, args, qt, prim, geo, np);
-    R *o = out + u;
-    o[0 * st] = to_r<R>(geo[G_ABX]);
-    o[1 * st] = to_r<R>(geo[G_ABY]);
-    o[2 * st] = to_r<R>(geo[G_ABZ]);
-    o[3 * st] = to_r<R>(geo[G_CDX]);
-    o[4 * st] = to_r<R>(geo[G_CDY]);
-    o[5 * st] = to_r<R>(geo[G_CDZ]);
-    o[6 * st] = to_r<R>(geo[G_SWAB]);
-    o[7 * st] = to_r<R>(geo[G_SWCD]);
-    o += kSetupGeo * st;
-    if (k.ltot == 0) {
-        double F0, F1;
-        if constexpr (sizeof(R) == 4)
-            boys_f01_mixed<false>(geo[G_T], tb.boys_t01, tb.boys_t01_f, F0, F1);
-        else
-            boys_f01<false>(geo[G_T], tb.boys_t01, F0, F1);
-        for (int f = 0; f < S_WZ; ++f) o[f * st] = (R)0;
-        o[S_WZ * st] = to_r<R>(geo[G_PREF] * F0);
-        return;
+    __shared__ double geo_s[kSetupUnits * G_N];
+    const int first = blockIdx.x * kSetupUnits, n = min(kSetupUnits, span.nu - first), tid = threadIdx.x;
+    out += first;
+    if (span.ps) {
+        const long long base = span.ps[0];
+        span_quartets(span, base, span.u0 + first, span.u0 + first + n - 1, range_s);
+        __syncthreads();
     }
-    const double p = geo[G_P], q2 = geo[G_Q], ipq = geo[G_IPQ];
-#pragma unroll 1
-    for (int mu = 0; mu < k.nrys; ++mu, o += k.sn * st) {
+    if (tid < n) {
+        int q = first + tid, prim = 0;
+        if (span.ps) {
+            const long long base = span.ps[0], u = span.u0 + first + tid;
+            q = quartet_of(span.ps, base, u, range_s[0], range_s[1]);
+            prim = (int)(u - (__ldg(span.ps + q) - base));
+        }
+        const int4 g = args.quartets[q];
+        const int4 qt = make_int4(pick(g, args.perm[0]), pick(g, args.perm[1]), pick(g, args.perm[2]),
+                                  pick(g, args.perm[3]));
+        double *geo = geo_s + tid * G_N;
+        int np = 0;
+        geometry_of<UnitGeo<SWAB, SWCD>>(sh, args, qt, prim, geo, np);
+        if (!k.direct) {  // the four-index path reads no transfer vectors
+            R *o = out + tid;
+            o[0 * st] = to_r<R>(geo[G_ABX]);
+            o[1 * st] = to_r<R>(geo[G_ABY]);
+            o[2 * st] = to_r<R>(geo[G_ABZ]);
+            o[3 * st] = to_r<R>(geo[G_CDX]);
+            o[4 * st] = to_r<R>(geo[G_CDY]);
+            o[5 * st] = to_r<R>(geo[G_CDZ]);
+            o[6 * st] = to_r<R>(geo[G_SWAB]);
+            o[7 * st] = to_r<R>(geo[G_SWCD]);
+        }
+    }
+    __syncthreads();
+    out += kSetupGeo * st;
+    for (int it = tid; it < kSetupUnits * k.nrys; it += 128) {
+        const int u = it % kSetupUnits, mu = it / kSetupUnits;
+        if (u >= n) continue;
+        const double *geo = geo_s + u * G_N;
+        R *o = out + mu * k.sn * st + u;
+        if (k.ltot == 0) {
+            double F0, F1;
+            if constexpr (sizeof(R) == 4)
+                boys_f01_mixed<false>(geo[G_T], tb.boys_t01, tb.boys_t01_f, F0, F1);
+            else
+                boys_f01<false>(geo[G_T], tb.boys_t01, F0, F1);
+            for (int f = 0; f < S_WZ; ++f) o[f * st] = (R)0;
+            o[S_WZ * st] = to_r<R>(geo[G_PREF] * F0);
+            continue;
+        }
         double x, w;
         rys_root<sizeof(R) == 4>(tb, k.nrys, mu, geo[G_T], x, w);
-        const double fq = q2 * x * ipq, fp = p * x * ipq;
+        const double ipq = geo[G_IPQ];
+        const double fq = geo[G_Q] * x * ipq, fp = geo[G_P] * x * ipq;
         o[S_WZ * st] = to_r<R>(geo[G_PREF] * w);
         o[S_B00 * st] = to_r<R>(0.5 * x * ipq);
         o[S_B10 * st] = to_r<R>((1.0 - fq) * (0.5 * geo[G_IP]));
@@ -116,14 +161,16 @@ unit_setup_kernel(ShellsDev sh, Tables tb, ClassArgs args, KernelInfo k, UnitSpa
             o[(S_C1X + s) * st] = to_r<R>(geo[G_QCX + s] + fp * pq);
         }
         if constexpr (sizeof(R) == 4) {
-            if (k.cb)
+            if (k.cb) {
 #pragma unroll
                 for (int s = 0; s < 3; ++s)
                     o[(k.cb + s) * st] = to_r<R>((geo[G_PAX + s] + geo[G_ABX + s]) - fq * geo[G_PQX + s]);
-            if (k.cd)
+            }
+            if (k.cd) {
 #pragma unroll
                 for (int s = 0; s < 3; ++s)
                     o[(k.cd + s) * st] = to_r<R>((geo[G_QCX + s] + geo[G_CDX + s]) + fp * geo[G_PQX + s]);
+            }
         }
     }
 }
@@ -136,8 +183,7 @@ __global__ void __launch_bounds__(kThreads)
 contract_kernel(ClassArgs args, int neri, UnitSpan span, R *values, R *carry, int parity) {
     __shared__ int q_s[2];
     const long long base = span.ps[0], u1 = span.u0 + span.nu;
-    if (threadIdx.x < 2)
-        q_s[threadIdx.x] = quartet_of(span.ps, base, threadIdx.x ? u1 - 1 : span.u0, 0, (int)span.nq - 1);
+    span_quartets(span, base, span.u0, u1 - 1, q_s);
     __syncthreads();
     const unsigned int n = (unsigned int)(q_s[1] - q_s[0] + 1) * (unsigned int)neri;
     const R *cin = carry + (size_t)parity * 2 * neri;
@@ -158,24 +204,38 @@ contract_kernel(ClassArgs args, int neri, UnitSpan span, R *values, R *carry, in
             v += neri;
             --left;
         }
-        // kBatch loads in flight: the chain of sums of a long quartet waits on memory otherwise
-        R x[kBatch];
-        for (; left > 0; left -= kBatch, v += (size_t)kBatch * neri) {
+        // the loads of the next kBatch units are under way while one batch is summed: the chain of a
+        // long quartet waits on memory otherwise
+        R x[kBatch], y2[kBatch];
+        auto fetch = [&](R (&d)[kBatch], int n) {
 #pragma unroll
             for (int i = 0; i < kBatch; ++i)
-                if (i < left) x[i] = v[(size_t)i * neri];
+                if (i < n) d[i] = v[(size_t)i * neri];
+            v += (size_t)kBatch * neri;
+        };
+        auto sum = [&](const R (&d)[kBatch], int n) {
 #pragma unroll
             for (int i = 0; i < kBatch; ++i)
-                if (i < left) {
+                if (i < n) {
                     if constexpr (sizeof(R) == 4) {
-                        const R y = __fsub_rn(x[i], comp);
+                        const R y = __fsub_rn(d[i], comp);
                         const R s = __fadd_rn(acc, y);
                         comp = __fsub_rn(__fsub_rn(s, acc), y);
                         acc = s;
                     } else {
-                        acc += x[i];
+                        acc += d[i];
                     }
                 }
+        };
+        fetch(x, left);
+        while (left > 0) {
+            fetch(y2, left - kBatch);
+            sum(x, left);
+            left -= kBatch;
+            if (left <= 0) break;
+            fetch(x, left - kBatch);
+            sum(y2, left);
+            left -= kBatch;
         }
         if (l > u1) {
             cout[o] = acc;
@@ -204,16 +264,13 @@ pack_kernel(ClassArgs args, int neri, int qt, UnitSpan span, const R *__restrict
     __shared__ unsigned long long part_raw_s[kThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long base = span.ps ? span.ps[0] : 0, u1 = span.u0 + span.nu;
-    if (tid == 0) {
-        if (span.ps) {
-            q_s[0] = quartet_of(span.ps, base, span.u0, 0, (int)span.nq - 1);
-            int b = quartet_of(span.ps, base, u1 - 1, 0, (int)span.nq - 1);
-            if (span.ps[b + 1] - base > u1) --b;  // continues in the next span
-            q_s[1] = b;
-        } else {  // values of whole quartets
-            q_s[0] = 0;
-            q_s[1] = span.nu - 1;
-        }
+    if (span.ps) {
+        span_quartets(span, base, span.u0, u1 - 1, q_s);
+        __syncthreads();
+        if (tid == 0 && span.ps[q_s[1] + 1] - base > u1) --q_s[1];  // continues in the next span
+    } else if (tid == 0) {  // values of whole quartets
+        q_s[0] = 0;
+        q_s[1] = span.nu - 1;
     }
     __syncthreads();
     const long long q0 = q_s[0] + (long long)blockIdx.x * qt;
@@ -310,7 +367,7 @@ pack_kernel(ClassArgs args, int neri, int qt, UnitSpan span, const R *__restrict
 template <typename R>
 cudaError_t setup_r(const ShellsDev &sh, const Tables &tb, const ClassArgs &a, const KernelInfo &k,
                     const UnitSpan &span, R *rec, int stride, cudaStream_t s) {
-    const unsigned blocks = (unsigned)((span.nu + 127) / 128);
+    const unsigned blocks = (unsigned)((span.nu + kSetupUnits - 1) / kSetupUnits);
     if (k.swab && k.swcd)
         unit_setup_kernel<R, true, true><<<blocks, 128, 0, s>>>(sh, tb, a, k, span, rec, stride);
     else if (k.swab)

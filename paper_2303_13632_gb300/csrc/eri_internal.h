@@ -108,6 +108,7 @@ struct KernelInfo {
     int sn;           // values per (quartet, root)
     int cb, cd;       // slots of C00 on B and C00' on D (0: none)
     bool swab, swcd;  // the VRR may be built on B (D)
+    bool direct;      // four-index path: the records' transfer vectors are not read
 };
 constexpr int kSetupGeo = 8;  // AB, CD and the HRR directions, ahead of the per-root values
 
@@ -116,7 +117,7 @@ constexpr int kSetupGeo = 8;  // AB, CD and the HRR directions, ahead of the per
 // sums the units of each quartet.
 struct UnitSpan {
     const long long *ps;  // exclusive prefix sum of the primitive quartets of the plan's quartets,
-                          // at the class's first quartet (nq + 1 entries)
+                          // at the class's first quartet (nq + 1 entries); null: a unit per quartet
     long long nq;         // quartets of the class
     long long u0;         // first unit of the span (units are counted from the class's first)
     int nu;               // units

@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "eri_device.cuh"
+#include "eri_internal.h"
 
 namespace eri {
 
@@ -42,7 +43,8 @@ template <>
 struct RTraits<double> {
     static __device__ __forceinline__ double round_away(double v) { return round(v); }
     static __device__ __forceinline__ double to_f64(double v) { return v; }
-    static __device__ __forceinline__ bool finite(double v) { return fabs(v) <= 1.7976931348623157e308; }
+    // on the integer pipe: a comparison would take the FP64 pipe
+    static __device__ __forceinline__ bool finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 };
 template <>
 struct RTraits<float> {
@@ -50,6 +52,10 @@ struct RTraits<float> {
     static __device__ __forceinline__ double to_f64(float v) { return f32_to_f64(v); }
     static __device__ __forceinline__ bool finite(float v) { return fabsf(v) <= 3.4028234663852886e38f; }
 };
+
+// Whether a flag stored as 0 or 1 in the recurrence type is set (its high bits, no FP64 comparison).
+__device__ __forceinline__ bool flag_of(double f) { return __double2hiint(f) != 0; }
+__device__ __forceinline__ bool flag_of(float f) { return __float_as_int(f) != 0; }
 
 // Two's complement bits of an integral value |v| <= 2^{bits-1} - 1.  In FP32 and for widths up
 // to 23 the sum v + 1.5 * 2^23 is exact and its low mantissa bits are the integer, which
@@ -152,6 +158,34 @@ __device__ __forceinline__ uint32_t shl(uint32_t v, int n) {
     uint32_t r;
     asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
     return r;
+}
+
+// Eight codes of B bits (halfwords or words at src, 16-byte aligned, upper bits zero) as B / 4 words.
+template <int B>
+__device__ __forceinline__ void pack_group(const unsigned char *src, uint32_t *out) {
+    uint32_t c[8];
+    const uint4 a = *reinterpret_cast<const uint4 *>(src);
+    if constexpr (B <= 16) {
+        const uint32_t r[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            c[2 * i] = r[i] & 0xffffu;
+            c[2 * i + 1] = r[i] >> 16;
+        }
+    } else {
+        const uint4 b = *reinterpret_cast<const uint4 *>(src + 16);
+        c[0] = a.x, c[1] = a.y, c[2] = a.z, c[3] = a.w, c[4] = b.x, c[5] = b.y, c[6] = b.z, c[7] = b.w;
+    }
+#pragma unroll
+    for (int w = 0; w < B / 4; ++w) {
+        uint32_t v = 0u;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int s = i * B - w * 32;
+            if (s > -B && s < 32) v |= s >= 0 ? c[i] << s : c[i] >> -s;
+        }
+        out[w] = v;
+    }
 }
 
 // max(m, |a|, |b|), NaN if one is
@@ -290,7 +324,7 @@ struct Cfg {
     static constexpr int ROW_OFF_STAGE = ROW_OFF_BMAX + (ROW_Q * 4 + 15) / 16 * 16;
     // staged codes (bytes, halfwords or words, kStagePad of them ahead) or FP32 values (bits = 0)
     static constexpr int row_smem(int bits) {
-        return ROW_OFF_STAGE + (ROW_Q * NERI + 2 * kStagePad) * (bits == 0 || bits > 16 ? 4 : (bits == 8 ? 1 : 2)) + 16;
+        return ROW_OFF_STAGE + (ROW_Q * NERI + 2 * kStagePad + 8) * (bits == 0 || bits > 16 ? 4 : (bits == 8 ? 1 : 2)) + 16;
     }
     // registers for three resident CTAs of 256 threads
     static constexpr int ROW_MINB = imax(1, 65536 / (ROW_THREADS * 84));
@@ -593,73 +627,45 @@ __device__ __forceinline__ void root_mixed(const Tables &tb, double T, int mu, d
     }
 }
 
-// Bra HRR (Eq. 7) of one VRR column g(e) (fixed k) into h[i][j], i <= La, j <= Lb.
-// Built on A (swab = false): (i, j+1) = (i+1, j) + AB (i, j), i.e. transfer to b.
-// Built on B (swab = true):  (i+1, j) = (i, j+1) + BA (i, j), i.e. transfer to a.
+// Transfer (Eq. 7) of one column g(0..N) into h[i][j], i <= A, j <= B, N = A + B.
+// Built on A (swap = false): (i, j+1) = (i+1, j) + AB (i, j), i.e. transfer to b.
+// Built on B (swap = true):  (i+1, j) = (i, j+1) + BA (i, j), i.e. transfer to a.
 // Transferring away from the centre nearer to P keeps the cancellation factor of the transfer
-// bounded (|AB| / |P - target| <= 2 for each step).
-template <class C>
-__device__ __forceinline__ void bra_hrr(const typename C::R (&g)[C::NAB + 1], typename C::R ab,
-                                        bool swab, typename C::R (&h)[C::La + 1][C::Lb + 1]) {
-    using R = typename C::R;
-    if (!swab) {
-        R t[C::Lb + 1][C::NAB + 1];
+// bounded (|AB| / |P - target| <= 2 for each step).  Both directions are rows of one triangle
+// t[n][e] = t[n-1][e+1] + s t[n-1][e] with s = AB or -AB, read as h[i][j] = t[j][i] or t[i][j]: lanes of
+// a warp that differ in the direction share its FMAs.
+template <int A, int B, typename R>
+__device__ __forceinline__ void transfer(const R (&g)[A + B + 1], R ab, bool swap, R (&h)[A + 1][B + 1]) {
+    constexpr int N = A + B, M = A > B ? A : B;
+    if constexpr (B == 0) {
 #pragma unroll
-        for (int e = 0; e <= C::NAB; ++e) t[0][e] = g[e];
-#pragma unroll
-        for (int j = 1; j <= C::Lb; ++j)
-#pragma unroll
-            for (int e = 0; e + j <= C::NAB; ++e) t[j][e] = fma(ab, t[j - 1][e], t[j - 1][e + 1]);
-#pragma unroll
-        for (int i = 0; i <= C::La; ++i)
-#pragma unroll
-            for (int j = 0; j <= C::Lb; ++j) h[i][j] = t[j][i];
+        for (int i = 0; i <= A; ++i) h[i][0] = g[i];
     } else {
-        R t[C::La + 1][C::NAB + 1];
+        const R s = swap ? -ab : ab;
+        R t[M + 1][N + 1];
 #pragma unroll
-        for (int e = 0; e <= C::NAB; ++e) t[0][e] = g[e];
+        for (int e = 0; e <= N; ++e) t[0][e] = g[e];
 #pragma unroll
-        for (int i = 1; i <= C::La; ++i)
+        for (int n = 1; n <= M; ++n)
 #pragma unroll
-            for (int e = 0; e + i <= C::NAB; ++e) t[i][e] = fma(-ab, t[i - 1][e], t[i - 1][e + 1]);
+            for (int e = 0; e + n <= N; ++e) t[n][e] = fma(s, t[n - 1][e], t[n - 1][e + 1]);
 #pragma unroll
-        for (int i = 0; i <= C::La; ++i)
+        for (int i = 0; i <= A; ++i)
 #pragma unroll
-            for (int j = 0; j <= C::Lb; ++j) h[i][j] = t[i][j];
+            for (int j = 0; j <= B; ++j) h[i][j] = swap ? t[i][j] : t[j][i];
     }
 }
 
-// Ket HRR of one transferred column s(0..NCD) (fixed i, j) into o[k][l], k <= Lc, l <= Ld;
-// transfer to d (swcd = false) or to c (swcd = true), as for the bra.
+// Bra transfer of a VRR column (fixed k), ket transfer of a transferred column (fixed i, j).
+template <class C>
+__device__ __forceinline__ void bra_hrr(const typename C::R (&g)[C::NAB + 1], typename C::R ab,
+                                        bool swab, typename C::R (&h)[C::La + 1][C::Lb + 1]) {
+    transfer<C::La, C::Lb>(g, ab, swab, h);
+}
 template <class C>
 __device__ __forceinline__ void ket_hrr(const typename C::R (&s)[C::NCD + 1], typename C::R cd,
                                         bool swcd, typename C::R (&o)[C::Lc + 1][C::Ld + 1]) {
-    using R = typename C::R;
-    if (!swcd) {
-        R t[C::Ld + 1][C::NCD + 1];
-#pragma unroll
-        for (int k = 0; k <= C::NCD; ++k) t[0][k] = s[k];
-#pragma unroll
-        for (int l = 1; l <= C::Ld; ++l)
-#pragma unroll
-            for (int k = 0; k + l <= C::NCD; ++k) t[l][k] = fma(cd, t[l - 1][k], t[l - 1][k + 1]);
-#pragma unroll
-        for (int k = 0; k <= C::Lc; ++k)
-#pragma unroll
-            for (int l = 0; l <= C::Ld; ++l) o[k][l] = t[l][k];
-    } else {
-        R t[C::Lc + 1][C::NCD + 1];
-#pragma unroll
-        for (int k = 0; k <= C::NCD; ++k) t[0][k] = s[k];
-#pragma unroll
-        for (int c = 1; c <= C::Lc; ++c)
-#pragma unroll
-            for (int k = 0; k + c <= C::NCD; ++k) t[c][k] = fma(-cd, t[c - 1][k], t[c - 1][k + 1]);
-#pragma unroll
-        for (int k = 0; k <= C::Lc; ++k)
-#pragma unroll
-            for (int l = 0; l <= C::Ld; ++l) o[k][l] = t[k][l];
-    }
+    transfer<C::Lc, C::Ld>(s, cd, swcd, o);
 }
 
 // I layout per quartet: [xi][mu][i][k][j][l] (the (j,l) block is contiguous for phase D).
@@ -678,7 +684,7 @@ __device__ __forceinline__ void phase_vrr(const typename C::R *bc, const typenam
     R c00 = b[S_C0X + xi], c01 = b[S_C1X + xi];
     R b00 = b[S_B00], b10 = b[S_B10], b01 = b[S_B01];
     R ab = rg[RG_ABX + xi];
-    const bool swab = rg[RG_SWAB] != (R)0;
+    const bool swab = flag_of(rg[RG_SWAB]);
     R prev[C::NAB + 1], cur[C::NAB + 1];
     // column k = 0: G(i+1, 0) = C00 G(i, 0) + i B10 G(i-1, 0)
     cur[0] = (xi == 2) ? b[S_WZ] : (R)1;
@@ -724,7 +730,7 @@ __device__ __forceinline__ void phase_vrr(const typename C::R *bc, const typenam
     }
     if constexpr (C::FUSE_BC) {
         R cd = rg[RG_CDX + xi];
-        const bool swcd = rg[RG_SWCD] != (R)0;
+        const bool swcd = flag_of(rg[RG_SWCD]);
 #pragma unroll
         for (int i = 0; i <= C::La; ++i)
 #pragma unroll
@@ -892,7 +898,7 @@ __device__ __forceinline__ void axis_2d(const typename C::R *b, const typename C
     R c00 = b[S_C0X + xi], c01 = b[S_C1X + xi];
     R b00 = b[S_B00], b10 = b[S_B10], b01 = b[S_B01];
     R ab = rg[RG_ABX + xi], cd = rg[RG_CDX + xi];
-    const bool swab = rg[RG_SWAB] != (R)0, swcd = rg[RG_SWCD] != (R)0;
+    const bool swab = flag_of(rg[RG_SWAB]), swcd = flag_of(rg[RG_SWCD]);
     R prev[C::NAB + 1], cur[C::NAB + 1];
     cur[0] = (xi == 2) ? b[S_WZ] : (R)1;
 #pragma unroll
@@ -952,7 +958,7 @@ __device__ __forceinline__ void phase_ket(const typename C::R *rg, int mu, int x
 #pragma unroll
     for (int k = 0; k <= C::NCD; ++k) s[k] = src[k];
     R o[C::Lc + 1][C::Ld + 1];
-    ket_hrr<C>(s, rg[RG_CDX + xi], rg[RG_SWCD] != (R)0, o);
+    ket_hrr<C>(s, rg[RG_CDX + xi], flag_of(rg[RG_SWCD]), o);
 #pragma unroll
     for (int k = 0; k <= C::Lc; ++k)
 #pragma unroll
@@ -1397,13 +1403,14 @@ rows_kernel(ClassArgs args) {
         const float *Iq = I_s + dq * 3 * C::NRYS * C::RIB;
         with_chunk<C::ROW_NCH>(ch, [&](auto k) { rows_quad<C, decltype(k)::value>(Iq, ox, oy, oz, acc); });
         // values and whole-byte codes are staged at the offset from a 16-byte boundary that their
-        // place in memory has; other codes behind kStagePad of them
+        // place in memory has; other codes behind kStagePad of them, groups of eight at vectors
         unsigned char *dst = nullptr;
         if (args.raw != nullptr)
             dst = reinterpret_cast<unsigned char *>(reinterpret_cast<float *>(args.raw) + q0 * C::NERI);
         else if (bits == 16 || bits == 8)
             dst = reinterpret_cast<unsigned char *>(args.packed) + q0 * C::NERI * (bits / 8);
-        unsigned char *st = stage + (dst != nullptr ? (int)(reinterpret_cast<uintptr_t>(dst) & 15) : kStagePad * size);
+        const int lead = (int)((unsigned long long)(q0 * C::NERI) & 7u);  // codes since the last multiple of 8
+        unsigned char *st = stage + (dst != nullptr ? (int)(reinterpret_cast<uintptr_t>(dst) & 15) : (kStagePad + lead) * size);
         // f(output, its staged place) over the thread's outputs
         auto outputs = [&](auto f) {
 #pragma unroll
@@ -1498,7 +1505,27 @@ rows_kernel(ClassArgs args) {
             // neighbour tile's bits
             const long long bit0 = q0 * (long long)C::NERI * bits, w0 = bit0 >> 5;
             const int nw = (int)(w1 - w0), head = (int)(bit0 & 31), tail = (int)(bit1 & 31);
-            for (int w = tid; w < nw; w += T) {
+            // widths that are a multiple of four: eight codes are `bits` / 4 whole words; the words ahead of
+            // the first whole group and behind the last one are gathered one by one below
+            int wlo = nw, wskip = 0;
+            if (bits == 12 || bits == 20) {
+                const int g0 = lead ? 1 : 0, g1 = (lead + nv) >> 3;  // whole groups, from the one `lead` is in
+                if (g1 > g0) {
+                    const int gw = bits / 4;
+                    wlo = (int)(((q0 * C::NERI >> 3) + g0) * gw - w0);
+                    wskip = (g1 - g0) * gw;
+                    uint32_t *out = args.packed + w0 + wlo;
+                    const unsigned char *grp = st - lead * size + g0 * 8 * size;
+                    for (int g = tid; g < g1 - g0; g += T) {
+                        if (bits == 12)
+                            pack_group<12>(grp + g * 16, out + g * 3);
+                        else
+                            pack_group<20>(grp + g * 32, out + g * 5);
+                    }
+                }
+            }
+            for (int w1st = tid; w1st < nw - wskip; w1st += T) {
+                const int w = w1st < wlo ? w1st : w1st + wskip;
                 const int b0 = w * 32 - head;  // the word's first bit, at or above -31
                 const int c = (int)__umulhi((unsigned int)(b0 + kStagePad * bits), bits_magic) - kStagePad;
                 int s = c * bits - b0;  // <= 0: the first code's place
@@ -1530,10 +1557,10 @@ rows_kernel(ClassArgs args) {
     }
 }
 
-// Setup stage of the split path (primitive quartets, K = 1): one thread per quartet computes
-// the Gaussian-product geometry, the Rys roots and weights and the B, C arrays in FP64 and
-// stores them (type R) field-major, so that every thread of this kernel does FP64 work and
-// the recurrence kernel that follows does none.
+// Setup stage of the split path (primitive quartets, K = 1) of the mixed path: one thread per quartet
+// computes the Gaussian-product geometry and the Rys roots and weights in FP64 and the B, C arrays in
+// two-float FP32 and stores them field-major, so that every thread of this kernel does FP64 work and
+// the recurrence kernel that follows does none.  (FP64: unit_setup_kernel, eri_contract.cu.)
 template <class C>
 __global__ void __launch_bounds__(128)
 eri_setup_kernel(ShellsDev sh, Tables tb, ClassArgs args, typename C::R *out, long long stride) {
@@ -1558,26 +1585,16 @@ eri_setup_kernel(ShellsDev sh, Tables tb, ClassArgs args, typename C::R *out, lo
         o[6 * st] = to_r<R>(geo[G_SWAB]);
         o[7 * st] = to_r<R>(geo[G_SWCD]);
     }
-    if constexpr (sizeof(R) == 4) {
-        SetupTF<C> pre;
-        pre.init(geo);
+    SetupTF<C> pre;
+    pre.init(geo);
 #pragma unroll 1
-        for (int mu = 0; mu < C::NRYS; ++mu) {
-            double x, w;
-            root_mixed<C>(tb, geo[G_T], mu, x, w);
-            float bc[C::SN];
-            pre.root(x, w, bc);
+    for (int mu = 0; mu < C::NRYS; ++mu) {
+        double x, w;
+        root_mixed<C>(tb, geo[G_T], mu, x, w);
+        float bc[C::SN];
+        pre.root(x, w, bc);
 #pragma unroll
-            for (int f = 0; f < C::SN; ++f) o[(C::SETUP_GEO + mu * C::SN + f) * st] = bc[f];
-        }
-    } else {
-#pragma unroll 1
-        for (int mu = 0; mu < C::NRYS; ++mu) {
-            R bc[C::SN];
-            phase_setup<C>(tb, geo, mu, bc);
-#pragma unroll
-            for (int f = 0; f < C::SN; ++f) o[(C::SETUP_GEO + mu * C::SN + f) * st] = bc[f];
-        }
+        for (int f = 0; f < C::SN; ++f) o[(C::SETUP_GEO + mu * C::SN + f) * st] = bc[f];
     }
 }
 
@@ -1884,6 +1901,23 @@ eri_tpq_kernel(ShellsDev sh, Tables tb, ClassArgs args) {
     tpq_tile<C, FORM>(sh, tb, args, blockIdx.x, smem);
 }
 
+template <class C>
+constexpr KernelInfo kernel_info() {
+    static_assert(C::SETUP_FIELDS * sizeof(typename C::R) <= kSetupFieldsMax * sizeof(double), "setup");
+    KernelInfo k{};
+    k.tpq = C::TPQ;
+    k.setup = C::USES_SETUP;
+    k.nrys = C::NRYS;
+    k.ltot = C::NAB + C::NCD;
+    k.sn = C::SN;
+    k.cb = C::DIRECT && C::Lb > 0 ? C::S_CB : 0;
+    k.cd = C::DIRECT && C::Ld > 0 ? C::S_CD : 0;
+    k.swab = C::SWAB_OK;
+    k.swcd = C::SWCD_OK;
+    k.direct = C::DIRECT;
+    return k;
+}
+
 // Host-side launch helper for one canonical class in one arithmetic type.  Without o.preset:
 // primitive (K = 1) quartets, through the setup kernel and o.scratch where the class uses it.
 // With o.preset: only the recurrence/quadrature kernel, over args.nq records of args.setup.
@@ -1910,9 +1944,15 @@ cudaError_t launch_class(const ShellsDev &sh, const Tables &tb, const ClassArgs 
         if (!o.scratch) return cudaErrorInvalidValue;
         a.setup = o.scratch;
         a.setup_stride = (args.nq + 31) / 32 * 32;
-        eri_setup_kernel<C><<<(unsigned)((args.nq + 127) / 128), 128, 0, stream>>>(
-            sh, tb, args, reinterpret_cast<R *>(o.scratch), a.setup_stride);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e;
+        if constexpr (sizeof(R) == 4) {
+            eri_setup_kernel<C><<<(unsigned)((args.nq + 127) / 128), 128, 0, stream>>>(
+                sh, tb, args, reinterpret_cast<R *>(o.scratch), a.setup_stride);
+            e = cudaGetLastError();
+        } else {
+            e = unit_setup(sh, tb, args, kernel_info<C>(), false, UnitSpan{nullptr, args.nq, 0, (int)args.nq}, o.scratch,
+                           (int)a.setup_stride, stream);
+        }
         if (e != cudaSuccess) return e;
     }
     if constexpr (C::TPQ) {

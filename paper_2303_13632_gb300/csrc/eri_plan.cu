@@ -1526,7 +1526,7 @@ eri_status_t eri_plan_class_kernels(eri_plan_t plan, int32_t cls, char *buf, siz
     if (units)
         name = "unit_setup_kernel + " + name + " + contract_kernel + pack_kernel";
     else if (g_info[k].setup)
-        name = std::string("eri_setup_kernel<") + cfg + "> + " + name;
+        name = (v == 0 ? std::string("unit_setup_kernel") : std::string("eri_setup_kernel<") + cfg + ">") + " + " + name;
     if (name.size() + 1 > len) return ERI_E_INVALID;
     std::memcpy(buf, name.c_str(), name.size() + 1);
     return ERI_OK;
