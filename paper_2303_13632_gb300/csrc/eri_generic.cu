@@ -29,7 +29,8 @@ namespace {
 
 constexpr int kGenThreads = 256;
 constexpr int kGenQmax = 64;      // quartets per tile
-constexpr int kGenUnits = 128;    // units (primitive quartets) per batch
+constexpr int kGenUnits = 128;    // units (primitive quartets) per batch of the setup stages
+constexpr int kGenBcBytes = 28 * 1024;  // shared memory of a batch's B, C records
 constexpr int kGenSmem = 96 * 1024;
 // B, C values per (unit, root): the slots of phase_setup plus C00 relative to B and C00'
 // relative to D
@@ -49,7 +50,8 @@ struct GenShape {
                      // so that the blocks the lanes of a warp build start in distinct banks
     int lanes;       // lanes per (unit, root, axis): (La+1)(Lb+1) rounded up to a power of two
     int q;           // quartets per tile
-    int units;       // units per batch
+    int setup;       // units per batch of the setup stages
+    int units;       // units per batch of the 2-D integrals
     unsigned m_neri, m_ncd;  // ceil(2^32 / d) for n_ERIQ, n_c n_d (0: d = 1)
     int geo_off, bc_off, i_off, smem;  // dynamic shared memory layout (bytes)
 };
@@ -74,14 +76,18 @@ GenShape gen_shape(const int L[4], bool contracted) {
     g.m_ncd = div_magic(g.n[2] * g.n[3]);
     const int tab = 2 * 4 * (g.n[0] * g.n[1] + g.n[2] * g.n[3]) + 4 * (kGenUnits + 2 * kGenQmax + 2);
     g.geo_off = (tab + 15) / 16 * 16;
-    const int perunit = G_N * 8 + g.nrys * kGenSNP * (int)sizeof(R) + 3 * g.nrys * g.iblkp * (int)sizeof(R);
-    g.units = std::max(1, std::min(kGenUnits, (kGenSmem - g.geo_off) / perunit));
+    // the records of a setup batch, and behind them the integrals of a smaller one, whose place the
+    // batch's geometry takes before
+    const int rec = g.nrys * kGenSNP * (int)sizeof(R), ints = 3 * g.nrys * g.iblkp * (int)sizeof(R);
+    g.setup = std::max(1, std::min(kGenUnits, kGenBcBytes / rec));
+    g.bc_off = g.geo_off;
+    g.i_off = (g.bc_off + g.setup * rec + 15) / 16 * 16;
+    g.units = std::max(1, std::min(g.setup, (kGenSmem - g.i_off) / ints));
+    g.geo_off = g.i_off;
+    g.smem = g.i_off + std::max(g.units * ints, g.setup * G_N * 8);
     // a tile of primitive quartets is one batch; contracted quartets have batches of their own, and
     // short tiles keep the longest of them from holding up the end of a launch
-    g.q = contracted ? (g.neri >= 64 ? 1 : 4) : std::min(kGenQmax, g.units);
-    g.bc_off = g.geo_off + g.units * G_N * 8;
-    g.i_off = (g.bc_off + g.units * g.nrys * kGenSNP * (int)sizeof(R) + 15) / 16 * 16;
-    g.smem = g.i_off + g.units * 3 * g.nrys * g.iblkp * (int)sizeof(R);
+    g.q = contracted ? (g.neri >= 64 ? 1 : 4) : std::min(std::min(kGenQmax, g.setup), std::max(g.units, 16384 / g.neri));
     return g;
 }
 
@@ -158,14 +164,16 @@ __device__ __forceinline__ void plane_recursion(const GenShape &g, const R *b, i
 
 // One tile: quartets [q0, q0 + qn) of the class of `args`, ERIs summed over primitive quartets
 // in FP64 into out[q * n_ERIQ + generic index], q = 0..qn-1 (out = the tile's first quartet).
-// The tile's primitive quartets are taken in batches of g.units, whatever quartet they belong to:
+// The tile's primitive quartets are taken in batches, whatever quartet they belong to, of g.setup for
+// the first two stages (short chains of FP64 work, nothing but their number hides their latency) and of
+// g.units for the others (their integrals fill the shared memory):
 //   geometry        one thread per unit
 //   roots, B and C  one thread per (unit, root)
 //   2-D integrals   plane_recursion, (La+1)(Lb+1) lanes per (unit, root, axis)
 //   quadrature      one thread per (quartet, output), or several that share the quartet's units
 // One primitive quartet per quartet at a time left most of the CTA idle in all but the last of these:
-// 35,000 quartets of a 40-atom molecule (K up to 6, FP32) from the work queue 133 -> 12.8 ms; the 369
-// classes with a g shell, 2^20 ERIs each, 16-bit codes 45 -> 38 ms (11.0 ms with the classes spread
+// 35,000 quartets of a 40-atom molecule (K up to 6, FP32) from the work queue 133 -> 9.0 ms; the 369
+// classes with a g shell, 2^20 ERIs each, 16-bit codes 45 -> 38 ms (10.6 ms with the classes spread
 // over side streams).  Bound by shared-memory reads: three per root and output for two operations.
 // Every thread of the CTA calls it; it begins and ends with a barrier.
 template <typename R>
@@ -210,20 +218,20 @@ __device__ __forceinline__ void generic_tile(const ShellsDev &sh, const Tables &
         for (int q = 0; q < qn; ++q) first_s[q + 1] += first_s[q];
     __syncthreads();
     const int total = first_s[qn];
-    for (int ub = 0; ub < total; ub += g.units) {
-        const int nu = min(g.units, total - ub);
-        for (int i = tid; i < nu; i += kGenThreads) {
+    for (int sb = 0; sb < total; sb += g.setup) {
+        const int ns = min(g.setup, total - sb);
+        for (int i = tid; i < ns; i += kGenThreads) {
             int lo = 0, hi = qn - 1;
             while (lo < hi) {
                 const int mid = (lo + hi + 1) / 2;
-                if (first_s[mid] <= ub + i) lo = mid; else hi = mid - 1;
+                if (first_s[mid] <= sb + i) lo = mid; else hi = mid - 1;
             }
             int np = 0;
-            geometry_of<GenGeo>(sh, args, shells_of(lo), ub + i - first_s[lo], geo_s + i * G_N, np);
+            geometry_of<GenGeo>(sh, args, shells_of(lo), sb + i - first_s[lo], geo_s + i * G_N, np);
             uq_s[i] = lo;
         }
         __syncthreads();
-        for (int it = tid; it < nu * g.nrys; it += kGenThreads) {
+        for (int it = tid; it < ns * g.nrys; it += kGenThreads) {
             const int u = it / g.nrys, mu = it - u * g.nrys;
             const double *geo = geo_s + u * G_N;
             double x, w;
@@ -244,45 +252,49 @@ __device__ __forceinline__ void generic_tile(const ShellsDev &sh, const Tables &
             b[S_WZ] = to_r<R>(geo[G_PREF] * w);
         }
         __syncthreads();
-        const int groups = nu * g.nrys * 3, nij = (La + 1) * (Lb + 1);
-        for (int it = tid; it - (tid & 31) < groups * g.lanes; it += kGenThreads) {
-            const int r = it / g.lanes, e = it % g.lanes;
-            const bool live = r < groups && e < nij;
-            const int m = r < groups ? r : 0;  // lanes past the last group repeat the first (not stored)
-            plane_recursion<R>(g, bc_s + (size_t)(m / 3) * kGenSNP, m % 3, e < nij ? e : 0, live,
-                               I_s + (size_t)m * g.iblkp);
-        }
-        __syncthreads();
-        // quadrature: `parts` neighbouring lanes share the units of one (quartet, output)
-        const int qa = uq_s[0], nseg = uq_s[nu - 1] - qa + 1, ms = 3 * g.iblkp;
-        int parts = 1;
-        while (parts < 32 && 2 * parts * nseg * g.neri <= kGenThreads && 2 * parts * nseg <= nu) parts *= 2;
-        const int items = nseg * g.neri * parts;
-        for (int it = tid; it - (tid & 31) < items; it += kGenThreads) {
-            const bool on = it < items;
-            const int t = on ? it / parts : 0, part = it & (parts - 1);
-            const int seg = div_by(t, g.m_neri), o = t - seg * g.neri, q = qa + seg;
-            const int ab = div_by(o, g.m_ncd), cd = o - ab * ncd;
-            const unsigned off = off_s[ab] + off_s[nab + cd];
-            const int u0 = max(first_s[q] - ub, 0), u1 = on ? min(first_s[q + 1] - ub, nu) : 0;
-            double sum = 0.0;
-            for (int u = u0 + part; u < u1; u += parts) {
-                const R *I0 = I_s + (size_t)u * g.nrys * ms;
-                const R *Ix = I0 + (off & 1023u), *Iy = I0 + g.iblkp + ((off >> 10) & 1023u),
-                        *Iz = I0 + 2 * g.iblkp + (off >> 20);
-                R s = (R)0;
-                for (int mu = 0; mu < g.nrys; ++mu, Ix += ms, Iy += ms, Iz += ms) s = fma(*Ix * *Iy, *Iz, s);
-                sum += RTraits<R>::to_f64(s);
+        for (int ub = sb; ub < sb + ns; ub += g.units) {
+            const int nu = min(g.units, sb + ns - ub);
+            const R *bc_u = bc_s + (size_t)(ub - sb) * g.nrys * kGenSNP;
+            const int groups = nu * g.nrys * 3, nij = (La + 1) * (Lb + 1);
+            for (int it = tid; it - (tid & 31) < groups * g.lanes; it += kGenThreads) {
+                const int r = it / g.lanes, e = it % g.lanes;
+                const bool live = r < groups && e < nij;
+                const int m = r < groups ? r : 0;  // lanes past the last group repeat the first (not stored)
+                plane_recursion<R>(g, bc_u + (size_t)(m / 3) * kGenSNP, m % 3, e < nij ? e : 0, live,
+                                   I_s + (size_t)m * g.iblkp);
             }
-            for (int d = parts / 2; d > 0; d >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, d, parts);
-            if (on && part == 0) {
-                double *dst = out + (long long)q * g.neri + pos_s[ab] + pos_s[nab + cd];
-                if (first_s[q] < ub) sum += *dst;
-                *dst = sum;
-                if (first_s[q + 1] <= ub + nu && !(fabs(sum) <= 1.7976931348623157e308)) atomicOr(args.err, 1);
+            __syncthreads();
+            // quadrature: `parts` neighbouring lanes share the units of one (quartet, output)
+            const int qa = uq_s[ub - sb], nseg = uq_s[ub - sb + nu - 1] - qa + 1, ms = 3 * g.iblkp;
+            int parts = 1;
+            while (parts < 32 && 2 * parts * nseg * g.neri <= kGenThreads && 2 * parts * nseg <= nu) parts *= 2;
+            const int items = nseg * g.neri * parts;
+            for (int it = tid; it - (tid & 31) < items; it += kGenThreads) {
+                const bool on = it < items;
+                const int t = on ? it / parts : 0, part = it & (parts - 1);
+                const int seg = div_by(t, g.m_neri), o = t - seg * g.neri, q = qa + seg;
+                const int ab = div_by(o, g.m_ncd), cd = o - ab * ncd;
+                const unsigned off = off_s[ab] + off_s[nab + cd];
+                const int u0 = max(first_s[q] - ub, 0), u1 = on ? min(first_s[q + 1] - ub, nu) : 0;
+                double sum = 0.0;
+                for (int u = u0 + part; u < u1; u += parts) {
+                    const R *I0 = I_s + (size_t)u * g.nrys * ms;
+                    const R *Ix = I0 + (off & 1023u), *Iy = I0 + g.iblkp + ((off >> 10) & 1023u),
+                            *Iz = I0 + 2 * g.iblkp + (off >> 20);
+                    R s = (R)0;
+                    for (int mu = 0; mu < g.nrys; ++mu, Ix += ms, Iy += ms, Iz += ms) s = fma(*Ix * *Iy, *Iz, s);
+                    sum += RTraits<R>::to_f64(s);
+                }
+                for (int d = parts / 2; d > 0; d >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, d, parts);
+                if (on && part == 0) {
+                    double *dst = out + (long long)q * g.neri + pos_s[ab] + pos_s[nab + cd];
+                    if (first_s[q] < ub) sum += *dst;
+                    *dst = sum;
+                    if (first_s[q + 1] <= ub + nu && !(fabs(sum) <= 1.7976931348623157e308)) atomicOr(args.err, 1);
+                }
             }
+            __syncthreads();
         }
-        __syncthreads();
     }
 }
 
@@ -409,15 +421,25 @@ cudaError_t launch_queue(const ShellsDev &sh, const Tables &tb, const QueueSpec 
                          bool mixed, bool contracted, int bits, int *err, void *d_table, unsigned long long *d_counter,
                          double *scratch, size_t scratch_bytes, int device, cudaStream_t stream) {
     if (n_classes <= 0) return cudaSuccess;
+    // the classes with the most work per quartet first: a long quartet of a high class that starts last
+    // keeps one CTA busy after all others are done (5 of 6.5 ms on a 40-atom molecule's 8,000 quartets)
+    std::vector<int> order(n_classes);
+    for (int i = 0; i < n_classes; ++i) order[i] = i;
+    auto work = [&](int i) {
+        const int *L = classes[i].L;
+        return (L[0] + L[1] + L[2] + L[3] + 2) * ncart(L[0]) * ncart(L[1]) * ncart(L[2]) * ncart(L[3]);
+    };
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return work(x) > work(y); });
     std::vector<QueueClass> qc(n_classes);
     long long tiles = 0;
     int smem = 0;
     long long slot = 1;
     for (int i = 0; i < n_classes; ++i) {
-        qc[i].a = classes[i].a;
-        qc[i].g = mixed ? gen_shape<float>(classes[i].L, contracted) : gen_shape<double>(classes[i].L, contracted);
+        const QueueSpec &c = classes[order[i]];
+        qc[i].a = c.a;
+        qc[i].g = mixed ? gen_shape<float>(c.L, contracted) : gen_shape<double>(c.L, contracted);
         qc[i].first_tile = tiles;
-        tiles += (classes[i].a.nq + qc[i].g.q - 1) / qc[i].g.q;
+        tiles += (c.a.nq + qc[i].g.q - 1) / qc[i].g.q;
         smem = std::max(smem, qc[i].g.smem);
         slot = std::max(slot, (long long)qc[i].g.q * qc[i].g.neri);
     }
