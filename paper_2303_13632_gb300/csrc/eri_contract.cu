@@ -186,8 +186,10 @@ contract_kernel(ClassArgs args, int neri, UnitSpan span, R *values, R *carry, in
     span_quartets(span, base, span.u0, u1 - 1, q_s);
     __syncthreads();
     const unsigned int n = (unsigned int)(q_s[1] - q_s[0] + 1) * (unsigned int)neri;
-    const R *cin = carry + (size_t)parity * 2 * neri;
-    R *cout = carry + (size_t)(1 - parity) * 2 * neri;
+    // two halves of kCarryBytes: a sum and, in FP32, its compensation per output
+    constexpr int kHalf = sizeof(R) == 4 ? 2 : 1;
+    const R *cin = carry + (size_t)parity * kHalf * neri;
+    R *cout = carry + (size_t)(1 - parity) * kHalf * neri;
     bool bad = false;
     for (unsigned int t = blockIdx.x * kThreads + threadIdx.x; t < n; t += gridDim.x * kThreads) {
         const int q = q_s[0] + (int)(t / (unsigned int)neri), o = (int)(t % (unsigned int)neri);

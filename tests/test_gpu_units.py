@@ -32,18 +32,25 @@ def test_cut_quartets_sum_to_the_same(L, degrees, n, precision, bits):
     for l in sorted(set(L)):
         Ls += [l] * len(degrees)
         ks += list(degrees)
+    # a quartet of another class, so that the call over all classes divides the scratch
+    other = 1 if set(L) == {0} else 0
+    Ls.append(other)
+    ks.append(2)
     shells = uneven_shells(rng, Ls, ks)
-    by = {l: [i for i, x in enumerate(Ls) if x == l] for l in set(L)}
+    by = {l: [i for i, x in enumerate(Ls[:-1]) if x == l] for l in set(L)}
     q = np.stack([rng.choice(by[l], n) for l in L], axis=1).astype(np.int32)
-    plan = api.eri_plan_create(shells, q, precision=precision)
+    plan = api.eri_plan_create(shells, np.concatenate([q, np.full((1, 4), len(Ls) - 1, dtype=np.int32)]),
+                               precision=precision)
     cls = W.class_id(*L)
+    fp64_first = api.eri_plan_class_info(plan, cls)[3]
+    first = api.eri_plan_class_info(plan, cls)[2]
     outs = []
     for whole in (False, True):
         if bits == 0:
             out = torch.full((api.eri_output_bytes(plan, 0)[0] // 8,), -1.0, dtype=torch.float64, device="cuda")
             api.eri_compute_class(plan, cls, out) if whole else api.eri_compute(plan, out)
             api.eri_sync(plan)
-            outs.append((out.cpu().numpy(),))
+            outs.append((out.cpu().numpy()[fp64_first:fp64_first + n * W.quartet_size(*L)],))
         else:
             nb, sb = api.eri_output_bytes(plan, bits)
             packed = torch.full((nb // 4,), -1, dtype=torch.int32, device="cuda")
@@ -53,7 +60,8 @@ def test_cut_quartets_sum_to_the_same(L, degrees, n, precision, bits):
             else:
                 api.eri_compute_compressed(plan, bits, packed, scales)
             api.eri_sync(plan)
-            outs.append((packed.cpu().numpy(), scales.cpu().numpy()))
+            off, seg = api.eri_packed_class_offset(plan, bits, cls)
+            outs.append((packed.cpu().numpy()[off // 4:(off + seg) // 4], scales.cpu().numpy()[first:first + n]))
     for x, y in zip(*outs):
         np.testing.assert_array_equal(x, y)
     some = np.arange(n) if np.prod(L) == 0 else np.array([0, 6, n - 1])
@@ -71,3 +79,18 @@ def test_cut_quartets_sum_to_the_same(L, degrees, n, precision, bits):
         # half a step, plus the path's own error: FP64 rounding, or 1e-5 of b_max in FP32
         own = 1e-10 if precision == "fp64" else 1e-5
         assert np.max(np.abs(codes * float(eps) - r)) <= 0.5 * eps * (1 + 1e-6) + own * np.abs(r).max()
+
+
+def test_classes_cut_side_by_side():
+    """Two classes on neighbouring streams, both cut inside quartets: each keeps its own carried sums."""
+    rng = np.random.default_rng(6)
+    shells = uneven_shells(rng, [2, 3, 3, 3, 3], [6, 6, 6, 6, 6])
+    q = np.array([[1, 2, 3, 4], [4, 3, 2, 1], [1, 2, 3, 0], [2, 4, 1, 0]], dtype=np.int32)
+    plan = api.eri_plan_create(shells, q, precision="fp64")
+    n = api.eri_output_bytes(plan, 0)[0] // 8
+    whole, each = (torch.full((n,), -1.0, dtype=torch.float64, device="cuda") for _ in range(2))
+    api.eri_compute(plan, whole)
+    for L in ((3, 3, 3, 3), (3, 3, 3, 2)):
+        api.eri_compute_class(plan, W.class_id(*L), each)
+    api.eri_sync(plan)
+    np.testing.assert_array_equal(whole.cpu().numpy(), each.cpu().numpy())
