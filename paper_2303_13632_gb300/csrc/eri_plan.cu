@@ -218,7 +218,9 @@ struct eri_plan_s {
     float *d_D32 = nullptr;      // FP32 copy of the density of eri_digest_jk (lazy)
     void *d_digest = nullptr;    // per-class parameters of eri_digest_jk's launch (lazy)
     void *d_queue = nullptr;     // class table and tile counter of the work-queue launch (lazy)
-    void *d_setup = nullptr;      // scratch of the split setup/recurrence path (lazy)
+    void *d_setup = nullptr;      // scratch: setup records, values of units or of g classes (primitive
+                                  // plans: on first use)
+    size_t scratch_bytes = 0;     // its size
     double *d_pairs = nullptr;    // primitive-pair table (n_prims^2 records), or null
     int *d_prim_shell = nullptr;  // shell of every primitive (with the pair table)
     std::vector<int> h_L, h_nprim;  // per shell, for eri_plan_update_shells
@@ -228,7 +230,7 @@ struct eri_plan_s {
     long long units[kNumClassIds] = {0};
     void *d_carry = nullptr;
     // side streams over which the classes of a call are spread, and the graph of the batched form
-    static constexpr int kSide = 8;
+    static constexpr int kSide = 16;
     cudaStream_t side[kSide] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[kSide] = {};
     // streamed copies to the host: copy stream and one event per class
@@ -402,11 +404,13 @@ int class_neri(int cls) {
     return ncart_h(L[0]) * ncart_h(L[1]) * ncart_h(L[2]) * ncart_h(L[3]);
 }
 
-// bytes of the plan's scratch (split setup records, or the FP64 values of the compressed output
-// of classes with a g shell)
+// bytes of a plan's scratch (split setup records, values of units, or the FP64 values of the
+// compressed output of classes with a g shell), and the least a contracted plan makes do with
 constexpr size_t kScratchBytes = (size_t)kSetupChunk * kSetupFieldsMax * sizeof(double);
+constexpr size_t kScratchMin = (size_t)64 << 20;
 
 cudaError_t ensure_scratch(eri_plan_s *p) {
+    p->scratch_bytes = p->d_setup ? p->scratch_bytes : kScratchBytes;
     return p->d_setup ? cudaSuccess : cudaMalloc(&p->d_setup, kScratchBytes);
 }
 
@@ -455,6 +459,17 @@ struct Slice {
 
 bool is_contracted(const eri_plan_s *p) { return p->max_nprim > 1; }
 
+// Side streams of a plan.  Sixteen keep the GPU fuller than eight on small contracted plans, whose
+// classes are chains of four short launches (a diatomic's 3,081 quartets 3.51 -> 3.16 ms, 17,000 of a
+// 40-atom molecule 1.49 -> 1.15 ms; 70,000 of it 8.58 -> 8.95 ms), and with the hundreds of classes
+// with a g shell (10.6 -> 9.6 ms at 2^20 ERIs each); the sweep over the s to f classes pays for the
+// longer fork (1.03 -> 1.10 ms at 2^14 ERIs per class).
+int side_count(const eri_plan_s *p) {
+    bool wide = is_contracted(p) && p->nq < (1 << 15);
+    for (int c = 256; c < kNumClassIds; ++c) wide = wide || p->count[c] > 0;
+    return wide ? eri_plan_s::kSide : eri_plan_s::kSide / 2;
+}
+
 // units of a span of class cls with `bytes` of scratch: a record and n_ERIQ values each
 int span_units(const KernelInfo &k, int neri, bool mixed, size_t bytes) {
     const size_t per = (size_t)(kSetupGeo + k.nrys * k.sn + neri) * (mixed ? sizeof(float) : sizeof(double));
@@ -481,7 +496,7 @@ eri_status_t launch_contracted(eri_plan_s *p, int cls, const ClassArgs &a, int v
         if (e != cudaSuccess) return cuda_status(e);
         total = ends[1] - ends[0];
     }
-    const size_t bytes = kScratchBytes / sl.count / 256 * 256;
+    const size_t bytes = p->scratch_bytes / sl.count / 256 * 256;
     char *records = static_cast<char *>(p->d_setup) + sl.index * bytes;
     char *carry = static_cast<char *>(p->d_carry) + sl.index * kCarryBytes;
     const int cap = span_units(info, neri, mixed, bytes);
@@ -519,7 +534,6 @@ eri_status_t launch_class_args(eri_plan_s *p, int cls, const ClassArgs &a, int v
     ShellsDev sh{p->d_cx, p->d_cy, p->d_cz, p->d_pofs, p->d_nprim, p->d_exps, p->d_cn};
     const int neri = class_neri(cls);
     const int bits = a.bits;
-    const size_t slice_bytes = kScratchBytes / sl.count / 256 * 256;
     if (class_has_g(c.cls)) {
         int L[4];
         class_ls(c.cls, L);
@@ -527,6 +541,7 @@ eri_status_t launch_class_args(eri_plan_s *p, int cls, const ClassArgs &a, int v
             cudaError_t e = ensure_scratch(p);
             if (e != cudaSuccess) return cuda_status(e);
         }
+        const size_t slice_bytes = p->scratch_bytes / sl.count / 256 * 256;
         return cuda_status(launch_generic(sh, p->tables, a, L, variant != 0, is_contracted(p),
                                           reinterpret_cast<double *>(static_cast<char *>(p->d_setup) + sl.index * slice_bytes),
                                           slice_bytes, stream));
@@ -541,7 +556,7 @@ eri_status_t launch_class_args(eri_plan_s *p, int cls, const ClassArgs &a, int v
         cudaError_t e = ensure_scratch(p);
         if (e != cudaSuccess) return cuda_status(e);
     }
-    o.scratch = static_cast<char *>(p->d_setup) + sl.index * slice_bytes;
+    o.scratch = static_cast<char *>(p->d_setup) + sl.index * (p->scratch_bytes / sl.count / 256 * 256);
     // chunks that fit the scratch (multiples of 32: every chunk starts on a packed word)
     const long long chunk = kSetupChunk / sl.count / 32 * 32;
     for (long long c0 = 0; c0 < a.nq; c0 += chunk) {
@@ -637,8 +652,7 @@ eri_status_t prepare_contracted(eri_plan_s *p) {
     size_t tmp = 0;
     cudaError_t e = plan_malloc(&d_counts, (n + 1) * sizeof(long long));
     if (e == cudaSuccess) e = plan_malloc(&p->d_pstart, (n + 1) * sizeof(long long));
-    if (e == cudaSuccess) e = plan_malloc(&p->d_setup, kScratchBytes);
-    if (e == cudaSuccess) e = plan_malloc(&p->d_carry, eri_plan_s::kSide * kCarryBytes);
+    if (e == cudaSuccess) e = plan_malloc(&p->d_carry, side_count(p) * kCarryBytes);
     if (e == cudaSuccess) e = unit_counts(p->d_quartets, n, p->d_nprim, d_counts, nullptr);
     if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(nullptr, tmp, d_counts, p->d_pstart, n + 1);
     if (e == cudaSuccess) e = plan_malloc(&d_tmp, std::max<size_t>(tmp, 1));
@@ -659,13 +673,28 @@ eri_status_t prepare_contracted(eri_plan_s *p) {
             p->units[c] = end - before;
             before = end;
         }
+    // a share for each side stream that holds the largest class in one span, within limits; FP64
+    // records and values, the larger ones
+    size_t share = kScratchMin / side_count(p);
+    for (int c = 0; c < kNumClassIds; ++c) {
+        if (p->count[c] == 0) continue;
+        if (class_has_g(c)) {
+            share = kScratchBytes / side_count(p);
+            continue;
+        }
+        const KernelInfo &k = g_info[canonicalise(c).cls * kNumVariants];
+        const double need = (double)((p->units[c] + 31) / 32 * 32) * (kSetupGeo + k.nrys * k.sn + class_neri(c)) * sizeof(double) + 256.0;
+        share = std::max(share, (size_t)std::min(need, (double)(kScratchBytes / side_count(p))));
+    }
+    p->scratch_bytes = std::min(kScratchBytes, share * side_count(p));
+    if ((e = plan_malloc(&p->d_setup, p->scratch_bytes)) != cudaSuccess) return cuda_status(e);
     return ensure_side_streams(p);
 }
 
 // side streams and events
 eri_status_t ensure_side_streams(eri_plan_s *p) {
     cudaError_t e = cudaSuccess;
-    for (int i = 0; e == cudaSuccess && i < eri_plan_s::kSide; ++i) {
+    for (int i = 0; e == cudaSuccess && i < side_count(p); ++i) {
         if (!p->side[i]) e = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking);
         if (e == cudaSuccess && !p->join_ev[i])
             e = cudaEventCreateWithFlags(&p->join_ev[i], cudaEventDisableTiming);
@@ -683,20 +712,19 @@ eri_status_t ensure_side_streams(eri_plan_s *p) {
 // 2^21 8.9 / 6.6 / 5.6 ms, 2^23 18.3 / 19.7 / 21.6 ms, 2^24 30.5 / 34.4 / 43.8 ms; FP64 at 2^19
 // 11.3 / 7.2 / 5.3 ms.  From about 2^25 quartets on (2^23 ERIs per class are 2^25.7) every class
 // fills the GPU by itself, and several at a time only spread the random reads of the pair table.
-// Sixteen streams gain another tenth on a small contracted molecule and lose it on the sweep.
 eri_status_t fork_streams(eri_plan_s *p, cudaStream_t stream, bool scratch, int *n) {
     *n = 0;
     int classes = 0;
     for (int c = 0; c < kNumClassIds; ++c) classes += p->count[c] > 0;
     if (classes < 2 || (!is_contracted(p) && p->nq >= (1LL << 25))) return ERI_OK;
-    if (!p->join_ev[eri_plan_s::kSide - 1] || !p->fork_ev || (scratch && !p->d_setup)) {
+    if (!p->join_ev[side_count(p) - 1] || !p->fork_ev || (scratch && !p->d_setup)) {
         cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return ERI_OK;
         eri_status_t e = ensure_side_streams(p);
         if (e == ERI_OK && scratch) e = cuda_status(ensure_scratch(p));
         if (e != ERI_OK) return e;
     }
-    *n = std::min(classes, (int)eri_plan_s::kSide);
+    *n = std::min(classes, side_count(p));
     return ERI_OK;
 }
 
@@ -1321,7 +1349,9 @@ eri_status_t eri_backward(eri_plan_t plan, const double *d_G, double *d_dR, doub
     int n = 0;
     eri_status_t fs = fork_streams(plan, st, false, &n);
     if (fs != ERI_OK) return fs;
-    if (n > 0) return on_side_streams(plan, st, n, run);
+    // eight streams at most: the adjoint's classes are one launch each and fill the GPU (16 classes, K = 3,
+    // 1024 quartets each: 12.7 ms on eight, 13.3 on sixteen)
+    if (n > 0) return on_side_streams(plan, st, std::min(n, eri_plan_s::kSide / 2), run);
     for (int c = 0; c < kNumClassIds; ++c)
         if (plan->count[c] > 0 && (fs = run(c, st, 0)) != ERI_OK) return fs;
     return ERI_OK;
@@ -1409,7 +1439,7 @@ eri_status_t eri_compute_compressed_queue(eri_plan_t plan, int32_t bits, void *d
                      is_contracted(plan), bits,
                      plan->d_err, plan->d_queue,
                      reinterpret_cast<unsigned long long *>(static_cast<char *>(plan->d_queue) + table),
-                     static_cast<double *>(plan->d_setup), kScratchBytes, plan->device, s);
+                     static_cast<double *>(plan->d_setup), plan->scratch_bytes, plan->device, s);
     return cuda_status(e);
 }
 
@@ -1544,7 +1574,7 @@ eri_status_t eri_plan_class_launches(eri_plan_t plan, int32_t cls, int32_t *n_la
     const int k = canonicalise(cls).cls * kNumVariants + v;
     if (!g_launch[k]) return ERI_E_UNSUPPORTED;
     if (is_contracted(plan)) {
-        const long long cap = span_units(g_info[k], class_neri(cls), v != 0, kScratchBytes);
+        const long long cap = span_units(g_info[k], class_neri(cls), v != 0, plan->scratch_bytes);
         *n_launches = 4 * (int32_t)((plan->units[cls] + cap - 1) / cap);
     } else {
         *n_launches = g_info[k].setup ? 2 * (int32_t)((plan->count[cls] + kSetupChunk - 1) / kSetupChunk) : 1;
