@@ -340,23 +340,24 @@ struct QueueClass {
     long long first_tile;  // first tile of the class in the queue
 };
 
+// The CTA's share of a queue: tiles by the counter until it is past the last one.  bits = 0: FP64
+// output, one tile per CTA (no counter, no slot).
 template <typename R>
-__global__ void __launch_bounds__(kGenThreads)
-eri_queue_kernel(ShellsDev sh, Tables tb, const QueueClass *__restrict__ classes, int n_classes,
-                 long long n_tiles, unsigned long long *counter, double *__restrict__ scratch,
-                 long long slot_doubles, int bits, int *err) {
-    extern __shared__ __align__(16) unsigned char smem[];
+__device__ __forceinline__ void queue_tiles(const ShellsDev &sh, const Tables &tb, const QueueClass *classes,
+                                            int n_classes, long long n_tiles, unsigned long long *counter,
+                                            double *__restrict__ scratch, long long slot_doubles, int bits,
+                                            unsigned char *smem) {
     __shared__ long long item_s;
     __shared__ int cls_s;
     __shared__ unsigned long long bmax_s[kGenQmax];
     __shared__ double inv_s[kGenQmax];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double *vals = scratch + (long long)blockIdx.x * slot_doubles;
-    const double M = (double)((1u << (bits - 1)) - 1u);
+    const double M = bits ? (double)((1u << (bits - 1)) - 1u) : 0.0;
     const uint32_t mask = (1u << bits) - 1u;
     for (;;) {
         if (tid == 0) {
-            item_s = (long long)atomicAdd(counter, 1ull);
+            item_s = bits ? (long long)atomicAdd(counter, 1ull) : (long long)blockIdx.x;
             int lo = 0, hi = n_classes - 1;  // last class whose first tile <= item
             while (lo < hi) {
                 const int mid = (lo + hi + 1) / 2;
@@ -372,7 +373,8 @@ eri_queue_kernel(ShellsDev sh, Tables tb, const QueueClass *__restrict__ classes
         const GenShape g = qc.g;
         const long long q0 = (item - qc.first_tile) * g.q;
         const int qn = (int)((a.nq - q0) < g.q ? (a.nq - q0) : g.q);
-        generic_tile<R>(sh, tb, a, g, q0, qn, vals, smem);
+        generic_tile<R>(sh, tb, a, g, q0, qn, bits ? vals : a.out_fp64 + q0 * (long long)g.neri, smem);
+        if (bits == 0) return;
         // b_max per quartet (non-negative IEEE values order like their bit patterns): all warps on
         // a large quartet, a warp per small one
         for (int q = tid; q < qn; q += kGenThreads) bmax_s[q] = 0ull;
@@ -415,52 +417,125 @@ eri_queue_kernel(ShellsDev sh, Tables tb, const QueueClass *__restrict__ classes
     }
 }
 
-}  // namespace
+template <typename R>
+__global__ void __launch_bounds__(kGenThreads)
+eri_queue_kernel(ShellsDev sh, Tables tb, const QueueClass *__restrict__ classes, int n_classes,
+                 long long n_tiles, unsigned long long *counter, double *__restrict__ scratch,
+                 long long slot_doubles, int bits) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    queue_tiles<R>(sh, tb, classes, n_classes, n_tiles, counter, scratch, slot_doubles, bits, smem);
+}
 
-cudaError_t launch_queue(const ShellsDev &sh, const Tables &tb, const QueueSpec *classes, int n_classes,
-                         bool mixed, bool contracted, int bits, int *err, void *d_table, unsigned long long *d_counter,
-                         double *scratch, size_t scratch_bytes, int device, cudaStream_t stream) {
-    if (n_classes <= 0) return cudaSuccess;
+// The same with the class table as a kernel parameter: calls over all classes run the classes with a g
+// shell in sets of kGenericSet while they are small.  They keep no table on the device for it, and a
+// captured launch carries its own.  With two launches per class the 369 classes took 3.24 ms however
+// few their quartets; at 2^15 ERIs per class in sets 0.42 ms, bound by the quadrature of generic_tile.
+struct GenSet {
+    QueueClass c[kGenericSet];
+};
+static_assert(sizeof(GenSet) + 512 <= 32764, "kernel parameters");
+
+template <typename R>
+__global__ void __launch_bounds__(kGenThreads)
+eri_generic_set_kernel(ShellsDev sh, Tables tb, const __grid_constant__ GenSet set, int n_classes, long long n_tiles,
+                       unsigned long long *counter, double *__restrict__ scratch, long long slot_doubles, int bits) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    queue_tiles<R>(sh, tb, set.c, n_classes, n_tiles, counter, scratch, slot_doubles, bits, smem);
+}
+
+// Table of a queue (n classes, into qc) and what its launch takes.
+struct QueueShape {
+    long long tiles = 0, slot = 1;  // tiles; FP64 values of the largest
+    int smem = 0;
+};
+
+QueueShape queue_table(const QueueSpec *classes, int n, bool mixed, bool contracted, QueueClass *qc) {
     // the classes with the most work per quartet first: a long quartet of a high class that starts last
     // keeps one CTA busy after all others are done (5 of 6.5 ms on a 40-atom molecule's 8,000 quartets)
-    std::vector<int> order(n_classes);
-    for (int i = 0; i < n_classes; ++i) order[i] = i;
+    std::vector<int> order(n);
+    for (int i = 0; i < n; ++i) order[i] = i;
     auto work = [&](int i) {
         const int *L = classes[i].L;
         return (L[0] + L[1] + L[2] + L[3] + 2) * ncart(L[0]) * ncart(L[1]) * ncart(L[2]) * ncart(L[3]);
     };
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return work(x) > work(y); });
-    std::vector<QueueClass> qc(n_classes);
-    long long tiles = 0;
-    int smem = 0;
-    long long slot = 1;
-    for (int i = 0; i < n_classes; ++i) {
+    QueueShape s;
+    for (int i = 0; i < n; ++i) {
         const QueueSpec &c = classes[order[i]];
         qc[i].a = c.a;
         qc[i].g = mixed ? gen_shape<float>(c.L, contracted) : gen_shape<double>(c.L, contracted);
-        qc[i].first_tile = tiles;
-        tiles += (c.a.nq + qc[i].g.q - 1) / qc[i].g.q;
-        smem = std::max(smem, qc[i].g.smem);
-        slot = std::max(slot, (long long)qc[i].g.q * qc[i].g.neri);
+        qc[i].first_tile = s.tiles;
+        s.tiles += (c.a.nq + qc[i].g.q - 1) / qc[i].g.q;
+        s.smem = std::max(s.smem, qc[i].g.smem);
+        s.slot = std::max(s.slot, (long long)qc[i].g.q * qc[i].g.neri);
     }
-    if (smem > 227 * 1024 - 2048) return cudaErrorInvalidValue;
-    void (*kern)(ShellsDev, Tables, const QueueClass *, int, long long, unsigned long long *, double *,
-                 long long, int, int *) = mixed ? eri_queue_kernel<float> : eri_queue_kernel<double>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
+    return s;
+}
+
+// Grid of a queue: the CTAs that the GPU holds at a time, as far as there are tiles and slots for them.
+template <class K>
+cudaError_t queue_grid(K kern, const QueueShape &s, size_t scratch_bytes, int device, long long *grid) {
     int per_sm = 0, sms = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGenThreads, smem)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device)) != cudaSuccess) return e;
-    long long grid = std::min<long long>(tiles, (long long)std::max(1, per_sm) * sms);
-    grid = std::min<long long>(grid, (long long)(scratch_bytes / (sizeof(double) * (size_t)slot)));
-    if (grid < 1) return cudaErrorInvalidValue;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGenThreads, s.smem);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e != cudaSuccess) return e;
+    *grid = std::min<long long>(s.tiles, (long long)std::max(1, per_sm) * sms);
+    *grid = std::min<long long>(*grid, (long long)(scratch_bytes / (sizeof(double) * (size_t)s.slot)));
+    return *grid < 1 ? cudaErrorInvalidValue : cudaSuccess;
+}
+
+template <typename R>
+cudaError_t run_set(const ShellsDev &sh, const Tables &tb, const QueueSpec *classes, int n, bool contracted, int bits,
+                    void *scratch, size_t scratch_bytes, int device, cudaStream_t stream) {
+    constexpr size_t kHead = 256;  // the counter, ahead of the slots
+    GenSet set;
+    const QueueShape s = queue_table(classes, n, sizeof(R) == 4, contracted, set.c);
+    if (s.smem > 227 * 1024 - 2048 || s.tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+    auto kern = eri_generic_set_kernel<R>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
+    if (e != cudaSuccess) return e;
+    long long grid = s.tiles;
+    if (bits) {
+        if (!scratch || scratch_bytes <= kHead) return cudaErrorInvalidValue;
+        if ((e = queue_grid(kern, s, scratch_bytes - kHead, device, &grid)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(scratch, 0, sizeof(unsigned long long), stream)) != cudaSuccess) return e;
+    }
+    kern<<<(unsigned)grid, kGenThreads, s.smem, stream>>>(
+        sh, tb, set, n, s.tiles, static_cast<unsigned long long *>(scratch),
+        bits ? reinterpret_cast<double *>(static_cast<char *>(scratch) + kHead) : nullptr, s.slot, bits);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_queue(const ShellsDev &sh, const Tables &tb, const QueueSpec *classes, int n_classes,
+                         bool mixed, bool contracted, int bits, void *d_table, unsigned long long *d_counter,
+                         double *scratch, size_t scratch_bytes, int device, cudaStream_t stream) {
+    if (n_classes <= 0) return cudaSuccess;
+    std::vector<QueueClass> qc(n_classes);
+    const QueueShape s = queue_table(classes, n_classes, mixed, contracted, qc.data());
+    if (s.smem > 227 * 1024 - 2048) return cudaErrorInvalidValue;
+    auto kern = mixed ? eri_queue_kernel<float> : eri_queue_kernel<double>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
+    if (e != cudaSuccess) return e;
+    long long grid = 0;
+    if ((e = queue_grid(kern, s, scratch_bytes, device, &grid)) != cudaSuccess) return e;
     if ((size_t)n_classes * sizeof(QueueClass) > queue_table_bytes()) return cudaErrorInvalidValue;
     e = cudaMemcpyAsync(d_table, qc.data(), (size_t)n_classes * sizeof(QueueClass), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(d_counter, 0, sizeof(unsigned long long), stream);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)grid, kGenThreads, smem, stream>>>(sh, tb, static_cast<const QueueClass *>(d_table), n_classes,
-                                                        tiles, d_counter, scratch, slot, bits, err);
+    kern<<<(unsigned)grid, kGenThreads, s.smem, stream>>>(sh, tb, static_cast<const QueueClass *>(d_table), n_classes,
+                                                          s.tiles, d_counter, scratch, s.slot, bits);
     return cudaGetLastError();
+}
+
+cudaError_t launch_generic_set(const ShellsDev &sh, const Tables &tb, const QueueSpec *classes, int n, bool mixed,
+                               bool contracted, int bits, void *scratch, size_t scratch_bytes, int device,
+                               cudaStream_t stream) {
+    if (n <= 0) return cudaSuccess;
+    if (n > kGenericSet) return cudaErrorInvalidValue;
+    return mixed ? run_set<float>(sh, tb, classes, n, contracted, bits, scratch, scratch_bytes, device, stream)
+                 : run_set<double>(sh, tb, classes, n, contracted, bits, scratch, scratch_bytes, device, stream);
 }
 
 size_t queue_table_bytes() { return (size_t)kNumClassIds * sizeof(QueueClass); }

@@ -69,8 +69,14 @@ struct QueueSpec {
 };
 size_t queue_table_bytes();
 cudaError_t launch_queue(const ShellsDev &sh, const Tables &tb, const QueueSpec *classes, int n_classes,
-                         bool mixed, bool contracted, int bits, int *err, void *d_table, unsigned long long *d_counter,
+                         bool mixed, bool contracted, int bits, void *d_table, unsigned long long *d_counter,
                          double *scratch, size_t scratch_bytes, int device, cudaStream_t stream);
+// Up to kGenericSet classes with a g shell in one launch, the table passed by value: FP64 output
+// (bits = 0, no scratch) or compressed (as launch_queue; scratch: a counter and the slots).
+constexpr int kGenericSet = 128;
+cudaError_t launch_generic_set(const ShellsDev &sh, const Tables &tb, const QueueSpec *classes, int n, bool mixed,
+                               bool contracted, int bits, void *scratch, size_t scratch_bytes, int device,
+                               cudaStream_t stream);
 
 // Quartets per launch of the split setup/recurrence path (a multiple of 32 so that every chunk
 // starts on a 32-bit word of the packed stream) and the widest setup record (n_Rys = 7).
@@ -83,7 +89,8 @@ constexpr double kPairTableMaxBytes = 16.0 * 1024 * 1024 * 1024;
 // Launcher of one canonical class kernel in one arithmetic variant.
 using LaunchFn = cudaError_t (*)(const ShellsDev &sh, const Tables &tb, const ClassArgs &args,
                                  cudaStream_t stream, const LaunchOpts &opts);
-// Variants: 0 = FP64, 1 = mixed, 2 = mixed with Kahan-compensated primitive sums.
+// Variants: 0 = FP64, 1 = mixed, 2 = mixed, contracted quartets (FP32 units,
+// summed by contract_kernel with Kahan steps).
 constexpr int kNumVariants = 3;
 
 // Launcher of one canonical class's adjoint kernel: `units` primitive quartets, ps their prefix sum

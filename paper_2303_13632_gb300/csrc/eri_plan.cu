@@ -728,22 +728,63 @@ eri_status_t fork_streams(eri_plan_s *p, cudaStream_t stream, bool scratch, int 
     return ERI_OK;
 }
 
-// The plan's non-empty classes on n side streams, forked from and joined back into `stream`: run(class,
-// stream, index of the stream) in decreasing order of work, dealt out in turn.
+// Classes launched together on one side stream: one class, or a set of classes with a g shell.
+struct Job {
+    std::vector<int> classes;
+    double work = 0;
+};
+
+double class_work(const eri_plan_s *p, int c) {
+    return (double)(is_contracted(p) ? p->units[c] : p->count[c]) * class_neri(c);
+}
+
+// Whether a call over all classes runs those with a g shell in sets: up to 10^8 primitive ERIs of them.
+// A set's CTAs have the shared memory of its highest class (two per SM), those of a class its own (up to
+// four), which tells once the classes fill the GPU by themselves.  The 369 classes, mixed, 16 bits,
+// a launch per class / in sets: 2^15 ERIs per class 3.24 / 0.42 ms, 2^20 9.6 / 11.8 ms; sets take
+// 1.53 ms at 2^17, in proportion from there on, and the other form is never below its 3.2 ms of launches.
+bool g_in_sets(const eri_plan_s *p) {
+    double work = 0;
+    for (int c = 256; c < kNumClassIds; ++c) work += class_work(p, c);
+    return work <= 1e8;
+}
+
+// The plan's non-empty classes, those with a g shell one by one or (sets) by precision in sets of
+// kGenericSet, the highest ones first; the jobs by decreasing work.
+std::vector<Job> jobs_of(const eri_plan_s *p, bool sets) {
+    std::vector<Job> jobs;
+    std::vector<int> g[kNumVariants];
+    auto add = [&](std::vector<int> cls) {
+        Job j;
+        for (int c : cls) j.work += class_work(p, c);
+        j.classes = std::move(cls);
+        jobs.push_back(std::move(j));
+    };
+    for (int c = 0; c < kNumClassIds; ++c) {
+        if (p->count[c] == 0) continue;
+        if (sets && class_has_g(c))
+            g[class_variant(p, c)].push_back(c);
+        else
+            add({c});
+    }
+    for (std::vector<int> &v : g) {
+        std::stable_sort(v.begin(), v.end(), [&](int x, int y) { return class_neri(x) > class_neri(y); });
+        for (size_t i = 0; i < v.size(); i += kGenericSet)
+            add(std::vector<int>(v.begin() + i, v.begin() + std::min(v.size(), i + kGenericSet)));
+    }
+    std::stable_sort(jobs.begin(), jobs.end(), [](const Job &x, const Job &y) { return x.work > y.work; });
+    return jobs;
+}
+
+// Jobs on n side streams, forked from and joined back into `stream`: run(job, stream, index of the
+// stream), dealt out in turn.
 template <class Run>
-eri_status_t on_side_streams(eri_plan_s *p, cudaStream_t stream, int n, Run run) {
+eri_status_t on_side_streams(eri_plan_s *p, cudaStream_t stream, int n, const std::vector<Job> &jobs, Run run) {
     cudaError_t e = cudaEventRecord(p->fork_ev, stream);
     for (int i = 0; e == cudaSuccess && i < n; ++i) e = cudaStreamWaitEvent(p->side[i], p->fork_ev, 0);
     if (e != cudaSuccess) return cuda_status(e);
-    std::vector<int> cls;
-    for (int c = 0; c < kNumClassIds; ++c)
-        if (p->count[c] > 0) cls.push_back(c);
-    auto work = [&](int c) {
-        return (is_contracted(p) && !class_has_g(c) ? p->units[c] : p->count[c]) * class_neri(c);
-    };
-    std::stable_sort(cls.begin(), cls.end(), [&](int x, int y) { return work(x) > work(y); });
     eri_status_t st = ERI_OK;
-    for (size_t i = 0; i < cls.size() && st == ERI_OK; ++i) st = run(cls[i], p->side[i % n], (int)(i % n));
+    for (size_t i = 0; i < jobs.size() && st == ERI_OK; ++i) st = run(jobs[i], p->side[i % n], (int)(i % n));
     // joined also after an error: the side streams' work stays ordered before the caller's
     for (int i = 0; i < n; ++i) {
         cudaError_t je = cudaEventRecord(p->join_ev[i], p->side[i]);
@@ -757,17 +798,35 @@ eri_status_t on_side_streams(eri_plan_s *p, cudaStream_t stream, int n, Run run)
 // tuned: with the kernel choices of eri_autotune.
 eri_status_t enqueue_forked(eri_plan_s *p, double *d_out, int bits, void *d_packed, float *d_scales,
                             bool tuned, int n, cudaStream_t stream) {
-    std::vector<size_t> off(kNumClassIds, 0);
-    size_t o = 0;
-    for (int c = 0; c < kNumClassIds; ++c) {
-        off[c] = o;
-        if (!d_out) o += packed_segment_bytes(p->count[c], class_neri(c), bits);
+    std::vector<size_t> off(kNumClassIds + 1, 0);
+    for (int c = 0; c < kNumClassIds; ++c)
+        off[c + 1] = off[c] + (d_out ? 0 : packed_segment_bytes(p->count[c], class_neri(c), bits));
+    const bool sets = g_in_sets(p);
+    const std::vector<Job> jobs = jobs_of(p, sets);
+    n = std::min(n, (int)jobs.size());
+    if (sets && off[kNumClassIds] > off[256]) {  // sets of classes OR their tiles' edge words into the output
+        cudaError_t e = cudaMemsetAsync(static_cast<char *>(d_packed) + off[256], 0, off[kNumClassIds] - off[256], stream);
+        if (e != cudaSuccess) return cuda_status(e);
     }
-    return on_side_streams(p, stream, n, [&](int c, cudaStream_t s, int i) {
-        const int variant = class_variant(p, c);
-        ClassArgs a = class_args(p, c, d_out, bits, d_packed, d_scales, off[c]);
-        const int phase = tuned && !class_has_g(c) ? p->tune_phase[canonicalise(c).cls * kNumVariants + variant] : 0;
-        return launch_class_args(p, c, a, variant, s, 0, Slice{i, n}, phase);
+    return on_side_streams(p, stream, n, jobs, [&](const Job &job, cudaStream_t s, int i) {
+        const int first = job.classes[0], variant = class_variant(p, first);
+        if (!sets || !class_has_g(first)) {
+            ClassArgs a = class_args(p, first, d_out, bits, d_packed, d_scales, off[first]);
+            const int phase = tuned && !class_has_g(first) ? p->tune_phase[canonicalise(first).cls * kNumVariants + variant] : 0;
+            return launch_class_args(p, first, a, variant, s, 0, Slice{i, n}, phase);
+        }
+        std::vector<QueueSpec> spec;
+        for (int c : job.classes) {
+            QueueSpec q;
+            class_ls(canonicalise(c).cls, q.L);
+            q.a = class_args(p, c, d_out, bits, d_packed, d_scales, off[c]);
+            spec.push_back(q);
+        }
+        ShellsDev sh{p->d_cx, p->d_cy, p->d_cz, p->d_pofs, p->d_nprim, p->d_exps, p->d_cn};
+        const size_t bytes = p->scratch_bytes / n / 256 * 256;
+        return cuda_status(launch_generic_set(sh, p->tables, spec.data(), (int)spec.size(), variant != 0, is_contracted(p),
+                                              d_out ? 0 : bits, static_cast<char *>(p->d_setup) + i * bytes, bytes,
+                                              p->device, s));
     });
 }
 
@@ -1351,7 +1410,9 @@ eri_status_t eri_backward(eri_plan_t plan, const double *d_G, double *d_dR, doub
     if (fs != ERI_OK) return fs;
     // eight streams at most: the adjoint's classes are one launch each and fill the GPU (16 classes, K = 3,
     // 1024 quartets each: 12.7 ms on eight, 13.3 on sixteen)
-    if (n > 0) return on_side_streams(plan, st, std::min(n, eri_plan_s::kSide / 2), run);
+    if (n > 0)
+        return on_side_streams(plan, st, std::min(n, eri_plan_s::kSide / 2), jobs_of(plan, false),
+                               [&](const Job &job, cudaStream_t s, int i) { return run(job.classes[0], s, i); });
     for (int c = 0; c < kNumClassIds; ++c)
         if (plan->count[c] > 0 && (fs = run(c, st, 0)) != ERI_OK) return fs;
     return ERI_OK;
@@ -1436,8 +1497,7 @@ eri_status_t eri_compute_compressed_queue(eri_plan_t plan, int32_t bits, void *d
     }
     ShellsDev sh{plan->d_cx, plan->d_cy, plan->d_cz, plan->d_pofs, plan->d_nprim, plan->d_exps, plan->d_cn};
     e = launch_queue(sh, plan->tables, spec.data(), (int)spec.size(), plan->precision == ERI_MIXED,
-                     is_contracted(plan), bits,
-                     plan->d_err, plan->d_queue,
+                     is_contracted(plan), bits, plan->d_queue,
                      reinterpret_cast<unsigned long long *>(static_cast<char *>(plan->d_queue) + table),
                      static_cast<double *>(plan->d_setup), plan->scratch_bytes, plan->device, s);
     return cuda_status(e);
