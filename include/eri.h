@@ -194,13 +194,16 @@ eri_status_t eri_plan_class_precision(eri_plan_t plan, int32_t cls, int32_t *pre
 
 /* Kernel launches eri_compute_class / eri_compute_compressed_class make for class cls in its
  * current precision: 1 for the fused kernels, 2 per chunk of 2^20 quartets (setup and
- * recurrence kernels) on the split path of primitive plans, 0 for an empty class.
+ * recurrence kernels) on the split path of primitive plans, 4 per span of primitive quartets that
+ * fills the plan's scratch (setup, recurrence, sums, compression) for contracted plans, 0 for an
+ * empty class.  (A call over all classes divides the scratch between its side streams and makes
+ * more, shorter launches of a class that does not fit its share.)
  * ERI_E_INVALID for a NULL plan or output, or cls not a class id. */
 eri_status_t eri_plan_class_launches(eri_plan_t plan, int32_t cls, int32_t *n_launches);
 
 /* Names of the kernel instantiation(s) eri_compute_compressed_class launches for class cls in
  * its current precision (for reports that group time by kernel, e.g. "eri_setup_kernel<Cfg<2, 1,
- * 1, 0, float>> + eri_class_kernel<Cfg<2, 1, 1, 0, float>, 0, 1>"), NUL-terminated into buf of
+ * 1, 0, float>> + eri_tpq_kernel<Cfg<2, 1, 1, 0, float>, 1>"), NUL-terminated into buf of
  * len bytes.  Host only; ERI_E_INVALID for a NULL plan or buffer, cls not a class id or a buffer
  * too short. */
 eri_status_t eri_plan_class_kernels(eri_plan_t plan, int32_t cls, char *buf, size_t len);
@@ -285,7 +288,12 @@ eri_status_t eri_pack_paper512_stream(const void *d_stream, int64_t n_quartets, 
 
 /* FP64 ERIs of every quartet (Eqs. 5-8 per primitive quartet, summed over primitives) into
  * d_out (eri_output_bytes(plan, 0, ...) bytes, class-sorted, see fp64_offset).
- * Asynchronous on `stream`; the launches per class are given by eri_plan_class_launches.
+ * Asynchronous on `stream`.  With several classes they are dealt out to side streams of the plan,
+ * forked from `stream` and joined back into it, each with its share of the plan's scratch (not for
+ * primitive plans of 2^25 quartets and more, whose classes run one after the other); to the caller
+ * everything is work of `stream`.  A contracted plan holds what its compute calls need from its
+ * creation on, so any of them may be captured; a primitive plan makes its scratch and side streams
+ * on first use.
  * ERI_E_INVALID for a NULL plan, a NULL d_out when the plan has quartets, or a d_out that is not
  * 8-byte aligned; ERI_E_CUDA if a launch fails.  Non-finite results are latched (eri_sync). */
 eri_status_t eri_compute(eri_plan_t plan, double *d_out, void *stream);
@@ -323,21 +331,16 @@ eri_status_t eri_compute_compressed_to_host(eri_plan_t plan, int32_t bits, void 
 eri_status_t eri_compute_compressed_class(eri_plan_t plan, int32_t cls, int32_t bits,
                                           void *d_packed, float *d_scales, void *stream);
 
-/* Batched form of eri_compute_compressed (same outputs, same layout): every class of the plan
- * runs as a persistent work-queue kernel (one grid of resident CTAs per class pulling tiles of
- * quartets from an atomic counter, so quartets of uneven contraction degree balance
- * dynamically), the classes spread over four streams forked from `stream`, the whole sequence
- * captured once into a CUDA graph and replayed on later calls with the same bits, precision
- * and output pointers.  The tile counters are plan-owned device memory.  The launch choice per
- * class (kernel family and grid) comes from eri_autotune when it has run.  Classes with a g
- * shell run their plain (non-persistent) launches, all on the first of the four streams since
- * they share the plan's scratch buffer; eri_autotune leaves them out.  Asynchronous. */
+/* Batched form of eri_compute_compressed (same outputs, same layout): the launches of every class
+ * of the plan, spread over side streams forked from `stream`, captured once into a CUDA graph and
+ * replayed on later calls with the same bits, precision and output pointers.  The kernel family
+ * per class comes from eri_autotune when it has run.  Asynchronous. */
 eri_status_t eri_compute_compressed_batched(eri_plan_t plan, int32_t bits, void *d_packed,
                                             float *d_scales, void *stream);
 
 /* eri_compute_compressed (same outputs, same layout) as ONE persistent launch of one kernel
- * for every class of the plan: the classes' quartets are cut into tiles (up to 128 quartets of
- * one class) that the resident CTAs pull from a single work queue (an atomic counter), so
+ * for every class of the plan: the classes' quartets are cut into tiles (up to 64 quartets of
+ * one class, the classes by decreasing work) that the resident CTAs pull from one work queue (an atomic counter), so
  * quartets of uneven class and contraction degree balance across the GPU without per-class
  * launches.  The kernel takes the angular momenta at run time (the kernel of the classes with a
  * g shell, see the class-id rule above): geometry, roots and B, C in FP64 (rounded to FP32 in
@@ -351,11 +354,11 @@ eri_status_t eri_compute_compressed_queue(eri_plan_t plan, int32_t bits, void *d
                                           float *d_scales, void *stream);
 
 /* Picks, per canonical class of the plan and for the plan's precision and `bits`, the faster
- * persistent launch (thread-per-quartet or shared-memory kernel where both exist; grid of all
- * resident CTAs, one or two CTAs per SM) by timing each candidate on the plan's own quartets
- * (outputs are written to d_packed/d_scales as a side effect).  Choices already recorded for
- * this GPU in the text file cache_path (may be NULL) are reused; new ones are appended.
- * Synchronous on `stream`. */
+ * kernel family for eri_compute_compressed_batched (thread-per-quartet or shared-memory kernel
+ * where both exist) by timing each candidate on the plan's own quartets (outputs are written to
+ * d_packed/d_scales as a side effect).  Choices already recorded for this GPU in the text file
+ * cache_path (may be NULL) are reused; new ones are appended (the last field of a line, once a grid
+ * size, is written 0 and ignored).  Synchronous on `stream`. */
 eri_status_t eri_autotune(eri_plan_t plan, int32_t bits, void *d_packed, float *d_scales,
                           const char *cache_path, void *stream);
 
@@ -366,14 +369,13 @@ eri_status_t eri_autotune(eri_plan_t plan, int32_t bits, void *d_packed, float *
  *                                                               shells' exps arrays)
  * using d g_a/dA_xi = 2 alpha g_{a+1_xi} - a_xi g_{a-1_xi} and d g_a/d alpha =
  * (2L+3)/(4 alpha) g_a - sum_xi g_{a+2_xi} (same coefficient and normalisation N(alpha, L));
- * the Rys recurrences (Eqs. 6-7) are recomputed on index ranges extended by two and
- * contracted with d_G (Eq. 8 with G weights).  Each class runs in its precision (the plan's, or
- * the per-class override): ERI_FP64 in FP64 throughout, for shells with L <= 2 (the extended
- * ranges of f shells exceed the per-CTA shared memory in FP64; such a plan returns
- * ERI_E_UNSUPPORTED before any device work); ERI_MIXED with the 2-D integrals on the extended
- * ranges by the FP32 four-index recursion, G rounded to FP32, the per-thread and per-warp sums
- * in FP32 and the geometry, roots, B and C (rounded once), the sums across warps, primitives and
- * quartets and both outputs in FP64, for every class up to f.  Plans with a g shell return
+ * the 2-D integrals are recomputed with n_Rys = floor((L+2)/2) + 1 roots, and the raised ones
+ * follow from them and their lowered forms inside the sums with d_G.  Each class runs in its
+ * precision (the plan's, or the per-class override): ERI_FP64 in FP64 throughout, for shells with
+ * L <= 2 (other plans return ERI_E_UNSUPPORTED before any device work); ERI_MIXED with the 2-D
+ * integrals by the FP32 four-index recursion, G rounded to FP32, FP32 sums (compensated over the
+ * primitive quartets of a quartet) and the geometry, roots, B and C (rounded once), the sums across
+ * warps and quartets and both outputs in FP64, for every class up to f.  Plans with a g shell return
  * ERI_E_UNSUPPORTED.  Both outputs are zeroed and then accumulated on `stream` (device atomics:
  * summation order, hence the last bits, can vary between runs). */
 eri_status_t eri_backward(eri_plan_t plan, const double *d_G, double *d_dR, double *d_dalpha,

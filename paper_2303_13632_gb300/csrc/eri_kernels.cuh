@@ -10,24 +10,24 @@
 //                     the ket with (C-D)_xi,
 //   quadrature Eq. 8: [ab|cd] = sum_mu prod_xi I(a_xi, b_xi, c_xi, d_xi, mu, xi), with the
 //                     weight and the Gaussian-product prefactor folded into the z origin,
-// sums the primitive quartets (contraction), and then either stores FP64 values or
-// compresses each quartet (Sec. II-D): b_max (max |x|), eps = b_max / (2^{n-1}-1) (Eq. 9),
-// q = ANINT(x eps^{-1}) (Eq. 10), packed into an n-bit little-endian stream.
+// and then either stores FP64 values or compresses each quartet (Sec. II-D): b_max (max |x|),
+// eps = b_max / (2^{n-1}-1) (Eq. 9), q = ANINT(x eps^{-1}) (Eq. 10), packed into an n-bit
+// little-endian stream.  Quartets of contracted shells run as their primitive quartets (units);
+// eri_contract.cu holds their setup, their sums and their compression.
 //
 // GPU mapping (replaces the FPGA's pipelined loops and private buffer copies, Sec. III-C..E):
-// a CTA owns a tile of Q quartets of one class and runs the stages as data-parallel phases
-// separated by __syncthreads():
-//   A0 geometry + prefactor   one thread per quartet                      (FP64)
-//   A1 roots/weights + B, C   one thread per (quartet, root)              (FP64 -> R)
-//   B  VRR + bra HRR          one thread per (quartet, root, axis)        (R)
-//   C  ket HRR                one thread per (quartet, root, axis, i, j)  (R)
-//   D  quadrature             one thread per (quartet, a, c, b-chunk), the b-chunk x d
-//                             outputs held in registers across primitives (R)
-//   E  b_max, eps, quantise, pack through shared memory, store          (compressed mode)
-// The intermediates I(i,j,k,l,mu,xi) of Table I live in shared memory; several CTAs per SM
-// overlap their phases, which is the GPU analogue of the paper's c_max concurrent quartets.
-// R = double gives the plain FP64 path, R = float the mixed path (FP64 setup/roots, FP32
-// recurrences and quadrature, Kahan-compensated sums over primitives).
+// the two halves of the work use different pipes and run as kernels of their own where a class
+// has more than a few outputs: the setup (geometry, prefactor, Boys, roots; FP64, bound by the FP64
+// pipe) writes a record per primitive quartet, and a kernel of one of three forms consumes it:
+//   tpq_tile     a thread per quartet, everything in registers: up to 100 outputs in FP32, a few in
+//                FP64; with the setup inline for the smallest classes
+//   rows_kernel  the larger FP32 classes: a lane per (root, axis, row) of the four-index recursion,
+//                the 2-D integrals of a tile in shared memory, outputs in registers
+//   class_tile   the FP64 classes: a CTA owns a tile of Q quartets and runs geometry, roots, VRR + bra
+//                HRR, ket HRR and quadrature as phases separated by __syncthreads(); several CTAs per
+//                SM overlap their phases
+// R = double gives the plain FP64 path, R = float the mixed path (FP64 setup and roots, FP32
+// recurrences and quadrature).
 #pragma once
 
 #include <type_traits>
@@ -263,7 +263,7 @@ struct Cfg {
     // primitive (K = 1) plans run the class through the setup kernel
     static constexpr bool USES_SETUP = !TPQ_SMALL;
     // FP32 recurrences with angular momentum on b or d use the four-index recursion
-    // (phase_direct, axis_direct): in FP32 the transfer relation amplifies rounding by up to
+    // (rows_direct, axis_direct): in FP32 the transfer relation amplifies rounding by up to
     // about 3^(Lb+Ld).  FP64 and the small inline-setup classes keep the VRR + HRR of Eqs. 6-7.
     static constexpr bool DIRECT = sizeof(R) == 4 && !TPQ_SMALL && (Lb + Ld) > 0;
     // VRR built on B (D) with the HRR transferring to a (c) where that is the better-
@@ -1598,7 +1598,7 @@ eri_setup_kernel(ShellsDev sh, Tables tb, ClassArgs args, typename C::R *out, lo
     }
 }
 
-// The four-index recursion of phase_direct for one (root, axis) in registers, in the layout of
+// The four-index recursion of rows_direct for one (root, axis) in registers, in the layout of
 // axis_2d (I[((i * (Lc+1) + k) * (Lb+1) + j) * (Ld+1) + l]); thread-per-quartet kernels.
 template <class C, bool ROUND>
 __device__ __forceinline__ void axis_direct(const typename C::R *b, int xi,
