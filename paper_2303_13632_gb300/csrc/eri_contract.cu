@@ -243,6 +243,22 @@ contract_kernel(ClassArgs args, int neri, UnitSpan span, R *values, R *carry, in
             cout[o] = acc;
             if constexpr (sizeof(R) == 4) cout[neri + o] = comp;
         } else {
+            // the zeros up to the longest quartet of the group: a Kahan step with zero changes the sum
+            // only where the compensation left over rounds it to a neighbour, so the others are not searched
+            if constexpr (sizeof(R) == 4) {
+                if (__fsub_rn(acc, comp) != acc) {
+                    const long long g0 = (long long)(q / span.group) * span.group;
+                    const long long g1 = min(g0 + span.group, span.nq);
+                    long long longest = 0;
+                    for (long long i = g0; i < g1; ++i) longest = max(longest, __ldg(span.ps + i + 1) - __ldg(span.ps + i));
+                    for (long long i = l - f; i < longest; ++i) {
+                        const R y = -comp, s = __fadd_rn(acc, y);
+                        if (!(s != acc)) break;
+                        comp = __fsub_rn(__fsub_rn(s, acc), y);
+                        acc = s;
+                    }
+                }
+            }
             bad |= !RTraits<R>::finite(acc);
             if constexpr (OUT64)
                 args.out_fp64[(long long)q * neri + o] = RTraits<R>::to_f64(acc);

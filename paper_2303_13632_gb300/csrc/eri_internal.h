@@ -116,6 +116,7 @@ struct KernelInfo {
     int cb, cd;       // slots of C00 on B and C00' on D (0: none)
     bool swab, swcd;  // the VRR may be built on B (D)
     bool direct;      // four-index path: the records' transfer vectors are not read
+    int group;        // quartets whose FP32 sums are of one length (UnitSpan::group)
 };
 constexpr int kSetupGeo = 8;  // AB, CD and the HRR directions, ahead of the per-root values
 
@@ -128,6 +129,8 @@ struct UnitSpan {
     long long nq;         // quartets of the class
     long long u0;         // first unit of the span (units are counted from the class's first)
     int nu;               // units
+    int group;            // FP32: the sums of `group` neighbouring quartets run over the longest one's primitive
+                          // quartets, zeros past a quartet's own (what the class's tile of whole quartets holds)
 };
 // Primitive quartets of each of n quartets; out[n] = 0.
 cudaError_t unit_counts(const int4 *q, long long n, const int *nprim, long long *out, cudaStream_t s);

@@ -1915,6 +1915,7 @@ constexpr KernelInfo kernel_info() {
     k.swab = C::SWAB_OK;
     k.swcd = C::SWCD_OK;
     k.direct = C::DIRECT;
+    k.group = imin(128, imin(C::QMAX_T, imax(1, C::SMEM_BUDGET / (C::PERQ + G_N * 8))));
     return k;
 }
 

@@ -486,6 +486,7 @@ eri_status_t launch_contracted(eri_plan_s *p, int cls, const ClassArgs &a, int v
     UnitSpan span{};
     span.ps = p->d_pstart + p->first[cls] + q_first;
     span.nq = a.nq;
+    span.group = info.group;
     long long total = p->units[cls];
     if (q_first != 0 || a.nq != p->count[cls]) {  // part of a class (plan-time calls only)
         long long ends[2];
