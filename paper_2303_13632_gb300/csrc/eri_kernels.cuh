@@ -1463,9 +1463,10 @@ rows_kernel(ClassArgs args) {
             const float eps = __uint_as_float(bmax_s[dq]) / M;
             const float inv = eps > 0.0f ? 1.0f / eps : 0.0f;
             if (item == 0) args.scales[q0 + dq] = eps;
-            // |x| <= M (1 + 3 2^-24), so up to 22 bits no code exceeds M; non-finite values, and an eps
-            // whose reciprocal overflows, take the checked form as well
-            if (bits > 22 || !(eps <= 3.4028234663852886e38f && inv <= 3.4028234663852886e38f)) {
+            // eps normal: |x| <= M (1 + 3 2^-24), so up to 22 bits no code exceeds M.  A subnormal eps is
+            // rounded by more than that (and its reciprocal can overflow): it takes the checked form, as
+            // non-finite values do
+            if (bits > 22 || !(eps >= 1.17549435e-38f && eps <= 3.4028234663852886e38f)) {
                 outputs([&](float v, unsigned char *e) {
                     float r = roundf(v * inv);
                     r = r > M ? M : (r < -M ? -M : r);
