@@ -32,6 +32,9 @@ constexpr int kGenQmax = 64;      // quartets per tile
 constexpr int kGenUnits = 128;    // units (primitive quartets) per batch of the setup stages
 constexpr int kGenBcBytes = 28 * 1024;  // shared memory of a batch's B, C records
 constexpr int kGenSmem = 96 * 1024;
+// Limit of the kernels' dynamic shared memory (the static part is below 2 KB).  It is state of the
+// function, shared by all host threads, so every launch sets the same one, whatever it takes itself.
+constexpr int kGenSmemLimit = 227 * 1024 - 2048;
 // B, C values per (unit, root): the slots of phase_setup plus C00 relative to B and C00'
 // relative to D
 constexpr int kGenCB = S_N, kGenCD = S_N + 3, kGenSN = S_N + 6;
@@ -311,7 +314,7 @@ template <typename R>
 cudaError_t run_values(const ShellsDev &sh, const Tables &tb, const ClassArgs &a, const GenShape &g,
                        double *out, cudaStream_t stream) {
     auto kern = eri_generic_kernel<R>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGenSmemLimit);
     if (e != cudaSuccess) return e;
     const long long tiles = (a.nq + g.q - 1) / g.q;
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
@@ -490,9 +493,9 @@ cudaError_t run_set(const ShellsDev &sh, const Tables &tb, const QueueSpec *clas
     constexpr size_t kHead = 256;  // the counter, ahead of the slots
     GenSet set;
     const QueueShape s = queue_table(classes, n, sizeof(R) == 4, contracted, set.c);
-    if (s.smem > 227 * 1024 - 2048 || s.tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+    if (s.smem > kGenSmemLimit || s.tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     auto kern = eri_generic_set_kernel<R>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGenSmemLimit);
     if (e != cudaSuccess) return e;
     long long grid = s.tiles;
     if (bits) {
@@ -514,9 +517,9 @@ cudaError_t launch_queue(const ShellsDev &sh, const Tables &tb, const QueueSpec 
     if (n_classes <= 0) return cudaSuccess;
     std::vector<QueueClass> qc(n_classes);
     const QueueShape s = queue_table(classes, n_classes, mixed, contracted, qc.data());
-    if (s.smem > 227 * 1024 - 2048) return cudaErrorInvalidValue;
+    if (s.smem > kGenSmemLimit) return cudaErrorInvalidValue;
     auto kern = mixed ? eri_queue_kernel<float> : eri_queue_kernel<double>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGenSmemLimit);
     if (e != cudaSuccess) return e;
     long long grid = 0;
     if ((e = queue_grid(kern, s, scratch_bytes, device, &grid)) != cudaSuccess) return e;
@@ -545,7 +548,7 @@ cudaError_t launch_generic(const ShellsDev &sh, const Tables &tb, const ClassArg
                            cudaStream_t stream) {
     if (a.nq <= 0) return cudaSuccess;
     const GenShape g = mixed ? gen_shape<float>(L, contracted) : gen_shape<double>(L, contracted);
-    if (g.smem > 227 * 1024) return cudaErrorInvalidValue;
+    if (g.smem > kGenSmemLimit) return cudaErrorInvalidValue;
     if (a.out_fp64)
         return mixed ? run_values<float>(sh, tb, a, g, a.out_fp64, stream)
                      : run_values<double>(sh, tb, a, g, a.out_fp64, stream);

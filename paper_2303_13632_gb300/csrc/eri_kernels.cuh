@@ -1978,7 +1978,9 @@ cudaError_t launch_class(const ShellsDev &sh, const Tables &tb, const ClassArgs 
     if constexpr (C::DIRECT) {
         auto k3 = rows_kernel<C>;
         const int smem = C::row_smem(args.out_fp64 || args.raw ? 0 : args.bits);
-        cudaError_t e = cudaFuncSetAttribute(k3, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        // the limit is state of the function, shared by all host threads: always the largest size, that of
+        // values, never one that another thread's launch exceeds
+        cudaError_t e = cudaFuncSetAttribute(k3, cudaFuncAttributeMaxDynamicSharedMemorySize, C::row_smem(0));
         if (e != cudaSuccess) return e;
         // at most eight CTAs per SM: with fewer resident, the last wave stays short
         const long long tiles = (args.nq + C::ROW_Q - 1) / C::ROW_Q;
