@@ -31,7 +31,7 @@ constexpr int kGenThreads = 256;
 constexpr int kGenQmax = 64;      // quartets per tile
 constexpr int kGenUnits = 128;    // units (primitive quartets) per batch of the setup stages
 constexpr int kGenBcBytes = 28 * 1024;  // shared memory of a batch's B, C records
-constexpr int kGenSmem = 96 * 1024;
+constexpr int kGenSmem = 96 * 1024, kGenSmemPrim = 72 * 1024;  // contracted plans, primitive plans
 // Limit of the kernels' dynamic shared memory (the static part is below 2 KB).  It is state of the
 // function, shared by all host threads, so every launch sets the same one, whatever it takes itself.
 constexpr int kGenSmemLimit = 227 * 1024 - 2048;
@@ -51,7 +51,7 @@ struct GenShape {
     int nrys, neri;  // roots, ERIs per quartet
     int iblkp;       // stride of the (La+1)(Lb+1)(Lc+1)(Ld+1) integrals of a (unit, root, axis), odd
                      // so that the blocks the lanes of a warp build start in distinct banks
-    int lanes;       // lanes per (unit, root, axis): (La+1)(Lb+1) rounded up to a power of two
+    int lanes;       // lanes per (unit, root, axis): (La+1)(Lb+1) rounded up to a power of two, or 1
     int q;           // quartets per tile
     int setup;       // units per batch of the setup stages
     int units;       // units per batch of the 2-D integrals
@@ -63,8 +63,19 @@ unsigned div_magic(int d) { return d == 1 ? 0u : (unsigned)(((1ull << 32) + d - 
 // n / d for n d < 2^32 with the magic of d
 __device__ __forceinline__ int div_by(int n, unsigned m) { return m ? (int)__umulhi((unsigned)n, m) : n; }
 
+// Shape of a class; q_most: quartets per tile of a primitive plan at most.
+//   Primitive plans: a tile is one batch of the setup stages, its records no more than the tile's, and 72 KB
+// of shared memory leave three CTAs per SM (96 KB and records for 26 to 128 units whatever the tile held
+// left two).  A second batch of the integrals that would be only partly filled is left to the next tile.
+//   Contracted quartets have setup batches of their own, and short tiles keep the longest of them from
+// holding up the end of a launch.
+//   FP64: the recursion on lanes costs 25 FP64 instructions per lane ahead of the first plane and five per
+// plane, on idle lanes too, and the FP64 pipe is what bounds it.  One thread per (unit, root, axis) issues
+// fewer but has their whole chain, so it takes the classes with few planes and the batches that fill a warp.
+//   369 classes in FP64, 2^15 / 2^20 / 2^22 ERIs each: 1.11 / 26.2 / 103.9 ms before these three rules,
+// 0.64 / 15.1 / 59.3 with them; one class at a time (the canonical ones) 23.0 -> 14.4 ms at 2^22.
 template <typename R>
-GenShape gen_shape(const int L[4], bool contracted) {
+GenShape gen_shape(const int L[4], bool contracted, int q_most = kGenQmax) {
     GenShape g{};
     for (int k = 0; k < 4; ++k) {
         g.L[k] = L[k];
@@ -73,24 +84,34 @@ GenShape gen_shape(const int L[4], bool contracted) {
     g.nrys = (L[0] + L[1] + L[2] + L[3]) / 2 + 1;
     g.neri = g.n[0] * g.n[1] * g.n[2] * g.n[3];
     g.iblkp = ((L[0] + 1) * (L[1] + 1) * (L[2] + 1) * (L[3] + 1)) | 1;
-    g.lanes = 1;
-    while (g.lanes < (L[0] + 1) * (L[1] + 1)) g.lanes *= 2;
     g.m_neri = div_magic(g.neri);
     g.m_ncd = div_magic(g.n[2] * g.n[3]);
     const int tab = 2 * 4 * (g.n[0] * g.n[1] + g.n[2] * g.n[3]) + 4 * (kGenUnits + 2 * kGenQmax + 2);
-    g.geo_off = (tab + 15) / 16 * 16;
+    g.bc_off = (tab + 15) / 16 * 16;
     // the records of a setup batch, and behind them the integrals of a smaller one, whose place the
     // batch's geometry takes before
     const int rec = g.nrys * kGenSNP * (int)sizeof(R), ints = 3 * g.nrys * g.iblkp * (int)sizeof(R);
+    const int budget = contracted ? kGenSmem : kGenSmemPrim;
+    auto records = [&](int setup) { return (g.bc_off + setup * rec + 15) / 16 * 16; };
+    auto units = [&](int setup) { return std::max(1, std::min(setup, (budget - records(setup)) / ints)); };
     g.setup = std::max(1, std::min(kGenUnits, kGenBcBytes / rec));
-    g.bc_off = g.geo_off;
-    g.i_off = (g.bc_off + g.setup * rec + 15) / 16 * 16;
-    g.units = std::max(1, std::min(g.setup, (kGenSmem - g.i_off) / ints));
+    if (contracted) {
+        g.q = g.neri >= 64 ? 1 : 4;  // whatever the call: the order of a quartet's sums depends on it
+    } else {
+        const int fit = std::max(1, (budget - g.bc_off) / (rec + ints));  // whose integrals fit at a time
+        g.q = std::min({q_most, kGenQmax, g.setup, std::max(fit, 16384 / g.neri)});
+        const int u = units(g.q);
+        if (g.q < 2 * u) g.q = std::min(g.q, u);
+        g.setup = g.q;
+    }
+    g.i_off = records(g.setup);
+    g.units = units(g.setup);
     g.geo_off = g.i_off;
     g.smem = g.i_off + std::max(g.units * ints, g.setup * G_N * 8);
-    // a tile of primitive quartets is one batch; contracted quartets have batches of their own, and
-    // short tiles keep the longest of them from holding up the end of a launch
-    g.q = contracted ? (g.neri >= 64 ? 1 : 4) : std::min(std::min(kGenQmax, g.setup), std::max(g.units, 16384 / g.neri));
+    const int planes = (L[2] + 1) * (L[3] + 1);
+    g.lanes = 1;
+    if (sizeof(R) == 4 || (planes > 6 && g.units * g.nrys * 3 < 36))
+        while (g.lanes < (L[0] + 1) * (L[1] + 1)) g.lanes *= 2;
     return g;
 }
 
@@ -165,6 +186,52 @@ __device__ __forceinline__ void plane_recursion(const GenShape &g, const R *b, i
     }
 }
 
+// The same by one thread, each value from the lower ones in shared memory, by the operations of
+// plane_recursion in their order.
+template <typename R>
+__device__ __forceinline__ void chain_recursion(const GenShape &g, const R *b, int xi, R *I) {
+    const int La = g.L[0], Lb = g.L[1], Lc = g.L[2], Ld = g.L[3];
+    const int sk = Ld + 1, sj = (Lc + 1) * sk, si = (Lb + 1) * sj;
+    const R cA = b[S_C0X + xi], cB = b[kGenCB + xi], cC = b[S_C1X + xi], cD = b[kGenCD + xi];
+    const R b00 = b[S_B00], b10 = b[S_B10], b01 = b[S_B01];
+    I[0] = xi == 2 ? b[S_WZ] : (R)1;
+    for (int i = 1; i <= La; ++i) {
+        R v = cA * I[(i - 1) * si];
+        if (i > 1) v = fma((R)(i - 1) * b10, I[(i - 2) * si], v);
+        I[i * si] = v;
+    }
+    for (int j = 1; j <= Lb; ++j)
+        for (int i = 0; i <= La; ++i) {
+            const int e = i * si + j * sj;
+            R v = cB * I[e - sj];
+            if (j > 1) v = fma((R)(j - 1) * b10, I[e - 2 * sj], v);
+            if (i > 0) v = fma((R)i * b10, I[e - si - sj], v);
+            I[e] = v;
+        }
+    for (int k = 1; k <= Lc; ++k)
+        for (int i = 0; i <= La; ++i)
+            for (int j = 0; j <= Lb; ++j) {
+                const int e = i * si + j * sj + k * sk;
+                R v = cC * I[e - sk];
+                if (k > 1) v = fma((R)(k - 1) * b01, I[e - 2 * sk], v);
+                if (i > 0) v = fma((R)i * b00, I[e - si - sk], v);
+                if (j > 0) v = fma((R)j * b00, I[e - sj - sk], v);
+                I[e] = v;
+            }
+    for (int l = 1; l <= Ld; ++l)
+        for (int k = 0; k <= Lc; ++k)
+            for (int i = 0; i <= La; ++i)
+                for (int j = 0; j <= Lb; ++j) {
+                    const int e = i * si + j * sj + k * sk + l;
+                    R v = cD * I[e - 1];
+                    if (l > 1) v = fma((R)(l - 1) * b01, I[e - 2], v);
+                    if (k > 0) v = fma((R)k * b01, I[e - sk - 1], v);
+                    if (i > 0) v = fma((R)i * b00, I[e - si - 1], v);
+                    if (j > 0) v = fma((R)j * b00, I[e - sj - 1], v);
+                    I[e] = v;
+                }
+}
+
 // One tile: quartets [q0, q0 + qn) of the class of `args`, ERIs summed over primitive quartets
 // in FP64 into out[q * n_ERIQ + generic index], q = 0..qn-1 (out = the tile's first quartet).
 // The tile's primitive quartets are taken in batches, whatever quartet they belong to, of g.setup for
@@ -172,7 +239,7 @@ __device__ __forceinline__ void plane_recursion(const GenShape &g, const R *b, i
 // g.units for the others (their integrals fill the shared memory):
 //   geometry        one thread per unit
 //   roots, B and C  one thread per (unit, root)
-//   2-D integrals   plane_recursion, (La+1)(Lb+1) lanes per (unit, root, axis)
+//   2-D integrals   plane_recursion, (La+1)(Lb+1) lanes per (unit, root, axis), or chain_recursion, one thread
 //   quadrature      one thread per (quartet, output), or several that share the quartet's units
 // One primitive quartet per quartet at a time left most of the CTA idle in all but the last of these:
 // 35,000 quartets of a 40-atom molecule (K up to 6, FP32) from the work queue 133 -> 9.0 ms; the 369
@@ -259,12 +326,17 @@ __device__ __forceinline__ void generic_tile(const ShellsDev &sh, const Tables &
             const int nu = min(g.units, sb + ns - ub);
             const R *bc_u = bc_s + (size_t)(ub - sb) * g.nrys * kGenSNP;
             const int groups = nu * g.nrys * 3, nij = (La + 1) * (Lb + 1);
-            for (int it = tid; it - (tid & 31) < groups * g.lanes; it += kGenThreads) {
-                const int r = it / g.lanes, e = it % g.lanes;
-                const bool live = r < groups && e < nij;
-                const int m = r < groups ? r : 0;  // lanes past the last group repeat the first (not stored)
-                plane_recursion<R>(g, bc_u + (size_t)(m / 3) * kGenSNP, m % 3, e < nij ? e : 0, live,
-                                   I_s + (size_t)m * g.iblkp);
+            if (sizeof(R) == 8 && g.lanes == 1) {
+                for (int it = tid; it < groups; it += kGenThreads)
+                    chain_recursion<R>(g, bc_u + (size_t)(it / 3) * kGenSNP, it % 3, I_s + (size_t)it * g.iblkp);
+            } else {
+                for (int it = tid; it - (tid & 31) < groups * g.lanes; it += kGenThreads) {
+                    const int r = it / g.lanes, e = it % g.lanes;
+                    const bool live = r < groups && e < nij;
+                    const int m = r < groups ? r : 0;  // lanes past the last group repeat the first (not stored)
+                    plane_recursion<R>(g, bc_u + (size_t)(m / 3) * kGenSNP, m % 3, e < nij ? e : 0, live,
+                                       I_s + (size_t)m * g.iblkp);
+                }
             }
             __syncthreads();
             // quadrature: `parts` neighbouring lanes share the units of one (quartet, output)
@@ -545,9 +617,14 @@ size_t queue_table_bytes() { return (size_t)kNumClassIds * sizeof(QueueClass); }
 
 cudaError_t launch_generic(const ShellsDev &sh, const Tables &tb, const ClassArgs &a, const int L[4],
                            bool mixed, bool contracted, double *scratch, size_t scratch_bytes,
-                           cudaStream_t stream) {
+                           int n_streams, cudaStream_t stream) {
     if (a.nq <= 0) return cudaSuccess;
-    const GenShape g = mixed ? gen_shape<float>(L, contracted) : gen_shape<double>(L, contracted);
+    // two tiles per SM of the stream's share at least: one tile's stages take the same time however few
+    // the others are (the canonical classes one at a time at 2^18 ERIs, FP64 10.4 -> 4.2 ms, FP32 with 16-bit
+    // codes 6.6 -> 4.3; with full tiles and the rules of gen_shape FP64 took 8.0)
+    const long long share = 2 * 152 / n_streams;
+    const int q_most = (int)std::min<long long>(kGenQmax, (a.nq + share - 1) / share);
+    const GenShape g = mixed ? gen_shape<float>(L, contracted, q_most) : gen_shape<double>(L, contracted, q_most);
     if (g.smem > kGenSmemLimit) return cudaErrorInvalidValue;
     if (a.out_fp64)
         return mixed ? run_values<float>(sh, tb, a, g, a.out_fp64, stream)

@@ -50,10 +50,10 @@ inline bool class_has_g(int cls) { return cls >= 256; }
 // quartets, permutation, output strides and output).  FP64 output is written to a.out_fp64;
 // compressed output goes through `scratch` (scratch_bytes of device memory, FP64 values of up to
 // scratch_bytes / (8 n_ERIQ) quartets at a time).  mixed: FP32 recurrences and quadrature from
-// FP64 setup values, FP64 sums over primitives.
+// FP64 setup values, FP64 sums over primitives.  n_streams: streams that share the GPU in this call.
 cudaError_t launch_generic(const ShellsDev &sh, const Tables &tb, const ClassArgs &a, const int L[4],
                            bool mixed, bool contracted, double *scratch, size_t scratch_bytes,
-                           cudaStream_t stream);
+                           int n_streams, cudaStream_t stream);
 // launches launch_generic makes for nq quartets of n_ERIQ = neri, and the kernel names
 int generic_launches(long long nq, int neri, bool compressed, size_t scratch_bytes);
 const char *generic_kernel_names(bool mixed, bool compressed);

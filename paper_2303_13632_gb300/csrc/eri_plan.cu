@@ -545,7 +545,7 @@ eri_status_t launch_class_args(eri_plan_s *p, int cls, const ClassArgs &a, int v
         const size_t slice_bytes = p->scratch_bytes / sl.count / 256 * 256;
         return cuda_status(launch_generic(sh, p->tables, a, L, variant != 0, is_contracted(p),
                                           reinterpret_cast<double *>(static_cast<char *>(p->d_setup) + sl.index * slice_bytes),
-                                          slice_bytes, stream));
+                                          slice_bytes, sl.count, stream));
     }
     LaunchFn fn = g_launch[c.cls * kNumVariants + variant];
     if (!fn) return ERI_E_UNSUPPORTED;
