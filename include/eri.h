@@ -373,10 +373,11 @@ eri_status_t eri_autotune(eri_plan_t plan, int32_t bits, void *d_packed, float *
  * follow from them and their lowered forms inside the sums with d_G.  Each class runs in its
  * precision (the plan's, or the per-class override): ERI_FP64 in FP64 throughout, for shells with
  * L <= 2 (other plans return ERI_E_UNSUPPORTED before any device work); ERI_MIXED with the 2-D
- * integrals by the FP32 four-index recursion, G rounded to FP32, FP32 sums (compensated over the
- * primitive quartets of a quartet) and the geometry, roots, B and C (rounded once), the sums across
- * warps and quartets and both outputs in FP64, for every class up to f.  Plans with a g shell return
- * ERI_E_UNSUPPORTED.  Both outputs are zeroed and then accumulated on `stream` (device atomics:
+ * integrals by the FP32 four-index recursion, G rounded to FP32, the sums over one root and axis of
+ * a primitive quartet in FP32; the sums of these over roots, axes, primitives and (exponents)
+ * neighbouring quartets that share the primitive are pairs of FP32 numbers (a sum and its rounding
+ * error), joined in FP64; geometry, roots, B and C (rounded once), everything beyond and both outputs
+ * in FP64, for every class up to f.  Plans with a g shell return ERI_E_UNSUPPORTED.  Both outputs are zeroed and then accumulated on `stream` (device atomics:
  * summation order, hence the last bits, can vary between runs). */
 eri_status_t eri_backward(eri_plan_t plan, const double *d_G, double *d_dR, double *d_dalpha,
                           void *stream);

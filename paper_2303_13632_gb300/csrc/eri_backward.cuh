@@ -33,16 +33,19 @@
 //      operations per output for all three axes; the partial W blocks go to shared memory
 //   3  one thread per (unit, axis, root, i0, i2): sums the partial blocks over the (a, c) with these
 //      components, forms the eight sums from the neighbouring blocks of I and adds to the centre and
-//      exponent gradients in registers (compensated in FP32) until the quartet or the primitive
-//      changes; then they are summed over the segment's lanes and added to global memory in FP64.
+//      exponent gradients in registers (in FP32 as pairs of a sum and its rounding error, exact to
+//      about 2^-40) until the quartet or the primitive changes; then the pairs are summed over the
+//      segment's lanes and added to global memory in FP64.
 // Step 3 of a unit and step 1 of the next one share a barrier interval (the first from the low
 // threads up, the second from the high ones down, I in two buffers): two barriers per QG units.
 // Bound by barriers between short steps and issue in FP32 (two CTAs per SM, 35% of the issue slots),
 // by the FP64 pipe in FP64.  Measured on the 16 classes of p and d shells, K = 3, forward and backward:
-// 1024 quartets per class in mixed precision 115 -> 12.7 ms, 384 in FP64 220 -> 46.7 ms.  Sharing the
-// barrier interval of steps 3 and 1 and summing exponent terms over a primitive's units instead of
-// once per unit took these from 14.6 and 54.4 ms; 36 instead of 18 G values per thread in FP64 (one
-// pass over the roots of [dd|dd], no b-chunks) from 50.4.
+// 1024 quartets per class in mixed precision 115 -> 14.0 ms, 384 in FP64 220 -> 46.9 ms.  In FP32 the
+// pairs cost 0.9 ms over compensated sums rounded to one number before the lanes are summed, and FP64
+// registers in their place 3.1 ms for the same results; relative error of both gradients against 64 bits
+// 6.4e-8 with them, 1.2e-7 without, 8.5e-8 with FP32 sums per primitive quartet and FP64 beyond.  36
+// instead of 18 G values per thread in FP64 (one pass over the roots of [dd|dd], no b-chunks) took that
+// from 50.4 ms.
 #pragma once
 
 #include "eri_kernels.cuh"
@@ -88,11 +91,18 @@ struct GCfg {
     static constexpr int OFF_BC = 0;
     static constexpr int OFF_META = align16(NBU * NRYS * SN * (int)sizeof(R));
     static constexpr int OFF_EA = align16(OFF_META + NBU * 8 * 4);
-    static constexpr int OFF_I = align16(OFF_EA + NBU * 8 * (int)sizeof(R));
+    static constexpr int OFF_I = align16(OFF_EA + NBU * 12 * (int)sizeof(R));
     static constexpr int OFF_W = align16(OFF_I + 2 * QG * I_VALS * (int)sizeof(R));  // I in two buffers
     // the batch's geometry is dead before steps 1 to 3 start
     static constexpr int SMEM = imax(OFF_W + QG * W_VALS * (int)sizeof(R), OFF_I + NBU * G_N * 8) + 16;
 };
+
+// a + b = sum + err exactly (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float a, float b, float &err) {
+    const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+    return s;
+}
 
 // Units of a class: its quartets' primitive quartets, quartet after quartet.
 struct GradUnits {
@@ -150,7 +160,9 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
     extern __shared__ __align__(16) unsigned char smem[];
     R *bc_s = reinterpret_cast<R *>(smem + C::OFF_BC);
     int *meta_s = reinterpret_cast<int *>(smem + C::OFF_META);  // quartet, its four shells' primitives
-    R *ea_s = reinterpret_cast<R *>(smem + C::OFF_EA);          // 2 alpha, (2L+3) / (4 alpha) of the four
+    // 2 alpha, (2L+3) / (4 alpha) of the four and what the latter's rounding to R leaves: it multiplies the
+    // same sign of term in every unit of the primitive, so its rounding would not average out
+    R *ea_s = reinterpret_cast<R *>(smem + C::OFF_EA);
     R *I_s = reinterpret_cast<R *>(smem + C::OFF_I);
     R *W_s = reinterpret_cast<R *>(smem + C::OFF_W);
     double *geo_s = reinterpret_cast<double *>(smem + C::OFF_I);
@@ -182,15 +194,15 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
     const int sg = tid / C::ST, sx = (tid - sg * C::ST) / C::SEG, se = (tid - sg * C::ST) % C::SEG;
     const bool s_on = sg < C::QG && se < C::SA;
     const int smu = se / C::AC, si = (se % C::AC) / C::NK, sk = se % C::NK;
-    // centre gradients of the quartet (0..3) and exponent gradients (4..7), with their compensation
-    R dacc[8], dcomp[8];
+    // centre gradients of the quartet (0..3) and exponent gradients (4..7); FP32: with their errors
+    R dacc[8], derr[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) dacc[k] = dcomp[k] = (R)0;
+    for (int k = 0; k < 8; ++k) dacc[k] = derr[k] = (R)0;
     auto add = [&](int k, R t) {
         if constexpr (sizeof(R) == 4) {
-            const R y = __fsub_rn(t, dcomp[k]), n = __fadd_rn(dacc[k], y);
-            dcomp[k] = __fsub_rn(__fsub_rn(n, dacc[k]), y);
-            dacc[k] = n;
+            R e;
+            dacc[k] = two_sum(dacc[k], t, e);
+            derr[k] += e;
         } else {
             dacc[k] += t;
         }
@@ -247,8 +259,11 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                 constexpr int Lk[4] = {C::La, C::Lb, C::Lc, C::Ld};
                 const double al = sh.exps[pk[k]];
                 meta_s[i * 8 + 1 + k] = pk[k];
-                ea_s[i * 8 + k] = to_r<R>(2.0 * al);
-                ea_s[i * 8 + 4 + k] = to_r<R>((0.25 * (2 * Lk[k] + 3)) / al);
+                const double ce = (0.25 * (2 * Lk[k] + 3)) / al;
+                const R ch = to_r<R>(ce);
+                ea_s[i * 12 + k] = to_r<R>(2.0 * al);
+                ea_s[i * 12 + 4 + k] = ch;
+                ea_s[i * 12 + 8 + k] = to_r<R>(ce - RTraits<R>::to_f64(ch));
             }
         }
         __syncthreads();
@@ -410,7 +425,7 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                     const R x2 = (R)2 * b00 * DK;
                     const R VP = fma(b10, fma(b10, DD, x2), b00 * b00 * KK) + b10 * S0;
                     const R VQ = fma(b01, fma(b01, KK, x2), b00 * b00 * DD) + b01 * S0;
-                    const R *ea = ea_s + (u0 + sg) * 8;
+                    const R *ea = ea_s + (u0 + sg) * 12;
                     const R cf[4] = {b[S_C0X + sx], b[C::S_CB + sx], b[S_C1X + sx], b[C::S_CD + sx]};
                     const R low[4] = {Sa, Sb, Sc, Sd};
                     const R e0 = sx == 0 ? S0 : (R)0;  // sum over mu of e0: the quartet's energy
@@ -419,7 +434,9 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                         const R p = k < 2 ? P : Q;
                         const R u1 = fma(cf[k], S0, p);
                         add(k, fma(ea[k], u1, -low[k]));
-                        add(4 + k, fma(ea[4 + k], e0, -fma(cf[k], u1 + p, k < 2 ? VP : VQ)));
+                        R x = -fma(cf[k], u1 + p, k < 2 ? VP : VQ);
+                        if constexpr (sizeof(R) == 4) x = fma(ea[8 + k], e0, x);
+                        add(4 + k, fma(ea[4 + k], e0, x));
                     }
                 }
             }
@@ -436,15 +453,29 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                 for (int k = 0; k < 4; ++k) ends |= (last || next[1 + k] != mine[1 + k]) ? 2u << k : 0u;
             }
             const unsigned int any = __reduce_or_sync(0xffffffffu, ends);
-            auto total = [&](int k, bool end) -> R {  // of the segment, on its first lane; the sum starts anew
-                R v = (R)0;
+            auto total = [&](int k, bool end) -> double {  // of the segment, on its first lane; the sum starts anew
+                R v = (R)0, err = (R)0;
                 if (end) {
-                    v = dacc[k] - dcomp[k];
-                    dacc[k] = dcomp[k] = (R)0;
+                    v = dacc[k];
+                    err = derr[k];
+                    dacc[k] = derr[k] = (R)0;
                 }
 #pragma unroll
-                for (int off = C::SW / 2; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off, C::SW);
-                return v;
+                for (int off = C::SW / 2; off > 0; off >>= 1) {
+                    const R o = __shfl_down_sync(0xffffffffu, v, off, C::SW);
+                    if constexpr (sizeof(R) == 4) {
+                        const R oe = __shfl_down_sync(0xffffffffu, err, off, C::SW);
+                        R e;
+                        v = two_sum(v, o, e);
+                        err += oe + e;
+                    } else {
+                        v += o;
+                    }
+                }
+                if constexpr (sizeof(R) == 4)  // (an infinite sum has no error term; plain conversions are the
+                    return RTraits<R>::finite(v) ? (double)v + (double)err : (double)v;  // faster ones here)
+                else
+                    return v;
             };
             const bool leader = se % C::SW == 0;
             if (any & 1u) {
@@ -453,16 +484,16 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                 if (end && leader) gqt = args.quartets[mine[0]];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const R v = total(k, end);
-                    if (end && leader) atomicAdd(dR + 3LL * pick(gqt, args.perm[k]) + sx, RTraits<R>::to_f64(v));
+                    const double v = total(k, end);
+                    if (end && leader) atomicAdd(dR + 3LL * pick(gqt, args.perm[k]) + sx, v);
                 }
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if (any & (2u << k)) {
                     const bool end = ends & (2u << k);
-                    const R v = total(4 + k, end);
-                    if (end && leader) atomicAdd(dalpha + mine[1 + k], RTraits<R>::to_f64(v));
+                    const double v = total(4 + k, end);
+                    if (end && leader) atomicAdd(dalpha + mine[1 + k], v);
                 }
         }
     }
