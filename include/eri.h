@@ -292,8 +292,8 @@ eri_status_t eri_pack_paper512_stream(const void *d_stream, int64_t n_quartets, 
  * forked from `stream` and joined back into it, each with its share of the plan's scratch (not for
  * primitive plans of 2^25 quartets and more, whose classes run one after the other); to the caller
  * everything is work of `stream`.  A contracted plan holds what its compute calls need from its
- * creation on, so any of them may be captured; a primitive plan makes its scratch and side streams
- * on first use.
+ * creation on, so any of them may be captured; a primitive plan makes its side streams and, where a
+ * class needs it, its scratch on first use.
  * ERI_E_INVALID for a NULL plan, a NULL d_out when the plan has quartets, or a d_out that is not
  * 8-byte aligned; ERI_E_CUDA if a launch fails.  Non-finite results are latched (eri_sync). */
 eri_status_t eri_compute(eri_plan_t plan, double *d_out, void *stream);

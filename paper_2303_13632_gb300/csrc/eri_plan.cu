@@ -704,6 +704,22 @@ eri_status_t ensure_side_streams(eri_plan_s *p) {
     return cuda_status(e);
 }
 
+// Whether a call over all classes uses the scratch: split setup records, FP64 values of compressed g
+// classes; `tuned`: with the kernel choices of eri_autotune, by which an inline class may be split.
+bool needs_scratch(const eri_plan_s *p, bool compressed, bool tuned) {
+    if (is_contracted(p)) return true;
+    for (int c = 0; c < kNumClassIds; ++c) {
+        if (p->count[c] == 0) continue;
+        if (class_has_g(c)) {
+            if (compressed) return true;
+            continue;
+        }
+        const int k = canonicalise(c).cls * kNumVariants + class_variant(p, c);
+        if (g_info[k].setup || (tuned && p->tune_phase[k])) return true;
+    }
+    return false;
+}
+
 // Side streams that a call over all classes spreads its classes over, so that small classes share the
 // GPU and the FP64 setup of one overlaps the recurrences of another; 0: none, the classes run on the
 // caller's stream one after the other.  A primitive plan makes its side streams (and, with
@@ -1277,7 +1293,7 @@ eri_status_t eri_compute(eri_plan_t plan, double *d_out, void *stream) {
     if (reinterpret_cast<uintptr_t>(d_out) % 8) return ERI_E_INVALID;
     cudaSetDevice(plan->device);
     int n = 0;
-    eri_status_t fs = fork_streams(plan, (cudaStream_t)stream, true, &n);
+    eri_status_t fs = fork_streams(plan, (cudaStream_t)stream, needs_scratch(plan, false, false), &n);
     if (fs != ERI_OK) return fs;
     if (n > 0) return enqueue_forked(plan, d_out, 0, nullptr, nullptr, false, n, (cudaStream_t)stream);
     for (int c = 0; c < kNumClassIds; ++c) {
@@ -1307,7 +1323,7 @@ eri_status_t eri_compute_compressed(eri_plan_t plan, int32_t bits, void *d_packe
         return ERI_E_INVALID;
     cudaSetDevice(plan->device);
     int n = 0;
-    eri_status_t fs = fork_streams(plan, (cudaStream_t)stream, true, &n);
+    eri_status_t fs = fork_streams(plan, (cudaStream_t)stream, needs_scratch(plan, true, false), &n);
     if (fs != ERI_OK) return fs;
     if (n > 0) return enqueue_forked(plan, nullptr, bits, d_packed, d_scales, false, n, (cudaStream_t)stream);
     size_t off = 0;
@@ -1428,7 +1444,8 @@ eri_status_t eri_compute_compressed_batched(eri_plan_t plan, int32_t bits, void 
     if (plan->nq == 0) return ERI_OK;
     cudaSetDevice(plan->device);
     eri_status_t st = ensure_side_streams(plan);
-    if (st == ERI_OK) st = cuda_status(ensure_scratch(plan));  // before the capture
+    const bool scratch = needs_scratch(plan, true, true);
+    if (st == ERI_OK && scratch) st = cuda_status(ensure_scratch(plan));  // before the capture
     if (st != ERI_OK) return st;
     if (!plan->graph || plan->g_bits != bits || plan->g_prec != plan->precision ||
         plan->g_packed != d_packed || plan->g_scales != d_scales) {
@@ -1447,7 +1464,7 @@ eri_status_t eri_compute_compressed_batched(eri_plan_t plan, int32_t bits, void 
         }
         // (the resources exist: one stream at least, for the plan's autotuned choices)
         int n = 0;
-        st = fork_streams(plan, origin, true, &n);
+        st = fork_streams(plan, origin, scratch, &n);
         if (st == ERI_OK) st = enqueue_forked(plan, nullptr, bits, d_packed, d_scales, true, std::max(1, n), origin);
         cudaGraph_t g = nullptr;
         e = cudaStreamEndCapture(origin, &g);
@@ -1509,8 +1526,7 @@ eri_status_t eri_autotune(eri_plan_t plan, int32_t bits, void *d_packed, float *
     if (!plan || bits < 2 || bits > 24) return ERI_E_INVALID;
     if (plan->nq > 0 && (!d_packed || !d_scales)) return ERI_E_INVALID;
     cudaSetDevice(plan->device);
-    eri_status_t st = cuda_status(ensure_scratch(plan));
-    if (st != ERI_OK) return st;
+    eri_status_t st = ERI_OK;
     cudaStream_t s = (cudaStream_t)stream;
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, plan->device) != cudaSuccess) return ERI_E_CUDA;
