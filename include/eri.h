@@ -291,9 +291,11 @@ eri_status_t eri_pack_paper512_stream(const void *d_stream, int64_t n_quartets, 
  * Asynchronous on `stream`.  With several classes they are dealt out to side streams of the plan,
  * forked from `stream` and joined back into it, each with its share of the plan's scratch (not for
  * primitive plans of 2^25 quartets and more, whose classes run one after the other); to the caller
- * everything is work of `stream`.  A contracted plan holds what its compute calls need from its
- * creation on, so any of them may be captured; a primitive plan makes its side streams and, where a
- * class needs it, its scratch on first use.
+ * everything is work of `stream`.  A contracted plan holds what eri_compute, eri_compute_class,
+ * eri_compute_compressed, eri_compute_compressed_class and eri_backward need from its creation on, so
+ * these may be captured (the process has to have loaded their kernels, by a call on any plan with the
+ * same classes and precision); a primitive plan makes its side streams and, where a class needs it, its
+ * scratch on first use, and every plan what the other compute calls need.
  * ERI_E_INVALID for a NULL plan, a NULL d_out when the plan has quartets, or a d_out that is not
  * 8-byte aligned; ERI_E_CUDA if a launch fails.  Non-finite results are latched (eri_sync). */
 eri_status_t eri_compute(eri_plan_t plan, double *d_out, void *stream);
