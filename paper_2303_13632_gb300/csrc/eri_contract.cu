@@ -85,6 +85,11 @@ __global__ void unit_counts_kernel(const int4 *__restrict__ q, long long n, cons
     out[i] = (long long)nprim[t.x] * nprim[t.y] * nprim[t.z] * nprim[t.w];
 }
 
+__global__ void class_ends_kernel(const long long *__restrict__ ps, const __grid_constant__ ClassEnds at,
+                                  long long *__restrict__ ends) {
+    for (int c = threadIdx.x; c < kNumClassIds; c += blockDim.x) ends[c] = ps[at.i[c]];
+}
+
 // Setup records of the units of a span, B and C formed in FP64 and rounded (as phase_setup): geometry
 // by one thread per unit, then roots, weights, B and C by one per (unit, root).  kSetupUnits units per
 // CTA: a warp for the geometry, all four for the roots, stores coalesced over the units.  Bound by the
@@ -425,6 +430,11 @@ cudaError_t contract_r(const ClassArgs &a, int neri, const UnitSpan &span, R *va
 
 cudaError_t unit_counts(const int4 *q, long long n, const int *nprim, long long *out, cudaStream_t s) {
     unit_counts_kernel<<<(unsigned)((n + 256) / 256), 256, 0, s>>>(q, n, nprim, out);
+    return cudaGetLastError();
+}
+
+cudaError_t class_ends(const long long *ps, const ClassEnds &at, long long *ends, cudaStream_t s) {
+    class_ends_kernel<<<1, 256, 0, s>>>(ps, at, ends);
     return cudaGetLastError();
 }
 

@@ -134,6 +134,12 @@ struct UnitSpan {
 };
 // Primitive quartets of each of n quartets; out[n] = 0.
 cudaError_t unit_counts(const int4 *q, long long n, const int *nprim, long long *out, cudaStream_t s);
+// ends[c] = ps[at.i[c]] for every class id c, in one launch: a copy to the host per class took 10 us each
+// (240 classes of a diatomic's plan).
+struct ClassEnds {
+    int i[kNumClassIds];
+};
+cudaError_t class_ends(const long long *ps, const ClassEnds &at, long long *ends, cudaStream_t s);
 // Records (layout of KernelInfo, field-major with `stride`) of the units of a span.
 cudaError_t unit_setup(const ShellsDev &sh, const Tables &tb, const ClassArgs &a, const KernelInfo &k,
                        bool mixed, const UnitSpan &span, void *records, int stride, cudaStream_t s);

@@ -644,50 +644,74 @@ eri_status_t launch_one(eri_plan_s *p, int cls, double *d_out, int bits, void *d
 
 eri_status_t ensure_side_streams(eri_plan_s *p);
 
+// Streams that a call over all classes can use: one per class at most.
+int stream_count(const eri_plan_s *p) {
+    int classes = 0;
+    for (int c = 0; c < kNumClassIds; ++c) classes += p->count[c] > 0;
+    return std::max(1, std::min(classes, side_count(p)));
+}
+
+// Scratch of a contracted plan: a share for each of n streams that holds its largest class in one span,
+// within limits (FP64 records and values, the larger ones; of a class with a g shell the FP64 values),
+// and a slot for every tile of the work queue, up to kScratchMin (with g shells kScratchBytes).
+size_t contracted_scratch(const eri_plan_s *p, int n) {
+    size_t share = 0, slots = 0, slot = 0;
+    bool g = false;
+    for (int c = 0; c < kNumClassIds; ++c) {
+        if (p->count[c] == 0) continue;
+        const int neri = class_neri(c);
+        size_t per = neri * sizeof(double);
+        long long units = p->count[c];
+        if (class_has_g(c)) {
+            g = true;
+        } else {
+            const KernelInfo &k = g_info[canonicalise(c).cls * kNumVariants];
+            per += (kSetupGeo + k.nrys * k.sn) * sizeof(double);
+            units = p->units[c];
+        }
+        const double need = (double)((units + 31) / 32 * 32) * per;
+        share = std::max(share, (size_t)std::min(need, (double)(kScratchBytes / n)));
+        slots += p->count[c];
+        slot = std::max(slot, std::max(neri, 256) * sizeof(double));  // four quartets below 64 values
+    }
+    const double queue = std::min((double)slots * slot, (double)(g ? kScratchBytes : kScratchMin));
+    share = std::max(share, (size_t)queue / n) + 512;  // slices and the counter of a set
+    return std::min(kScratchBytes, (share + 255) / 256 * 256 * n);
+}
+
 // What the compute calls of a contracted plan need: the prefix sum of the primitive quartets, the
 // scratch, the carried sums and the side streams.  Called once the class layout is known.
 eri_status_t prepare_contracted(eri_plan_s *p) {
     const long long n = p->nq;
-    long long *d_counts = nullptr;
-    void *d_tmp = nullptr;
+    const int streams = stream_count(p);
+    char *d_tmp = nullptr;  // the scan's storage, then the classes' ends
     size_t tmp = 0;
-    cudaError_t e = plan_malloc(&d_counts, (n + 1) * sizeof(long long));
-    if (e == cudaSuccess) e = plan_malloc(&p->d_pstart, (n + 1) * sizeof(long long));
-    if (e == cudaSuccess) e = plan_malloc(&p->d_carry, side_count(p) * kCarryBytes);
-    if (e == cudaSuccess) e = unit_counts(p->d_quartets, n, p->d_nprim, d_counts, nullptr);
-    if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(nullptr, tmp, d_counts, p->d_pstart, n + 1);
-    if (e == cudaSuccess) e = plan_malloc(&d_tmp, std::max<size_t>(tmp, 1));
-    if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(d_tmp, tmp, d_counts, p->d_pstart, n + 1);
-    for (int c = 0; e == cudaSuccess && c < kNumClassIds; ++c)
-        if (p->count[c] > 0)
-            e = cudaMemcpyAsync(&p->units[c], p->d_pstart + p->first[c] + p->count[c], sizeof(long long),
-                                cudaMemcpyDeviceToHost, nullptr);
+    cudaError_t e = plan_malloc(&p->d_pstart, (n + 1) * sizeof(long long));
+    if (e == cudaSuccess) e = plan_malloc(&p->d_carry, streams * kCarryBytes);
+    if (e == cudaSuccess) e = unit_counts(p->d_quartets, n, p->d_nprim, p->d_pstart, nullptr);
+    if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(nullptr, tmp, p->d_pstart, p->d_pstart, n + 1);
+    tmp = (tmp + 255) / 256 * 256;
+    if (e == cudaSuccess) e = plan_malloc(&d_tmp, tmp + kNumClassIds * sizeof(long long));
+    if (e == cudaSuccess) e = cub::DeviceScan::ExclusiveSum(d_tmp, tmp, p->d_pstart, p->d_pstart, n + 1);
+    ClassEnds at{};
+    for (int c = 0; c < kNumClassIds; ++c) at.i[c] = (int)(p->count[c] > 0 ? p->first[c] + p->count[c] : 0);
+    std::vector<long long> ends(kNumClassIds);
+    if (e == cudaSuccess) {
+        long long *d_ends = reinterpret_cast<long long *>(d_tmp + tmp);
+        e = class_ends(p->d_pstart, at, d_ends, nullptr);
+        if (e == cudaSuccess) e = cudaMemcpy(ends.data(), d_ends, kNumClassIds * sizeof(long long), cudaMemcpyDeviceToHost);
+    }
     const cudaError_t se = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = se;
-    cudaFree(d_counts);
     cudaFree(d_tmp);
     if (e != cudaSuccess) return cuda_status(e);
-    long long before = 0;  // the copies hold the prefix at each class's end
+    long long before = 0;
     for (int c = 0; c < kNumClassIds; ++c)
         if (p->count[c] > 0) {
-            const long long end = p->units[c];
-            p->units[c] = end - before;
-            before = end;
+            p->units[c] = ends[c] - before;
+            before = ends[c];
         }
-    // a share for each side stream that holds the largest class in one span, within limits; FP64
-    // records and values, the larger ones
-    size_t share = kScratchMin / side_count(p);
-    for (int c = 0; c < kNumClassIds; ++c) {
-        if (p->count[c] == 0) continue;
-        if (class_has_g(c)) {
-            share = kScratchBytes / side_count(p);
-            continue;
-        }
-        const KernelInfo &k = g_info[canonicalise(c).cls * kNumVariants];
-        const double need = (double)((p->units[c] + 31) / 32 * 32) * (kSetupGeo + k.nrys * k.sn + class_neri(c)) * sizeof(double) + 256.0;
-        share = std::max(share, (size_t)std::min(need, (double)(kScratchBytes / side_count(p))));
-    }
-    p->scratch_bytes = std::min(kScratchBytes, share * side_count(p));
+    p->scratch_bytes = contracted_scratch(p, streams);
     if ((e = plan_malloc(&p->d_setup, p->scratch_bytes)) != cudaSuccess) return cuda_status(e);
     return ensure_side_streams(p);
 }
@@ -695,7 +719,7 @@ eri_status_t prepare_contracted(eri_plan_s *p) {
 // side streams and events
 eri_status_t ensure_side_streams(eri_plan_s *p) {
     cudaError_t e = cudaSuccess;
-    for (int i = 0; e == cudaSuccess && i < side_count(p); ++i) {
+    for (int i = 0, n = stream_count(p); e == cudaSuccess && i < n; ++i) {
         if (!p->side[i]) e = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking);
         if (e == cudaSuccess && !p->join_ev[i])
             e = cudaEventCreateWithFlags(&p->join_ev[i], cudaEventDisableTiming);
@@ -731,17 +755,16 @@ bool needs_scratch(const eri_plan_s *p, bool compressed, bool tuned) {
 // fills the GPU by itself, and several at a time only spread the random reads of the pair table.
 eri_status_t fork_streams(eri_plan_s *p, cudaStream_t stream, bool scratch, int *n) {
     *n = 0;
-    int classes = 0;
-    for (int c = 0; c < kNumClassIds; ++c) classes += p->count[c] > 0;
-    if (classes < 2 || (!is_contracted(p) && p->nq >= (1LL << 25))) return ERI_OK;
-    if (!p->join_ev[side_count(p) - 1] || !p->fork_ev || (scratch && !p->d_setup)) {
+    const int most = stream_count(p);
+    if (most < 2 || (!is_contracted(p) && p->nq >= (1LL << 25))) return ERI_OK;
+    if (!p->join_ev[most - 1] || !p->fork_ev || (scratch && !p->d_setup)) {
         cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return ERI_OK;
         eri_status_t e = ensure_side_streams(p);
         if (e == ERI_OK && scratch) e = cuda_status(ensure_scratch(p));
         if (e != ERI_OK) return e;
     }
-    *n = std::min(classes, side_count(p));
+    *n = most;
     return ERI_OK;
 }
 

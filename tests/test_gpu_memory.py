@@ -46,3 +46,22 @@ def test_primitive_calls_without_scratch(precision, classes):
     left, plan = taken(call)
     assert left < 32 * MB
     plan.destroy()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_small_contracted_plan(precision):
+    """A contracted plan's scratch follows its classes: of these quartets of p and d shells, K = 2, a class
+    has at most 12, 192 primitive quartets of up to 1,296 outputs and 117 record values, 2.2 MB in FP64 on a
+    stream for each of 7 classes.  All of it is made with the plan."""
+    rng = np.random.default_rng(4)
+    pool = W.random_contracted_pool(rng, 2, K=2, Ls=(1, 2))
+    q = np.array([(i, j, k, l) for i in range(4) for j in range(i + 1) for k in range(i + 1) for l in range(k + 1)],
+                 dtype=np.int32)
+    assert max(np.unique(pool.L[q], axis=0, return_counts=True)[1]) == 12
+
+    left, plan = taken(lambda: api.eri_plan_create(pool, q, precision=precision))
+    assert left < 32 * MB
+    out = torch.empty(api.eri_output_bytes(plan, 0)[0] // 8, dtype=torch.float64, device="cuda")
+    more, _ = taken(lambda: api.eri_compute(plan, out))
+    assert more < 4 * MB
+    plan.destroy()
