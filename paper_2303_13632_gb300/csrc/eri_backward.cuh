@@ -48,6 +48,7 @@
 // from 50.4 ms.
 #pragma once
 
+#include "eri_bwd_table.h"
 #include "eri_kernels.cuh"
 
 namespace eri {
@@ -329,13 +330,10 @@ __device__ __forceinline__ void backward_units(const ShellsDev &sh, const Tables
                     R Wb[JL];
 #pragma unroll
                     for (int t = 0; t < JL; ++t) Wb[t] = (R)0;
-                    // components with value v along the axis: x: r = La - v fixed, y and z: r = v..La
-                    // (r = La - a_x; index r (r+1) / 2 + a_z)
                     for (int na = 0; na <= C::La - si; ++na) {
-                        const int ra = sx == 0 ? C::La - si : si + na, za = sx == 0 ? na : (sx == 1 ? ra - si : si);
+                        const int ca = axis_component(C::La, sx, si, na);
                         for (int nc = 0; nc <= C::Lc - sk; ++nc) {
-                            const int rc = sx == 0 ? C::Lc - sk : sk + nc, zc = sx == 0 ? nc : (sx == 1 ? rc - sk : sk);
-                            const R *p = Wu + ((ra * (ra + 1) / 2 + za) * C::NC + rc * (rc + 1) / 2 + zc) * JP;
+                            const R *p = Wu + (ca * C::NC + axis_component(C::Lc, sx, sk, nc)) * JP;
 #pragma unroll
                             for (int ch = 0; ch < C::NCH; ++ch, p += C::NA * C::NC * JP) {
                                 R v[JL];

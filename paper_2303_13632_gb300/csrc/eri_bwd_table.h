@@ -1,8 +1,11 @@
-// eri_bwd_table.h -- index table of the adjoint's contraction grouped by axis (plain C++17, evaluated
-// at compile time), written out entry by entry.  The adjoint kernel (eri_backward.cuh) forms the same
-// groups from its thread layout and reads no table; this header states them for the CPU test.
+// eri_bwd_table.h -- indices of the adjoint's contraction grouped by axis (plain C++17, no CUDA needed,
+// so that a CPU test reads the same code).
 //
-// The adjoint contracts G with the 2-D integrals axis by axis: for axis x and the x-components
+// axis_component is what the adjoint kernel (eri_backward.cuh) walks a group by: the components of one
+// shell with a given value along an axis.
+//
+// BwdTab writes the groups of whole quartets out entry by entry; no kernel reads it.  The adjoint
+// contracts G with the 2-D integrals axis by axis: for axis x and the x-components
 // w = (i0, i1, i2, i3) of the four centres, W = sum of G I_y I_z over the outputs sharing them
 // (y, z the axes after x in cyclic order).  The table lists, for each axis, the outputs group by
 // group: entries start[w] .. start[w + 1] - 1 of e[x * N ..] belong to w (groups in the order
@@ -15,7 +18,21 @@
 
 namespace eri {
 
+#ifdef __CUDACC__
+#define ERI_BWD_FN __host__ __device__
+#else
+#define ERI_BWD_FN
+#endif
+
 constexpr int bwd_ncart(int L) { return (L + 1) * (L + 2) / 2; }
+
+// Index, in output order, of the n-th of the L - v + 1 components with value v along axis x: a component
+// (a_x, a_y, a_z) has index r (r + 1) / 2 + a_z with r = L - a_x, so r = L - v is fixed for the first axis
+// and runs over v..L for the others.
+ERI_BWD_FN constexpr int axis_component(int L, int x, int v, int n) {
+    const int r = x == 0 ? L - v : v + n, z = x == 2 ? v : n;
+    return r * (r + 1) / 2 + z;
+}
 
 template <int A, int B, int Cc, int D>
 struct BwdTab {
