@@ -918,7 +918,7 @@ def run_gradient(args):
     for prec in ("mixed", "fp64"):
         t_roof = flops = 0.0
         for c in cls_list_:
-            f64, rr = perfmodel.adjoint_flops_per_quartet(c, prec)
+            f64, rr = perfmodel.adjoint_sum_flops(c, prec)
             if prec == "fp64":
                 f64, rr = f64 + rr, 0
             t_roof += prim_quartets * (f64 / (p64 * 1e12) + rr / (p32 * 1e12))

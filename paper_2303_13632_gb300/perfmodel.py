@@ -76,9 +76,30 @@ def flops_per_quartet(cls, precision: str = "fp64"):
     return f64, vrr + hrr + quad + comp + (60 * n - roots64) + (20 * n - bc64)
 
 
+def adjoint_sum_flops(cls, precision: str = "fp64"):
+    """(fp64_flops, rr_flops) of the adjoint (eri_backward) per primitive quartet of class cls, by sums
+    over the class's own 2-D integrals:
+      setup        40 + 20 n' + 60 n'  geometry, B and C, n' = floor((L + 2) / 2) + 1 roots: FP64, except
+                                       two thirds of the roots in the recurrence type on the mixed path
+      recurrences  15 per root and tuple w = (i0, i1, i2, i3) of components along an axis: three axes, a
+                   product and two FMAs each                                              (R)
+      blocks       8 per root and output: W = sum G I_y I_z along the three axes          (R)
+      gathering    1 per root, axis, (a, c) pair and (i1, i3): the blocks of one (i0, i2) (R)
+      sums         30 per root, axis and w: W times I and its lowered forms, eight sums   (R)
+      derivatives  68 per root, axis and (i0, i2): the raised integrals of four centres   (R)"""
+    La, Lb, Lc, Ld = canonical(cls)
+    n = (La + Lb + Lc + Ld + 2) // 2 + 1
+    neri = ncart(La) * ncart(Lb) * ncart(Lc) * ncart(Ld)
+    wn = (La + 1) * (Lb + 1) * (Lc + 1) * (Ld + 1)
+    roots64 = 60 * n if precision == "fp64" else 20 * n
+    rr = (15 * n * wn + 8 * n * neri + 3 * n * ncart(La) * ncart(Lc) * (Lb + 1) * (Ld + 1) + 90 * n * wn
+          + 3 * 68 * n * (La + 1) * (Lc + 1))
+    return 40 + 20 * n + roots64, rr + (60 * n - roots64)
+
+
 def adjoint_flops_per_quartet(cls, precision: str = "fp64"):
-    """(fp64_flops, rr_flops) of the adjoint (eri_backward) per primitive quartet of class cls,
-    counted like flops_per_quartet:
+    """(fp64_flops, rr_flops) per primitive quartet of class cls of an adjoint on 2-D integrals extended
+    by two (the kernels form the sums of adjoint_sum_flops instead), counted like flops_per_quartet:
       setup       40 + 20 n' + 60 n'   geometry, B and C, roots on the extended class (every L + 2,
                                        n' = floor((L + 2) / 2) + 1 roots): FP64, except two thirds
                                        of the roots (40 n') in the recurrence type on the mixed
