@@ -1466,7 +1466,7 @@ rows_kernel(ClassArgs args) {
             // eps normal: |x| <= M (1 + 3 2^-24), so up to 22 bits no code exceeds M.  A subnormal eps is
             // rounded by more than that (and its reciprocal can overflow): it takes the checked form, as
             // non-finite values do
-            if (bits > 22 || !(eps >= 1.17549435e-38f && eps <= 3.4028234663852886e38f)) {
+            if (bits > 22 || !(eps <= 3.4028234663852886e38f && inv <= 8.507059173023462e37f)) {  // 2^126
                 outputs([&](float v, unsigned char *e) {
                     float r = roundf(v * inv);
                     r = r > M ? M : (r < -M ? -M : r);
