@@ -40,10 +40,10 @@
 // threads up, the second from the high ones down, I in two buffers): two barriers per QG units.
 // Bound by barriers between short steps and issue in FP32 (two CTAs per SM, 35% of the issue slots),
 // by the FP64 pipe in FP64.  Measured on the 16 classes of p and d shells, K = 3, forward and backward:
-// 1024 quartets per class in mixed precision 115 -> 14.0 ms, 384 in FP64 220 -> 46.9 ms.  In FP32 the
+// 1024 quartets per class in mixed precision 115 -> 13.3 ms, 384 in FP64 220 -> 47.3 ms.  In FP32 the
 // pairs cost 0.9 ms over compensated sums rounded to one number before the lanes are summed, and FP64
 // registers in their place 3.1 ms for the same results; relative error of both gradients against 64 bits
-// 6.4e-8 with them, 1.2e-7 without, 8.5e-8 with FP32 sums per primitive quartet and FP64 beyond.  36
+// 5.8e-8 with them, 1.2e-7 without, 8.5e-8 with FP32 sums per primitive quartet and FP64 beyond.  36
 // instead of 18 G values per thread in FP64 (one pass over the roots of [dd|dd], no b-chunks) took that
 // from 50.4 ms.
 #pragma once

@@ -4,7 +4,8 @@
 // from one to over a thousand of them, uneven within a class.  Walking them one after the other in
 // the CTA that owns the quartet leaves the GPU to the longest quartet and the few threads of each
 // phase; here every primitive quartet is a unit of its own, as in a primitive plan:
-//   unit_setup_kernel   one thread per unit: geometry, roots and weights, B and C (FP64)
+//   unit_setup_kernel   one thread per unit: geometry; then one per (unit, root): root and weight, B and
+//                       C (FP64)
 //   class kernel        the class's recurrence and quadrature kernel over the units' records
 //   contract_kernel     one thread per (quartet, output): the sum over the quartet's units, in
 //                       order, so that the FP32 Kahan sums are those of a sequential loop
@@ -14,10 +15,11 @@
 // fill the scratch; a quartet may be cut, its partial sums are carried to the next span.
 //
 // Measured against the primitive loop inside the class kernel: a diatomic's 3,081 unique quartets
-// (s, s, p, p, d, f per atom, K up to 6, FP64) 501 -> 5.4 ms; 70,000 quartets of a 40-atom molecule
-// (K up to 6, FP32, 16-bit codes) 300 -> 10.3 ms, same codes bit for bit.  The sums are bound by the
-// latency of a long quartet's chain: with 32 values of a chain in flight instead of 8 those two
-// fell from 7.1 and 11.6 ms.
+// (s, s, p, p, d, f per atom, K up to 6, FP64) 501 -> 3.2 ms; 70,000 quartets of a 40-atom molecule
+// (K up to 6, FP32, 16-bit codes) 300 -> 8.6 ms, same codes bit for bit.  The sums are bound by the
+// latency of a long quartet's chain: kBatch values of it are added while the next kBatch are loaded
+// (with 32 values in flight instead of 8, before the setup ran by (unit, root), those two fell from 7.1
+// and 11.6 to 5.4 and 10.3 ms).
 #include <algorithm>
 #include <type_traits>
 

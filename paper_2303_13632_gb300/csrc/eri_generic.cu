@@ -73,7 +73,7 @@ __device__ __forceinline__ int div_by(int n, unsigned m) { return m ? (int)__umu
 // plane, on idle lanes too, and the FP64 pipe is what bounds it.  One thread per (unit, root, axis) issues
 // fewer but has their whole chain, so it takes the classes with few planes and the batches that fill a warp.
 //   369 classes in FP64, 2^15 / 2^20 / 2^22 ERIs each: 1.11 / 26.2 / 103.9 ms before these three rules,
-// 0.64 / 15.1 / 59.3 with them; one class at a time (the canonical ones) 23.0 -> 14.4 ms at 2^22.
+// 0.64 / 15.2 / 59.5 with them; one class at a time (the canonical ones) 23.0 -> 13.9 ms at 2^22.
 template <typename R>
 GenShape gen_shape(const int L[4], bool contracted, int q_most = kGenQmax) {
     GenShape g{};

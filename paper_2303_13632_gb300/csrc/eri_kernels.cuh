@@ -83,10 +83,11 @@ __host__ __device__ constexpr int pow2ceil(int n) { return n <= 1 ? 1 : 2 * pow2
 
 // (j, l) blocks of 2-D integrals in shared memory, moved as vectors: V values per access (16 bytes
 // where the block is long enough), P values from one block (i, k) to the next k, ROW from one i to
-// the next.  Both are an odd number of vectors, so that the vectors of a quarter warp (the rows that
-// rows_direct stores, the blocks that the quadrature loads) fall into distinct banks: with scalar
-// stores and rows of a multiple of 32 values, [fd|fd] spent 48 of 110 million shared-memory
-// wavefronts on store conflicts.
+// the next.  Both are an odd number of vectors, so that the rows of a (root, axis) and the blocks of a
+// row start in distinct banks: with scalar stores and rows of a multiple of 32 values, [fd|fd] spent 48
+// of 110 million shared-memory wavefronts on store conflicts.  The strides from one (root, axis) to the
+// next are not odd (52 and 312 vectors in [fd|fd]), so rows that a quarter warp stores for several of them
+// still meet: counted over the layout 576 wavefronts per tile where 216 would do, 540 for 270 in [fd|dd].
 template <int JL, int NK, int BYTES>
 struct JBlock {
     static constexpr int V = JL == 1 ? 1 : (BYTES == 8 || JL == 2 ? 2 : 4);

@@ -779,10 +779,10 @@ double class_work(const eri_plan_s *p, int c) {
 }
 
 // Whether a call over all classes runs those with a g shell in sets: up to 10^8 primitive ERIs of them.
-// A set's CTAs have the shared memory of its highest class (two per SM), those of a class its own (up to
-// four), which tells once the classes fill the GPU by themselves.  The 369 classes, mixed, 16 bits,
-// a launch per class / in sets: 2^15 ERIs per class 3.24 / 0.42 ms, 2^20 9.6 / 11.8 ms; sets take
-// 1.53 ms at 2^17, in proportion from there on, and the other form is never below its 3.2 ms of launches.
+// A set's CTAs have the shared memory of its highest class, those of a class its own, which tells once the
+// classes fill the GPU by themselves.  The 369 classes, a launch per class / in sets: mixed with 16-bit
+// codes 1.88 / 0.45 ms at 2^15 ERIs per class, 3.90 / 2.53 at 2^18 (9.7e7 in all), 9.78 / 9.89 at 2^20; FP64
+// 1.82 / 0.63, 4.71 / 4.25 and 15.2 / 16.8, so that from 2^19 on (7.78 / 8.43) it loses.
 bool g_in_sets(const eri_plan_s *p) {
     double work = 0;
     for (int c = 256; c < kNumClassIds; ++c) work += class_work(p, c);
